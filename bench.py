@@ -490,15 +490,15 @@ def canny_run(torch, pipe, stream, bufs, steps, hbm_peak, want_cpu):
            "parity": "batched == plain bit for bit in this run; bit-exact with the oracle (tests/test_gpu_canny.py)"}
     out["hbm"]["frac"] = out["hbm"]["achieved"] / hbm_peak
     nms_ms = kern.get("canny_nms", 0.0)
-    if nms_ms > 0:  # the stencil pass alone: the planes read once, strong and candidate planes written
-        gbs = 3.0 * px / (nms_ms / 1000.0) / 1e9
+    if nms_ms > 0:  # the stencil pass alone: the planes read once, strong and candidate bit planes written
+        gbs = 1.25 * px / (nms_ms / 1000.0) / 1e9
         out["nms_kernel"] = {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
-                             "alg_bytes_per_px": 3}
+                             "alg_bytes_per_px": 1.25}
     cnt_ms = kern.get("canny_counts", 0.0)
     if cnt_ms > 0:  # the counts pass alone: edges and labels read once
         gbs = 5.0 * px / (cnt_ms / 1000.0) / 1e9
         out["counts_kernel"] = {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
-                                "alg_bytes_per_px": 5}
+                                "alg_bytes_per_px": 3.25}
     if want_cpu:
         import time
         import oracle
@@ -567,8 +567,8 @@ def rbc_run(torch, pipe, stream, steps, hbm_peak, want_cpu):
                    "alg_bytes_per_px": RBC_BYTES_PER_PX, "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"},
            "parity": "tile 0 equals the oracle bit for bit in this run; tests/test_gpu_rbc.py"}
     pl = kern.get("rbc_planes")
-    if pl:   # the planes pass alone: RGB read, marker and mask written
-        g = 5.0 * H * W / (pl / 1000.0) / 1e9
+    if pl:   # the planes pass alone: RGB read, marker and mask bits written
+        g = 3.25 * H * W / (pl / 1000.0) / 1e9
         out["planes_kernel"] = {"achieved": g, "peak": hbm_peak, "unit": "GB/s", "frac": g / hbm_peak,
                                 "alg_bytes_per_px": 5}
     if want_cpu:

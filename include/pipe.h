@@ -240,9 +240,9 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
  *  rgb_dev: H rows of 3*W bytes (R,G,B) at pitch_bytes >= 3*W; out_dev: a
  *  W x H uint8 plane, caller-owned, not overlapping the input;
  *  0 <= t_lo <= t_hi <= 255 (the workload uses 40 and 100).  The pipe owns
- *  the scratch (a W x H mask plane, one seed flag per 64x64 work tile and a
- *  work queue), allocated on the first call of a larger size, which
- *  synchronises `stream`.
+ *  the scratch (marker and mask as bit planes and a queue of 64x64 work
+ *  tiles, shared with the Canny calls), allocated on the first call of a
+ *  larger size, which synchronises `stream`.
  * Returns PIPE_EINVAL on a bad argument (nothing is launched); otherwise
  * the work is asynchronous on `stream`. */
 int rbc_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes, int t_lo, int t_hi,
@@ -269,10 +269,10 @@ int rbc_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
  *  img_dev, edges_dev: W x H uint8 planes, caller-owned, not overlapping;
  *  labels_dev: W x H int32 (may be NULL when n_objects = 0); counts_dev:
  *  n_objects int32.  0 <= low <= high; 0 <= radius <= 4.  The hysteresis
- *  runs the segmentation's reconstruction kernel, started from the 64x64
- *  work tiles that hold a strong pixel, on pipe-owned scratch (a W x H
- *  candidate plane, one seed flag per work tile and a work queue), allocated
- *  on the first call of a larger size, which synchronises `stream`.
+ *  grows the strong pixels through the candidates from the 64x64 work tiles
+ *  that hold one, on pipe-owned scratch (both as bit planes and a work
+ *  queue), allocated on the first call of a larger size, which synchronises
+ *  `stream`.
  * Returns PIPE_EINVAL on a bad argument (nothing is launched); otherwise
  * the work is asynchronous on `stream`. */
 int canny_tile(pipe_t p, const uint8_t* img_dev, const int32_t* labels_dev, int W, int H, int n_objects, int low,
@@ -280,16 +280,15 @@ int canny_tile(pipe_t p, const uint8_t* img_dev, const int32_t* labels_dev, int 
 
 /* Batched form of canny_tile: the edges and edge counts of n tiles of any
  * sizes in one launch per pass (one suppression launch over all tiles, one
- * reconstruction queue for every tile's hysteresis, one counts launch), so
+ * queue for every tile's hysteresis, one counts launch), so
  * that many tiles share the GPU.  Results are identical to canny_tile on
  * each tile alone.
  *  tiles[i]: img (W x H uint8), edges (W x H uint8, not overlapping img),
  *    labels (W x H int32; may be NULL when n_objects = 0), n_objects (host
  *    int), counts (n_objects int32); 1 <= n <= 4096; low, high, radius as
- *    for canny_tile.  The pipe's scratch covers all tiles at once (a
- *    candidate byte per pixel, a seed flag per work tile, the queue),
- *    allocated on the first call of a larger size, which synchronises
- *    `stream`.
+ *    for canny_tile.  The pipe's scratch covers all tiles at once (the bit
+ *    planes and the queue), allocated on the first call of a larger size,
+ *    which synchronises `stream`.
  * Returns PIPE_EINVAL on a bad argument (nothing is launched); otherwise
  * the work is asynchronous on `stream`. */
 typedef struct {

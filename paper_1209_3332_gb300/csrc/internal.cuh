@@ -70,7 +70,6 @@ struct Shared {
     int processed;                      // tile processings (diagnostic)
     int nobj;                           // object items of a batched feature pass
     int next_obj;                       // the batched feature pass draws its objects from this counter
-    int nseed;                          // work tiles of a seeded reconstruction queued at the start
 };
 
 struct Launch {
@@ -162,39 +161,6 @@ void upload_deconv_tables(const int32_t* lut256, const int32_t* wq3);
 void launch_deconv(const Launch& L, cudaStream_t s, Profiler* pf);
 int recon_grid(int device);
 void launch_recon(const Launch& L, int grid_cap, cudaStream_t s, Profiler* pf);
-// The reconstruction started from a sparse marker: only the work tiles whose
-// flag is set (a marker pixel in the tile or its one-pixel halo) are queued
-// at the start; the others are at a fixed point and wait to be requested.
-// flags: one int per work tile of the launch, set by the kernel that wrote the
-// marker and zeroed by the caller before it; L.sh->nseed must be zeroed too.
-void launch_recon_seeded(const Launch& L, const int* flags, int grid_cap, cudaStream_t s, Profiler* pf);
-
-// Sets the seed flags of a 16-pixel chunk at (x0, y) of an image with rtx x
-// rty work tiles (x0 a multiple of 16, so the chunk lies in one work tile):
-// the tile holding it, and the neighbours whose one-pixel halo holds one of
-// its marker pixels (bit p of m: pixel x0 + p is a marker pixel).
-// The work tiles (RT x RT, rtx x rty of them) whose tile or one-pixel halo
-// holds pixel (x, y), as bits of a 3 x 3 neighbourhood: bit (dy + 1) * 3 +
-// (dx + 1) for the tile at offset (dx, dy) from the pixel's own.
-__device__ __forceinline__ unsigned seed_bits_px(int rtx, int rty, int x, int y) {
-    const int tx = x / RT, ty = y / RT, xr = x - tx * RT, yr = y - ty * RT;
-    const int dxl = (xr == 0 && tx > 0) ? -1 : 0, dxh = (xr == RT - 1 && tx + 1 < rtx) ? 1 : 0;
-    const int dyl = (yr == 0 && ty > 0) ? -1 : 0, dyh = (yr == RT - 1 && ty + 1 < rty) ? 1 : 0;
-    unsigned m = 0;
-    for (int dy = dyl; dy <= dyh; dy++)
-        for (int dx = dxl; dx <= dxh; dx++) m |= 1u << ((dy + 1) * 3 + dx + 1);
-    return m;
-}
-
-__device__ __forceinline__ void flag_seed_tiles(int* flags, int rtx, int rty, int x0, int y, unsigned m) {
-    if (!m) return;
-    const int tx = x0 / RT, ty = y / RT, yr = y - ty * RT;
-    const int ylo = (yr == 0 && ty > 0) ? ty - 1 : ty, yhi = (yr == RT - 1 && ty + 1 < rty) ? ty + 1 : ty;
-    const int xlo = ((x0 & (RT - 1)) == 0 && (m & 1u) && tx > 0) ? tx - 1 : tx;
-    const int xhi = (((x0 + 15) & (RT - 1)) == RT - 1 && (m & 0x8000u) && tx + 1 < rtx) ? tx + 1 : tx;
-    for (int yy = ylo; yy <= yhi; yy++)
-        for (int xx = xlo; xx <= xhi; xx++) flags[yy * rtx + xx] = 1;
-}
 void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cudaStream_t s, Profiler* pf);
 size_t edt_rows_smem(int RB, int Wmax);
 void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf);
@@ -207,33 +173,75 @@ void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, in
 void launch_features_batched(const Launch& L, int grid, cudaStream_t s, Profiler* pf);
 // per object 1..K of a label plane: its box (xmin, ymin, xmax, ymax); empty (xmax < xmin) if absent
 void launch_object_boxes(const int32_t* labels, int W, int H, int K, int4* bbox, cudaStream_t s, Profiler* pf);
-// One tile of a Canny launch (plain: one tile; batched: many).
+// One tile of a Canny launch (plain: one tile; batched: many), or of another
+// growth of a binary marker through a binary mask.
 struct CannyDesc {
     const uint8_t* img;      // W x H plane
     const int32_t* labels;   // W x H labels (may be null when K == 0)
-    uint8_t* edges;          // strong pixels (0/1), grown into the edge map by the hysteresis
-    uint8_t* cand;           // candidates (0/1): the hysteresis mask
+    uint8_t* edges;          // the grown marker as bytes (0/1)
     int32_t* counts;         // K edge counts
     int W, H, K;
     int bx;                  // 32-pixel blocks per row
     int blk_base;            // first 32x32 block of this tile in the counts launch
     int nms_base;            // first warp of this tile in the suppression launch
-    int rt_base;             // first work tile of this tile in the reconstruction launch
+    int rt_base;             // first work tile of this tile
 };
-// Blocks of a tile in the Canny launches (32 x 32 pixels each).
+// The descriptors of a launch: up to NEAR travel in the launch parameters,
+// more are in device memory.
+struct CannyTab {
+    static constexpr int NEAR = 8;
+    int n;
+    const CannyDesc* far;
+    CannyDesc near[NEAR];
+    __device__ __forceinline__ const CannyDesc& operator[](int i) const { return n <= NEAR ? near[i] : far[i]; }
+    // the tile of launch item b, by the tiles' first items
+    __device__ __forceinline__ int find(int b, int CannyDesc::*base) const {
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((*this)[mid].*base <= b) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+};
+CannyTab make_canny_tab(const std::vector<CannyDesc>& v, CannyDesc* far, cudaStream_t s);
+// Growth of a marker through a mask (k_grow.cu): bit planes of 64 64-bit words
+// per work tile, and the state of its queue.
+struct GrowShared {  // the words that every worker's atomics meet at, in lines of their own
+    unsigned long long tp;          // tail << 32 | groups not finished and tiles queued or running
+    int err;                        // first device-side error
+    alignas(256) int head;          // queue head
+    alignas(256) int next;          // next group of tiles
+};
+struct GrowLaunch {
+    CannyTab tab;
+    unsigned long long *mask, *marker;  // the marker grows in place
+    unsigned long long* slots;          // [n_rt], zeroed before the launches
+    int* state;                         // [n_rt], zeroed
+    uint8_t* any;                       // [n_rt] the work tile holds a marker pixel
+    GrowShared* sh;
+    int n_rt;
+    int group;                          // work tiles drawn at a time at the start, 1 to 32
+    long long wait_budget;
+};
+// by one thread of the kernel that writes the planes
+__device__ __forceinline__ void grow_reset(const GrowLaunch& G) {
+    G.sh->tp = (unsigned long long)((G.n_rt + G.group - 1) / G.group);
+    G.sh->head = G.sh->err = G.sh->next = 0;
+}
+int grow_grid(int device);
+int grow_group(int n_rt);  // GrowLaunch::group for a launch of n_rt work tiles
+// grows the marker and writes it to every tile's edges as bytes
+void launch_grow(const GrowLaunch& G, int grid_cap, cudaStream_t s, Profiler* pf);
+// Blocks (32 x 32 pixels) and suppression warps of a tile in the Canny launches.
 int canny_blocks(int W, int H);
 int canny_nms_warps(int W, int H);
-void upload_canny_descs(CannyDesc* dst, const std::vector<CannyDesc>& v, cudaStream_t s);
-// descs: host copy; d_descs: device array of the same length.  Zeroes the
-// counts, writes strong pixels into edges and candidates into cand, and sets
-// the seed flags (indexed by rt_base + work tile) of the work tiles the
-// strong pixels touch.
-void launch_canny_nms(const std::vector<CannyDesc>& descs, CannyDesc* d_descs, int low, int high, int* flags,
-                      cudaStream_t s, Profiler* pf);
+// Zeroes the counts; writes the strong pixels into the marker and the
+// candidates into the mask.
+void launch_canny_nms(const GrowLaunch& G, int warps, int low, int high, cudaStream_t s, Profiler* pf);
 // Edge counts of every tile: each edge pixel adds one to every object 1..K
 // with a pixel within its disk of radius r (the disk dilation of the object).
-void launch_canny_counts(const std::vector<CannyDesc>& descs, CannyDesc* d_descs, int r, cudaStream_t s,
-                         Profiler* pf);
+void launch_canny_counts(const GrowLaunch& G, int blocks, int r, cudaStream_t s, Profiler* pf);
 // One tile of a batched watershed split.
 struct WsDesc {
     const int32_t* labels;
@@ -258,11 +266,9 @@ size_t watershed_scratch_bytes(int W, int H);
 void launch_watershed(const int32_t* labels, const int32_t* edt, int W, int H, int K, int h, int32_t* out,
                       int32_t* n_basins, int4* bbox, int* cnt, int* next, void* scratch, int* status, int sms,
                       cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Profiler* pf);
-// RBC detection planes: d = R - max(G, B); marker (0/1) = d >= t_hi into
-// marker, mask (0/1) = d >= t_lo into mask, and the seed flags of the work
-// tiles (RT x RT) that the marker pixels touch.
-void launch_rbc_planes(const uint8_t* rgb, size_t pitch, int W, int H, int t_lo, int t_hi, uint8_t* marker,
-                       uint8_t* mask, int* flags, cudaStream_t s, Profiler* pf);
+// RBC detection planes: d = R - max(G, B); marker = d >= t_hi, mask = d >= t_lo.
+void launch_rbc_planes(const GrowLaunch& G, const uint8_t* rgb, size_t pitch, int t_lo, int t_hi, cudaStream_t s,
+                       Profiler* pf);
 void launch_unpack_bits(const uint32_t* bits, int W, int H, int cbx, uint8_t* out, cudaStream_t s,
                         Profiler* pf);
 

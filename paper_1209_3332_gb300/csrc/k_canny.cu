@@ -11,38 +11,26 @@
 //   p survives iff m(p) > m(a) and m(p) >= m(b); candidate iff it survives
 //     with m > low, strong iff it survives with m > high;
 //   edges = candidates 8-connected through candidates to a strong pixel.
-// Every kernel takes an array of tile descriptors, so one launch covers any
-// number of tiles (the plain form is the batched form of one tile), a CTA
-// finding its tile by binary search over the tiles' first blocks.
+// Every kernel takes a table of tile descriptors, so one launch covers any
+// number of tiles (the plain form is the batched form of one tile), a warp
+// finding its tile by binary search over the tiles' first items.
 // k_canny_nms writes the strong pixels (the marker) and the candidates (the
-// mask) as 0/1 planes from one 32x32 block per CTA staged with a 2-px halo,
-// and flags the 64x64 work tiles the strong pixels touch; the hysteresis is
-// then the reconstruction by dilation of the marker under the mask, run by
-// the reconstruction kernel of the segmentation from the flagged work tiles
-// only.  The counts are a stencil pass over the same blocks: each edge pixel
-// adds one to every object with a pixel within its disk -- the same count
-// as the edge pixels within each object's disk dilation, with the labels
-// and edges read once, coalesced.
+// mask) as bit planes, 64x64 work tile by work tile; the hysteresis is the
+// growth of the marker through the mask (k_grow.cu), which also writes the
+// edge map as bytes.  The counts are a stencil pass over 32x32 blocks: each
+// edge pixel adds one to every object with a pixel within its disk -- the
+// same count as the edge pixels within each object's disk dilation, with the
+// labels read only around edges.
 #include "internal.cuh"
 
 namespace nucseg {
 
 constexpr int CT = 32;                 // block of the counts pass: CT x CT pixels
-
-// the tile of launch item b, by binary search over the tiles' first items
-__device__ __forceinline__ int find_desc(const CannyDesc* __restrict__ D, int n, int b, int CannyDesc::*base) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (D[mid].*base <= b) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
+typedef unsigned long long u64;
 
 // ---- suppression: one warp streams a strip of 128 columns (4 per lane) down
-// a segment of 64 rows (one work-tile row), keeping the last three image rows,
-// the magnitudes of the last three rows and the Sobel pair of the current row
-// in registers ------------------------------------------------------------------
+// a segment of 64 rows (one work-tile row), keeping four image rows and the
+// magnitudes of three in registers ---------------------------------------------------
 constexpr int NS_COLS = 128, NS_ROWS = 64;
 constexpr int NS_WARPS = 4;          // warps per CTA
 
@@ -97,11 +85,6 @@ __device__ __forceinline__ Row8 ns_load_row(const uint8_t* __restrict__ I, int W
     return ns_row(ns_fetch(I, W, H, y, cx0, vec, lane), lane);
 }
 
-struct Sob6 {                        // columns cx0 - 1 .. cx0 + 4 of one row (index j = column - cx0 + 1)
-    int m[6];                        // L1 magnitude, 0 off the image
-    int ax[4], ay[4], same[4];       // |gx|, |gy| and whether gx, gy have one sign, columns cx0 .. cx0 + 3
-};
-
 __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -118,50 +101,61 @@ __device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
 // vs = A + 2B + C and vd = C - A per column, gx(c) = vs(c+1) - vs(c-1) and
 // gy(c) = vd(c-1) + 2 vd(c) + vd(c+1).  Signed values carry a bias (256 on
 // vd, 1024 on gx and gy) so that every lane stays in [0, 2^16) and packed
-// adds never borrow across lanes.  colmask: per pair, 0xffff on the lanes of
-// columns inside the image; m is 0 elsewhere and on a row off the image.
-__device__ __forceinline__ Sob6 ns_sobel(const Row8& A, const Row8& B, const Row8& C, const uint32_t colmask[3],
-                                         bool row_in) {
-    constexpr uint32_t B256 = 0x01000100u, B1024 = 0x04000400u;
+// adds never borrow across lanes.
+constexpr uint32_t B256 = 0x01000100u, B1024 = 0x04000400u;
+struct Grad {
+    uint32_t x[3], y[3];  // gx + 1024, gy + 1024
+};
+__device__ __forceinline__ Grad ns_grad(const Row8& A, const Row8& B, const Row8& C) {
     uint32_t V[4], Dv[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         V[k] = A.p[k] + (B.p[k] << 1) + C.p[k];
         Dv[k] = C.p[k] + B256 - A.p[k];
     }
-    const uint32_t rm = row_in ? 0xffffffffu : 0u;
-    uint32_t SX[3], SY[3], AX[3], AY[3];
+    Grad g;
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        SX[k] = V[k + 1] + B1024 - V[k];
-        SY[k] = Dv[k] + (__byte_perm(Dv[k], Dv[k + 1], 0x5432) << 1) + Dv[k + 1];
-        AX[k] = max2(SX[k], B1024) - min2(SX[k], B1024);
-        AY[k] = max2(SY[k], B1024) - min2(SY[k], B1024);
+        g.x[k] = V[k + 1] + B1024 - V[k];
+        g.y[k] = Dv[k] + (__byte_perm(Dv[k], Dv[k + 1], 0x5432) << 1) + Dv[k + 1];
     }
-    Sob6 o;
+    return g;
+}
+__device__ __forceinline__ uint32_t abs2(uint32_t biased) { return max2(biased, B1024) - min2(biased, B1024); }
+
+// L1 magnitudes of the three column pairs.  colmask: per pair, 0xffff on the
+// lanes of columns inside the image; m is 0 elsewhere and on a row off the image.
+struct Mag {
+    uint32_t m[3];
+    __device__ __forceinline__ int at(int j) const { return (int)((m[j >> 1] >> (16 * (j & 1))) & 0xffffu); }
+};
+__device__ __forceinline__ Mag ns_mag(const Grad& g, const uint32_t colmask[3], bool row_in) {
+    Mag o;
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const uint32_t M = (AX[k] + AY[k]) & colmask[k] & rm;
-        o.m[2 * k] = (int)(M & 0xffffu);
-        o.m[2 * k + 1] = (int)(M >> 16);
-    }
-    // columns 0..3 are the high lane of pair 0, both lanes of pair 1, the low lane of pair 2
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        const int k = (c + 1) >> 1, sh = (c & 1) ? 0 : 16;
-        o.ax[c] = (int)((AX[k] >> sh) & 0xffffu);
-        o.ay[c] = (int)((AY[k] >> sh) & 0xffffu);
-        o.same[c] = (((SX[k] >> sh) & 0xffffu) > 1024u) == (((SY[k] >> sh) & 0xffffu) > 1024u);
-    }
+    for (int k = 0; k < 3; k++) o.m[k] = row_in ? (abs2(g.x[k]) + abs2(g.y[k])) & colmask[k] : 0u;
     return o;
 }
 
-__global__ void __launch_bounds__(32 * NS_WARPS, 4) k_canny_nms(const CannyDesc* __restrict__ D, int n, int n_warps,
-                                                            int low, int high, int* __restrict__ flags) {
-    const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * NS_WARPS + (threadIdx.x >> 5);
+// floor(v tan 22.5 deg) for 0 <= v <= 1020, where it equals (v * 27146) >> 16
+// (tan 22.5 deg is irrational, so a <= tan22(b) is a < b tan 22.5 deg for b > 0)
+__device__ __forceinline__ int tan22(int v) { return (v * 27146) >> 16; }
+
+// One warp per strip of 128 columns (two work tiles) and 64 rows (one work
+// tile).  Magnitudes are computed for every pixel; the suppression itself
+// runs only on rows where some lane has a magnitude above low, which leaves
+// out about half of the rows on the benchmark tile (8 planes of 4096^2: 290 us,
+// 502 with the suppression of every pixel and byte planes; rows fetched two
+// ahead instead of one: no change).  Bound: instruction issue (1 B read and
+// 1/4 B written per pixel, 25 us).  The strip's marker and mask bits are
+// gathered in shared memory, four columns per lane and row.
+__global__ void __launch_bounds__(32 * NS_WARPS, 6) k_canny_nms(const __grid_constant__ GrowLaunch G, int n_warps,
+                                                                int low, int high) {
+    __shared__ __align__(16) uint8_t bits[NS_WARPS][2][NS_ROWS][NS_COLS / 8];  // marker, mask
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gw = blockIdx.x * NS_WARPS + warp;
+    if (blockIdx.x == 0 && threadIdx.x == 0) grow_reset(G);
     if (gw >= n_warps) return;
-    const CannyDesc& d = D[find_desc(D, n, gw, &CannyDesc::nms_base)];
+    const CannyDesc& d = G.tab[G.tab.find(gw, &CannyDesc::nms_base)];
     const uint8_t* __restrict__ I = d.img;
     const int W = d.W, H = d.H, wi = gw - d.nms_base;
     const int strips = (W + NS_COLS - 1) / NS_COLS, nw = strips * ((H + NS_ROWS - 1) / NS_ROWS);
@@ -169,172 +163,187 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 4) k_canny_nms(const CannyDesc*
     const int cx0 = strip * NS_COLS + 4 * lane, ya = seg * NS_ROWS, yb = min(ya + NS_ROWS, H);
     // this warp's share of the counts to zero
     for (long long i = (long long)wi * 32 + lane; i < d.K; i += (long long)nw * 32) d.counts[i] = 0;
+#pragma unroll
+    for (int i = 0; i < 2 * NS_ROWS * NS_COLS / 8 / (32 * 16); i++)
+        reinterpret_cast<uint4*>(&bits[warp][0][0][0])[i * 32 + lane] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
     const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(I) & 3) == 0;
-    const bool out_vec = vec && (reinterpret_cast<uintptr_t>(d.edges) & 3) == 0 &&
-                         (reinterpret_cast<uintptr_t>(d.cand) & 3) == 0;
     uint32_t colmask[3];  // pair k holds columns cx0 + 2k - 1 and cx0 + 2k
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         const int x = cx0 + 2 * k - 1;
         colmask[k] = ((x >= 0 && x < W) ? 0xffffu : 0u) | ((x + 1 >= 0 && x + 1 < W) ? 0xffff0000u : 0u);
     }
+    const uint32_t low2 = (uint32_t)min(low, 0xffff) * 0x00010001u;
     Row8 P = ns_load_row(I, W, H, ya - 1, cx0, vec, lane);
     Row8 Q = ns_load_row(I, W, H, ya, cx0, vec, lane);
-    Sob6 prev = ns_sobel(ns_load_row(I, W, H, ya - 2, cx0, vec, lane), P, Q, colmask, ya - 1 >= 0);
-    Sob6 cur = ns_sobel(P, Q, ns_load_row(I, W, H, ya + 1, cx0, vec, lane), colmask, true);
-    P = Q;
-    Q = ns_load_row(I, W, H, ya + 1, cx0, vec, lane);
-    const int rtx = (W + RT - 1) / RT, rty = (H + RT - 1) / RT;
-    unsigned seed = 0u;
+    Row8 N = ns_load_row(I, W, H, ya + 1, cx0, vec, lane);
+    Mag prev = ns_mag(ns_grad(ns_load_row(I, W, H, ya - 2, cx0, vec, lane), P, Q), colmask, ya - 1 >= 0);
+    Mag cur = ns_mag(ns_grad(P, Q, N), colmask, true);
     RowFetch fn = ns_fetch(I, W, H, ya + 2, cx0, vec, lane);  // one row ahead of its use
 #pragma unroll 1
     for (int y = ya; y < yb; y++) {
-        const Row8 N = ns_row(fn, lane);
+        const Row8 M = ns_row(fn, lane);  // rows P, Q, N, M: y - 1 .. y + 2
         fn = ns_fetch(I, W, H, y + 3, cx0, vec, lane);
-        const Sob6 next = ns_sobel(P, Q, N, colmask, y + 1 < H);
-        uint32_t ws = 0, wc = 0;
+        const Mag next = ns_mag(ns_grad(Q, N, M), colmask, y + 1 < H);
+        // columns cx0 .. cx0 + 3 are the high lane of pair 0, pair 1, the low lane of pair 2
+        const uint32_t top = max2(max2(cur.m[0] >> 16, cur.m[1]), cur.m[2] & 0xffffu);
+        if (__any_sync(0xffffffffu, max2(top, low2) != low2)) {
+            const Grad g = ns_grad(P, Q, N);
+            unsigned v = 0;  // bits 0-3: strong, 4-7: candidates
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const int j = c + 1;
-            const int ax = cur.ax[c], ay = cur.ay[c], m = cur.m[j];
-            int ma, mb;
-            if ((ax + ay) * (ax + ay) < 2 * ax * ax) {                  // horizontal
-                ma = cur.m[j - 1]; mb = cur.m[j + 1];
-            } else if (ay > ax && (ay - ax) * (ay - ax) > 2 * ax * ax) {  // vertical
-                ma = prev.m[j]; mb = next.m[j];
-            } else if (cur.same[c]) {                                   // along (+x, +y)
-                ma = prev.m[j - 1]; mb = next.m[j + 1];
-            } else {                                                    // along (+x, -y)
-                ma = prev.m[j + 1]; mb = next.m[j - 1];
+            for (int c = 0; c < 4; c++) {
+                const int j = c + 1, sh = 16 * (j & 1), m = cur.at(j);
+                const int gx = (int)((g.x[j >> 1] >> sh) & 0xffffu) - 1024, gy = (int)((g.y[j >> 1] >> sh) & 0xffffu) - 1024;
+                const int ax = abs(gx), ay = abs(gy);
+                const bool hor = ay <= tan22(ax), ver = ax <= tan22(ay), same = (gx ^ gy) >= 0;
+                // a on the previous row (left for the horizontal sector), b opposite
+                const int ma = hor ? cur.at(j - 1) : ver ? prev.at(j) : same ? prev.at(j - 1) : prev.at(j + 1);
+                const int mb = hor ? cur.at(j + 1) : ver ? next.at(j) : same ? next.at(j + 1) : next.at(j - 1);
+                const bool keep = m > ma && m >= mb && m > low;
+                v |= (keep ? 16u << c : 0u) | (keep && m > high ? 1u << c : 0u);
             }
-            const bool keep = m > ma && m >= mb;
-            ws |= (uint32_t)(keep && m > high) << (8 * c);
-            wc |= (uint32_t)(keep && m > low) << (8 * c);
-        }
-        if (cx0 < W) {
-            const size_t o = (size_t)y * W + cx0;
-            if (out_vec) {
-                *reinterpret_cast<uint32_t*>(d.edges + o) = ws;
-                *reinterpret_cast<uint32_t*>(d.cand + o) = wc;
-            } else {
-                for (int c = 0; c < 4 && cx0 + c < W; c++) {
-                    d.edges[o + c] = (uint8_t)(ws >> (8 * c));
-                    d.cand[o + c] = (uint8_t)(wc >> (8 * c));
-                }
-            }
-            if (ws) {
-#pragma unroll
-                for (int c = 0; c < 4; c++)
-                    if ((ws >> (8 * c)) & 1u) seed |= seed_bits_px(rtx, rty, cx0 + c, y);
-            }
+            // bytes of 8 columns: the even lane of a pair writes the marker, the odd one the mask
+            const unsigned o = __shfl_xor_sync(0xffffffffu, v, 1);
+            bits[warp][lane & 1][y - ya][lane >> 1] =
+                (uint8_t)((lane & 1) ? (o >> 4) | (v & 0xf0u) : (v & 15u) | (o << 4));
         }
         prev = cur;
         cur = next;
         P = Q;
         Q = N;
+        N = M;
     }
-    // lanes 0-15 and 16-31 each lie in one work tile: one flag store per touched work tile
-    const unsigned lo = __reduce_or_sync(0xffffffffu, lane < 16 ? seed : 0u);
-    const unsigned hi = __reduce_or_sync(0xffffffffu, lane >= 16 ? seed : 0u);
-    if ((lane == 0 || lane == 16) && cx0 < W) {
-        const unsigned m9 = lane == 0 ? lo : hi;
-        const int tx = cx0 / RT, ty = ya / RT;
-        for (int b = 0; b < 9; b++)
-            if ((m9 >> b) & 1u) flags[d.rt_base + (ty + b / 3 - 1) * rtx + (tx + b % 3 - 1)] = 1;
+    __syncwarp();
+    const int rtx = (W + RT - 1) / RT;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {  // the strip's two work tiles: rows 2 l and 2 l + 1 from lane l
+        const int tx = 2 * strip + h;
+        if (tx >= rtx) break;
+        const size_t t = (size_t)d.rt_base + (size_t)seg * rtx + tx;
+        u64 w[2][2];
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+#pragma unroll
+            for (int r = 0; r < 2; r++) w[q][r] = *reinterpret_cast<const u64*>(&bits[warp][q][2 * lane + r][8 * h]);
+        reinterpret_cast<ulonglong2*>(G.marker + t * RT)[lane] = make_ulonglong2(w[0][0], w[0][1]);
+        reinterpret_cast<ulonglong2*>(G.mask + t * RT)[lane] = make_ulonglong2(w[1][0], w[1][1]);
+        const bool any = __any_sync(0xffffffffu, (w[0][0] | w[0][1]) != 0ull);
+        if (lane == 0) G.any[t] = any;
     }
 }
 
+// ---- edge counts: one warp per 32x32 block with an edge pixel ---------------------
+// The warp lists the block's edge pixels (a few dozen of 1024), stages the
+// labels of the rows within r of them with a 4-pixel margin (0 off the
+// image, and for labels outside 1..K) and one bit per staged pixel that holds
+// an object, and takes the listed pixels 32 at a time, one per lane: the
+// bits under the disk's chord of each row pick the labels to look at.  Each
+// edge pixel adds one to every distinct object in its disk (the first four
+// remembered in registers, beyond that an object is new iff no earlier disk
+// offset holds it).  8 tiles of 4096^2: 223 us (465 with a CTA per block, a
+// thread per pixel and a label read for every disk offset; 246 with four label
+// loads of a lane in flight instead of seven).  Bound: the latency of the label
+// loads of the blocks that hold edges (about half), 24 warps per SM by shared
+// memory.
 constexpr int CR_MAX = 4;                 // largest disk radius of the counts
-constexpr int CC_S = CT + 2 * CR_MAX;     // staged labels: the block and a CR_MAX-pixel halo (40 x 40)
+constexpr int CC_S = CT + 2 * CR_MAX;     // staged labels: the block and a CR_MAX-pixel margin (40 x 40)
+constexpr int CC_WARPS = 4;
 
-// Edge counts, one 32x32 block per CTA: the edge bytes of the block, then
-// (for a block with an edge pixel) the labels of the block and a 4-pixel
-// halo (0 off the image, and for labels outside 1..K), staged in shared
-// memory with 16-byte loads where the rows allow; each edge pixel adds one
-// to every distinct object in its disk (the first four remembered in
-// registers, beyond that an object is new iff no earlier disk offset holds
-// it).
-__global__ void __launch_bounds__(256) k_canny_counts(const CannyDesc* __restrict__ D, int n, int r) {
-    __shared__ __align__(16) int32_t sl[CC_S][CC_S];
-    __shared__ __align__(16) uint8_t se[CT][CT];
-    const int t = threadIdx.x;
-    const CannyDesc& d = D[find_desc(D, n, blockIdx.x, &CannyDesc::blk_base)];
-    const int K = d.K;
+struct CountStage {
+    int32_t lab[CC_S][CC_S];
+    u64 occ[CC_S];           // bit x: lab[y][x] != 0
+    uint16_t list[CT * CT];  // edge pixels, y << 5 | x
+};
+
+__global__ void __launch_bounds__(CC_WARPS * 32) k_canny_counts(const __grid_constant__ GrowLaunch G, int n_blocks, int r) {
+    extern __shared__ __align__(16) unsigned char cc_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    CountStage& S = reinterpret_cast<CountStage*>(cc_smem)[warp];
+    const int gb = blockIdx.x * CC_WARPS + warp;
+    if (gb >= n_blocks) return;
+    const CannyDesc& d = G.tab[G.tab.find(gb, &CannyDesc::blk_base)];
+    const int K = d.K, W = d.W, H = d.H, bl = gb - d.blk_base;
     if (K <= 0) return;
-    const int W = d.W, H = d.H, bl = blockIdx.x - d.blk_base;
-    const int by = bl / d.bx, x0 = (bl - by * d.bx) * CT, y0 = by * CT;
-    int any = 0;
-    if (t < 64) {  // the block's edge bytes: one 16-byte row half per thread
-        const int ly = t >> 1, lx = (t & 1) * 16, gy = y0 + ly, gx = x0 + lx;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        const uint8_t* src = d.edges + (size_t)gy * W + gx;
-        if (gy < H) {
-            if (gx + 16 <= W && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-                v = *reinterpret_cast<const uint4*>(src);
-            } else {
-                uint32_t w[4] = {0, 0, 0, 0};
+    const int by = bl / d.bx, bx = bl - by * d.bx, x0 = bx * CT, y0 = by * CT;
+    const size_t t = (size_t)d.rt_base + (size_t)(by >> 1) * ((W + RT - 1) / RT) + (bx >> 1);
+    const uint32_t e = reinterpret_cast<const uint32_t*>(G.marker + t * RT + (by & 1) * CT + lane)[bx & 1];
+    const unsigned rows = __ballot_sync(0xffffffffu, e != 0u);  // block rows with an edge pixel
+    if (!rows) return;
+    int at = __popc(e), n;
 #pragma unroll
-                for (int k = 0; k < 16; k++)
-                    if (gx + k < W) w[k >> 2] |= (uint32_t)src[k] << (8 * (k & 3));
-                v = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        *reinterpret_cast<uint4*>(&se[ly][lx]) = v;
-        any = (v.x | v.y | v.z | v.w) != 0;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += v;
     }
-    if (!__syncthreads_or(any)) return;       // no edge pixel: no label is needed
+    n = __shfl_sync(0xffffffffu, at, 31);
+    at -= __popc(e);
+    for (uint32_t m = e; m; m &= m - 1) S.list[at++] = (uint16_t)(lane << 5 | (__ffs(m) - 1));
+    // staged rows needed: within r of a row with an edge pixel (staged row = block row + CR_MAX)
+    u64 need = 0;
+    for (int dy = CR_MAX - r; dy <= CR_MAX + r; dy++) need |= (u64)rows << dy;
     const bool vec = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(d.labels) & 15) == 0;
-    // 400 four-label groups over 256 threads: both of a thread's loads are
-    // issued before either is stored, so their latencies overlap
+    if (lane < CC_S) S.occ[lane] = 0ull;
+    if (lane < CC_S - 32) S.occ[lane + 32] = 0ull;
+    __syncwarp();
     constexpr int NQ = CC_S * (CC_S / 4);
-    int4 v[2];
+    constexpr int CU = 7;  // loads of a lane in flight
+#pragma unroll 1
+    for (int i0 = 0; i0 < NQ; i0 += CU * 32) {
+        int4 v[CU];
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-        const int i = t + 256 * u;
-        const int ly = i / (CC_S / 4), q = i - ly * (CC_S / 4);
-        const int gy = y0 - CR_MAX + ly, gx = x0 - CR_MAX + 4 * q;
-        v[u] = make_int4(0, 0, 0, 0);
-        if (i < NQ && (unsigned)gy < (unsigned)H) {
-            const int32_t* src = d.labels + (size_t)gy * W + gx;
-            if (vec && gx >= 0 && gx + 4 <= W) {
-                v[u] = __ldg(reinterpret_cast<const int4*>(src));
-            } else {
-                int e[4];
+        for (int u = 0; u < CU; u++) {
+            const int i = i0 + 32 * u + lane, ly = i / (CC_S / 4), q = i - ly * (CC_S / 4);
+            const int gy = y0 - CR_MAX + ly, gx = x0 - CR_MAX + 4 * q;
+            v[u] = make_int4(0, 0, 0, 0);
+            if (i < NQ && ((need >> ly) & 1u) && (unsigned)gy < (unsigned)H) {
+                const int32_t* src = d.labels + (size_t)gy * W + gx;
+                if (vec && gx >= 0 && gx + 4 <= W) {
+                    v[u] = __ldg(reinterpret_cast<const int4*>(src));
+                } else {
+                    int w[4];
 #pragma unroll
-                for (int k = 0; k < 4; k++) e[k] = (unsigned)(gx + k) < (unsigned)W ? __ldg(src + k) : 0;
-                v[u] = make_int4(e[0], e[1], e[2], e[3]);
+                    for (int k = 0; k < 4; k++) w[k] = (unsigned)(gx + k) < (unsigned)W ? __ldg(src + k) : 0;
+                    v[u] = make_int4(w[0], w[1], w[2], w[3]);
+                }
             }
         }
-    }
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-        const int i = t + 256 * u;
-        if (i >= NQ) break;
-        const int ly = i / (CC_S / 4), q = i - ly * (CC_S / 4);
-        int4 w = v[u];
-        w.x = (w.x >= 1 && w.x <= K) ? w.x : 0;
-        w.y = (w.y >= 1 && w.y <= K) ? w.y : 0;
-        w.z = (w.z >= 1 && w.z <= K) ? w.z : 0;
-        w.w = (w.w >= 1 && w.w <= K) ? w.w : 0;
-        *reinterpret_cast<int4*>(&sl[ly][4 * q]) = w;
+        for (int u = 0; u < CU; u++) {
+            const int i = i0 + 32 * u + lane, ly = i / (CC_S / 4), q = i - ly * (CC_S / 4);
+            if (i >= NQ || !(v[u].x | v[u].y | v[u].z | v[u].w)) continue;
+            int4 w = v[u];
+            w.x = (w.x >= 1 && w.x <= K) ? w.x : 0;
+            w.y = (w.y >= 1 && w.y <= K) ? w.y : 0;
+            w.z = (w.z >= 1 && w.z <= K) ? w.z : 0;
+            w.w = (w.w >= 1 && w.w <= K) ? w.w : 0;
+            *reinterpret_cast<int4*>(&S.lab[ly][4 * q]) = w;  // read only where occ is set
+            const u64 o = (u64)((w.x != 0) | (w.y != 0) << 1 | (w.z != 0) << 2 | (w.w != 0) << 3) << (4 * q);
+            if (o) atomicOr(&S.occ[ly], o);
+        }
     }
-    __syncthreads();
+    __syncwarp();
     const int r2 = r * r;
-    for (int i = t; i < CT * CT; i += 256) {
-        const int ly = i / CT, lx = i - ly * CT;
-        if (!se[ly][lx]) continue;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        if (i0 + lane >= n) break;
+        const int p = S.list[i0 + lane], ly = p >> 5, lx = p & 31;
         int seen0 = 0, seen1 = 0, seen2 = 0, seen3 = 0, nseen = 0;
-        for (int dy = -r; dy <= r; dy++)
-            for (int dx = -r; dx <= r; dx++) {
-                if (dx * dx + dy * dy > r2) continue;
-                const int v = sl[ly + CR_MAX + dy][lx + CR_MAX + dx];
-                if (!v || v == seen0 || v == seen1 || v == seen2 || v == seen3) continue;
+        for (int dy = -r; dy <= r; dy++) {
+            int w = r;  // half-width of the disk's chord
+            while (w * w + dy * dy > r2) w--;
+            const int row = ly + CR_MAX + dy;
+            u64 m = (S.occ[row] >> (lx + CR_MAX - w)) & ((2ull << (2 * w)) - 1ull);
+            for (; m; m &= m - 1) {
+                const int dx = __ffsll((long long)m) - 1 - w;
+                const int v = S.lab[row][lx + CR_MAX + dx];
+                if (v == seen0 || v == seen1 || v == seen2 || v == seen3) continue;
                 bool fresh = true;
                 if (nseen >= 4) {  // look for v at an earlier disk offset
                     for (int ey = -r; ey <= dy && fresh; ey++)
                         for (int ex = -r; ex <= r; ex++) {
                             if (ey == dy && ex >= dx) break;
-                            if (ex * ex + ey * ey <= r2 && sl[ly + CR_MAX + ey][lx + CR_MAX + ex] == v) {
+                            if (ex * ex + ey * ey <= r2 && ((S.occ[ly + CR_MAX + ey] >> (lx + CR_MAX + ex)) & 1u) &&
+                                S.lab[ly + CR_MAX + ey][lx + CR_MAX + ex] == v) {
                                 fresh = false;
                                 break;
                             }
@@ -346,54 +355,22 @@ __global__ void __launch_bounds__(256) k_canny_counts(const CannyDesc* __restric
                 else if (nseen == 3) seen3 = v;
                 nseen++;
             }
+        }
     }
 }
 
 int canny_blocks(int W, int H) { return ((W + CT - 1) / CT) * ((H + CT - 1) / CT); }
-
-// descriptors reach the device through kernel parameters (no host staging
-// buffer has to outlive the call)
-constexpr int CANNY_DESC_PACK = 8;
-struct CannyDescPack {
-    CannyDesc d[CANNY_DESC_PACK];
-    int n, first;
-};
-__global__ void k_set_canny_desc(CannyDesc* dst, CannyDescPack p) {
-    if (threadIdx.x < p.n) dst[p.first + threadIdx.x] = p.d[threadIdx.x];
-}
-void upload_canny_descs(CannyDesc* dst, const std::vector<CannyDesc>& v, cudaStream_t s) {
-    for (int i = 0; i < (int)v.size(); i += CANNY_DESC_PACK) {
-        CannyDescPack pk;
-        pk.first = i;
-        pk.n = (int)v.size() - i < CANNY_DESC_PACK ? (int)v.size() - i : CANNY_DESC_PACK;
-        for (int k = 0; k < pk.n; k++) pk.d[k] = v[i + k];
-        k_set_canny_desc<<<1, 32, 0, s>>>(dst, pk);
-    }
-}
-
 int canny_nms_warps(int W, int H) { return ((W + NS_COLS - 1) / NS_COLS) * ((H + NS_ROWS - 1) / NS_ROWS); }
 
-void launch_canny_nms(const std::vector<CannyDesc>& descs, CannyDesc* d_descs, int low, int high, int* flags,
-                      cudaStream_t s, Profiler* pf) {
-    int warps = 0;
-    for (auto& d : descs) warps += canny_nms_warps(d.W, d.H);
-    if (!warps) return;
+void launch_canny_nms(const GrowLaunch& G, int warps, int low, int high, cudaStream_t s, Profiler* pf) {
     pf->begin("canny_nms", s);
-    k_canny_nms<<<(warps + NS_WARPS - 1) / NS_WARPS, 32 * NS_WARPS, 0, s>>>(d_descs, (int)descs.size(), warps, low,
-                                                                          high, flags);
+    k_canny_nms<<<(warps + NS_WARPS - 1) / NS_WARPS, 32 * NS_WARPS, 0, s>>>(G, warps, low, high);
     pf->end("canny_nms", s);
 }
 
-void launch_canny_counts(const std::vector<CannyDesc>& descs, CannyDesc* d_descs, int r, cudaStream_t s,
-                         Profiler* pf) {
-    int blocks = 0, K = 0;
-    for (auto& d : descs) {
-        blocks += canny_blocks(d.W, d.H);
-        K += d.K;
-    }
-    if (!blocks || !K) return;
+void launch_canny_counts(const GrowLaunch& G, int blocks, int r, cudaStream_t s, Profiler* pf) {
     pf->begin("canny_counts", s);
-    k_canny_counts<<<blocks, 256, 0, s>>>(d_descs, (int)descs.size(), r);
+    k_canny_counts<<<(blocks + CC_WARPS - 1) / CC_WARPS, CC_WARPS * 32, CC_WARPS * sizeof(CountStage), s>>>(G, blocks, r);
     pf->end("canny_counts", s);
 }
 

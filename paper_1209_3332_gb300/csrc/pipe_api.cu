@@ -311,13 +311,9 @@ struct pipe_s {
     DevBuf ws_status;   // watershed_tile: device status word
     DevBuf ws_desc;     // watershed_batch: tile descriptors
     cudaStream_t ws_side = nullptr;        // watershed_tile: large boxes overlap the small ones here
-    LaunchCtx rbc;      // rbc_tile: the reconstruction of the RBC markers runs on this context
-    DevBuf rbc_mask;    // rbc_tile: the mask plane
-    DevBuf rbc_flags;   // rbc_tile: seed flags, one int per work tile
-    LaunchCtx canny;    // canny_tile: the hysteresis runs the reconstruction on this context
-    DevBuf canny_cand;  // canny_tile / canny_batch: candidate planes (the reconstruction's masks)
-    DevBuf canny_flags; // canny_tile / canny_batch: seed flags, one int per work tile
-    DevBuf canny_desc;  // canny_tile / canny_batch: tile descriptors
+    DevBuf grow;        // rbc_tile, canny_tile, canny_batch: bit planes and queue of the growth
+    DevBuf canny_desc;  // canny_batch: tile descriptors
+    int grow_cap = 1;   // resident CTAs of the growth
     cudaEvent_t ws_fork = nullptr, ws_join = nullptr;
     // batched form
     LaunchCtx batch;
@@ -450,10 +446,33 @@ int upload_desc(const Launch& L, const std::vector<TileDev>& td, cudaStream_t s)
     return PIPE_OK;
 }
 
-int max_width(const std::vector<TileDev>& td) {
-    int w = 1;
-    for (auto& t : td) w = std::max(w, t.W);
-    return w;
+// The growth of binary markers over the tiles of cd, n_rt work tiles in all:
+// bit planes, queue and descriptors (a larger call than any before grows them,
+// which synchronises s).
+int make_grow(pipe_t p, const std::vector<CannyDesc>& cd, int n_rt, cudaStream_t s, GrowLaunch* out) {
+    const size_t plane = al256((size_t)n_rt * RT * 8), queue = (size_t)n_rt * 12;
+    const size_t need = al256(sizeof(GrowShared)) + 2 * plane + al256(queue) + al256((size_t)n_rt);
+    const size_t desc = cd.size() > CannyTab::NEAR ? sizeof(CannyDesc) * cd.size() : 0;
+    if (p->grow.n < need || p->canny_desc.n < desc) {
+        CK(cudaStreamSynchronize(s));
+        int rc;
+        if ((rc = p->grow.ensure(need)) || (rc = p->canny_desc.ensure(desc))) return rc;
+    }
+    char* b = (char*)p->grow.p;
+    out->sh = (GrowShared*)b;
+    b += al256(sizeof(GrowShared));
+    out->mask = (unsigned long long*)b;
+    out->marker = (unsigned long long*)(b + plane);
+    b += 2 * plane;
+    out->slots = (unsigned long long*)b;
+    out->state = (int*)(b + (size_t)n_rt * 8);
+    out->any = (uint8_t*)(b + al256(queue));
+    out->n_rt = n_rt;
+    out->group = grow_group(n_rt);
+    out->wait_budget = p->prm.wait_budget_cycles;
+    CK(cudaMemsetAsync(out->slots, 0, queue, s));
+    out->tab = make_canny_tab(cd, (CannyDesc*)p->canny_desc.p, s);
+    return PIPE_OK;
 }
 
 // The whole path over the descriptors of L (segmentation, and features when
@@ -705,6 +724,7 @@ int pipe_create(const pipe_params* params, int device, pipe_t* out) {
     deconv_tables(lut, wq);
     upload_deconv_tables(lut, wq);
     p->recon_cap = std::max(1, recon_grid(device));
+    p->grow_cap = std::max(1, grow_grid(device));
     if (prm.autotune_cache) {
         p->tune_file = prm.autotune_cache;
         load_tune_file(p);
@@ -728,12 +748,7 @@ void pipe_destroy(pipe_t p) {
     p->fbbox.release();
     p->morph_tmp.release();
     p->ws_obj.release();
-    rel(p->rbc);
-    p->rbc_mask.release();
-    p->rbc_flags.release();
-    rel(p->canny);
-    p->canny_cand.release();
-    p->canny_flags.release();
+    p->grow.release();
     p->canny_desc.release();
     p->ws_scratch.release();
     p->ws_status.release();
@@ -938,75 +953,35 @@ int rbc_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
     if (rgb_dev < out_dev + N && out_dev < rgb_end) return PIPE_EINVAL;  // the planes overlap
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(p->device));
-    const int rtx = (W + RT - 1) / RT, rty = (H + RT - 1) / RT, n_rt = rtx * rty;
-    if (p->rbc_mask.n < N || p->rbc_flags.n < sizeof(int) * (size_t)n_rt || p->rbc.wl.n < wl_bytes(n_rt) ||
-        !p->rbc.shared.p) {
-        CK(cudaStreamSynchronize(s));
-        const bool fresh = !p->rbc.shared.p;
-        int rc;
-        if ((rc = p->rbc_mask.ensure(N)) || (rc = p->rbc_flags.ensure(sizeof(int) * (size_t)n_rt)) ||
-            (rc = ensure_ctx(p->rbc, 1, n_rt, 0)))
-            return rc;
-        if (fresh) CK(cudaMemset(p->rbc.shared.p, 0, p->rbc.shared.n));
-    }
-    std::vector<TileDev> td(1);
-    std::memset(&td[0], 0, sizeof(TileDev));
-    td[0].W = W;
-    td[0].H = H;
-    td[0].R = out_dev;
-    td[0].hem8 = (uint8_t*)p->rbc_mask.p;
-    td[0].rtx = rtx;
-    td[0].rty = rty;
-    Launch L = make_launch(p, p->rbc, td, n_rt, 4);
-    int* flags = (int*)p->rbc_flags.p;
-    // 1. red dominance: the marker into out_dev, the mask into the pipe's
-    //    plane, and the work tiles the marker touches
-    CK(cudaMemsetAsync(flags, 0, sizeof(int) * (size_t)n_rt, s));
-    CK(cudaMemsetAsync(&L.sh->nseed, 0, sizeof(int), s));
-    launch_rbc_planes(rgb_dev, pitch_bytes, W, H, t_lo, t_hi, out_dev, (uint8_t*)p->rbc_mask.p, flags, s, &p->prof);
-    // 2. reconstruction by dilation of the marker under the mask, started from
-    //    the flagged work tiles only
-    int rc;
-    if ((rc = upload_desc(L, td, s))) return rc;
-    launch_recon_seeded(L, flags, p->recon_cap, s, &p->prof);
+    std::vector<CannyDesc> cd(1);
+    std::memset(&cd[0], 0, sizeof(CannyDesc));
+    cd[0].W = W;
+    cd[0].H = H;
+    cd[0].edges = out_dev;
+    GrowLaunch G;
+    const int rc = make_grow(p, cd, ((W + RT - 1) / RT) * ((H + RT - 1) / RT), s, &G);
+    if (rc) return rc;
+    // red dominance into the marker and the mask, then the growth of the marker
+    launch_rbc_planes(G, rgb_dev, pitch_bytes, t_lo, t_hi, s, &p->prof);
+    launch_grow(G, p->grow_cap, s, &p->prof);
     CK(cudaGetLastError());
     return PIPE_OK;
 }
 
 namespace {
 
-// Canny of n tiles: one NMS launch over all of them, one reconstruction
-// queue for every tile's hysteresis (seeded from the work tiles that hold a
-// strong pixel), one counts launch.  Arguments already checked.
+// Canny of n tiles: one NMS launch over all of them, one queue for every
+// tile's hysteresis, one counts launch.  Arguments already checked.
 int canny_run(pipe_t p, const edge_tile* tiles, int n, int low, int high, int radius, cudaStream_t s) {
-    size_t cand_bytes = 0;
-    int n_rt = 0;
-    for (int i = 0; i < n; i++) {
-        cand_bytes += al256((size_t)tiles[i].W * tiles[i].H);
-        n_rt += ((tiles[i].W + RT - 1) / RT) * ((tiles[i].H + RT - 1) / RT);
-    }
-    const size_t desc_bytes = sizeof(CannyDesc) * (size_t)n, flag_bytes = sizeof(int) * (size_t)n_rt;
-    if (p->canny_cand.n < cand_bytes || p->canny_flags.n < flag_bytes || p->canny_desc.n < desc_bytes ||
-        p->canny.wl.n < wl_bytes(n_rt) || p->canny.tiles.n < tiles_bytes(n) || p->canny.shared.n < shared_bytes(n) ||
-        !p->canny.shared.p) {
-        CK(cudaStreamSynchronize(s));
-        int rc;
-        if ((rc = p->canny_cand.ensure(cand_bytes)) || (rc = p->canny_flags.ensure(flag_bytes)) ||
-            (rc = p->canny_desc.ensure(desc_bytes)) || (rc = ensure_ctx(p->canny, n, n_rt, 0)))
-            return rc;
-        CK(cudaMemset(p->canny.shared.p, 0, p->canny.shared.n));
-    }
     std::vector<CannyDesc> cd(n);
-    std::vector<TileDev> td(n);
-    char* cand = (char*)p->canny_cand.p;
     int blk = 0, nw = 0, rt = 0;
+    bool counts = false;
     for (int i = 0; i < n; i++) {
         const edge_tile& t = tiles[i];
         CannyDesc& c = cd[i];
         c.img = t.img;
         c.labels = t.labels;
         c.edges = t.edges;
-        c.cand = (uint8_t*)cand;
         c.counts = t.counts;
         c.W = t.W;
         c.H = t.H;
@@ -1017,32 +992,18 @@ int canny_run(pipe_t p, const edge_tile* tiles, int n, int low, int high, int ra
         c.rt_base = rt;
         blk += canny_blocks(t.W, t.H);
         nw += canny_nms_warps(t.W, t.H);
-        cand += al256((size_t)t.W * t.H);
-        TileDev& d = td[i];
-        std::memset(&d, 0, sizeof(TileDev));
-        d.W = t.W;
-        d.H = t.H;
-        d.R = t.edges;
-        d.hem8 = c.cand;
-        d.rtx = (t.W + RT - 1) / RT;
-        d.rty = (t.H + RT - 1) / RT;
-        rt += d.rtx * d.rty;
+        rt += ((t.W + RT - 1) / RT) * ((t.H + RT - 1) / RT);
+        counts |= t.n_objects > 0;
     }
-    CannyDesc* dcd = (CannyDesc*)p->canny_desc.p;
-    int* flags = (int*)p->canny_flags.p;
-    Launch L = make_launch(p, p->canny, td, n_rt, 4);  // rt_base in the same order as above
-    upload_canny_descs(dcd, cd, s);
-    CK(cudaMemsetAsync(flags, 0, flag_bytes, s));
-    CK(cudaMemsetAsync(&L.sh->nseed, 0, sizeof(int), s));
-    // 1. gradient and non-maximum suppression: strong pixels into the edge
-    //    planes, candidates into the pipe's planes, counts zeroed, seed flags
-    launch_canny_nms(cd, dcd, low, high, flags, s, &p->prof);
-    // 2. hysteresis: reconstruction by dilation of the strong pixels under the candidates
-    int rc;
-    if ((rc = upload_desc(L, td, s))) return rc;
-    launch_recon_seeded(L, flags, p->recon_cap, s, &p->prof);
+    GrowLaunch G;
+    const int rc = make_grow(p, cd, rt, s, &G);
+    if (rc) return rc;
+    // 1. gradient and non-maximum suppression: strong pixels and candidates; counts zeroed
+    launch_canny_nms(G, nw, low, high, s, &p->prof);
+    // 2. hysteresis: the strong pixels grown through the candidates, into the edge planes
+    launch_grow(G, p->grow_cap, s, &p->prof);
     // 3. edge pixels within each object's disk dilation
-    launch_canny_counts(cd, dcd, radius, s, &p->prof);
+    if (counts) launch_canny_counts(G, blk, radius, s, &p->prof);
     CK(cudaGetLastError());
     return PIPE_OK;
 }
@@ -1172,8 +1133,12 @@ int pipe_status_read(pipe_t p) {
     };
     check(p->plain, 1);
     check(p->batch, p->batch_ntiles);
-    check(p->canny, 1);
-    check(p->rbc, 1);
+    if (p->grow.p) {
+        GrowShared sh;
+        if (cudaMemcpy(&sh, p->grow.p, sizeof(sh), cudaMemcpyDeviceToHost) != cudaSuccess) return PIPE_ECUDA;
+        if (sh.err && result == PIPE_OK) result = sh.err;
+        cudaMemset((char*)p->grow.p + offsetof(GrowShared, err), 0, sizeof(int));
+    }
     if (p->ws_status.p) {
         int st = 0;
         if (cudaMemcpy(&st, p->ws_status.p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return PIPE_ECUDA;

@@ -187,3 +187,27 @@ def test_batch_argument_checks(pipe):
         pipe.canny_batch([dict(img=I, edges=E, n_objects=2, counts=C)])       # objects without labels
     with pytest.raises(P.PipeError):
         pipe.canny_batch([])
+
+
+@pytest.mark.parametrize("n", [8, 9, 17])
+def test_batch_descriptor_tables(pipe, n):
+    """Up to 8 descriptors travel in the launch parameters, more in device
+    memory; the tiles differ in size, so each must meet its own."""
+    import torch
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(n)
+    imgs = [np.kron(rng.integers(0, 256, (5 + i, 9 + 2 * i), dtype=np.uint8), np.ones((7, 7), np.uint8)) for i in range(n)]
+    tiles = [dict(img=torch.from_numpy(a).to(dev), edges=torch.full(a.shape, 7, dtype=torch.uint8, device=dev)) for a in imgs]
+    pipe.canny_batch(tiles)
+    torch.cuda.synchronize()
+    for a, t in zip(imgs, tiles):
+        assert np.array_equal(t["edges"].cpu().numpy(), oracle.canny(a))
+
+
+@pytest.mark.parametrize("W,H", [(64 * 64, 31 * 64 + 1), (64 * 128 - 3, 64 * 128)])
+def test_growth_draws_of_several_tiles(pipe, W, H):
+    """Planes of 2048 and 16384 work tiles, from which the growth draws two
+    and four tiles at a time."""
+    rng = np.random.default_rng(W)
+    img = np.kron(rng.integers(0, 256, ((H + 15) // 16, (W + 15) // 16), dtype=np.uint8), np.ones((16, 16), np.uint8))[:H, :W]
+    check(pipe, img)
