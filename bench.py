@@ -495,10 +495,10 @@ def canny_run(torch, pipe, stream, bufs, steps, hbm_peak, want_cpu):
         out["nms_kernel"] = {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                              "alg_bytes_per_px": 1.25}
     cnt_ms = kern.get("canny_counts", 0.0)
-    if cnt_ms > 0:  # the counts pass alone: edges and labels read once
-        gbs = 5.0 * px / (cnt_ms / 1000.0) / 1e9
+    if cnt_ms > 0:  # the counts pass alone: edge bits and labels read once
+        gbs = 4.125 * px / (cnt_ms / 1000.0) / 1e9
         out["counts_kernel"] = {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
-                                "alg_bytes_per_px": 3.25}
+                                "alg_bytes_per_px": 4.125}
     if want_cpu:
         import time
         import oracle
@@ -570,7 +570,7 @@ def rbc_run(torch, pipe, stream, steps, hbm_peak, want_cpu):
     if pl:   # the planes pass alone: RGB read, marker and mask bits written
         g = 3.25 * H * W / (pl / 1000.0) / 1e9
         out["planes_kernel"] = {"achieved": g, "peak": hbm_peak, "unit": "GB/s", "frac": g / hbm_peak,
-                                "alg_bytes_per_px": 5}
+                                "alg_bytes_per_px": 3.25}
     if want_cpu:
         out["cpu_oracle"] = {"tiles_per_s": 1.0 / cpu_s, "cores": 1, "sample": "the oracle on tile 0, %.2f s" % cpu_s}
     return out
