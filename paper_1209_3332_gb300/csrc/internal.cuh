@@ -66,10 +66,11 @@ constexpr int LAUNCH_TAB = 64;    // tiles whose block bases travel in the launc
 // Shared state of one launch sequence (device memory).
 struct Shared {
     unsigned long long tp;              // reconstruction worklist: tail << 32 | pending
-    int head, err;                      // worklist head; first device-side error
+    alignas(256) int head;              // worklist head
+    alignas(256) int next_obj;          // the batched feature pass draws its objects from this counter
+    alignas(256) int nobj;              // object items of a batched feature pass
+    int err;                            // first device-side error
     int processed;                      // tile processings (diagnostic)
-    int nobj;                           // object items of a batched feature pass
-    int next_obj;                       // the batched feature pass draws its objects from this counter
 };
 
 struct Launch {

@@ -128,8 +128,11 @@ __device__ __forceinline__ bool budget_over(long long t0, long long budget) {
 // << ITEM_BITS | the work tile's index within its image, with bit 31 set on
 // the tile's first visit (queued by k_wl_init).  The tail and the
 // count of queued-or-running tiles (pending) share one 64-bit word, so a push
-// moves both with one atomic.  A consumer holding a ticket waits until its
-// item arrives or until no tile is queued or running any more.
+// moves both with one atomic, and a visit's pushes and the release of its tile
+// are one atomic together: the workers' atomics on one word are served one
+// after the other, about 2.8 ns each, and head and tail lie in lines of their
+// own.  A consumer holding a ticket waits until its item arrives or until no
+// tile is queued or running any more.
 
 constexpr int ITEM_BITS = 18;  // work tiles per image <= (16384 / 64)^2 = 2^16 < 2^18
 constexpr unsigned ITEM_MASK = (1u << ITEM_BITS) - 1;
@@ -143,9 +146,9 @@ __device__ __forceinline__ void st_vol64(unsigned long long* p, unsigned long lo
     *(volatile unsigned long long*)p = v;
 }
 
-__device__ void wl_push(const Launch& L, unsigned item) {
+// puts item into position i of the queue
+__device__ void wl_put(const Launch& L, unsigned i, unsigned item) {
     const unsigned cap = (unsigned)L.n_rt;
-    const unsigned i = (unsigned)(atomicAdd(&L.sh->tp, (1ull << 32) | 1ull) >> 32);
     unsigned long long* slot = L.wl_slots + i % cap;
     long long t0 = clock64();
     while ((unsigned)(ld_vol64(slot) >> 32) != i) {
@@ -155,19 +158,16 @@ __device__ void wl_push(const Launch& L, unsigned item) {
     st_vol64(slot, ((unsigned long long)(i + 1) << 32) | item);
 }
 
-// work tile k of image ti, whose first work tile has global index base
-__device__ void wl_request(const Launch& L, int ti, int base, int k) {
-    const int t = base + k;
+// marks work tile t (global index) as wanted; true if the caller has to queue it
+__device__ bool wl_want(const Launch& L, int t) {
     for (int it = 0; it < 1024; it++) {
         int s = atomicCAS(&L.wl_state[t], WL_IDLE, WL_QUEUED);
-        if (s == WL_IDLE) {
-            wl_push(L, ((unsigned)ti << ITEM_BITS) | (unsigned)k);
-            return;
-        }
-        if (s == WL_QUEUED || s == WL_DIRTY) return;
-        if (atomicCAS(&L.wl_state[t], WL_RUNNING, WL_DIRTY) == WL_RUNNING) return;
+        if (s == WL_IDLE) return true;
+        if (s == WL_QUEUED || s == WL_DIRTY) return false;
+        if (atomicCAS(&L.wl_state[t], WL_RUNNING, WL_DIRTY) == WL_RUNNING) return false;
     }
     atomicCAS(&L.sh->err, 0, ST_TIMEOUT);
+    return false;
 }
 
 // takes the next item; false when the queue is drained (or on error)
@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
         }
         __syncwarp();
         for (;;) {
-            int nr = 0;
+            int nr = 0, queue = -1;
             bool more = false;
             bool go = sweep_now || (full_check ? can_raise(S, lane) : border_can_raise(S, lane));
             sweep_now = false;
@@ -742,28 +742,32 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
                         default: target = k; break;
                     }
                     S.flags[lane] = 0;
-                    if (target >= 0) wl_request(L, ti, base, target);
+                    if (target >= 0 && wl_want(L, base + target)) queue = target;
                 }
             }
-            // every request (and the pending count it adds) comes before this
-            // tile stops counting as running
-            __syncwarp();
-            if (grew) continue;  // the fresher halo may raise pixels: check again
-            int again = 0;
+            const unsigned qm = __ballot_sync(FULL, queue >= 0);
+            // The tile is released (unless its fresher halo is to be looked at
+            // again) before the wanted neighbours enter the queue; until the one
+            // atomic that adds them and takes the tile off, it counts as pending.
+            // No fence is needed before the release: every write-back above was
+            // followed by one.
+            int again = grew ? 1 : 0;
+            unsigned at = 0;
             if (lane == 0) {
-                // no fence needed here: every write-back above was followed by
-                // one, and the requests' pending counts precede this update in
-                // the counter's order through the warp barrier
-                const int st = atomicCAS(&L.wl_state[t], WL_RUNNING, WL_IDLE);
-                if (st == WL_RUNNING) {
-                    atomicAdd(&L.sh->tp, ~0ull);  // pending - 1
-                } else {
-                    // a neighbour raised the halo meanwhile: take the tile again
-                    atomicExch(&L.wl_state[t], WL_RUNNING);
-                    again = 1;
+                if (!grew && atomicCAS(&L.wl_state[t], WL_RUNNING, WL_IDLE) != WL_RUNNING) {
+                    atomicExch(&L.wl_state[t], WL_RUNNING);  // a neighbour raised the halo meanwhile
+                    again = 2;
                 }
+                const int n = __popc(qm), less = again ? 0 : 1;
+                if (n || less)
+                    at = (unsigned)(atomicAdd(&L.sh->tp, ((unsigned long long)n << 32) + (unsigned long long)(long long)(n - less)) >> 32);
             }
-            if (!__shfl_sync(FULL, again, 0)) break;
+            at = __shfl_sync(FULL, at, 0);
+            if (queue >= 0) wl_put(L, at + __popc(qm & ((1u << lane) - 1u)), ((unsigned)ti << ITEM_BITS) | (unsigned)queue);
+            again = __shfl_sync(FULL, again, 0);
+            __syncwarp();
+            if (again == 1) continue;  // the fresher halo may raise pixels: check again
+            if (!again) break;
             visits++;
             __threadfence();
             if (__any_sync(FULL, ld_vol(&L.sh->err) != 0)) break;
