@@ -15,9 +15,8 @@
 //  * a row sweep gives each lane two adjacent columns, a column sweep two
 //    adjacent rows; the pair is updated with 16x2-bit SIMD max/min
 //    (new = min(max(R, max of the three pixels of the line before), M)),
-//    the two outer neighbours come from the adjacent lanes by shuffle, and
-//    the halo reaches the edge lanes as a third operand of the max (the
-//    other lanes read zeros there), so no lane needs a branch or a select;
+//    and the two outer neighbours come from the adjacent lanes by shuffle; the
+//    halo is let into the border pixels once, before the first round;
 //  * a sweep reads each block once per two lines and never reads what
 //    another lane stored during it.
 // After each round an exact, chain-free test decides whether another is
@@ -45,39 +44,24 @@ constexpr unsigned FULL = 0xffffffffu;
 // first line of each pair (row -1, column -1) in bits 0-7, the second
 // (row RT, column RT) in bits 16-23, which is where a pixel pair of the
 // neighbouring edge lane needs it; the corners appear in a row and in a
-// column line.  Z is a line of zeros, the halo operand of the inner lanes.
-// B0 keeps the four border lines as they were when neighbours were last
+// column line.  B0 keeps the four border lines as they were when neighbours were last
 // queued for them (top, bottom, left, right).
 struct WarpTile {
     uint2 B[NB * BS];
     uint32_t HRow[2][HL];
     uint32_t HC[2][HL];
-    uint32_t Z[HL];
     uint8_t HMr[2][HL + 2];  // M of the halo rows
     uint8_t HMc[2][HL + 2];  // M of the halo columns
     uint8_t B0[4][RT];
     int flags[9];            // neighbours to queue: up, down, left, right, UL, UR, DL, DR, self
 };
 
-// R / M byte of interior pixel (y, x)
-__device__ __forceinline__ uint8_t& rpx(WarpTile& S, int y, int x) {
-    return reinterpret_cast<uint8_t*>(&S.B[(y >> 1) * BS + (x >> 1)].x)[((y & 1) << 1) | (x & 1)];
-}
-__device__ __forceinline__ uint8_t mpx(const WarpTile& S, int y, int x) {
-    return reinterpret_cast<const uint8_t*>(&S.B[(y >> 1) * BS + (x >> 1)].y)[((y & 1) << 1) | (x & 1)];
-}
-// R and M of halo pixel (hy, hx)
+// R of halo pixel (hy, hx), and setting its R and M
 __device__ __forceinline__ int halo_r(const WarpTile& S, int hy, int hx) {
     if (hy == -1) return (int)(S.HRow[0][hx + 1] & 0xffu);
     if (hy == RT) return (int)(S.HRow[1][hx + 1] >> 16);
     if (hx == -1) return (int)(S.HC[0][hy + 1] & 0xffu);
     return (int)(S.HC[1][hy + 1] >> 16);
-}
-__device__ __forceinline__ int halo_m(const WarpTile& S, int hy, int hx) {
-    if (hy == -1) return S.HMr[0][hx + 1];
-    if (hy == RT) return S.HMr[1][hx + 1];
-    if (hx == -1) return S.HMc[0][hy + 1];
-    return S.HMc[1][hy + 1];
 }
 __device__ __forceinline__ void set_halo_r(WarpTile& S, int hy, int hx, uint32_t r) {
     if (hy == -1) S.HRow[0][hx + 1] = r;
@@ -109,9 +93,6 @@ constexpr uint32_t ROW0 = 0x4140, ROW1 = 0x4342, COL0 = 0x4240, COL1 = 0x4341;
 constexpr uint32_t PACK_ROWS = 0x6420, PACK_COLS = 0x6240;
 // (left neighbour's high lane, own low lane) and (own high lane, right neighbour's low lane)
 constexpr uint32_t FROM_LEFT = 0x1076, FROM_RIGHT = 0x5432;
-// two halo-line words -> a pixel pair (first line: bits 0-7; second line: bits 16-23)
-constexpr uint32_t LINE0_PAIR = 0x5410, LINE1_PAIR = 0x7632;
-
 __device__ __forceinline__ int ld_vol(const int* p) { return *(const volatile int*)p; }
 
 __device__ __forceinline__ bool budget_over(long long t0, long long budget) {
@@ -409,25 +390,23 @@ __device__ __forceinline__ bool merge_halo(WarpTile& S, const uint8_t hr[9], int
 // and values only grow towards the unique fixed point whatever the order.
 // P is the pixel pair of the line before (columns 2l, 2l + 1); its outer
 // neighbours come from lanes l - 1 and l + 1 (the edge lanes get their own
-// pair back, harmlessly, and the halo column through E).
-__device__ __forceinline__ uint32_t line_step(uint32_t& P, uint32_t R, uint32_t M, uint32_t e) {
+// pair back: its far pixel is a neighbour too).  The halo takes no part: it
+// has been let into the border pixels before (let_in_halo).
+__device__ __forceinline__ uint32_t line_step(uint32_t& P, uint32_t R, uint32_t M) {
     const uint32_t L = __shfl_up_sync(FULL, P, 1), Rt = __shfl_down_sync(FULL, P, 1);
-    const uint32_t w = __vimax3_u16x2(__byte_perm(P, L, FROM_LEFT), P, __byte_perm(P, Rt, FROM_RIGHT));
-    P = min2(__vimax3_u16x2(R, w, e), M);
+    P = min2(__vimax3_u16x2(__byte_perm(P, L, FROM_LEFT), __byte_perm(P, Rt, FROM_RIGHT), max2(P, R)), M);
     return P;
 }
 
 __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
-    const uint32_t* E = lane == 0 ? S.HC[0] : lane == 31 ? S.HC[1] : S.Z;
-    uint32_t Pd = __byte_perm(S.HRow[0][2 * lane + 1], S.HRow[0][2 * lane + 2], LINE0_PAIR);
-    uint32_t Pu = __byte_perm(S.HRow[1][2 * lane + 1], S.HRow[1][2 * lane + 2], LINE1_PAIR);
+    uint32_t Pd = 0u, Pu = 0u;
     // down: block row k, rows 2k then 2k + 1; up: block row NB-1-k, rows 2(NB-1-k) + 1 then 2(NB-1-k)
     auto step = [&](uint2 bd, uint2 bu, int k) {
         const int jd = k, ju = NB - 1 - k;
-        const uint32_t d0 = line_step(Pd, __byte_perm(bd.x, 0u, ROW0), __byte_perm(bd.y, 0u, ROW0), E[2 * jd]);
-        const uint32_t u1 = line_step(Pu, __byte_perm(bu.x, 0u, ROW1), __byte_perm(bu.y, 0u, ROW1), E[2 * ju + 3]);
-        const uint32_t d1 = line_step(Pd, __byte_perm(bd.x, 0u, ROW1), __byte_perm(bd.y, 0u, ROW1), E[2 * jd + 1]);
-        const uint32_t u0 = line_step(Pu, __byte_perm(bu.x, 0u, ROW0), __byte_perm(bu.y, 0u, ROW0), E[2 * ju + 2]);
+        const uint32_t d0 = line_step(Pd, __byte_perm(bd.x, 0u, ROW0), __byte_perm(bd.y, 0u, ROW0));
+        const uint32_t u1 = line_step(Pu, __byte_perm(bu.x, 0u, ROW1), __byte_perm(bu.y, 0u, ROW1));
+        const uint32_t d1 = line_step(Pd, __byte_perm(bd.x, 0u, ROW1), __byte_perm(bd.y, 0u, ROW1));
+        const uint32_t u0 = line_step(Pu, __byte_perm(bu.x, 0u, ROW0), __byte_perm(bu.y, 0u, ROW0));
         S.B[jd * BS + lane].x = __byte_perm(d0, d1, PACK_ROWS);
         S.B[ju * BS + lane].x = __byte_perm(u0, u1, PACK_ROWS);
     };
@@ -454,18 +433,15 @@ __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
 }
 
 // The column sweep pair: right (columns 0 -> RT-1) and left (RT-1 -> 0) at
-// once, lane l owning block row l (rows 2l, 2l + 1) in both chains; the halo
-// rows reach the edge lanes through E.
+// once, lane l owning block row l (rows 2l, 2l + 1) in both chains.
 __device__ __forceinline__ void col_sweeps(WarpTile& S, int lane) {
-    const uint32_t* E = lane == 0 ? S.HRow[0] : lane == 31 ? S.HRow[1] : S.Z;
-    uint32_t Cr = __byte_perm(S.HC[0][2 * lane + 1], S.HC[0][2 * lane + 2], LINE0_PAIR);
-    uint32_t Cl = __byte_perm(S.HC[1][2 * lane + 1], S.HC[1][2 * lane + 2], LINE1_PAIR);
+    uint32_t Cr = 0u, Cl = 0u;
     auto step = [&](uint2 br, uint2 bl, int k) {
         const int ir = k, il = NB - 1 - k;
-        const uint32_t r0 = line_step(Cr, __byte_perm(br.x, 0u, COL0), __byte_perm(br.y, 0u, COL0), E[2 * ir]);
-        const uint32_t l1 = line_step(Cl, __byte_perm(bl.x, 0u, COL1), __byte_perm(bl.y, 0u, COL1), E[2 * il + 3]);
-        const uint32_t r1 = line_step(Cr, __byte_perm(br.x, 0u, COL1), __byte_perm(br.y, 0u, COL1), E[2 * ir + 1]);
-        const uint32_t l0 = line_step(Cl, __byte_perm(bl.x, 0u, COL0), __byte_perm(bl.y, 0u, COL0), E[2 * il + 2]);
+        const uint32_t r0 = line_step(Cr, __byte_perm(br.x, 0u, COL0), __byte_perm(br.y, 0u, COL0));
+        const uint32_t l1 = line_step(Cl, __byte_perm(bl.x, 0u, COL1), __byte_perm(bl.y, 0u, COL1));
+        const uint32_t r1 = line_step(Cr, __byte_perm(br.x, 0u, COL1), __byte_perm(br.y, 0u, COL1));
+        const uint32_t l0 = line_step(Cl, __byte_perm(bl.x, 0u, COL0), __byte_perm(bl.y, 0u, COL0));
         S.B[lane * BS + ir].x = __byte_perm(r0, r1, PACK_COLS);
         S.B[lane * BS + il].x = __byte_perm(l0, l1, PACK_COLS);
     };
@@ -501,24 +477,23 @@ __device__ __forceinline__ void sweep_round(WarpTile& S, int lane) {
 }
 
 // Whether some pixel of the tile can still be raised by one of its 8
-// neighbours: the exact convergence test, two pixels per lane and row, with
-// no dependent chain; it stops at the first 16-row group that has one.
+// neighbours in the tile: the exact convergence test, two pixels per lane and
+// row, with no dependent chain; it stops at the first 16-row group that has one.
 __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
-    const uint32_t* E = lane == 0 ? S.HC[0] : lane == 31 ? S.HC[1] : S.Z;
-    // maximum of R over the three columns around each pixel of a pair in row y
-    auto hmax = [&](uint32_t R, int y) -> uint32_t {
+    // maximum of R over the three columns around each pixel of a pair of a row
+    auto hmax = [&](uint32_t R) -> uint32_t {
         const uint32_t L = __shfl_up_sync(FULL, R, 1), Rt = __shfl_down_sync(FULL, R, 1);
-        return __vimax3_u16x2(__byte_perm(R, L, FROM_LEFT), __byte_perm(R, Rt, FROM_RIGHT), max2(R, E[y + 1]));
+        return __vimax3_u16x2(__byte_perm(R, L, FROM_LEFT), __byte_perm(R, Rt, FROM_RIGHT), R);
     };
-    uint32_t hp = hmax(__byte_perm(S.HRow[0][2 * lane + 1], S.HRow[0][2 * lane + 2], LINE0_PAIR), -1);
+    uint32_t hp = 0u;
     uint2 b = S.B[lane];
     uint32_t R0 = __byte_perm(b.x, 0u, ROW0), M0 = __byte_perm(b.y, 0u, ROW0);
-    uint32_t h0 = hmax(R0, 0);
+    uint32_t h0 = hmax(R0);
     bool v = false;
     // block row j: rows 2j (R0, M0, h0) and 2j + 1; R2 is row 2j + 2
     auto block_row = [&](uint32_t R2, uint32_t M2, int j) {
         const uint32_t R1 = __byte_perm(b.x, 0u, ROW1), M1 = __byte_perm(b.y, 0u, ROW1);
-        const uint32_t h1 = hmax(R1, 2 * j + 1), h2 = hmax(R2, 2 * j + 2);
+        const uint32_t h1 = hmax(R1), h2 = hmax(R2);
         v |= min2(__vimax3_u16x2(hp, h0, h1), M0) != R0;
         v |= min2(__vimax3_u16x2(h0, h1, h2), M1) != R1;
         hp = h1;
@@ -536,7 +511,7 @@ __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
                 block_row(__byte_perm(nb.x, 0u, ROW0), __byte_perm(nb.y, 0u, ROW0), j);
                 b = nb;
             } else {
-                block_row(__byte_perm(S.HRow[1][2 * lane + 1], S.HRow[1][2 * lane + 2], LINE1_PAIR), 0u, j);
+                block_row(0u, 0u, j);
             }
         }
         if (__any_sync(FULL, v)) return true;
@@ -544,42 +519,37 @@ __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
     return false;
 }
 
-// Whether a halo pixel can raise a pixel of the tile border.  When the
-// tile's interior was at a fixed point before the halo grew, only border
-// pixels can have become raisable, so this is the exact test in that case.
-__device__ __forceinline__ bool border_can_raise(WarpTile& S, int lane) {
-    // lane l: border pixels 2l and 2l + 1 of each side from one block word of
-    // R and one of M, and the four halo pixels around them (the halo lines
-    // hold the corners too, with the same values as the halo rows)
-    const uint2 bt = S.B[lane], bb = S.B[(NB - 1) * BS + lane];
-    const uint2 bl = S.B[lane * BS], br = S.B[lane * BS + NB - 1];
+// Lets the halo into the tile: raises each border pixel by the halo pixels
+// around it; true if one grew.  The halo only acts through the border, so the
+// sweeps and the test need not look at it (they read a halo word per line
+// before), and when the tile was at a fixed point before the halo grew, no
+// pixel can be raised if no border pixel grew here.
+__device__ __forceinline__ bool let_in_halo(WarpTile& S, int lane) {
+    // lane l: border pixels 2l and 2l + 1 of a side in one block word, and the
+    // four halo pixels around them (the halo lines hold the corners too, with
+    // the same values as the halo rows)
     const int i = 2 * lane;
-    auto raisable = [](int h0, int h1, int h2, uint32_t r, uint32_t m, int sh) -> bool {
-        const int mh = max(max(h0, h1), h2);
-        return min(mh, (int)((m >> sh) & 0xffu)) > (int)((r >> sh) & 0xffu);
-    };
     bool v = false;
-    {
-        const int a = S.HRow[0][i] & 0xff, b = S.HRow[0][i + 1] & 0xff, c = S.HRow[0][i + 2] & 0xff,
-                  d = S.HRow[0][i + 3] & 0xff;
-        v |= raisable(a, b, c, bt.x, bt.y, 0) | raisable(b, c, d, bt.x, bt.y, 8);  // top row
-    }
-    {
-        const int a = S.HRow[1][i] >> 16, b = S.HRow[1][i + 1] >> 16, c = S.HRow[1][i + 2] >> 16,
-                  d = S.HRow[1][i + 3] >> 16;
-        v |= raisable(a, b, c, bb.x, bb.y, 16) | raisable(b, c, d, bb.x, bb.y, 24);  // bottom row
-    }
-    {
-        const int a = S.HC[0][i] & 0xff, b = S.HC[0][i + 1] & 0xff, c = S.HC[0][i + 2] & 0xff,
-                  d = S.HC[0][i + 3] & 0xff;
-        v |= raisable(a, b, c, bl.x, bl.y, 0) | raisable(b, c, d, bl.x, bl.y, 16);  // left column
-    }
-    {
-        const int a = S.HC[1][i] >> 16, b = S.HC[1][i + 1] >> 16, c = S.HC[1][i + 2] >> 16,
-                  d = S.HC[1][i + 3] >> 16;
-        v |= raisable(a, b, c, br.x, br.y, 8) | raisable(b, c, d, br.x, br.y, 24);  // right column
-    }
-    return __any_sync(FULL, v);
+    // pixels at bits s0 and s1 of w.x, under the halo values a, b, c, d
+    auto raise = [&](uint2* w, int a, int b, int c, int d, int s0, int s1) {
+        const uint2 q = *w;
+        const int r0 = (int)((q.x >> s0) & 0xffu), r1 = (int)((q.x >> s1) & 0xffu);
+        const int n0 = max(r0, min(max(max(a, b), c), (int)((q.y >> s0) & 0xffu)));
+        const int n1 = max(r1, min(max(max(b, c), d), (int)((q.y >> s1) & 0xffu)));
+        if (n0 != r0 || n1 != r1) {
+            w->x = q.x + ((uint32_t)(n0 - r0) << s0) + ((uint32_t)(n1 - r1) << s1);
+            v = true;
+        }
+    };
+    raise(&S.B[lane], S.HRow[0][i] & 0xff, S.HRow[0][i + 1] & 0xff, S.HRow[0][i + 2] & 0xff, S.HRow[0][i + 3] & 0xff, 0, 8);
+    raise(&S.B[(NB - 1) * BS + lane], S.HRow[1][i] >> 16, S.HRow[1][i + 1] >> 16, S.HRow[1][i + 2] >> 16,
+          S.HRow[1][i + 3] >> 16, 16, 24);
+    __syncwarp();  // the corner blocks belong to a row and to a column
+    raise(&S.B[lane * BS], S.HC[0][i] & 0xff, S.HC[0][i + 1] & 0xff, S.HC[0][i + 2] & 0xff, S.HC[0][i + 3] & 0xff, 0, 16);
+    raise(&S.B[lane * BS + NB - 1], S.HC[1][i] >> 16, S.HC[1][i + 1] >> 16, S.HC[1][i + 2] >> 16, S.HC[1][i + 3] >> 16, 8, 24);
+    const bool any = __any_sync(FULL, v);
+    __syncwarp();
+    return any;
 }
 
 // ---- neighbour requests ---------------------------------------------------------------
@@ -660,7 +630,6 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
     const int lane = threadIdx.x;
     int visits = 0;  // tile processings of this worker (diagnostic), added once at exit
     if (lane < 9) S.flags[lane] = 0;
-    for (int i = lane; i < HL; i += 32) S.Z[i] = 0u;
     __syncwarp();
     for (;;) {
         unsigned item = 0;
@@ -704,7 +673,7 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
         for (;;) {
             int nr = 0, queue = -1;
             bool more = false;
-            bool go = sweep_now || (full_check ? can_raise(S, lane) : border_can_raise(S, lane));
+            bool go = let_in_halo(S, lane) || sweep_now || (full_check && can_raise(S, lane));
             sweep_now = false;
             while (go) {
                 if (nr >= MAX_ROUNDS) { more = true; break; }
