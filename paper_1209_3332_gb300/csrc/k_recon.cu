@@ -76,7 +76,9 @@ __device__ __forceinline__ void set_halo_m(WarpTile& S, int hy, int hx, uint8_t 
     if (hx == RT) S.HMc[1][hy + 1] = m;
 }
 
-// 16x2-bit SIMD helpers (values are bytes zero-extended to 16-bit lanes)
+// 16x2-bit SIMD helpers.  A pixel pair is two 16-bit lanes with the pixel in
+// the high byte; the low bytes are left as they come, since they cannot change
+// the high byte of a maximum or a minimum, so no permute has to clear them.
 __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -88,11 +90,16 @@ __device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
     return d;
 }
 // byte permutes: a block word -> the pixel pair of row a (ROW0/ROW1) or of
-// column b (COL0/COL1) as two 16-bit lanes; two row or column pairs -> a block word
-constexpr uint32_t ROW0 = 0x4140, ROW1 = 0x4342, COL0 = 0x4240, COL1 = 0x4341;
-constexpr uint32_t PACK_ROWS = 0x6420, PACK_COLS = 0x6240;
-// (left neighbour's high lane, own low lane) and (own high lane, right neighbour's low lane)
-constexpr uint32_t FROM_LEFT = 0x1076, FROM_RIGHT = 0x5432;
+// column 0 (COL0; the pair of column 1 is the word itself); two row or column
+// pairs -> a block word
+constexpr uint32_t ROW0 = 0x1404, ROW1 = 0x3424, COL0 = 0x2404;
+constexpr uint32_t PACK_ROWS = 0x7531, PACK_COLS = 0x7351;
+// the two chains' pairs as one word for the shuffles: bytes 0 and 2 of the
+// first, 1 and 3 of the second; and back: (left neighbour's second pixel, own
+// first) and (own second, right neighbour's first) of either chain
+constexpr uint32_t PACK_CHAINS = 0x7351;
+constexpr uint32_t LEFT_A = 0x4020, RIGHT_A = 0x4020, LEFT_B = 0x5030, RIGHT_B = 0x5030;
+
 __device__ __forceinline__ int ld_vol(const int* p) { return *(const volatile int*)p; }
 
 __device__ __forceinline__ bool budget_over(long long t0, long long budget) {
@@ -388,14 +395,16 @@ __device__ __forceinline__ bool merge_halo(WarpTile& S, const uint8_t hr[9], int
 // chain is still one full directional sweep (every row after the line
 // before it), so a round of the two pairs propagates as the four sweeps do,
 // and values only grow towards the unique fixed point whatever the order.
-// P is the pixel pair of the line before (columns 2l, 2l + 1); its outer
-// neighbours come from lanes l - 1 and l + 1 (the edge lanes get their own
-// pair back: its far pixel is a neighbour too).  The halo takes no part: it
-// has been let into the border pixels before (let_in_halo).
-__device__ __forceinline__ uint32_t line_step(uint32_t& P, uint32_t R, uint32_t M) {
+// A and B are the two chains' pixel pairs of the line before; their outer
+// neighbours come from lanes l - 1 and l + 1, both chains in one word per
+// direction (the edge lanes get their own pair back: its far pixel is a
+// neighbour too).  The halo takes no part: it has been let into the border
+// pixels before (let_in_halo).
+__device__ __forceinline__ void line_step(uint32_t& A, uint32_t& B, uint32_t RA, uint32_t MA, uint32_t RB, uint32_t MB) {
+    const uint32_t P = __byte_perm(A, B, PACK_CHAINS);
     const uint32_t L = __shfl_up_sync(FULL, P, 1), Rt = __shfl_down_sync(FULL, P, 1);
-    P = min2(__vimax3_u16x2(__byte_perm(P, L, FROM_LEFT), __byte_perm(P, Rt, FROM_RIGHT), max2(P, R)), M);
-    return P;
+    A = min2(__vimax3_u16x2(__byte_perm(L, P, LEFT_A), __byte_perm(P, Rt, RIGHT_A), max2(A, RA)), MA);
+    B = min2(__vimax3_u16x2(__byte_perm(L, P, LEFT_B), __byte_perm(P, Rt, RIGHT_B), max2(B, RB)), MB);
 }
 
 __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
@@ -403,10 +412,12 @@ __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
     // down: block row k, rows 2k then 2k + 1; up: block row NB-1-k, rows 2(NB-1-k) + 1 then 2(NB-1-k)
     auto step = [&](uint2 bd, uint2 bu, int k) {
         const int jd = k, ju = NB - 1 - k;
-        const uint32_t d0 = line_step(Pd, __byte_perm(bd.x, 0u, ROW0), __byte_perm(bd.y, 0u, ROW0));
-        const uint32_t u1 = line_step(Pu, __byte_perm(bu.x, 0u, ROW1), __byte_perm(bu.y, 0u, ROW1));
-        const uint32_t d1 = line_step(Pd, __byte_perm(bd.x, 0u, ROW1), __byte_perm(bd.y, 0u, ROW1));
-        const uint32_t u0 = line_step(Pu, __byte_perm(bu.x, 0u, ROW0), __byte_perm(bu.y, 0u, ROW0));
+        line_step(Pd, Pu, __byte_perm(bd.x, 0u, ROW0), __byte_perm(bd.y, 0u, ROW0), __byte_perm(bu.x, 0u, ROW1),
+                  __byte_perm(bu.y, 0u, ROW1));
+        const uint32_t d0 = Pd, u1 = Pu;
+        line_step(Pd, Pu, __byte_perm(bd.x, 0u, ROW1), __byte_perm(bd.y, 0u, ROW1), __byte_perm(bu.x, 0u, ROW0),
+                  __byte_perm(bu.y, 0u, ROW0));
+        const uint32_t d1 = Pd, u0 = Pu;
         S.B[jd * BS + lane].x = __byte_perm(d0, d1, PACK_ROWS);
         S.B[ju * BS + lane].x = __byte_perm(u0, u1, PACK_ROWS);
     };
@@ -438,10 +449,10 @@ __device__ __forceinline__ void col_sweeps(WarpTile& S, int lane) {
     uint32_t Cr = 0u, Cl = 0u;
     auto step = [&](uint2 br, uint2 bl, int k) {
         const int ir = k, il = NB - 1 - k;
-        const uint32_t r0 = line_step(Cr, __byte_perm(br.x, 0u, COL0), __byte_perm(br.y, 0u, COL0));
-        const uint32_t l1 = line_step(Cl, __byte_perm(bl.x, 0u, COL1), __byte_perm(bl.y, 0u, COL1));
-        const uint32_t r1 = line_step(Cr, __byte_perm(br.x, 0u, COL1), __byte_perm(br.y, 0u, COL1));
-        const uint32_t l0 = line_step(Cl, __byte_perm(bl.x, 0u, COL0), __byte_perm(bl.y, 0u, COL0));
+        line_step(Cr, Cl, __byte_perm(br.x, 0u, COL0), __byte_perm(br.y, 0u, COL0), bl.x, bl.y);
+        const uint32_t r0 = Cr, l1 = Cl;
+        line_step(Cr, Cl, br.x, br.y, __byte_perm(bl.x, 0u, COL0), __byte_perm(bl.y, 0u, COL0));
+        const uint32_t r1 = Cr, l0 = Cl;
         S.B[lane * BS + ir].x = __byte_perm(r0, r1, PACK_COLS);
         S.B[lane * BS + il].x = __byte_perm(l0, l1, PACK_COLS);
     };
@@ -480,41 +491,37 @@ __device__ __forceinline__ void sweep_round(WarpTile& S, int lane) {
 // neighbours in the tile: the exact convergence test, two pixels per lane and
 // row, with no dependent chain; it stops at the first 16-row group that has one.
 __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
-    // maximum of R over the three columns around each pixel of a pair of a row
-    auto hmax = [&](uint32_t R) -> uint32_t {
-        const uint32_t L = __shfl_up_sync(FULL, R, 1), Rt = __shfl_down_sync(FULL, R, 1);
-        return __vimax3_u16x2(__byte_perm(R, L, FROM_LEFT), __byte_perm(R, Rt, FROM_RIGHT), R);
+    // maxima of R over the three columns around each pixel, for the two rows
+    // of a block row: the neighbours' block words hold both rows
+    auto hmax = [&](uint32_t w, uint32_t& top, uint32_t& bot) {
+        const uint32_t L = __shfl_up_sync(FULL, w, 1), Rt = __shfl_down_sync(FULL, w, 1);
+        top = __vimax3_u16x2(__byte_perm(L, w, 0x4010), __byte_perm(w, Rt, 0x4010), __byte_perm(w, 0u, ROW0));
+        bot = __vimax3_u16x2(__byte_perm(L, w, 0x6030), __byte_perm(w, Rt, 0x6030), __byte_perm(w, 0u, ROW1));
     };
-    uint32_t hp = 0u;
+    uint32_t hp = 0u, h0, h1;  // maxima of the row before block row j, and of its two rows
     uint2 b = S.B[lane];
-    uint32_t R0 = __byte_perm(b.x, 0u, ROW0), M0 = __byte_perm(b.y, 0u, ROW0);
-    uint32_t h0 = hmax(R0);
-    bool v = false;
-    // block row j: rows 2j (R0, M0, h0) and 2j + 1; R2 is row 2j + 2
-    auto block_row = [&](uint32_t R2, uint32_t M2, int j) {
-        const uint32_t R1 = __byte_perm(b.x, 0u, ROW1), M1 = __byte_perm(b.y, 0u, ROW1);
-        const uint32_t h1 = hmax(R1), h2 = hmax(R2);
-        v |= min2(__vimax3_u16x2(hp, h0, h1), M0) != R0;
-        v |= min2(__vimax3_u16x2(h0, h1, h2), M1) != R1;
-        hp = h1;
-        h0 = h2;
-        R0 = R2;
-        M0 = M2;
-    };
+    hmax(b.x, h0, h1);
+    uint32_t v = 0u;
 #pragma unroll 1
     for (int g = 0; g < NB / 8; g++) {
 #pragma unroll
         for (int jj = 0; jj < 8; jj++) {
             const int j = g * 8 + jj;
+            uint2 nb = make_uint2(0u, 0u);
+            uint32_t n0 = 0u, n1 = 0u;
             if (j + 1 < NB) {
-                const uint2 nb = S.B[(j + 1) * BS + lane];
-                block_row(__byte_perm(nb.x, 0u, ROW0), __byte_perm(nb.y, 0u, ROW0), j);
-                b = nb;
-            } else {
-                block_row(0u, 0u, j);
+                nb = S.B[(j + 1) * BS + lane];
+                hmax(nb.x, n0, n1);
             }
+            const uint32_t r0 = min2(__vimax3_u16x2(hp, h0, h1), __byte_perm(b.y, 0u, ROW0));
+            const uint32_t r1 = min2(__vimax3_u16x2(h0, h1, n0), __byte_perm(b.y, 0u, ROW1));
+            v |= __byte_perm(r0, r1, PACK_ROWS) ^ b.x;
+            hp = h1;
+            h0 = n0;
+            h1 = n1;
+            b = nb;
         }
-        if (__any_sync(FULL, v)) return true;
+        if (__any_sync(FULL, v != 0u)) return true;
     }
     return false;
 }
