@@ -30,7 +30,8 @@ struct TileDev {
     size_t pitch;                 // RGB row pitch in bytes
     const uint8_t* rgb;
     uint8_t* hem8;                // H*W
-    uint8_t* R;                   // H*W reconstruction (workspace)
+    uint8_t* R;                   // reconstruction (workspace), rows of rp bytes
+    int rp;                       // W rounded up to 16: R's rows start on 16-byte boundaries
     int32_t* labels;              // H*W
     int32_t* edt;                 // H*W (may be null: EDT skipped)
     int32_t* n_objects;           // [1]
@@ -105,6 +106,47 @@ __device__ __forceinline__ void set_status(int* status, int code) {
     atomicCAS(status, 0, code);
 }
 
+// 4 N consecutive bytes from p on, any alignment, from N + 1 aligned words; all
+// of [p - 3, p + 4 N + 4) must be readable.
+template <int N>
+__device__ __forceinline__ void load_unaligned(const uint8_t* p, uint32_t (&out)[N]) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(a & ~(uintptr_t)3);
+    const uint32_t sel = 0x3210u + 0x1111u * (uint32_t)(a & 3);
+    uint32_t v[N + 1];
+#pragma unroll
+    for (int i = 0; i <= N; i++) v[i] = __ldg(w + i);
+#pragma unroll
+    for (int i = 0; i < N; i++) out[i] = __byte_perm(v[i], v[i + 1], sel);
+}
+
+// zeroes the pixels from n on (n < 16)
+__device__ __forceinline__ uint4 clip_px16(uint4 v, int n) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; i++) w[i] &= n >= 4 * i + 4 ? 0xffffffffu : n <= 4 * i ? 0u : (1u << (8 * (n - 4 * i))) - 1u;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Pixels x .. x + 15 of row y of a W x H byte plane, 0 beyond the row's end: a
+// 16-byte load where that is aligned, the aligned words that hold them where
+// these lie within the plane, bytes otherwise.  x < W, y < H.
+__device__ __forceinline__ uint4 load_px16(const uint8_t* __restrict__ plane, int W, int H, int x, int y) {
+    const uint8_t* p = plane + (size_t)y * W + x;
+    const int n = W - x;  // valid pixels
+    if (n >= 16 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) return __ldg(reinterpret_cast<const uint4*>(p));
+    uint32_t w[4] = {0, 0, 0, 0};
+    const size_t left = (size_t)(H - y) * W - x;  // bytes of the plane from p on
+    if (left >= 20 && p >= plane + 3) {
+        load_unaligned<4>(p, w);
+        if (n < 16) return clip_px16(make_uint4(w[0], w[1], w[2], w[3]), n);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; k++)
+            if (k < n) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
 // Object boxes from one row segment of FB_SEG labels, one warp: each lane
 // reads 4 labels at a time; the lanes holding the same label (one
 // __match_any_sync group per label value) combine their column range and

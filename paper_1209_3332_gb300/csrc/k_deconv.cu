@@ -64,13 +64,23 @@ __device__ __forceinline__ void deconv_item(const TileDev* __restrict__ tiles, i
     int x0 = cx * 16;
     const uint8_t* src = t.rgb + (size_t)y * t.pitch + (size_t)x0 * 3;
     uint8_t* dh = t.hem8 + (size_t)y * t.W + x0;
-    uint8_t* dr = t.R + (size_t)y * t.W + x0;
-    bool full = x0 + 16 <= t.W;
-    if (full && ((reinterpret_cast<uintptr_t>(src) & 15) == 0)) {
-        uint4 a = __ldcs(reinterpret_cast<const uint4*>(src));
-        uint4 b = __ldcs(reinterpret_cast<const uint4*>(src) + 1);
-        uint4 c = __ldcs(reinterpret_cast<const uint4*>(src) + 2);
-        uint32_t w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+    uint8_t* dr = t.R + (size_t)y * t.rp + x0;
+    // rows that do not start on 16-byte boundaries (odd widths) are read as the
+    // aligned words around them, except at the buffer's ends
+    const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+    const bool inside = (y > 0 || x0 > 0) && (y + 1 < t.H || x0 + 18 <= t.W);
+    if (x0 + 16 <= t.W && (aligned || inside)) {
+        uint32_t w[12];
+        if (aligned) {
+            const uint4 a = __ldcs(reinterpret_cast<const uint4*>(src));
+            const uint4 b = __ldcs(reinterpret_cast<const uint4*>(src) + 1);
+            const uint4 c = __ldcs(reinterpret_cast<const uint4*>(src) + 2);
+            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+            w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+            w[8] = c.x; w[9] = c.y; w[10] = c.z; w[11] = c.w;
+        } else {
+            load_unaligned<12>(src, w);
+        }
         uint32_t hv[4] = {0, 0, 0, 0}, rv[4] = {0, 0, 0, 0}, mkmax = 0;
         // byte k of the 48 loaded bytes, zero-extended
         auto byte_at = [&](int k) -> uint32_t { return __byte_perm(w[k >> 2], 0u, 0x4440 | (k & 3)); };
@@ -83,15 +93,19 @@ __device__ __forceinline__ void deconv_item(const TileDev* __restrict__ tiles, i
             mkmax = max(mkmax, mk);
         }
         if (rt_src && mkmax >= SRC_MARKER) rt_src[t.rt_base + (y / RT) * t.rtx + x0 / RT] = 1;
-        if ((reinterpret_cast<uintptr_t>(dh) & 15) == 0 && (reinterpret_cast<uintptr_t>(dr) & 15) == 0) {
+        *reinterpret_cast<uint4*>(dr) = make_uint4(rv[0], rv[1], rv[2], rv[3]);
+        const unsigned a = (unsigned)(reinterpret_cast<uintptr_t>(dh) & 3);
+        if ((reinterpret_cast<uintptr_t>(dh) & 15) == 0) {
             *reinterpret_cast<uint4*>(dh) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-            *reinterpret_cast<uint4*>(dr) = make_uint4(rv[0], rv[1], rv[2], rv[3]);
-        } else {
+        } else if (a == 0) {
 #pragma unroll
-            for (int p = 0; p < 16; p++) {
-                dh[p] = (uint8_t)(hv[p >> 2] >> ((p & 3) * 8));
-                dr[p] = (uint8_t)(rv[p >> 2] >> ((p & 3) * 8));
-            }
+            for (int i = 0; i < 4; i++) reinterpret_cast<uint32_t*>(dh)[i] = hv[i];
+        } else {  // 4 - a bytes, three words, a bytes
+            const unsigned head = 4 - a, sel = 0x3210u + 0x1111u * head;
+            for (unsigned i = 0; i < head; i++) dh[i] = (uint8_t)(hv[0] >> (8 * i));
+#pragma unroll
+            for (int i = 0; i < 3; i++) reinterpret_cast<uint32_t*>(dh + head)[i] = __byte_perm(hv[i], hv[i + 1], sel);
+            for (unsigned i = 0; i < a; i++) dh[12 + head + i] = (uint8_t)(hv[3] >> (8 * (head + i)));
         }
     } else {
         int n = min(16, t.W - x0);

@@ -275,38 +275,32 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_fill_local(Launch L) {
     // has no borrow between bytes; each byte plus 256 - thr (in its own
     // 16-bit lane) carries into bit 8 of the lane exactly when it is >= thr
     const uint32_t bias2 = (uint32_t)max(0, 256 - L.thr) * 0x00010001u;
-    if (g.bw == 32 && (T.W & 15) == 0 &&
-        ((reinterpret_cast<uintptr_t>(T.hem8) | reinterpret_cast<uintptr_t>(T.R)) & 15) == 0) {
-        // lanes 2r and 2r+1 read the two 16-byte halves of row r (then of row
-        // r+16), so every load covers 16 whole sectors; each half yields 16
-        // foreground bits, and two shuffles assemble row y's word in lane y
-        uint32_t half[2];
+    // lanes 2r and 2r+1 read the two 16-pixel halves of row r (then of row
+    // r+16), so every load covers whole sectors; each half yields 16 foreground
+    // bits, and two shuffles assemble row y's word in lane y
+    uint32_t half[2];
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int row = (lane >> 1) + 16 * i;
-            half[i] = 0;
-            if (row < g.bh) {
-                const size_t o = (size_t)(g.y0 + row) * T.W + g.x0 + (lane & 1) * 16;
-                const uint4 hv = __ldg(reinterpret_cast<const uint4*>(T.hem8 + o));
-                const uint4 rv = __ldcg(reinterpret_cast<const uint4*>(T.R + o));
-                const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, rw[4] = {rv.x, rv.y, rv.z, rv.w};
+    for (int i = 0; i < 2; i++) {
+        const int row = (lane >> 1) + 16 * i, x = g.x0 + (lane & 1) * 16, y = g.y0 + row;
+        half[i] = 0;
+        if (row < g.bh && x < T.W) {
+            const uint4 hv = load_px16(T.hem8, T.W, T.H, x, y);
+            const uint4 rv = __ldcg(reinterpret_cast<const uint4*>(T.R + (size_t)y * T.rp + x));
+            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, rw[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const uint32_t d = hw[k] - rw[k];
-                    const uint32_t e = (d & 0x00ff00ffu) + bias2, o = ((d >> 8) & 0x00ff00ffu) + bias2;
-                    half[i] |= (((e >> 8) & 1u) | ((o >> 7) & 2u) | ((e >> 22) & 4u) | ((o >> 21) & 8u)) << (k * 4);
-                }
+            for (int k = 0; k < 4; k++) {
+                const uint32_t d = hw[k] - rw[k];
+                const uint32_t e = (d & 0x00ff00ffu) + bias2, o = ((d >> 8) & 0x00ff00ffu) + bias2;
+                half[i] |= (((e >> 8) & 1u) | ((o >> 7) & 2u) | ((e >> 22) & 4u) | ((o >> 21) & 8u)) << (k * 4);
             }
         }
+    }
+    {
         const int src = 2 * (lane & 15);
         const uint32_t lo0 = __shfl_sync(FULLM, half[0], src), hi0 = __shfl_sync(FULLM, half[0], src + 1);
         const uint32_t lo1 = __shfl_sync(FULLM, half[1], src), hi1 = __shfl_sync(FULLM, half[1], src + 1);
-        fg = lane < 16 ? (lo0 | (hi0 << 16)) : (lo1 | (hi1 << 16));
-        if (lane >= g.bh) fg = 0;
-    } else if (lane < g.bh) {
-        const size_t o = (size_t)(g.y0 + lane) * T.W + g.x0;
-        for (int x = 0; x < g.bw; x++)
-            if ((int)T.hem8[o + x] - (int)__ldcg(T.R + o + x) >= L.thr) fg |= 1u << x;
+        // (what R's row padding leaves beyond the row's end is masked out)
+        fg = lane < g.bh ? (lane < 16 ? (lo0 | (hi0 << 16)) : (lo1 | (hi1 << 16))) & vm : 0u;
     }
     if (lane < g.bh) T.fgbits[block_word(T, g, lane)] = fg;
     const uint32_t bg = lane < g.bh ? (~fg & vm) : 0u;
@@ -645,11 +639,6 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int wa
             }
         }
     }
-    // label of the run starting at column s of this row
-    auto run_label = [&](int s) -> int {
-        const int v = par[lane * CB + s];
-        return (v & LAB_FLAG) ? (v & ~LAB_FLAG) : (par[v] & ~LAB_FLAG);
-    };
     if (g.bw == CB && (T.W & 3) == 0) {
         // lanes 8r..8r+7 write row 4q+r, four labels each: every store covers
         // four whole 128-byte rows of the block
@@ -674,9 +663,18 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int wa
                     make_int4(v[0], v[1], v[2], v[3]);
             }
         }
-    } else if (lane < g.bh) {
-        int32_t* dst = T.labels + (size_t)gy * T.W + g.x0;
-        for (int x = 0; x < g.bw; x++) dst[x] = ((kept >> x) & 1u) ? run_label(run_start(st, x)) : 0;
+    } else {
+        // rows that are not 16-byte aligned: one row per step, a pixel per lane
+#pragma unroll 4
+        for (int y = 0; y < g.bh; y++) {
+            const uint32_t sty = __shfl_sync(FULLM, st, y), kpy = __shfl_sync(FULLM, kept, y);
+            int lab = 0;
+            if ((kpy >> lane) & 1u) {
+                const int e = par[y * CB + run_start(sty, lane)];
+                lab = (e & LAB_FLAG) ? (e & ~LAB_FLAG) : (par[e] & ~LAB_FLAG);
+            }
+            if (lane < g.bw) T.labels[(size_t)(g.y0 + y) * T.W + g.x0 + lane] = lab;
+        }
     }
     // EDT input: this chunk's 32 kept bits of each column, as one word per
     // column: a 32x32 bit transpose across the lanes in five exchange stages

@@ -265,63 +265,75 @@ __device__ __forceinline__ void halo_coord(int q, int lane, int& hy, int& hx) {
 }
 __device__ __forceinline__ bool halo_lane(int q, int lane) { return q < 8 || lane < 4; }
 
+// the image of a visit, in registers (a descriptor in memory would be read
+// again after every fence)
+struct Img {
+    uint8_t* R;
+    const uint8_t* hem8;
+    int W, H, rp;
+};
+
 // R (and M) of this lane's halo pixels, 0 outside the image
-__device__ __forceinline__ void load_halo(uint8_t hr[9], uint8_t* hm, const uint8_t* Rg, const uint8_t* Mg, int W,
-                                          int H, int x0, int y0, int lane) {
+__device__ __forceinline__ void load_halo(uint8_t hr[9], uint8_t* hm, const Img& T, int x0, int y0, int lane) {
 #pragma unroll
     for (int q = 0; q < 9; q++) {
         int hy, hx;
         halo_coord(q, lane, hy, hx);
         const int gy = y0 + hy, gx = x0 + hx;
-        const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W && halo_lane(q, lane);
-        const size_t o = (size_t)gy * W + gx;
-        hr[q] = in ? __ldcg(Rg + o) : (uint8_t)0;
-        if (hm) hm[q] = in ? __ldg(Mg + o) : (uint8_t)0;
+        const bool in = gy >= 0 && gy < T.H && gx >= 0 && gx < T.W && halo_lane(q, lane);
+        hr[q] = in ? __ldcg(T.R + (size_t)gy * T.rp + gx) : (uint8_t)0;
+        if (hm) hm[q] = in ? __ldg(T.hem8 + (size_t)gy * T.W + gx) : (uint8_t)0;
     }
 }
 
-__device__ __forceinline__ bool fast_rows(const uint8_t* p, const uint8_t* q, int W, int x0) {
-    return (W & 15) == 0 && x0 + RT <= W && ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(q)) & 15) == 0;
-}
-
-__device__ __forceinline__ void load_tile(WarpTile& S, const uint8_t* Rg, const uint8_t* Mg, int W, int H, int x0,
-                                          int y0, int lane) {
+// Stages the tile.  Lane: block row jj of a group of 8, 16-pixel segment seg;
+// rows 2j and 2j + 1 of R and M, eight blocks built from them.  R's rows are
+// 16-byte aligned; hem8's are where W is a multiple of 16 (odd widths read the
+// aligned words around them: with byte loads for both planes a 1025 x 2049
+// image took 381 us).
+__device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int y0, int lane) {
     uint8_t hr[9], hm[9];
-    load_halo(hr, hm, Rg, Mg, W, H, x0, y0, lane);
-    if (fast_rows(Rg, Mg, W, x0)) {
-        // lane: block row jj of a group of 8, 16-pixel segment seg; rows 2j and
-        // 2j + 1 of R and M with 16-byte loads, eight blocks built from them
-        const int jj = lane >> 2, seg = lane & 3;
+    load_halo(hr, hm, T, x0, y0, lane);
+    const uint8_t* const Rg = T.R;
+    const uint8_t* const Mg = T.hem8;
+    const int W = T.W, H = T.H;
+    const int jj = lane >> 2, seg = lane & 3, x = x0 + seg * 16;
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    auto put = [&](int j, uint4 rt, uint4 rb, uint4 mt, uint4 mb) {
+        const uint32_t rtw[4] = {rt.x, rt.y, rt.z, rt.w}, rbw[4] = {rb.x, rb.y, rb.z, rb.w};
+        const uint32_t mtw[4] = {mt.x, mt.y, mt.z, mt.w}, mbw[4] = {mb.x, mb.y, mb.z, mb.w};
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            uint2* d = &S.B[j * BS + seg * 8 + 2 * u];
+            d[0] = make_uint2(__byte_perm(rtw[u], rbw[u], 0x5410), __byte_perm(mtw[u], mbw[u], 0x5410));
+            d[1] = make_uint2(__byte_perm(rtw[u], rbw[u], 0x7632), __byte_perm(mtw[u], mbw[u], 0x7632));
+        }
+    };
+    if ((W & 15) == 0 && x0 + RT <= W && (reinterpret_cast<uintptr_t>(Mg) & 15) == 0) {
 #pragma unroll 2
         for (int g = 0; g < NB / 8; g++) {
             const int j = g * 8 + jj, gy = y0 + 2 * j;
-            const size_t o = (size_t)gy * W + x0 + seg * 16;
-            const uint4 z = make_uint4(0, 0, 0, 0);
+            const size_t o = (size_t)gy * W + x;
             const uint4 rt = gy < H ? __ldcg(reinterpret_cast<const uint4*>(Rg + o)) : z;
             const uint4 rb = gy + 1 < H ? __ldcg(reinterpret_cast<const uint4*>(Rg + o + W)) : z;
             const uint4 mt = gy < H ? __ldg(reinterpret_cast<const uint4*>(Mg + o)) : z;
             const uint4 mb = gy + 1 < H ? __ldg(reinterpret_cast<const uint4*>(Mg + o + W)) : z;
-            const uint32_t rtw[4] = {rt.x, rt.y, rt.z, rt.w}, rbw[4] = {rb.x, rb.y, rb.z, rb.w};
-            const uint32_t mtw[4] = {mt.x, mt.y, mt.z, mt.w}, mbw[4] = {mb.x, mb.y, mb.z, mb.w};
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                uint2* d = &S.B[j * BS + seg * 8 + 2 * u];
-                d[0] = make_uint2(__byte_perm(rtw[u], rbw[u], 0x5410), __byte_perm(mtw[u], mbw[u], 0x5410));
-                d[1] = make_uint2(__byte_perm(rtw[u], rbw[u], 0x7632), __byte_perm(mtw[u], mbw[u], 0x7632));
-            }
+            put(j, rt, rb, mt, mb);
         }
     } else {
-        for (int j = 0; j < NB; j++) {
-            uint32_t rw = 0, mw = 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int gy = y0 + 2 * j + (q >> 1), gx = x0 + 2 * lane + (q & 1);
-                const bool in = gy < H && gx < W;
-                const size_t o = (size_t)gy * W + gx;
-                rw |= (in ? (uint32_t)__ldcg(Rg + o) : 0u) << (8 * q);
-                mw |= (in ? (uint32_t)__ldg(Mg + o) : 0u) << (8 * q);
+#pragma unroll 1
+        for (int g = 0; g < NB / 8; g++) {
+            const int j = g * 8 + jj, gy = y0 + 2 * j;
+            const bool in0 = x < W && gy < H, in1 = x < W && gy + 1 < H;
+            const uint8_t* r = Rg + (size_t)gy * T.rp + x;
+            uint4 rt = in0 ? __ldcg(reinterpret_cast<const uint4*>(r)) : z;
+            uint4 rb = in1 ? __ldcg(reinterpret_cast<const uint4*>(r + T.rp)) : z;
+            const uint4 mt = in0 ? load_px16(Mg, W, H, x, gy) : z, mb = in1 ? load_px16(Mg, W, H, x, gy + 1) : z;
+            if (W - x < 16) {  // R's row padding
+                rt = clip_px16(rt, max(W - x, 0));
+                rb = clip_px16(rb, max(W - x, 0));
             }
-            S.B[j * BS + lane] = make_uint2(rw, mw);
+            put(j, rt, rb, mt, mb);
         }
     }
 #pragma unroll
@@ -334,34 +346,24 @@ __device__ __forceinline__ void load_tile(WarpTile& S, const uint8_t* Rg, const 
     }
 }
 
-// Writes the tile's R back: 16-byte stores where rows are 16-byte aligned.
-__device__ __forceinline__ void store_tile(WarpTile& S, uint8_t* Rg, int W, int H, int x0, int y0, int lane) {
-    if (fast_rows(Rg, Rg, W, x0)) {
-        const int jj = lane >> 2, seg = lane & 3;
+// Writes the tile's R back (row padding takes zeros).
+__device__ __forceinline__ void store_tile(WarpTile& S, const Img& T, int x0, int y0, int lane) {
+    const int jj = lane >> 2, seg = lane & 3, x = x0 + seg * 16;
+    if (x >= T.W) return;
 #pragma unroll 1
-        for (int g = 0; g < NB / 8; g++) {
-            const int j = g * 8 + jj, gy = y0 + 2 * j;
-            uint32_t top[4], bot[4];
+    for (int g = 0; g < NB / 8; g++) {
+        const int j = g * 8 + jj, gy = y0 + 2 * j;
+        uint32_t top[4], bot[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const uint2* s = &S.B[j * BS + seg * 8 + 2 * u];
-                const uint32_t a = s[0].x, b = s[1].x;
-                top[u] = __byte_perm(a, b, 0x5410);
-                bot[u] = __byte_perm(a, b, 0x7632);
-            }
-            const size_t o = (size_t)gy * W + x0 + seg * 16;
-            if (gy < H) __stcg(reinterpret_cast<uint4*>(Rg + o), make_uint4(top[0], top[1], top[2], top[3]));
-            if (gy + 1 < H) __stcg(reinterpret_cast<uint4*>(Rg + o + W), make_uint4(bot[0], bot[1], bot[2], bot[3]));
+        for (int u = 0; u < 4; u++) {
+            const uint2* s = &S.B[j * BS + seg * 8 + 2 * u];
+            const uint32_t a = s[0].x, b = s[1].x;
+            top[u] = __byte_perm(a, b, 0x5410);
+            bot[u] = __byte_perm(a, b, 0x7632);
         }
-    } else {
-        for (int j = 0; j < NB; j++) {
-            const uint32_t rw = S.B[j * BS + lane].x;
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int gy = y0 + 2 * j + (q >> 1), gx = x0 + 2 * lane + (q & 1);
-                if (gy < H && gx < W) __stcg(Rg + (size_t)gy * W + gx, (uint8_t)(rw >> (8 * q)));
-            }
-        }
+        uint8_t* const r = T.R + (size_t)gy * T.rp + x;
+        if (gy < T.H) __stcg(reinterpret_cast<uint4*>(r), make_uint4(top[0], top[1], top[2], top[3]));
+        if (gy + 1 < T.H) __stcg(reinterpret_cast<uint4*>(r + T.rp), make_uint4(bot[0], bot[1], bot[2], bot[3]));
     }
 }
 
@@ -623,17 +625,16 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
         // only its border can have become raisable; its first visit starts
         // from the marker and sweeps at once
         bool sweep_now = (item & ITEM_FIRST) != 0, full_check = false;
-        const TileDev& T = L.tiles[ti];
-        const int W = T.W, H = T.H, rx = T.rtx, ry = T.rty, base = T.rt_base;
-        uint8_t* const Rg = T.R;
-        const uint8_t* const Mg = T.hem8;
+        const TileDev& D = L.tiles[ti];
+        const Img T{D.R, D.hem8, D.W, D.H, D.rp};
+        const int rx = D.rtx, ry = D.rty, base = D.rt_base;
         const int t = base + k, ty = k / rx, tx = k - ty * rx;
         const int x0 = tx * RT, y0 = ty * RT;
         if (lane == 0) atomicExch(&L.wl_state[t], WL_RUNNING);
         visits++;
         __threadfence();
         __syncwarp();
-        load_tile(S, Rg, Mg, W, H, x0, y0, lane);
+        load_tile(S, T, x0, y0, lane);
         __syncwarp();
         // the border as loaded is the reference for the first requests (lane l:
         // border pixels 2l, 2l + 1 of each side, from one block word per side)
@@ -668,8 +669,8 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
                 // issued before the write-back so that the two overlap (a stale
                 // value can only cause a needless request)
                 uint8_t hr[9];
-                load_halo(hr, nullptr, Rg, Mg, W, H, x0, y0, lane);
-                store_tile(S, Rg, W, H, x0, y0, lane);
+                load_halo(hr, nullptr, T, x0, y0, lane);
+                store_tile(S, T, x0, y0, lane);
                 // the stores drain while the requests are worked out in shared memory
                 grew = __any_sync(FULL, merge_halo(S, hr, lane));
                 __syncwarp();
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
             if (__any_sync(FULL, ld_vol(&L.sh->err) != 0)) break;
             // only the halo can have changed: the interior belongs to this worker
             uint8_t hr[9];
-            load_halo(hr, nullptr, Rg, Mg, W, H, x0, y0, lane);
+            load_halo(hr, nullptr, T, x0, y0, lane);
             merge_halo(S, hr, lane);
             __syncwarp();
         }

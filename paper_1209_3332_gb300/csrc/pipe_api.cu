@@ -180,6 +180,8 @@ std::string tune_str(const Tune& t) {
     return std::to_string(t.recon_grid) + " " + std::to_string(t.edt_rb) + " " + std::to_string(t.feat_grid);
 }
 
+int r_pitch(int W) { return (W + 15) & ~15; }
+
 Geo geometry(int W, int H, int feats_cap) {
     Geo g;
     g.W = W;
@@ -193,7 +195,7 @@ Geo geometry(int W, int H, int feats_cap) {
     size_t words = (size_t)H * g.wpr;
     g.nchunks = (int)((words + SCAN_CHUNK - 1) / SCAN_CHUNK);
     size_t b = 0;
-    b += al256(g.N);                              // R
+    b += al256((size_t)H * r_pitch(W));           // R
     b += 2 * al256(g.N * 4);                      // P, A
     b += al256((size_t)g.cbx * g.cby * RL_CAP * 4);  // per-block root lists
     b += al256((size_t)g.cbx * g.cby * 4);        // per-block root counts
@@ -214,7 +216,8 @@ void carve(TileDev& t, const Geo& g, char* base) {
     size_t words = (size_t)g.H * g.wpr;
     char* p = base;
     auto take = [&](size_t n) { char* r = p; p += al256(n); return r; };
-    t.R = (uint8_t*)take(g.N);
+    t.R = (uint8_t*)take((size_t)g.H * r_pitch(g.W));
+    t.rp = r_pitch(g.W);
     t.P = (int32_t*)take(g.N * 4);
     t.A = (int32_t*)take(g.N * 4);
     t.rootlist = (int32_t*)take((size_t)g.cbx * g.cby * RL_CAP * 4);
@@ -1153,7 +1156,7 @@ int pipe_debug_plane(pipe_t p, int which, void* dst_dev, pipe_stream_t stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const TileDev& t = p->last_plain;
     if (which == 0) {
-        CK(cudaMemcpyAsync(dst_dev, t.R, (size_t)t.W * t.H, cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpy2DAsync(dst_dev, t.W, t.R, t.rp, t.W, t.H, cudaMemcpyDeviceToDevice, s));
     } else {
         launch_unpack_bits(which == 1 ? t.fgbits : t.filledbits, t.W, t.H, t.cbx, (uint8_t*)dst_dev, s, &p->prof);
         CK(cudaGetLastError());

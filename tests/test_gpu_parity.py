@@ -110,3 +110,29 @@ def test_holes_of_every_size(pipe):
     g, r = check(pipe, rgb)
     holes = int(r["filled"].sum()) - int(r["fg"].sum())
     assert holes > 20000  # the rings' insides were filled
+
+
+@pytest.mark.parametrize("W,H,off,pad", [(16, 1, 1, 0), (17, 2, 2, 1), (35, 3, 3, 5), (64, 65, 1, 0), (79, 33, 2, 7),
+                                         (130, 67, 3, 0), (193, 129, 1, 2)])
+def test_unaligned_buffers(pipe, W, H, off, pad):
+    """RGB rows and a hem8 plane that start on no 4-byte boundary, at widths
+    around the 16-pixel loads and the 64-pixel work tiles."""
+    import torch
+    import synth
+    rgb = synth.tile(W, H, 31 + W, n_nuclei=max(1, W * H // 400), frac_cluster=0.3)
+    dev = torch.device("cuda", 0)
+    pitch = 3 * W + pad
+    src = torch.zeros(off + H * pitch, dtype=torch.uint8, device=dev)
+    view = src[off:].view(H, pitch)[:, :3 * W]
+    view.copy_(torch.from_numpy(rgb.reshape(H, 3 * W)).to(dev))
+    hem = torch.full((off + H * W,), 7, dtype=torch.uint8, device=dev)[off:].view(H, W)
+    lab = torch.empty((H, W), dtype=torch.int32, device=dev)
+    edt = torch.empty_like(lab)
+    nobj = torch.zeros(1, dtype=torch.int32, device=dev)
+    pipe.seg_tile(view.view(H, W, 3) if pad == 0 else view.as_strided((H, W, 3), (pitch, 3, 1)), hem, lab, edt, nobj)
+    R = torch.empty((H, W), dtype=torch.uint8, device=dev)
+    pipe.debug_plane(0, R)
+    torch.cuda.synchronize()
+    ref = oracle_all(rgb)
+    assert_planes_equal(dict(hem8=hem.cpu().numpy(), R=R.cpu().numpy(), labels=lab.cpu().numpy(), edt=edt.cpu().numpy(),
+                             K=int(nobj.item())), ref)
