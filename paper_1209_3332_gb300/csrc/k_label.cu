@@ -214,26 +214,51 @@ __device__ __forceinline__ int gidx(const TileDev& T, const WarpGeo& g, int li) 
 constexpr int PAR_IDX = 0x3ff;
 __device__ __forceinline__ int par_root(UF par, int i) { return par[i] & PAR_IDX; }
 
+// What the later passes read of a block before anything else (blkroots): the
+// number of its local roots and, so that most of them need no more,
+//  * BLK_PURE: every pixel of the block is in the class, so its one root is
+//    its first pixel;
+//  * per side (left, right, top, bottom): every pixel has the same local root,
+//    or none (BLK_UNIFORM), and no pixel is in the class (BLK_EMPTY).
+// Blocks without a class pixel, and pure ones, publish no edge roots.
+constexpr int BLK_COUNT = 0x3ff;
+constexpr int BLK_UNIFORM = 1 << 16, BLK_EMPTY = 1 << 20, BLK_PURE = 1 << 24;
+constexpr int BLK_ALL_UNIFORM = 15 * BLK_UNIFORM, BLK_ALL_EMPTY = 15 * BLK_EMPTY;
+constexpr int HOLE_BIT = 1 << 30;  // between the fill and the labelling: a background component is a hole
+enum Side { LEFT = 0, RIGHT = 1, TOP = 2, BOTTOM = 3 };
+
 // Edge roots: [0,CB) left column, [CB,2CB) right column (x=31), [2CB,3CB)
 // top row, [3CB,4CB) bottom row (y=31); -1 where the pixel is not in the class.
-__device__ __forceinline__ void publish_edges(const TileDev& T, const WarpGeo& g, uint32_t w, uint32_t st,
-                                              UF par, int lane) {
+// Returns the block's side flags.
+__device__ __forceinline__ int publish_edges(const TileDev& T, const WarpGeo& g, uint32_t w, uint32_t st,
+                                             UF par, int lane) {
     int* e = T.border + (size_t)g.lb * 4 * CB;
-    e[lane] = (w & 1u) ? gidx(T, g, par_root(par, lane * CB)) : -1;
-    e[CB + lane] = (w >> 31) ? gidx(T, g, par_root(par, lane * CB + run_start(st, 31))) : -1;
     uint32_t w0 = __shfl_sync(FULLM, w, 0), s0 = __shfl_sync(FULLM, st, 0);
     uint32_t w31 = __shfl_sync(FULLM, w, 31), s31 = __shfl_sync(FULLM, st, 31);
-    e[2 * CB + lane] = ((w0 >> lane) & 1u) ? gidx(T, g, par_root(par, run_start(s0, lane))) : -1;
-    e[3 * CB + lane] = ((w31 >> lane) & 1u) ? gidx(T, g, par_root(par, 31 * CB + run_start(s31, lane))) : -1;
+    const int r[4] = {(w & 1u) ? gidx(T, g, par_root(par, lane * CB)) : -1,
+                      (w >> 31) ? gidx(T, g, par_root(par, lane * CB + run_start(st, 31))) : -1,
+                      ((w0 >> lane) & 1u) ? gidx(T, g, par_root(par, run_start(s0, lane))) : -1,
+                      ((w31 >> lane) & 1u) ? gidx(T, g, par_root(par, 31 * CB + run_start(s31, lane))) : -1};
+    int flags = 0;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        e[q * CB + lane] = r[q];
+        const bool out = lane >= (q < 2 ? g.bh : g.bw);  // beyond the image: part of no side
+        const int first = __shfl_sync(FULLM, r[q], 0);
+        if (__all_sync(FULLM, out || r[q] == first)) flags |= BLK_UNIFORM << q;
+        if (__all_sync(FULLM, r[q] < 0)) flags |= BLK_EMPTY << q;
+    }
+    return flags;
 }
 
 // Record this block's local roots (run starts that are roots) in the block's
 // own slice of the root list (RL_CAP entries: a 32x32 block has at most 512
 // 4-connected and 256 8-connected components) and initialise P/A at their
 // global index with payload pay(root).  No global counter is involved.
+// Returns the number of roots on lane 31.
 template <typename Pay>
-__device__ __forceinline__ void register_roots(const TileDev& T, const WarpGeo& g, uint32_t st, UF par,
-                                               Pay pay, int lane) {
+__device__ __forceinline__ int register_roots(const TileDev& T, const WarpGeo& g, uint32_t st, UF par,
+                                              Pay pay, int lane) {
     uint32_t rs = 0;
     for (uint32_t m = st; m; m &= m - 1) {
         int s = __ffs(m) - 1;
@@ -254,7 +279,7 @@ __device__ __forceinline__ void register_roots(const TileDev& T, const WarpGeo& 
         T.A[gi] = pay(li);
         list[k++] = gi;
     }
-    if (lane == 31) T.blkroots[g.lb] = incl;
+    return incl;
 }
 
 
@@ -303,6 +328,16 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_fill_local(Launch L) {
         fg = lane < g.bh ? (lane < 16 ? (lo0 | (hi0 << 16)) : (lo1 | (hi1 << 16))) & vm : 0u;
     }
     if (lane < g.bh) T.fgbits[block_word(T, g, lane)] = fg;
+    if (__ballot_sync(FULLM, fg != 0u) == 0u) {  // only background (more than half of the blocks)
+        if (lane == 0) {
+            const int gi = g.y0 * T.W + g.x0;
+            T.P[gi] = gi;
+            T.A[gi] = g.bx == 0 || g.by == 0 || g.bx == T.cbx - 1 || g.by == T.cby - 1;
+            T.rootlist[(size_t)g.lb * RL_CAP] = gi;
+            T.blkroots[g.lb] = 1 | BLK_PURE | BLK_ALL_UNIFORM;
+        }
+        return;
+    }
     const uint32_t bg = lane < g.bh ? (~fg & vm) : 0u;
     const uint32_t st = bg & ~(bg << 1);
     warp_ccl<4>(bg, st, lane, par);
@@ -321,18 +356,22 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_fill_local(Launch L) {
         }
     }
     __syncwarp();
-    register_roots(T, g, st, par, [&](int li) { return (int)((touch[li >> 5] >> (li & 31)) & 1u); }, lane);
-    publish_edges(T, g, bg, st, par, lane);
+    const int n = register_roots(T, g, st, par, [&](int li) { return (int)((touch[li >> 5] >> (li & 31)) & 1u); }, lane);
+    const int flags = publish_edges(T, g, bg, st, par, lane);
+    if (lane == 31) T.blkroots[g.lb] = n | flags;
 }
 
 // ---- merge facing edge pixels of neighbouring blocks ------------------------------
-template <int CONN>
+// the root of edge pixel j of a side of block (bx, by), -1 where there is none
 __device__ __forceinline__ int edge_root(const TileDev& T, int bx, int by, int side, int j) {
     if (bx < 0 || by < 0 || bx >= T.cbx || by >= T.cby || j < 0 || j >= CB) return -1;
-    return T.border[(size_t)(by * T.cbx + bx) * 4 * CB + side * CB + j];
+    const int lb = by * T.cbx + bx, f = T.blkroots[lb];
+    if (f & BLK_PURE)
+        return (side < 2 ? by * CB + j < T.H : bx * CB + j < T.W) ? by * CB * T.W + bx * CB : -1;
+    if ((f & BLK_COUNT) == 0) return -1;
+    return T.border[(size_t)lb * 4 * CB + side * CB + j];
 }
 
-// One warp per block: lanes walk the right column and then the bottom row.
 // Consecutive edge pixels mostly repeat the same pair of local roots, so a
 // lane unions only when its pair differs from the previous lane's.
 __device__ __forceinline__ void union_dedup(int* P, int a, int b, int lane) {
@@ -341,47 +380,116 @@ __device__ __forceinline__ void union_dedup(int* P, int a, int b, int lane) {
     if (a >= 0 && b >= 0 && !same) g_union(P, a, b);
 }
 
+// One warp: the facing pixels of block (bx, by) and the block(s) to its right
+// (side 0) or below it (side 1), one edge pixel per lane.
 template <int CONN>
-__global__ void __launch_bounds__(CCL_WARPS * 32) k_merge(Launch L) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gb = blockIdx.x * CCL_WARPS + warp;
-    if (gb >= L.n_cb) return;
-    const WarpGeo g = warp_geo(L, gb);
-    const TileDev T = L.tiles[g.ti];  // by value: stores below cannot force reloads
-    const int* e = T.border + (size_t)g.lb * 4 * CB;
-    // right column pixel (lane, 31) against the next block(s) to the right
-    {
-        int a = e[CB + lane];
-        int b = edge_root<CONN>(T, g.bx + 1, g.by, 0, lane);
-        union_dedup(T.P, a, b, lane);
+__device__ __forceinline__ void merge_edge(const TileDev& T, int bx, int by, int side, int lane) {
+    if (side == 0) {  // right column pixel (lane, 31)
+        const int a = edge_root(T, bx, by, RIGHT, lane);
+        union_dedup(T.P, a, edge_root(T, bx + 1, by, LEFT, lane), lane);
         if (CONN == 8) {
-            int up = lane == 0 ? edge_root<CONN>(T, g.bx + 1, g.by - 1, 0, CB - 1)
-                               : edge_root<CONN>(T, g.bx + 1, g.by, 0, lane - 1);
-            union_dedup(T.P, a, up, lane);
-            int dn = lane == CB - 1 ? edge_root<CONN>(T, g.bx + 1, g.by + 1, 0, 0)
-                                    : edge_root<CONN>(T, g.bx + 1, g.by, 0, lane + 1);
-            union_dedup(T.P, a, dn, lane);
+            union_dedup(T.P, a, lane == 0 ? edge_root(T, bx + 1, by - 1, LEFT, CB - 1)
+                                          : edge_root(T, bx + 1, by, LEFT, lane - 1), lane);
+            union_dedup(T.P, a, lane == CB - 1 ? edge_root(T, bx + 1, by + 1, LEFT, 0)
+                                               : edge_root(T, bx + 1, by, LEFT, lane + 1), lane);
         }
-    }
-    // bottom row pixel (31, lane) against the block(s) below
-    {
-        int a = e[3 * CB + lane];
-        int b = edge_root<CONN>(T, g.bx, g.by + 1, 2, lane);
-        union_dedup(T.P, a, b, lane);
+    } else {          // bottom row pixel (31, lane)
+        const int a = edge_root(T, bx, by, BOTTOM, lane);
+        union_dedup(T.P, a, edge_root(T, bx, by + 1, TOP, lane), lane);
         if (CONN == 8) {
-            int l = lane == 0 ? edge_root<CONN>(T, g.bx - 1, g.by + 1, 2, CB - 1)
-                              : edge_root<CONN>(T, g.bx, g.by + 1, 2, lane - 1);
-            union_dedup(T.P, a, l, lane);
-            int r = lane == CB - 1 ? edge_root<CONN>(T, g.bx + 1, g.by + 1, 2, 0)
-                                   : edge_root<CONN>(T, g.bx, g.by + 1, 2, lane + 1);
-            union_dedup(T.P, a, r, lane);
+            union_dedup(T.P, a, lane == 0 ? edge_root(T, bx - 1, by + 1, TOP, CB - 1)
+                                          : edge_root(T, bx, by + 1, TOP, lane - 1), lane);
+            union_dedup(T.P, a, lane == CB - 1 ? edge_root(T, bx + 1, by + 1, TOP, 0)
+                                               : edge_root(T, bx, by + 1, TOP, lane + 1), lane);
         }
     }
 }
 
-// ---- root-list passes (grid-stride over every tile's list) -----------------------
-constexpr int HOLE_BIT = 1 << 30;  // in a block's root count between the fill and the labelling
-// mode 0: border flag of a local root -> its global root
+// A warp takes `per` blocks (a power of two up to 8); lane i decides from the
+// flags of block i what there is to do, and the edges that need a look at their
+// pixels are then walked by the whole warp, one after the other.
+// Background (CONN 4): two facing sides with one root each, by far the most
+// common case, are one union by the lane.  To the right these form chains:
+// blocks of a warp that such pairs connect in a row are joined to the smallest
+// of their roots at once, not link by link; downwards, pairs whose roots have
+// become the same are joined once per warp.
+// Foreground (CONN 8): most sides hold no pixel.
+// 16 tiles of 4096^2: 93 and 67 us (247 and 109 with a warp per block that
+// walks all of its edge pixels).  Bound: the latency of the finds.
+template <int CONN>
+__global__ void __launch_bounds__(CCL_WARPS * 32) k_merge(Launch L, int per) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = (blockIdx.x * CCL_WARPS + warp) * per, gb = first + lane;
+    if (first >= L.n_cb) return;
+    const bool in = lane < per && gb < L.n_cb;
+    bool right = false, below = false;       // the edge is to be walked
+    int ra = -1, rb = -1, da = -1, db = -1;  // CONN 4: one pair per side
+    int* P = nullptr;
+    bool pass = false;                       // left and right side have the same root
+    if (in) {
+        const TileDev& T = L.tiles[tile_of_block(L, gb)];
+        const int lb = gb - T.cb_base, by = lb / T.cbx, bx = lb - by * T.cbx, f = T.blkroots[lb];
+        const bool hr = bx + 1 < T.cbx, hd = by + 1 < T.cby;
+        if (CONN == 8) {
+            right = hr && (f & BLK_COUNT) && !(f & (BLK_EMPTY << RIGHT));
+            below = hd && (f & BLK_COUNT) && !(f & (BLK_EMPTY << BOTTOM));
+        } else {
+            P = T.P;
+            // the root of a uniform side
+            auto root = [&](int q, int fq, int x, int y, int side) -> int {
+                if (fq & BLK_PURE) return y * CB * T.W + x * CB;
+                return (fq & (BLK_EMPTY << side)) || !(fq & BLK_COUNT) ? -1 : T.border[(size_t)q * 4 * CB + side * CB];
+            };
+            const int fr = hr ? T.blkroots[lb + 1] : 0, fd = hd ? T.blkroots[lb + T.cbx] : 0;
+            const bool ur = hr && (f & (BLK_UNIFORM << RIGHT)) && (fr & (BLK_UNIFORM << LEFT));
+            const bool ud = hd && (f & (BLK_UNIFORM << BOTTOM)) && (fd & (BLK_UNIFORM << TOP));
+            right = hr && !ur;
+            below = hd && !ud;
+            if (ur) {
+                ra = root(lb, f, bx, by, RIGHT);
+                rb = root(lb + 1, fr, bx + 1, by, LEFT);
+                if (f & (BLK_UNIFORM << LEFT)) pass = root(lb, f, bx, by, LEFT) == ra;
+            }
+            if (ud) {
+                da = root(lb, f, bx, by, BOTTOM);
+                db = root(lb + T.cbx, fd, bx, by + 1, TOP);
+            }
+        }
+    }
+    if (CONN == 4) {
+        const unsigned cont = __ballot_sync(FULLM, ra >= 0 && rb >= 0), passm = __ballot_sync(FULLM, pass);
+        // a chain starts at a pair that the pair before does not lead into
+        const unsigned starts = cont & ~((cont << 1) & passm);
+        if ((cont >> lane) & 1u) {
+            const int s = 31 - __clz(starts & below_or_at(lane));
+            const unsigned later = starts & ~below_or_at(s);
+            const unsigned seg = cont & ~((1u << s) - 1u) & (later ? (later & (0u - later)) - 1u : FULLM);
+            const int m = (int)__reduce_min_sync(seg, (unsigned)ra);
+            if (ra != m) g_union(P, ra, m);
+            if (lane == 31 - __clz(seg)) g_union(P, rb, m);
+        }
+        __syncwarp();
+        const bool pair = da >= 0 && db >= 0;
+        const int fa = pair ? g_find(P, da) : -1, fb = pair ? g_find(P, db) : -1;
+        // P belongs to an image: roots of two images in one warp may share an index
+        const unsigned grp = __match_any_sync(FULLM, fa) & __match_any_sync(FULLM, fb) &
+                             __match_any_sync(FULLM, (unsigned long long)(uintptr_t)P);
+        if (pair && fa != fb && lane == __ffs(grp) - 1) g_union(P, fa, fb);
+        __syncwarp();
+    }
+    const unsigned wr = __ballot_sync(FULLM, right), wb = __ballot_sync(FULLM, below);
+    for (unsigned m = wr | wb; m; m &= m - 1) {
+        const int i = __ffs(m) - 1, b = first + i;
+        const TileDev& T = L.tiles[tile_of_block(L, b)];
+        const int lb = b - T.cb_base, by = lb / T.cbx, bx = lb - by * T.cbx;
+        if ((wr >> i) & 1u) merge_edge<CONN>(T, bx, by, 0, lane);
+        if ((wb >> i) & 1u) merge_edge<CONN>(T, bx, by, 1, lane);
+    }
+}
+
+// ---- root-list passes ---------------------------------------------------------------
+// mode 0: border flag of a local root -> its global root (only blocks on the
+//         image border hold one)
 // mode 1: copy the global root's flag back to every local root; compress P;
 //         mark the blocks that hold a hole (HOLE_BIT in their root count)
 //         (the labelling pass must read the flag at its own local roots: a
@@ -389,51 +497,81 @@ constexpr int HOLE_BIT = 1 << 30;  // in a block's root count between the fill a
 //         that pass overwrites while other blocks would still follow links to it)
 // mode 2: add local areas into the global root; compress P
 // mode 3: mark kept global roots in the root bitmap
-// Each warp strides over the labelling blocks (a grid of a warp per block,
-// or of a few CTAs per SM: most blocks have one or two roots).
-__global__ void __launch_bounds__(CCL_WARPS * 32) k_roots(Launch L, int mode) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int gb = blockIdx.x * CCL_WARPS + warp; gb < L.n_cb; gb += gridDim.x * CCL_WARPS) {
-        const int ti = tile_of_block(L, gb);
-        const TileDev T = L.tiles[ti];  // by value: stores below cannot force reloads
-        const int lb = gb - T.cb_base;
-        const int n = T.blkroots[lb];
-        const int* list = T.rootlist + (size_t)lb * RL_CAP;
-        bool hole = false;  // mode 1: a background component of this block is a hole
-        for (int j = lane; j < n; j += 32) {
-            int r = list[j];
-            if (mode == 0) {
-                if (T.A[r]) {
-                    int g = g_find(T.P, r);
-                    if (g != r) T.A[g] = 1;
-                }
-            } else if (mode == 1) {
-                int g = g_find(T.P, r);
-                int f = T.A[r];
-                if (g != r) {
-                    f = __ldcg(T.A + g);
-                    T.A[r] = f;
-                    T.P[r] = g;
-                }
-                hole |= f == 0;
-            } else if (mode == 2) {
-                int g = g_find(T.P, r);
-                if (g != r) {
-                    atomicAdd(T.A + g, T.A[r]);
-                    T.P[r] = g;
-                }
-            } else {
-                if (T.P[r] == r) {
-                    int a = T.A[r];
-                    if (a >= L.amin && a <= L.amax) {
-                        int y = r / T.W, x = r - y * T.W;
-                        atomicOr(T.rootbits + (size_t)y * T.wpr + (x >> 5), 1u << (x & 31));
-                    }
-                }
-            }
+// A warp takes the roots of `per` blocks as one list (most blocks have one or
+// two, or none).  16 tiles of 4096^2: 13, 53, 17 and 16 us (212 in all with a
+// warp per block).
+template <int MODE>
+__device__ __forceinline__ bool root_pass(const Launch& L, const TileDev& T, int r) {
+    if (MODE == 0) {
+        if (T.A[r]) {
+            const int g = g_find(T.P, r);
+            if (g != r) T.A[g] = 1;
         }
-        if (mode == 1 && __any_sync(FULLM, hole) && lane == 0) T.blkroots[lb] = n | HOLE_BIT;
+    } else if (MODE == 1) {
+        const int g = g_find(T.P, r);
+        int f = T.A[r];
+        if (g != r) {
+            f = __ldcg(T.A + g);
+            T.A[r] = f;
+            T.P[r] = g;
+        }
+        return f == 0;  // a hole
+    } else if (MODE == 2) {
+        const int g = g_find(T.P, r);
+        if (g != r) {
+            atomicAdd(T.A + g, T.A[r]);
+            T.P[r] = g;
+        }
+    } else if (T.P[r] == r) {
+        const int a = T.A[r];
+        if (a >= L.amin && a <= L.amax) {
+            const int y = r / T.W, x = r - y * T.W;
+            atomicOr(T.rootbits + (size_t)y * T.wpr + (x >> 5), 1u << (x & 31));
+        }
     }
+    return false;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(CCL_WARPS * 32) k_roots(Launch L, int per) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = (blockIdx.x * CCL_WARPS + warp) * per, gb = first + lane;
+    if (first >= L.n_cb) return;
+    int ti = 0, lb = 0, f = 0, n = 0;
+    if (lane < per && gb < L.n_cb) {
+        ti = tile_of_block(L, gb);
+        const TileDev& T = L.tiles[ti];
+        lb = gb - T.cb_base;
+        f = T.blkroots[lb];
+        n = f & BLK_COUNT;
+        if (MODE == 0) {
+            const int by = lb / T.cbx, bx = lb - by * T.cbx;
+            if (bx > 0 && by > 0 && bx < T.cbx - 1 && by < T.cby - 1) n = 0;
+        }
+    }
+    int end = n;  // roots of the blocks up to and with this lane's
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const int y = __shfl_up_sync(FULLM, end, o);
+        if (lane >= o) end += y;
+    }
+    const int total = __shfl_sync(FULLM, end, per - 1);
+    unsigned holes = 0;  // blocks with a hole
+    for (int i0 = 0; i0 < total; i0 += 32) {
+        const int i = i0 + lane;
+        int src = 0;  // the block that holds root i
+        for (int o = per >> 1; o > 0; o >>= 1)
+            if (__shfl_sync(FULLM, end, src + o - 1) <= i) src += o;
+        const int j = i - (__shfl_sync(FULLM, end, src) - __shfl_sync(FULLM, n, src));
+        const int ot = __shfl_sync(FULLM, ti, src), ob = __shfl_sync(FULLM, lb, src);
+        bool h = false;
+        if (i < total) {
+            const TileDev& T = L.tiles[ot];
+            h = root_pass<MODE>(L, T, T.rootlist[(size_t)ob * RL_CAP + j]);
+        }
+        if (MODE == 1) holes |= __reduce_or_sync(FULLM, h ? 1u << src : 0u);
+    }
+    if (MODE == 1 && ((holes >> lane) & 1u)) L.tiles[ti].blkroots[lb] = f | HOLE_BIT;
 }
 
 // ---- K4a: holes -> filled; foreground local components ----------------------------
@@ -452,7 +590,16 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_label_local(Launch L) {
     // background runs whose component does not reach the border are holes;
     // only blocks that hold one (most hold none) label their background again
     uint32_t filled = fg;
-    if (__ldcg(T.blkroots + g.lb) & HOLE_BIT) {
+    const bool hole = __ldcg(T.blkroots + g.lb) & HOLE_BIT;
+    if (!hole && __ballot_sync(FULLM, fg != 0u) == 0u) {  // no foreground
+        if (lane < g.bh) {
+            T.filledbits[wblk] = 0u;
+            T.rootbits[wrow] = 0u;
+        }
+        if (lane == 0) T.blkroots[g.lb] = BLK_ALL_UNIFORM | BLK_ALL_EMPTY;
+        return;
+    }
+    if (hole) {
         const uint32_t bg = lane < g.bh ? (~fg & vm) : 0u;
         const uint32_t sb = bg & ~(bg << 1);
         warp_ccl<4>(bg, sb, lane, par);
@@ -475,8 +622,9 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_label_local(Launch L) {
         atomicAdd(&par[par_root(par, lane * CB + s)], __popc(run_mask(filled, s)) << 16);
     }
     __syncwarp();
-    register_roots(T, g, st, par, [&](int li) { return par[li] >> 16; }, lane);
-    publish_edges(T, g, filled, st, par, lane);
+    const int n = register_roots(T, g, st, par, [&](int li) { return par[li] >> 16; }, lane);
+    const int flags = publish_edges(T, g, filled, st, par, lane);
+    if (lane == 31) T.blkroots[g.lb] = n | flags;
 }
 
 // ---- K4e: exclusive popcount prefix of the root bitmap ----------------------------
@@ -573,6 +721,20 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int wa
     const WarpGeo g = warp_geo(L, gb);
     const TileDev T = L.tiles[g.ti];  // by value: stores below cannot force reloads
     const uint32_t filled = lane < g.bh ? T.filledbits[block_word(T, g, lane)] : 0u;
+    if (__ballot_sync(FULLM, filled != 0u) == 0u) {  // no object: zeros
+        if (T.edt && lane < g.bw) T.colbits[(size_t)g.by * T.W + g.x0 + lane] = 0u;
+        int32_t* dst = T.labels + (size_t)g.y0 * T.W + g.x0;
+        if (g.bw == CB && (T.W & 3) == 0) {
+#pragma unroll
+            for (int q = 0; q < CB / 4; q++) {
+                const int y = 4 * q + (lane >> 3);
+                if (y < g.bh) reinterpret_cast<int4*>(dst + (size_t)y * T.W)[lane & 7] = make_int4(0, 0, 0, 0);
+            }
+        } else if (lane < g.bw) {
+            for (int y = 0; y < g.bh; y++) dst[(size_t)y * T.W + lane] = 0;
+        }
+        return;
+    }
     const uint32_t st = filled & ~(filled << 1);
     warp_ccl<8>(filled, st, lane, par);
     // roots of this lane's row: label (0 if filtered out) into the root's entry
@@ -738,30 +900,35 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
     pf->begin("fill_local", s);
     k_fill_local<<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s>>>(L);
     pf->end("fill_local", s);
-    const int wg = (L.n_cb + CCL_WARPS - 1) / CCL_WARPS;
-    // the area and keep passes stride over the blocks with a few CTAs per SM;
-    // the flag passes, whose finds wait on global links, keep a warp per block
-    const int rg = std::min(wg, sms * 16);
+    // Blocks per warp of the merge and root passes: as many as leave one wave of
+    // resident warps, up to 8.  On 16 tiles of 4096^2 more blocks per warp mean
+    // fewer waves of a latency-bound kernel; on one small tile a warp per block
+    // spreads its few edges (512^2, merges with 32 blocks per warp: 33 and 28 us).
+    int per = 1;
+    while (per < 8 && L.n_cb > per * sms * 64) per *= 2;
+    const int pg = (L.n_cb + CCL_WARPS * per - 1) / (CCL_WARPS * per), pt = CCL_WARPS * 32;
     pf->begin("fill_merge", s);
-    k_merge<4><<<wg, CCL_WARPS * 32, 0, s>>>(L);
+    k_merge<4><<<pg, pt, 0, s>>>(L, per);
     pf->end("fill_merge", s);
     pf->begin("fill_roots_flag", s);
-    k_roots<<<wg, CCL_WARPS * 32, 0, s>>>(L, 0);
+    k_roots<0><<<pg, pt, 0, s>>>(L, per);
     pf->end("fill_roots_flag", s);
     pf->begin("fill_roots_copy", s);
-    k_roots<<<wg, CCL_WARPS * 32, 0, s>>>(L, 1);
+    k_roots<1><<<pg, pt, 0, s>>>(L, per);
     pf->end("fill_roots_copy", s);
     pf->begin("label_local", s);
     k_label_local<<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s>>>(L);
     pf->end("label_local", s);
     pf->begin("label_merge", s);
-    k_merge<8><<<wg, CCL_WARPS * 32, 0, s>>>(L);
+    // (a warp per block: edges with foreground are all walked, and 8 blocks per
+    // warp take 102 us instead of 38 on four tiles dense with nuclei)
+    k_merge<8><<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, pt, 0, s>>>(L, 1);
     pf->end("label_merge", s);
     pf->begin("label_roots_area", s);
-    k_roots<<<rg, CCL_WARPS * 32, 0, s>>>(L, 2);
+    k_roots<2><<<pg, pt, 0, s>>>(L, per);
     pf->end("label_roots_area", s);
     pf->begin("label_roots_keep", s);
-    k_roots<<<rg, CCL_WARPS * 32, 0, s>>>(L, 3);
+    k_roots<3><<<pg, pt, 0, s>>>(L, per);
     pf->end("label_roots_keep", s);
     pf->begin("scan_chunks", s);
     k_scan_chunks<<<L.n_chunks, SCAN_THREADS, 0, s>>>(L, 0);

@@ -256,3 +256,40 @@ def test_served_concurrent_polls_keep_each_tickets_results(pipe):
     for a, b in zip(got, ref):
         assert a["n_objects"] == b["n_objects"]
         assert_same_feats(a["feats"], b["feats"], "concurrent polls")
+
+
+@pytest.mark.parametrize("n", [1, 600, 1200, 2400])
+def test_many_small_tiles_in_one_batch(n):
+    """20 labelling blocks per tile, so that the merge and root passes take
+    1, 2, 4 and 8 blocks per warp and a warp's blocks span several tiles:
+    nuclei, noise (many components per block), rings (holes), nothing."""
+    import torch
+    import paper_1209_3332_gb300 as P
+    W, H = 130, 100
+    rng = np.random.default_rng(5)
+    yy, xx = np.mgrid[0:H, 0:W]
+    rings = np.full((H, W, 3), (225, 215, 228), np.uint8)
+    for cx, cy, r in ((30, 30, 12), (64, 64, 9), (95, 33, 14), (100, 80, 10)):
+        d = np.hypot(xx - cx, yy - cy)
+        rings[(d <= r) & (d > r - 4)] = (90, 60, 140)
+    kinds = [synth.tile(W, H, 3, n_nuclei=25, frac_cluster=0.4), rng.integers(0, 256, (H, W, 3)).astype(np.uint8), rings,
+             np.full((H, W, 3), 230, np.uint8), synth.tile(W, H, 4, n_nuclei=0), synth.tile(W, H, 5, n_nuclei=60, frac_chain=0.5)]
+    refs = [oracle_all(k) for k in kinds]
+    pipe = P.Pipe(0, autotune=0)
+    dev = torch.device("cuda", 0)
+    rgb = [torch.from_numpy(np.ascontiguousarray(k)).to(dev) for k in kinds]
+    hem = torch.empty((n, H, W), dtype=torch.uint8, device=dev)
+    lab = torch.full((n, H, W), -1, dtype=torch.int32, device=dev)
+    edt = torch.empty((n, H, W), dtype=torch.int32, device=dev)
+    nobj = torch.zeros(n, dtype=torch.int32, device=dev)
+    feats = torch.zeros((n, 700, 15), dtype=torch.float32, device=dev)
+    pipe.seg_features_batch([dict(rgb=rgb[i % len(kinds)], hem8=hem[i], labels=lab[i], edt=edt[i], n_objects=nobj[i:i + 1],
+                                  feats=feats[i]) for i in range(n)])
+    torch.cuda.synchronize()
+    assert pipe.status() == P.PIPE_OK
+    for k, r in enumerate(refs[:n]):
+        want = torch.from_numpy(r["labels"]).to(dev), torch.from_numpy(r["edt"]).to(dev)
+        assert bool((nobj[k::len(kinds)] == r["K"]).all())
+        assert bool((lab[k::len(kinds)] == want[0]).all()) and bool((edt[k::len(kinds)] == want[1]).all())
+        assert_feats_close(feats[k].cpu().numpy()[:r["K"]], r["feats"])
+    pipe.close()
