@@ -49,6 +49,7 @@ constexpr int WS_WARPS = 4;      // objects in flight per CTA of the small-box k
 constexpr int WS_STAGE = 1024;   // staged box (with margin) capacity per warp of that kernel, pixels
 constexpr int WS_PX_BYTES = 14;  // stage bytes per pixel: e 4, w 4, dr 2, two frontier lists 2 + 2
 constexpr int WS_LARGE_SMEM = 96 * 1024;  // dynamic stage of a large-box CTA (one warp)
+constexpr int WS_OUT_PASSES = 8;  // passes that spread "on no marker" before the union-find
 constexpr unsigned WFULL = 0xffffffffu;
 
 __device__ __forceinline__ int ws_isqrt(int v) {  // floor(sqrt(v)), exact
@@ -134,6 +135,12 @@ __device__ __forceinline__ bool ws_nb_in(const B& b, int q) {
     else return b.in(q);
 }
 
+// neighbour j (0..7, raster order) of pixel s of a shared-memory box
+__device__ __forceinline__ int ws_nb8(const SBox& b, int s, int j) {
+    const int k = j < 4 ? j : j + 1;
+    return s + (k / 3 - 1) * b.ww + (k % 3 - 1);
+}
+
 template <class B>
 __device__ __forceinline__ int ws_find(const B& b, int x) {
     // path halving: a non-root is pointed at its grandparent (an ancestor,
@@ -208,29 +215,14 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
         if (!__any_sync(WFULL, ch)) break;
     }
 
-    // 2. plateaus of equal R: union-find, then the non-maximal flag on roots
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
-        const int s = b.stor(it);
-        if (b.in(s)) b.w[s] = (Wt)s;
-    }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
-        const int s = b.stor(it);
-        if (!b.in(s)) continue;
-        const int r = b.dr[s] >> 8;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {  // the neighbours before s in raster order
-            const int q = b.nb(it, s, j < 3 ? -1 : 0, j < 3 ? j - 1 : -1);
-            if (!ws_nb_in(b, q)) continue;
-            if ((int)(b.dr[q] >> 8) == r) ws_unite(b, s, q);
-        }
-    }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
-        const int s = b.stor(it);
-        if (b.in(s)) b.w[s] = (Wt)ws_find(b, s);
-    }
-    __syncwarp();
+    // 2. markers.  Pixels with a higher neighbour are on no marker, and neither
+    // are pixels of equal R beside one of those: a few passes of that leave
+    // little but the markers themselves.  What is left is joined by union-find
+    // (adjacent pixels left over have equal R: of two different ones the lower
+    // has a higher neighbour), and a component beside a pixel of equal R that
+    // was left out is no marker either (only possible if the passes were cut
+    // short, by a plateau longer than they reach).
+    constexpr Wt OUT = UNNAMED - 1;  // on no marker
     for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s)) continue;
@@ -240,16 +232,92 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
         for (int j = 0; j < 9; j++) {
             if (j == 4) continue;
             const int q = b.nb(it, s, j / 3 - 1, j % 3 - 1);
-            if (!ws_nb_in(b, q)) continue;
-            higher |= (int)(b.dr[q] >> 8) > r;
+            if constexpr (B::GLOBAL) {
+                if (!ws_nb_in(b, q)) continue;
+            }
+            higher |= (int)(b.dr[q] >> 8) > r;  // 0 off the object
         }
-        if (higher) atomicOr((Wt*)(b.w + (int)(b.w[s] & IDX)), FLAG);
+        b.w[s] = higher ? OUT : (Wt)s;
     }
     __syncwarp();
+    // Whether a pixel left over touches one of equal R that is out.  In shared
+    // memory all sixteen words are read at once and then compared (branches
+    // between them cost about 2000 cycles per pixel instead of 300).
+    auto beside_out = [&](const Walk& it, int s) -> bool {
+        const int r = b.dr[s] >> 8;
+        bool out = false;
+        if constexpr (B::GLOBAL) {
+#pragma unroll
+            for (int j = 0; j < 9; j++) {
+                if (j == 4) continue;
+                const int q = b.nb(it, s, j / 3 - 1, j % 3 - 1);
+                if (!ws_nb_in(b, q)) continue;
+                out |= (int)(b.dr[q] >> 8) == r && b.w[q] == OUT;
+            }
+        } else {
+            unsigned dq[8];
+            Wt wq[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const int q = ws_nb8(b, s, j);
+                dq[j] = b.dr[q];
+                wq[j] = b.w[q];
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j++) out |= ((int)(dq[j] >> 8) == r) & (wq[j] == OUT);
+        }
+        return out;
+    };
+    bool settled = false;
+    for (int pass = 0; pass < WS_OUT_PASSES && !settled; pass++) {
+        bool ch = false;
+        for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+            const int s = b.stor(it);
+            if (!b.in(s) || b.w[s] == OUT || !beside_out(it, s)) continue;
+            b.w[s] = OUT;
+            ch = true;
+        }
+        __syncwarp();
+        settled = !__any_sync(WFULL, ch);
+    }
+    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+        const int s = b.stor(it);
+        if (!b.in(s) || b.w[s] == OUT) continue;
+        unsigned with = 0;  // the neighbours before s in raster order to join
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int q = b.nb(it, s, j < 3 ? -1 : 0, j < 3 ? j - 1 : -1);
+            if constexpr (B::GLOBAL) {
+                if (!ws_nb_in(b, q) || b.w[q] == OUT) continue;
+                with |= 1u << j;
+            } else {
+                with |= (unsigned)(b.in(q) & (b.w[q] != OUT)) << j;
+            }
+        }
+        for (; with; with &= with - 1) {
+            const int j = __ffs(with) - 1;
+            ws_unite(b, s, b.nb(it, s, j < 3 ? -1 : 0, j < 3 ? j - 1 : -1));
+        }
+    }
+    __syncwarp();
+    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+        const int s = b.stor(it);
+        if (b.in(s) && b.w[s] != OUT) b.w[s] = (Wt)ws_find(b, s);
+    }
+    __syncwarp();
+    if (!settled) {
+        for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+            const int s = b.stor(it);
+            if (!b.in(s) || b.w[s] == OUT || !beside_out(it, s)) continue;
+            atomicOr((Wt*)(b.w + (int)(b.w[s] & IDX)), FLAG);
+        }
+        __syncwarp();
+    }
     for (Walk it(lane, b.ww); it.f < b.n; it.next()) {  // bit 8 of dr: a marker pixel (R no longer needed)
         const int s = b.stor(it);
         if (!b.in(s)) continue;
-        const bool mk = !(b.w[(int)(b.w[s] & IDX)] & FLAG);
+        const Wt w = b.w[s];
+        const bool mk = w != OUT && !(b.w[(int)(w & IDX)] & FLAG);
         b.dr[s] = (uint16_t)((b.dr[s] & 0xFF) | (mk ? 0x100 : 0));
     }
     __syncwarp();
@@ -318,81 +386,93 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
                 const unsigned old = atomicOr((unsigned*)(a & ~(uintptr_t)3), 0x400u << sh);
                 return !((old >> sh) & 0x400u);
             };
+            // the unnamed object pixels around s that are not in F yet, as a list
+            // entry each, behind the n entries of `to`; all lanes call it together
+            auto append = [&](bool named, int s, volatile uint16_t* to, int n) -> int {
+                unsigned open = 0, mine = 0;
+                if (named) {
+                    Wt wq[8];
+                    unsigned dq[8];
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const int q = ws_nb8(b, s, j);
+                        wq[j] = b.w[q];
+                        dq[j] = b.dr[q];
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; j++)
+                        open |= (unsigned)((wq[j] == UNNAMED) & ((dq[j] & 0xFF) != 0) & !(dq[j] & 0x400)) << j;
+                }
+                for (; open; open &= open - 1) {
+                    const int j = __ffs(open) - 1;
+                    if (enter(ws_nb8(b, s, j))) mine |= 1u << j;
+                }
+                const int c = __popc(mine);
+                int at = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(WFULL, at, o);
+                    if (lane >= o) at += v;
+                }
+                const int total = __shfl_sync(WFULL, at, 31);
+                at += n - c;
+                for (; mine; mine &= mine - 1) to[at++] = (uint16_t)ws_nb8(b, s, __ffs(mine) - 1);
+                return n + total;
+            };
             volatile uint16_t* cur = b.la;
             volatile uint16_t* nxt = b.lb;
             int m = 0;
             for (int f0 = 0; f0 < b.n; f0 += 32) {  // neighbours of the markers
                 const int s = f0 + lane;
                 const bool mk = s < b.n && b.w[s] != UNNAMED;
-#pragma unroll
-                for (int j = 0; j < 9; j++) {
-                    if (j == 4) continue;
-                    const int q = s + (j / 3 - 1) * b.ww + (j % 3 - 1);
-                    const bool add = mk && b.in(q) && b.w[q] == UNNAMED && enter(q);
-                    const unsigned bal = __ballot_sync(WFULL, add);
-                    if (add) cur[m + __popc(bal & lt)] = (uint16_t)q;
-                    m += __popc(bal);
-                }
+                if (__any_sync(WFULL, mk)) m = append(mk, s, cur, m);
             }
             __syncwarp();
+            // every entry has a neighbour named in an earlier wave, so the next L
+            // is known before a wave: no wave names nothing
             int L = 256;
             for (unsigned wave = 1; m > 0; wave++) {
                 if (wave >= cap) {
                     if (lane == 0) set_status(status, ST_OVERFLOW);
                     return 0;
                 }
-                int named = 0, fmax = -1, nm = 0;
+                int fmax = 0, nm = 0;
+                for (int i = lane; i < m; i += 32) fmax = max(fmax, (int)(b.dr[cur[i]] & 0xFF));
+                L = min(L, (int)__reduce_max_sync(WFULL, (unsigned)fmax));
                 for (int i0 = 0; i0 < m; i0 += 32) {
                     const int i = i0 + lane;
                     const int s = i < m ? (int)cur[i] : -1;
-                    bool took = false;
-                    if (s >= 0) {
+                    const bool took = s >= 0 && (int)(b.dr[s] & 0xFF) >= L;
+                    if (took) {
                         int be = 0;
                         Wt bn = IDX;
+                        Wt wq[8];
+                        int eq[8];
 #pragma unroll
-                        for (int j = 0; j < 9; j++) {
-                            if (j == 4) continue;
-                            const int q = s + (j / 3 - 1) * b.ww + (j % 3 - 1);
-                            const Wt wq = b.w[q];
-                            if ((wq >> B::SH) >= (Wt)wave) continue;  // unnamed, or named in this wave
-                            const int eq = b.e[q];
-                            const Wt nq = wq & IDX;
-                            if (eq > be || (eq == be && nq < bn)) {
-                                be = eq;
+                        for (int j = 0; j < 8; j++) {
+                            const int q = ws_nb8(b, s, j);
+                            wq[j] = b.w[q];
+                            eq[j] = b.e[q];
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            const bool old = (wq[j] >> B::SH) < (Wt)wave;  // named in an earlier wave
+                            const Wt nq = wq[j] & IDX;
+                            if (old & ((eq[j] > be) | ((eq[j] == be) & (nq < bn)))) {
+                                be = eq[j];
                                 bn = nq;
                             }
                         }
-                        if (be > 0) {
-                            const int d = b.dr[s] & 0xFF;
-                            fmax = max(fmax, d);
-                            if (d >= L) {
-                                b.w[s] = ((Wt)wave << B::SH) | bn;
-                                named++;
-                                took = true;
-                            }
-                        }
+                        b.w[s] = ((Wt)wave << B::SH) | bn;
                     }
                     const bool keep = s >= 0 && !took;
                     unsigned bal = __ballot_sync(WFULL, keep);
                     if (keep) nxt[nm + __popc(bal & lt)] = (uint16_t)s;
                     nm += __popc(bal);
-#pragma unroll
-                    for (int j = 0; j < 9; j++) {  // unnamed neighbours of a pixel just named enter F
-                        if (j == 4) continue;
-                        const int q = s + (j / 3 - 1) * b.ww + (j % 3 - 1);
-                        const bool add = took && b.in(q) && b.w[q] == UNNAMED && enter(q);
-                        bal = __ballot_sync(WFULL, add);
-                        if (add) nxt[nm + __popc(bal & lt)] = (uint16_t)q;
-                        nm += __popc(bal);
-                    }
+                    // unnamed neighbours of a pixel just named enter F
+                    if (__any_sync(WFULL, took)) nm = append(took, s, nxt, nm);
                 }
                 __syncwarp();
-                named = __reduce_add_sync(WFULL, (unsigned)named);
-                fmax = (int)__reduce_max_sync(WFULL, (unsigned)(fmax + 1)) - 1;
-                if (!named) {
-                    if (fmax < 0) break;
-                    L = fmax;
-                }
                 volatile uint16_t* t = cur;
                 cur = nxt;
                 nxt = t;
