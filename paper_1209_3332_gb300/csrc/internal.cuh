@@ -296,19 +296,15 @@ struct WsDesc {
     int obj_base;         // first object item of this tile
     int seg_base;         // first box row segment of this tile
 };
-// descs: host copy; d_descs: device array of the same length
+// descs: host copy; d_descs: device array of the same length; cnt: an int per
+// object (basin counts, then their exclusive prefix); next: WS_COUNTERS ints and
+// an int per object (draw counters and lists, set up by the launcher); status: a
+// device int; side: a second stream for the larger boxes (fork and join through
+// the two events)
+constexpr int WS_COUNTERS = 5;
 void launch_watershed_batch(const std::vector<WsDesc>& descs, WsDesc* d_descs, int h, int4* bbox, int* cnt,
                             int* next, void* scratch, size_t scratch_px, int* status, int sms, cudaStream_t s,
                             cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Profiler* pf);
-// scratch of the watershed's out-of-stage boxes: a 64-bit and a 16-bit word per pixel
-size_t watershed_scratch_bytes(int W, int H);
-// cnt: K ints (per-object basin counts, then their exclusive prefix); next: 3 + K device ints (the
-// large-box draw counter, the large-box list length and the small-box draw counter, zeroed by the
-// launcher, then the large-box list); status: a device int
-// side: a second stream for the large boxes (fork/join through the two events)
-void launch_watershed(const int32_t* labels, const int32_t* edt, int W, int H, int K, int h, int32_t* out,
-                      int32_t* n_basins, int4* bbox, int* cnt, int* next, void* scratch, int* status, int sms,
-                      cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Profiler* pf);
 // RBC detection planes: d = R - max(G, B); marker = d >= t_hi, mask = d >= t_lo.
 void launch_rbc_planes(const GrowLaunch& G, const uint8_t* rgb, size_t pitch, int t_lo, int t_hi, cudaStream_t s,
                        Profiler* pf);

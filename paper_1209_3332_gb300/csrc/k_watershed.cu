@@ -41,14 +41,17 @@
 // beyond that stage run the same steps (with a full-box scan per wave) on
 // image-sized scratch planes in global memory.  A scan of the per-object
 // basin counts and a pass adding each object's offset finish the numbering.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace nucseg {
 
-constexpr int WS_WARPS = 4;      // objects in flight per CTA of the small-box kernel (one per warp)
-constexpr int WS_STAGE = 1024;   // staged box (with margin) capacity per warp of that kernel, pixels
+constexpr int WS_WARPS = 4;      // warps per CTA: one object each (small boxes) or one together
+constexpr int WS_STAGE = 384;    // staged box (with margin) capacity per warp of the small-box kernel, pixels
+constexpr int WS_MIDDLE = 1024;  // staged box capacity of a CTA with the small stage
 constexpr int WS_PX_BYTES = 14;  // stage bytes per pixel: e 4, w 4, dr 2, two frontier lists 2 + 2
-constexpr int WS_LARGE_SMEM = 96 * 1024;  // dynamic stage of a large-box CTA (one warp)
+constexpr int WS_LARGE_SMEM = 96 * 1024;  // dynamic stage of a CTA with the large stage
 constexpr int WS_OUT_PASSES = 8;  // passes that spread "on no marker" before the union-find
 constexpr unsigned WFULL = 0xffffffffu;
 
@@ -60,24 +63,54 @@ __device__ __forceinline__ int ws_isqrt(int v) {  // floor(sqrt(v)), exact
     return r;
 }
 
-// Flat positions f = lane, lane+32, ... of a row-major box of width ww, with
+// The threads that split one object: a warp, or the NW warps of a CTA.
+template <int NW>
+struct Team {
+    static constexpr int N = 32 * NW;
+    int t;    // thread of the team
+    int* sh;  // NW > 1: shared, the lengths of the two frontier lists, a result, and a word per warp
+    __device__ __forceinline__ int lane() const { return t & 31; }
+    __device__ __forceinline__ void sync() const {
+        if constexpr (NW == 1) __syncwarp(); else __syncthreads();
+    }
+    // sync, and whether p held for some thread
+    __device__ __forceinline__ bool any(bool p) const {
+        if constexpr (NW == 1) { __syncwarp(); return __any_sync(WFULL, p); }
+        else return __syncthreads_or(p);
+    }
+    // the largest v >= 0
+    __device__ __forceinline__ int max_of(int v) const {
+        v = (int)__reduce_max_sync(WFULL, (unsigned)v);
+        if constexpr (NW > 1) {
+            __syncthreads();
+            if (lane() == 0) sh[3 + (t >> 5)] = v;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < NW; i++) v = max(v, sh[3 + i]);
+        }
+        return v;
+    }
+};
+
+// Flat positions f = f0, f0 + STEP, ... of a row-major box of width ww, with
 // (y, x) of f kept without a division per step.
-struct Walk {
+template <int STEP>
+struct WalkBy {
     int f, y, x, qy, qx, ww;
-    __device__ __forceinline__ Walk(int f0, int ww_) : f(f0), ww(ww_) {
+    __device__ __forceinline__ WalkBy(int f0, int ww_) : f(f0), ww(ww_) {
         y = f0 / ww;
         x = f0 - y * ww;
-        qy = 32 / ww;
-        qx = 32 - qy * ww;
+        qy = STEP / ww;
+        qx = STEP - qy * ww;
     }
     __device__ __forceinline__ void next() {
-        f += 32;
+        f += STEP;
         x += qx;
         y += qy;
         if (x >= ww) { x -= ww; y++; }
     }
     __device__ __forceinline__ void prev() {
-        f -= 32;
+        f -= STEP;
         x -= qx;
         y -= qy;
         if (x < 0) { x += ww; y--; }
@@ -97,10 +130,13 @@ struct SBox {
     volatile uint16_t *la, *lb;                 // frontier lists, n entries each
     int ww, n;                                  // walk width, flat size
     int gx0, gy0, W;                            // image position of flat (0, 0)
-    __device__ __forceinline__ int stor(const Walk& it) const { return it.f; }
+    template <class WK>
+    __device__ __forceinline__ int stor(const WK& it) const { return it.f; }
     __device__ __forceinline__ bool in(int s) const { return (dr[s] & 0xFF) != 0; }
-    __device__ __forceinline__ int nb(const Walk&, int s, int dy, int dx) const { return s + dy * ww + dx; }
-    __device__ __forceinline__ size_t gidx(const Walk& it) const {
+    template <class WK>
+    __device__ __forceinline__ int nb(const WK&, int s, int dy, int dx) const { return s + dy * ww + dx; }
+    template <class WK>
+    __device__ __forceinline__ size_t gidx(const WK& it) const {
         return (size_t)(gy0 + it.y) * W + (gx0 + it.x);
     }
 };
@@ -118,13 +154,16 @@ struct GBox {
     int k;
     int ww, bh, n;
     int gx0, gy0, W;
-    __device__ __forceinline__ int stor(const Walk& it) const { return it.y * W + it.x; }
+    template <class WK>
+    __device__ __forceinline__ int stor(const WK& it) const { return it.y * W + it.x; }
     __device__ __forceinline__ bool in(int s) const { return lab[s] == k; }
-    __device__ __forceinline__ int nb(const Walk& it, int s, int dy, int dx) const {
+    template <class WK>
+    __device__ __forceinline__ int nb(const WK& it, int s, int dy, int dx) const {
         return ((unsigned)(it.y + dy) < (unsigned)bh && (unsigned)(it.x + dx) < (unsigned)ww) ? s + dy * W + dx
                                                                                               : -1;
     }
-    __device__ __forceinline__ size_t gidx(const Walk& it) const {
+    template <class WK>
+    __device__ __forceinline__ size_t gidx(const WK& it) const {
         return (size_t)(gy0 + it.y) * W + (gx0 + it.x);
     }
 };
@@ -173,9 +212,11 @@ __device__ __forceinline__ void ws_unite(const B& b, int a, int c) {
 
 // The four steps on one object.  Returns the number of basins (0 on a wave
 // count beyond the cap, after setting the status word).
-template <class B>
-__device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
+template <class B, int NW>
+__device__ int ws_object(const B& b, const Team<NW>& team, int32_t* out, int* status) {
     using Wt = typename B::Wt;
+    using Walk = WalkBy<Team<NW>::N>;
+    const int t = team.t, lane = team.lane();
     constexpr Wt IDX = ((Wt)1 << B::SH) - 1;
     constexpr Wt FLAG = (Wt)1 << (sizeof(Wt) * 8 - 1);
     constexpr Wt UNNAMED = ~(Wt)0;
@@ -205,14 +246,13 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
             }
         };
         if ((pass & 1) == 0) {
-            for (Walk it(lane, b.ww); it.f < b.n; it.next()) relax(it);
+            for (Walk it(t, b.ww); it.f < b.n; it.next()) relax(it);
         } else {
-            const int last = b.n - 1 - lane;
+            const int last = b.n - 1 - t;
             if (last >= 0)
                 for (Walk it(last, b.ww); it.f >= 0; it.prev()) relax(it);
         }
-        __syncwarp();
-        if (!__any_sync(WFULL, ch)) break;
+        if (!team.any(ch)) break;
     }
 
     // 2. markers.  Pixels with a higher neighbour are on no marker, and neither
@@ -223,7 +263,7 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
     // was left out is no marker either (only possible if the passes were cut
     // short, by a plateau longer than they reach).
     constexpr Wt OUT = UNNAMED - 1;  // on no marker
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         const int r = b.dr[s] >> 8;
@@ -239,7 +279,7 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
         }
         b.w[s] = higher ? OUT : (Wt)s;
     }
-    __syncwarp();
+    team.sync();
     // Whether a pixel left over touches one of equal R that is out.  In shared
     // memory all sixteen words are read at once and then compared (branches
     // between them cost about 2000 cycles per pixel instead of 300).
@@ -271,16 +311,15 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
     bool settled = false;
     for (int pass = 0; pass < WS_OUT_PASSES && !settled; pass++) {
         bool ch = false;
-        for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+        for (Walk it(t, b.ww); it.f < b.n; it.next()) {
             const int s = b.stor(it);
             if (!b.in(s) || b.w[s] == OUT || !beside_out(it, s)) continue;
             b.w[s] = OUT;
             ch = true;
         }
-        __syncwarp();
-        settled = !__any_sync(WFULL, ch);
+        settled = !team.any(ch);
     }
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s) || b.w[s] == OUT) continue;
         unsigned with = 0;  // the neighbours before s in raster order to join
@@ -299,34 +338,34 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
             ws_unite(b, s, b.nb(it, s, j < 3 ? -1 : 0, j < 3 ? j - 1 : -1));
         }
     }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    team.sync();
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (b.in(s) && b.w[s] != OUT) b.w[s] = (Wt)ws_find(b, s);
     }
-    __syncwarp();
+    team.sync();
     if (!settled) {
-        for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+        for (Walk it(t, b.ww); it.f < b.n; it.next()) {
             const int s = b.stor(it);
             if (!b.in(s) || b.w[s] == OUT || !beside_out(it, s)) continue;
             atomicOr((Wt*)(b.w + (int)(b.w[s] & IDX)), FLAG);
         }
-        __syncwarp();
+        team.sync();
     }
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {  // bit 8 of dr: a marker pixel (R no longer needed)
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {  // bit 8 of dr: a marker pixel (R no longer needed)
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         const Wt w = b.w[s];
         const bool mk = w != OUT && !(b.w[(int)(w & IDX)] & FLAG);
         b.dr[s] = (uint16_t)((b.dr[s] & 0xFF) | (mk ? 0x100 : 0));
     }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {  // markers: stamp 0, name = root
+    team.sync();
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {  // markers: stamp 0, name = root
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         b.w[s] = (b.dr[s] & 0x100) ? (b.w[s] & IDX) : UNNAMED;
     }
-    __syncwarp();
+    team.sync();
 
     // 3. flooding in synchronous waves
     {
@@ -336,11 +375,11 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
             int L = 256;  // above every d: the first pass only measures F
             for (unsigned wave = 1;; wave++) {
                 if (wave >= cap) {
-                    if (lane == 0) set_status(status, ST_OVERFLOW);
+                    if (t == 0) set_status(status, ST_OVERFLOW);
                     return 0;
                 }
                 int named = 0, fmax = -1;
-                for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+                for (Walk it(t, b.ww); it.f < b.n; it.next()) {
                     const int s = b.stor(it);
                     if (!b.in(s) || b.w[s] != UNNAMED) continue;
                     int be = 0;
@@ -368,10 +407,9 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
                         }
                     }
                 }
-                __syncwarp();
-                named = __reduce_add_sync(WFULL, (unsigned)named);
-                fmax = (int)__reduce_max_sync(WFULL, (unsigned)(fmax + 1)) - 1;
-                if (!named) {
+                const bool some = team.any(named > 0);
+                fmax = team.max_of(fmax + 1) - 1;
+                if (!some) {
                     if (fmax < 0) break;
                     L = fmax;
                 }
@@ -379,16 +417,17 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
         } else {
             // F as a list: entries enter once (bit 10 of dr, set atomically on
             // the 32-bit word holding it; nothing else writes dr meanwhile)
-            const unsigned lt = (1u << lane) - 1;
             auto enter = [&](int q) -> bool {
                 const uintptr_t a = (uintptr_t)(b.dr + q);
                 const unsigned sh = (unsigned)(a & 2) * 8;
                 const unsigned old = atomicOr((unsigned*)(a & ~(uintptr_t)3), 0x400u << sh);
                 return !((old >> sh) & 0x400u);
             };
-            // the unnamed object pixels around s that are not in F yet, as a list
-            // entry each, behind the n entries of `to`; all lanes call it together
-            auto append = [&](bool named, int s, volatile uint16_t* to, int n) -> int {
+            // Puts `self` (if keep) and, if named, the unnamed object pixels around
+            // s that are not in F yet into list `to`; the lanes of a warp call it
+            // together.  The list's length is in len (a warp alone) or shared.
+            int len = 0;
+            auto append = [&](bool keep, bool named, int s, volatile uint16_t* to, int which) {
                 unsigned open = 0, mine = 0;
                 if (named) {
                     Wt wq[8];
@@ -407,7 +446,7 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
                     const int j = __ffs(open) - 1;
                     if (enter(ws_nb8(b, s, j))) mine |= 1u << j;
                 }
-                const int c = __popc(mine);
+                const int c = __popc(mine) + (keep ? 1 : 0);
                 int at = c;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -415,31 +454,56 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
                     if (lane >= o) at += v;
                 }
                 const int total = __shfl_sync(WFULL, at, 31);
-                at += n - c;
+                int base = len;
+                if constexpr (NW > 1) {
+                    if (lane == 0) base = atomicAdd(&team.sh[which], total);
+                    base = __shfl_sync(WFULL, base, 0);
+                } else {
+                    len += total;
+                }
+                at += base - c;
+                if (keep) to[at++] = (uint16_t)s;
                 for (; mine; mine &= mine - 1) to[at++] = (uint16_t)ws_nb8(b, s, __ffs(mine) - 1);
-                return n + total;
+            };
+            // the length of list `which` after all appends; the other one starts empty
+            auto length = [&](int which) -> int {
+                team.sync();
+                if constexpr (NW > 1) {
+                    const int m = *(volatile int*)&team.sh[which];
+                    if (t == 0) team.sh[1 - which] = 0;  // seen before the next append: a wave's max_of lies between
+                    return m;
+                } else {
+                    const int m = len;
+                    len = 0;
+                    return m;
+                }
             };
             volatile uint16_t* cur = b.la;
             volatile uint16_t* nxt = b.lb;
-            int m = 0;
-            for (int f0 = 0; f0 < b.n; f0 += 32) {  // neighbours of the markers
+            int which = 0;
+            if constexpr (NW > 1) {
+                if (t == 0) team.sh[0] = 0;
+                team.sync();
+            }
+            for (int f0 = t - lane; f0 < b.n; f0 += Team<NW>::N) {  // neighbours of the markers
                 const int s = f0 + lane;
                 const bool mk = s < b.n && b.w[s] != UNNAMED;
-                if (__any_sync(WFULL, mk)) m = append(mk, s, cur, m);
+                if (__any_sync(WFULL, mk)) append(false, mk, s, cur, which);
             }
-            __syncwarp();
+            int m = length(which);
             // every entry has a neighbour named in an earlier wave, so the next L
             // is known before a wave: no wave names nothing
             int L = 256;
             for (unsigned wave = 1; m > 0; wave++) {
                 if (wave >= cap) {
-                    if (lane == 0) set_status(status, ST_OVERFLOW);
+                    if (t == 0) set_status(status, ST_OVERFLOW);
                     return 0;
                 }
-                int fmax = 0, nm = 0;
-                for (int i = lane; i < m; i += 32) fmax = max(fmax, (int)(b.dr[cur[i]] & 0xFF));
-                L = min(L, (int)__reduce_max_sync(WFULL, (unsigned)fmax));
-                for (int i0 = 0; i0 < m; i0 += 32) {
+                int fmax = 0;
+                for (int i = t; i < m; i += Team<NW>::N) fmax = max(fmax, (int)(b.dr[cur[i]] & 0xFF));
+                L = min(L, team.max_of(fmax));
+                which = 1 - which;
+                for (int i0 = t - lane; i0 < m; i0 += Team<NW>::N) {
                     const int i = i0 + lane;
                     const int s = i < m ? (int)cur[i] : -1;
                     const bool took = s >= 0 && (int)(b.dr[s] & 0xFF) >= L;
@@ -465,62 +529,58 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
                         }
                         b.w[s] = ((Wt)wave << B::SH) | bn;
                     }
-                    const bool keep = s >= 0 && !took;
-                    unsigned bal = __ballot_sync(WFULL, keep);
-                    if (keep) nxt[nm + __popc(bal & lt)] = (uint16_t)s;
-                    nm += __popc(bal);
-                    // unnamed neighbours of a pixel just named enter F
-                    if (__any_sync(WFULL, took)) nm = append(took, s, nxt, nm);
+                    append(s >= 0 && !took, took, s, nxt, which);
                 }
-                __syncwarp();
-                volatile uint16_t* t = cur;
+                m = length(which);
+                volatile uint16_t* sw = cur;
                 cur = nxt;
-                nxt = t;
-                m = nm;
+                nxt = sw;
             }
         }
     }
 
     // 4. ranks of the basins by first pixel
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {  // roots: first-pixel field to "none"
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {  // roots: first-pixel field to "none"
         const int s = b.stor(it);
         if (b.in(s) && (int)(b.w[s] & IDX) == s) b.w[s] = (IDX << B::SH) | (Wt)s;
     }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    team.sync();
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         const Wt nm = b.w[s] & IDX;
         atomicMin((Wt*)(b.w + (int)nm), ((Wt)s << B::SH) | nm);
     }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {  // bit 9 of dr: the first pixel of its basin
+    team.sync();
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {  // bit 9 of dr: the first pixel of its basin
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         const int nm = (int)(b.w[s] & IDX);
         if ((int)(b.w[nm] >> B::SH) == s) b.dr[s] = (uint16_t)(b.dr[s] | 0x200);
     }
-    __syncwarp();
+    team.sync();
     int run = 0;
-    for (int f0 = 0; f0 < b.n; f0 += 32) {  // raster order: rank = first pixels up to this one
-        const int f = f0 + lane;
-        bool first = false;
-        int s = 0;
-        if (f < b.n) {
-            const Walk it(f, b.ww);
-            s = b.stor(it);
-            first = b.in(s) && (b.dr[s] & 0x200);
+    if (t < 32) {
+        for (int f0 = 0; f0 < b.n; f0 += 32) {  // raster order: rank = first pixels up to this one
+            const int f = f0 + lane;
+            bool first = false;
+            int s = 0;
+            if (f < b.n) {
+                const Walk it(f, b.ww);
+                s = b.stor(it);
+                first = b.in(s) && (b.dr[s] & 0x200);
+            }
+            const unsigned bal = __ballot_sync(WFULL, first);
+            if (first) {
+                const Wt nm = b.w[s] & IDX;
+                const int rank = run + __popc(bal & ((1u << lane) - 1)) + 1;
+                b.w[(int)nm] = ((Wt)rank << B::SH) | nm;
+            }
+            run += __popc(bal);
         }
-        const unsigned bal = __ballot_sync(WFULL, first);
-        if (first) {
-            const Wt nm = b.w[s] & IDX;
-            const int rank = run + __popc(bal & ((1u << lane) - 1)) + 1;
-            b.w[(int)nm] = ((Wt)rank << B::SH) | nm;
-        }
-        run += __popc(bal);
     }
-    __syncwarp();
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    team.sync();
+    for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         out[b.gidx(it)] = (int32_t)(b.w[(int)(b.w[s] & IDX)] >> B::SH);
@@ -529,9 +589,11 @@ __device__ int ws_object(const B& b, int lane, int32_t* out, int* status) {
 }
 
 // Large boxes: the same steps on global scratch planes, kept out of line.
+template <int NW>
 __device__ __noinline__ int ws_object_global(const int32_t* labels, const int32_t* edt, int W, int k, int4 bx,
                                              int h, uint16_t* gdr, unsigned long long* gw, int32_t* out,
-                                             int* status, int lane) {
+                                             int* status, const Team<NW>& team) {
+    using Walk = WalkBy<Team<NW>::N>;
     GBox b;
     const size_t o = (size_t)bx.y * W + bx.x;
     b.dr = gdr + o;
@@ -545,22 +607,24 @@ __device__ __noinline__ int ws_object_global(const int32_t* labels, const int32_
     b.gx0 = bx.x;
     b.gy0 = bx.y;
     b.W = W;
-    for (Walk it(lane, b.ww); it.f < b.n; it.next()) {
+    for (Walk it(team.t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
         if (!b.in(s)) continue;
         const int d = min(255, ws_isqrt(b.e[s]));
         b.dr[s] = (uint16_t)(d | ((d > h ? d - h : 0) << 8));
     }
-    __syncwarp();
-    return ws_object(b, lane, out, status);
+    team.sync();
+    return ws_object(b, team, out, status);
 }
 
 // Stages one object's box plus margin into a shared-memory stage of `cap`
 // pixels (e, w, dr and the two frontier lists, laid out back to back) and
 // splits it there.
+template <int NW>
 __device__ __forceinline__ int ws_staged(const int32_t* __restrict__ labels, const int32_t* __restrict__ edt,
                                          int W, int H, int k, int4 bx, int h, char* stage, int cap,
-                                         int32_t* out, int* status, int lane) {
+                                         int32_t* out, int* status, const Team<NW>& team) {
+    using Walk = WalkBy<Team<NW>::N>;
     const int BW = bx.z - bx.x + 3, BH = bx.w - bx.y + 3;
     SBox b;
     b.e = (int32_t*)stage;
@@ -573,7 +637,7 @@ __device__ __forceinline__ int ws_staged(const int32_t* __restrict__ labels, con
     b.gx0 = bx.x - 1;
     b.gy0 = bx.y - 1;
     b.W = W;
-    for (Walk it(lane, BW); it.f < b.n; it.next()) {
+    for (Walk it(team.t, BW); it.f < b.n; it.next()) {
         const int gy = b.gy0 + it.y, gx = b.gx0 + it.x;
         int ev = 0;
         if ((unsigned)gy < (unsigned)H && (unsigned)gx < (unsigned)W) {
@@ -585,69 +649,98 @@ __device__ __forceinline__ int ws_staged(const int32_t* __restrict__ labels, con
         b.e[it.f] = ev;
         b.w[it.f] = 0xffffffffu;
     }
-    __syncwarp();
-    return ws_object(b, lane, out, status);
+    team.sync();
+    return ws_object(b, team, out, status);
 }
 
 __device__ __forceinline__ int ws_box_px(int4 bx) { return (bx.z - bx.x + 3) * (bx.w - bx.y + 3); }
 
-// The next entry for this warp from a launch-wide counter (entries go to
-// whichever warp is free, so a warp that drew a slow object takes no more).
-__device__ __forceinline__ int ws_next(int* next, int lane) {
+// The next entry for this team from a launch-wide counter (entries go to
+// whichever team is free, so one that drew a slow object takes no more).
+template <int NW>
+__device__ __forceinline__ int ws_next(int* next, const Team<NW>& team) {
     int v = 0;
-    if (lane == 0) v = atomicAdd(next, 1);
-    return __shfl_sync(WFULL, v, 0);
+    if constexpr (NW == 1) {
+        if (team.t == 0) v = atomicAdd(next, 1);
+        return __shfl_sync(WFULL, v, 0);
+    } else {
+        __syncthreads();
+        if (team.t == 0) team.sh[2] = atomicAdd(next, 1);
+        __syncthreads();
+        return *(volatile int*)&team.sh[2];
+    }
 }
 
-// Sorts the objects before the two object kernels: an absent object
-// (empty box) gets count 0; an object whose box exceeds the small stage is
-// appended to the large list (next[1] entries).
+// Sorts the objects before the object kernels.  An absent object (empty box)
+// gets count 0.  By its box an object goes to a warp (k_ws_objects), or to a CTA
+// with a small or a large stage (k_ws_team), listed from the front and from the
+// back of `list`: next[1] and next[4] entries.
+// next: large drawn, large listed, small drawn, middle drawn, middle listed
 __global__ void k_ws_classify(const int4* __restrict__ bbox, int total, int* cnt, int* next, int* list) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
     const int4 bx = bbox[i];
     if (bx.z < bx.x) cnt[i] = 0;
-    else if (ws_box_px(bx) > WS_STAGE) list[atomicAdd(next + 1, 1)] = i;
+    else if (ws_box_px(bx) > WS_MIDDLE) list[atomicAdd(next + 1, 1)] = i;
+    else if (ws_box_px(bx) > WS_STAGE) list[total - 1 - atomicAdd(next + 4, 1)] = i;
+}
+
+// The objects of one tile or of many: items are objects numbered across the
+// tiles; the tile of an item is the last descriptor whose obj_base is <= the
+// item (seg_base likewise for box segments).
+__device__ __forceinline__ int ws_desc_of(const WsDesc* __restrict__ D, int n, int item, bool by_seg) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((by_seg ? D[mid].seg_base : D[mid].obj_base) <= item) lo = mid; else hi = mid - 1;
+    }
+    return lo;
 }
 
 // Small boxes: persistent warps drawing objects from a launch-wide counter
 // (next[2]), WS_STAGE pixels of stage each.  Writes the basin's rank inside
 // the object to out and the basin count to cnt[object]; absent objects and
 // larger boxes were sorted out by k_ws_classify.
-__global__ void __launch_bounds__(WS_WARPS * 32) k_ws_objects(const int32_t* __restrict__ labels,
-                                                               const int32_t* __restrict__ edt, int W, int H,
-                                                               int K, int h, const int4* __restrict__ bbox,
-                                                               int32_t* out, int* cnt, int* next, int* status) {
+__global__ void __launch_bounds__(WS_WARPS * 32) k_ws_objects(const WsDesc* __restrict__ D, int n, int total, int h,
+                                                               const int4* __restrict__ bbox, int* cnt, int* next,
+                                                               int* status) {
     extern __shared__ __align__(16) char ws_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5;
+    const Team<1> team{(int)threadIdx.x & 31, nullptr};
     char* stage = ws_smem + (size_t)warp * WS_STAGE * WS_PX_BYTES;
-    for (int obj = ws_next(next + 2, lane); obj < K; obj = ws_next(next + 2, lane)) {
-        const int4 bx = bbox[obj];
+    for (int item = ws_next(next + 2, team); item < total; item = ws_next(next + 2, team)) {
+        const int4 bx = bbox[item];
         if (bx.z < bx.x || ws_box_px(bx) > WS_STAGE) continue;
-        const int c = ws_staged(labels, edt, W, H, obj + 1, bx, h, stage, WS_STAGE, out, status, lane);
-        if (lane == 0) cnt[obj] = c;
+        const WsDesc& T = D[ws_desc_of(D, n, item, false)];
+        const int c = ws_staged(T.labels, T.edt, T.W, T.H, item - T.obj_base + 1, bx, h, stage, WS_STAGE, T.out,
+                                status, team);
+        if (team.t == 0) cnt[item] = c;
         __syncwarp();
     }
 }
 
-// Large boxes: one warp per CTA with a stage of `cap` pixels, drawing from
-// the large list (next[0] the draw counter, next[1] its length); boxes
-// beyond the stage run on the global scratch planes.
-__global__ void __launch_bounds__(32) k_ws_large(const int32_t* __restrict__ labels, const int32_t* __restrict__ edt,
-                                                 int W, int H, int h, const int4* __restrict__ bbox, int32_t* out,
-                                                 int* cnt, int cap, uint16_t* gdr, unsigned long long* gw, int* next,
-                                                 const int* __restrict__ list, int* status) {
+// Larger boxes: the warps of a CTA split one object, with a stage of `cap`
+// pixels; drawn from a list (entries list[0], list[step], ...); boxes beyond the
+// stage run on the global scratch planes.
+__global__ void __launch_bounds__(WS_WARPS * 32) k_ws_team(const WsDesc* __restrict__ D, int n, int h,
+                                                           const int4* __restrict__ bbox, int* cnt, int cap,
+                                                           uint16_t* gdr, unsigned long long* gw, int* draw,
+                                                           const int* __restrict__ listed, const int* __restrict__ list,
+                                                           int step, int* status) {
     extern __shared__ __align__(16) char ws_smem[];
-    const int lane = threadIdx.x;
-    const int nl = next[1];
-    for (int i = ws_next(next, lane); i < nl; i = ws_next(next, lane)) {
-        const int obj = list[i];
-        const int4 bx = bbox[obj];
+    __shared__ int sh[3 + WS_WARPS];
+    const Team<WS_WARPS> team{(int)threadIdx.x, sh};
+    const int nl = *listed;
+    for (int i = ws_next(draw, team); i < nl; i = ws_next(draw, team)) {
+        const int item = list[i * step];
+        const int4 bx = bbox[item];
+        const WsDesc& T = D[ws_desc_of(D, n, item, false)];
+        const int k = item - T.obj_base + 1;
         const int c = ws_box_px(bx) <= cap
-                          ? ws_staged(labels, edt, W, H, obj + 1, bx, h, ws_smem, cap, out, status, lane)
-                          : ws_object_global(labels, edt, W, obj + 1, bx, h, gdr, gw, out, status, lane);
-        if (lane == 0) cnt[obj] = c;
-        __syncwarp();
+                          ? ws_staged(T.labels, T.edt, T.W, T.H, k, bx, h, ws_smem, cap, T.out, status, team)
+                          : ws_object_global(T.labels, T.edt, T.W, k, bx, h, gdr + T.px_base, gw + T.px_base,
+                                             T.out, status, team);
+        if (team.t == 0) cnt[item] = c;
     }
 }
 
@@ -688,44 +781,14 @@ __device__ __forceinline__ void ws_scan_block(int* cnt, int K, int32_t* n_basins
     if (t == 0) *n_basins = carry;
 }
 
-__global__ void __launch_bounds__(1024) k_ws_scan(int* cnt, int K, int32_t* n_basins) {
-    ws_scan_block(cnt, K, n_basins);
-}
-
 // out += o on the pixels of object k inside box bx (one warp).
 __device__ __forceinline__ void ws_offset_obj(const int32_t* __restrict__ labels, int W, int k, int4 bx, int o,
                                               int32_t* out, int lane) {
     const int bw = bx.z - bx.x + 1, n = bw * (bx.w - bx.y + 1);
-    for (Walk it(lane, bw); it.f < n; it.next()) {
+    for (WalkBy<32> it(lane, bw); it.f < n; it.next()) {
         const size_t g = (size_t)(bx.y + it.y) * W + (bx.x + it.x);
         if (labels[g] == k) out[g] += o;
     }
-}
-
-// out += the object's first basin number - 1 on the object's pixels.
-__global__ void __launch_bounds__(256) k_ws_offset(const int32_t* __restrict__ labels, int W, int K,
-                                                   const int4* __restrict__ bbox, const int* __restrict__ off,
-                                                   int32_t* out) {
-    const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int obj = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); obj < K; obj += nw) {
-        const int o = off[obj];
-        const int4 bx = bbox[obj];
-        if (o == 0 || bx.z < bx.x) continue;
-        ws_offset_obj(labels, W, obj + 1, bx, o, out, lane);
-    }
-}
-
-// ---- batched form: the objects of many tiles in one launch per pass ----------------
-// Items are objects numbered across the tiles; the tile of an item is the last
-// descriptor whose obj_base is <= the item (seg_base likewise for box segments).
-__device__ __forceinline__ int ws_desc_of(const WsDesc* __restrict__ D, int n, int item, bool by_seg) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((by_seg ? D[mid].seg_base : D[mid].obj_base) <= item) lo = mid; else hi = mid - 1;
-    }
-    return lo;
 }
 
 constexpr int WS_DESC_PACK = 16;
@@ -738,12 +801,12 @@ __global__ void k_ws_set_desc(WsDesc* dst, WsDescPack pk) {
     if ((int)threadIdx.x < pk.n) dst[pk.first + threadIdx.x] = pk.d[threadIdx.x];
 }
 
-__global__ void k_ws_bbox_init_b(int4* bbox, int total) {
+__global__ void k_ws_bbox_init(int4* bbox, int total) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < total) bbox[i] = make_int4(0x7fffffff, 0x7fffffff, -1, -1);
 }
 
-__global__ void __launch_bounds__(256) k_ws_bbox_b(const WsDesc* __restrict__ D, int n, int total_segs,
+__global__ void __launch_bounds__(256) k_ws_bbox(const WsDesc* __restrict__ D, int n, int total_segs,
                                                    int4* bbox) {
     const int lane = threadIdx.x & 31;
     const int gw = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -754,50 +817,12 @@ __global__ void __launch_bounds__(256) k_ws_bbox_b(const WsDesc* __restrict__ D,
     bbox_segment(T.labels + (size_t)y * T.W, T.W, T.K, y, xs, bbox + T.obj_base, lane);
 }
 
-__global__ void __launch_bounds__(WS_WARPS * 32) k_ws_objects_b(const WsDesc* __restrict__ D, int n, int total,
-                                                                 int h, const int4* __restrict__ bbox, int* cnt,
-                                                                 int* next, int* status) {
-    extern __shared__ __align__(16) char ws_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    char* stage = ws_smem + (size_t)warp * WS_STAGE * WS_PX_BYTES;
-    for (int item = ws_next(next + 2, lane); item < total; item = ws_next(next + 2, lane)) {
-        const int4 bx = bbox[item];
-        if (bx.z < bx.x || ws_box_px(bx) > WS_STAGE) continue;
-        const WsDesc& T = D[ws_desc_of(D, n, item, false)];
-        const int c = ws_staged(T.labels, T.edt, T.W, T.H, item - T.obj_base + 1, bx, h, stage, WS_STAGE, T.out,
-                                status, lane);
-        if (lane == 0) cnt[item] = c;
-        __syncwarp();
-    }
-}
-
-__global__ void __launch_bounds__(32) k_ws_large_b(const WsDesc* __restrict__ D, int n, int h,
-                                                   const int4* __restrict__ bbox, int* cnt, int cap, uint16_t* gdr,
-                                                   unsigned long long* gw, int* next, const int* __restrict__ list,
-                                                   int* status) {
-    extern __shared__ __align__(16) char ws_smem[];
-    const int lane = threadIdx.x;
-    const int nl = next[1];
-    for (int i = ws_next(next, lane); i < nl; i = ws_next(next, lane)) {
-        const int item = list[i];
-        const int4 bx = bbox[item];
-        const WsDesc& T = D[ws_desc_of(D, n, item, false)];
-        const int k = item - T.obj_base + 1;
-        const int c = ws_box_px(bx) <= cap
-                          ? ws_staged(T.labels, T.edt, T.W, T.H, k, bx, h, ws_smem, cap, T.out, status, lane)
-                          : ws_object_global(T.labels, T.edt, T.W, k, bx, h, gdr + T.px_base, gw + T.px_base,
-                                             T.out, status, lane);
-        if (lane == 0) cnt[item] = c;
-        __syncwarp();
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_ws_scan_b(const WsDesc* __restrict__ D, int* cnt) {
+__global__ void __launch_bounds__(1024) k_ws_scan(const WsDesc* __restrict__ D, int* cnt) {
     const WsDesc& T = D[blockIdx.x];
     ws_scan_block(cnt + T.obj_base, T.K, T.n_basins);
 }
 
-__global__ void __launch_bounds__(256) k_ws_offset_b(const WsDesc* __restrict__ D, int n, int total,
+__global__ void __launch_bounds__(256) k_ws_offset(const WsDesc* __restrict__ D, int n, int total,
                                                      const int4* __restrict__ bbox, const int* __restrict__ off) {
     const int lane = threadIdx.x & 31;
     const int nw = gridDim.x * (blockDim.x >> 5);
@@ -810,70 +835,16 @@ __global__ void __launch_bounds__(256) k_ws_offset_b(const WsDesc* __restrict__ 
     }
 }
 
-size_t watershed_scratch_bytes(int W, int H) {
-    return (size_t)W * H * (sizeof(unsigned long long) + sizeof(uint16_t));
-}
-
-void launch_watershed(const int32_t* labels, const int32_t* edt, int W, int H, int K, int h, int32_t* out,
-                      int32_t* n_basins, int4* bbox, int* cnt, int* next, void* scratch, int* status, int sms,
-                      cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Profiler* pf) {
-    static bool attrs[64] = {};  // opt-in shared memory above 48 KB, once per device
-    const int small_smem = WS_WARPS * WS_STAGE * WS_PX_BYTES;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attrs[dev]) {
-        cudaFuncSetAttribute(k_ws_objects, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem);
-        cudaFuncSetAttribute(k_ws_large, cudaFuncAttributeMaxDynamicSharedMemorySize, WS_LARGE_SMEM);
-        if (dev >= 0 && dev < 64) attrs[dev] = true;
-    }
-    const size_t N = (size_t)W * H;
-    cudaMemsetAsync(out, 0, N * sizeof(int32_t), s);
-    if (K <= 0) {
-        cudaMemsetAsync(n_basins, 0, sizeof(int32_t), s);
-        return;
-    }
-    launch_object_boxes(labels, W, H, K, bbox, s, pf);
-    unsigned long long* gw = (unsigned long long*)scratch;
-    uint16_t* gdr = (uint16_t*)(gw + N);
-    int* list = next + 3;
-    cudaMemsetAsync(next, 0, 3 * sizeof(int), s);
-    pf->begin("ws_classify", s);
-    k_ws_classify<<<(K + 255) / 256, 256, 0, s>>>(bbox, K, cnt, next, list);
-    pf->end("ws_classify", s);
-    // the large boxes on the (higher-priority) side stream, overlapping the small ones
-    cudaEventRecord(fork, s);
-    cudaStreamWaitEvent(side, fork, 0);
-    pf->begin("ws_large", side);
-    k_ws_large<<<K < sms ? K : sms, 32, WS_LARGE_SMEM, side>>>(labels, edt, W, H, h, bbox, out, cnt,
-                                                           WS_LARGE_SMEM / WS_PX_BYTES, gdr, gw, next, list,
-                                                           status);
-    pf->end("ws_large", side);
-    cudaEventRecord(join, side);
-    const int ctas = (K + WS_WARPS - 1) / WS_WARPS;
-    pf->begin("ws_objects", s);
-    k_ws_objects<<<ctas < sms * 4 ? ctas : sms * 4, WS_WARPS * 32, small_smem, s>>>(labels, edt, W, H, K, h, bbox,
-                                                                                 out, cnt, next, status);
-    pf->end("ws_objects", s);
-    cudaStreamWaitEvent(s, join, 0);
-    pf->begin("ws_scan", s);
-    k_ws_scan<<<1, 1024, 0, s>>>(cnt, K, n_basins);
-    pf->end("ws_scan", s);
-    const int octas = (K + 7) / 8;
-    pf->begin("ws_offset", s);
-    k_ws_offset<<<octas < sms * 8 ? octas : sms * 8, 256, 0, s>>>(labels, W, K, bbox, cnt, out);
-    pf->end("ws_offset", s);
-}
-
 void launch_watershed_batch(const std::vector<WsDesc>& descs, WsDesc* d_descs, int h, int4* bbox, int* cnt,
                             int* next, void* scratch, size_t scratch_px, int* status, int sms, cudaStream_t s,
                             cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Profiler* pf) {
     static bool attrs[64] = {};  // opt-in shared memory above 48 KB, once per device
-    const int small_smem = WS_WARPS * WS_STAGE * WS_PX_BYTES;
+    const int small_smem = WS_WARPS * WS_STAGE * WS_PX_BYTES, mid_smem = WS_MIDDLE * WS_PX_BYTES;
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attrs[dev]) {
-        cudaFuncSetAttribute(k_ws_objects_b, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem);
-        cudaFuncSetAttribute(k_ws_large_b, cudaFuncAttributeMaxDynamicSharedMemorySize, WS_LARGE_SMEM);
+        cudaFuncSetAttribute(k_ws_objects, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem);
+        cudaFuncSetAttribute(k_ws_team, cudaFuncAttributeMaxDynamicSharedMemorySize, WS_LARGE_SMEM);
         if (dev >= 0 && dev < 64) attrs[dev] = true;
     }
     const int n = (int)descs.size();
@@ -894,37 +865,41 @@ void launch_watershed_batch(const std::vector<WsDesc>& descs, WsDesc* d_descs, i
         unsigned long long* gw = (unsigned long long*)scratch;
         uint16_t* gdr = (uint16_t*)(gw + scratch_px);
         pf->begin("ws_bbox_init", s);
-        k_ws_bbox_init_b<<<(total + 255) / 256, 256, 0, s>>>(bbox, total);
+        k_ws_bbox_init<<<(total + 255) / 256, 256, 0, s>>>(bbox, total);
         pf->end("ws_bbox_init", s);
         pf->begin("ws_bbox", s);
-        k_ws_bbox_b<<<(unsigned)(((long long)segs * 32 + 255) / 256), 256, 0, s>>>(d_descs, n, segs, bbox);
+        k_ws_bbox<<<(unsigned)(((long long)segs * 32 + 255) / 256), 256, 0, s>>>(d_descs, n, segs, bbox);
         pf->end("ws_bbox", s);
-        int* list = next + 3;
-        cudaMemsetAsync(next, 0, 3 * sizeof(int), s);
+        int* list = next + WS_COUNTERS;
+        cudaMemsetAsync(next, 0, WS_COUNTERS * sizeof(int), s);
         pf->begin("ws_classify", s);
         k_ws_classify<<<(total + 255) / 256, 256, 0, s>>>(bbox, total, cnt, next, list);
         pf->end("ws_classify", s);
+        // the larger boxes on the (higher-priority) side stream, overlapping the small ones
         cudaEventRecord(fork, s);
         cudaStreamWaitEvent(side, fork, 0);
         pf->begin("ws_large", side);
-        k_ws_large_b<<<total < sms ? total : sms, 32, WS_LARGE_SMEM, side>>>(
-            d_descs, n, h, bbox, cnt, WS_LARGE_SMEM / WS_PX_BYTES, gdr, gw, next, list, status);
+        k_ws_team<<<std::min(total, sms * 2), WS_WARPS * 32, WS_LARGE_SMEM, side>>>(
+            d_descs, n, h, bbox, cnt, WS_LARGE_SMEM / WS_PX_BYTES, gdr, gw, next, next + 1, list, 1, status);
         pf->end("ws_large", side);
+        pf->begin("ws_middle", side);
+        k_ws_team<<<std::min(total, sms * 8), WS_WARPS * 32, mid_smem, side>>>(
+            d_descs, n, h, bbox, cnt, WS_MIDDLE, gdr, gw, next + 3, next + 4, list + total - 1, -1, status);
+        pf->end("ws_middle", side);
         cudaEventRecord(join, side);
         const int ctas = (total + WS_WARPS - 1) / WS_WARPS;
         pf->begin("ws_objects", s);
-        k_ws_objects_b<<<ctas < sms * 4 ? ctas : sms * 4, WS_WARPS * 32, small_smem, s>>>(d_descs, n, total, h, bbox,
-                                                                                        cnt, next, status);
+        k_ws_objects<<<std::min(ctas, sms * 10), WS_WARPS * 32, small_smem, s>>>(d_descs, n, total, h, bbox, cnt, next, status);
         pf->end("ws_objects", s);
         cudaStreamWaitEvent(s, join, 0);
     }
     pf->begin("ws_scan", s);
-    k_ws_scan_b<<<n, 1024, 0, s>>>(d_descs, cnt);
+    k_ws_scan<<<n, 1024, 0, s>>>(d_descs, cnt);
     pf->end("ws_scan", s);
     if (total > 0) {
         const int octas = (total + 7) / 8;
         pf->begin("ws_offset", s);
-        k_ws_offset_b<<<octas < sms * 8 ? octas : sms * 8, 256, 0, s>>>(d_descs, n, total, bbox, cnt);
+        k_ws_offset<<<octas < sms * 8 ? octas : sms * 8, 256, 0, s>>>(d_descs, n, total, bbox, cnt);
         pf->end("ws_offset", s);
     }
 }

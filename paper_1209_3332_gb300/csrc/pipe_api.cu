@@ -846,42 +846,8 @@ int morph_open_tile(pipe_t p, const uint8_t* src_dev, int W, int H, int radius, 
 
 int watershed_tile(pipe_t p, const int32_t* labels_dev, const int32_t* edt_dev, int W, int H, int n_objects,
                    int h, int32_t* out_dev, int32_t* n_basins_dev, pipe_stream_t stream) {
-    if (!p || !labels_dev || !edt_dev || !out_dev || !n_basins_dev || n_objects < 0 || h < 0 || h > 255)
-        return PIPE_EINVAL;
-    if (!valid_size(W, H)) return PIPE_EINVAL;
-    const size_t N = (size_t)W * H;
-    auto overlap = [N](const void* a, const void* b) {
-        const char *x = (const char*)a, *y = (const char*)b;
-        return x < y + N * 4 && y < x + N * 4;
-    };
-    if (overlap(out_dev, labels_dev) || overlap(out_dev, edt_dev)) return PIPE_EINVAL;
-    cudaStream_t s = (cudaStream_t)stream;
-    CK(cudaSetDevice(p->device));
-    const size_t need_obj = (size_t)std::max(n_objects, 1) * (sizeof(int4) + 2 * sizeof(int)) + 3 * sizeof(int);
-    const size_t need_scr = watershed_scratch_bytes(W, H);
-    if (p->ws_obj.n < need_obj || p->ws_scratch.n < need_scr || !p->ws_status.p) {
-        CK(cudaStreamSynchronize(s));
-        int rc;
-        if ((rc = p->ws_obj.ensure(need_obj)) || (rc = p->ws_scratch.ensure(need_scr))) return rc;
-        if (!p->ws_status.p) {
-            if ((rc = p->ws_status.ensure(sizeof(int)))) return rc;
-            CK(cudaMemset(p->ws_status.p, 0, sizeof(int)));
-        }
-    }
-    if (!p->ws_side) {
-        int lo_pri = 0, hi_pri = 0;  // the large boxes go first when SM room frees up
-        CK(cudaDeviceGetStreamPriorityRange(&lo_pri, &hi_pri));
-        CK(cudaStreamCreateWithPriority(&p->ws_side, cudaStreamNonBlocking, hi_pri));
-        CK(cudaEventCreateWithFlags(&p->ws_fork, cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&p->ws_join, cudaEventDisableTiming));
-    }
-    int4* bbox = (int4*)p->ws_obj.p;
-    int* cnt = (int*)(bbox + std::max(n_objects, 1));
-    int* next = cnt + std::max(n_objects, 1);
-    launch_watershed(labels_dev, edt_dev, W, H, n_objects, h, out_dev, n_basins_dev, bbox, cnt, next, p->ws_scratch.p,
-                     (int*)p->ws_status.p, p->sms, s, p->ws_side, p->ws_fork, p->ws_join, &p->prof);
-    CK(cudaGetLastError());
-    return PIPE_OK;
+    const ws_tile t{labels_dev, edt_dev, W, H, n_objects, out_dev, n_basins_dev};
+    return watershed_batch(p, &t, 1, h, stream);
 }
 
 int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t stream) {
@@ -908,7 +874,7 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
         objs += (size_t)t.n_objects;
         px += N;
     }
-    if (objs > (size_t)INT32_MAX / 32) return PIPE_EINVAL;
+    if (n > 1 && objs > (size_t)INT32_MAX / 32) return PIPE_EINVAL;
     long long segs = 0;
     for (auto& x : d) {
         x.seg_base = (int)segs;
@@ -917,7 +883,7 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
     if (segs * 32 > INT32_MAX) return PIPE_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(p->device));
-    const size_t need_obj = std::max(objs, (size_t)1) * (sizeof(int4) + 2 * sizeof(int)) + 3 * sizeof(int);
+    const size_t need_obj = std::max(objs, (size_t)1) * (sizeof(int4) + 2 * sizeof(int)) + WS_COUNTERS * sizeof(int);
     const size_t need_scr = px * (sizeof(unsigned long long) + sizeof(uint16_t));
     const size_t need_desc = sizeof(WsDesc) * (size_t)n;
     if (p->ws_obj.n < need_obj || p->ws_scratch.n < need_scr || p->ws_desc.n < need_desc || !p->ws_status.p) {
