@@ -196,7 +196,7 @@ int morph_open_tile(pipe_t p, const uint8_t* src_dev, int W, int H, int radius, 
  *    pixel); n_objects = K of seg_tile; 0 <= h <= 255 (the marker height).
  *  out_dev: W x H int32, caller-owned, must not overlap labels or edt;
  *  n_basins_dev: one int32 receiving the number of basins.
- *  Objects whose bounding box with a 1-pixel margin exceeds 1024 pixels run
+ *  Objects whose bounding box with a 1-pixel margin exceeds 384 pixels run
  *  on a pipe-owned side stream (forked from and joined back to `stream`, so
  *  the call stays in `stream` order); boxes beyond 7021 pixels are processed
  *  from image-sized scratch planes the pipe owns (10 bytes per pixel,

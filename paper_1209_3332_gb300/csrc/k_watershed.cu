@@ -17,30 +17,32 @@
 //
 // Objects are independent: two labels are never 8-adjacent (they would be
 // one component), and d = 0 off the object keeps R, the plateaus and the
-// flooding inside it.  So one warp owns one object: its bounding box plus a
-// 1-px margin is staged in shared memory (d, R and later flags in one 16-bit
-// word per pixel, edt, and one 32-bit work word), and every step runs there
-// with __syncwarp between passes:
+// flooding inside it.  So a team of threads owns one object: its bounding box
+// plus a 1-px margin is staged in shared memory (d, R and later flags in one
+// 16-bit word per pixel, edt, and one 32-bit work word), and every step runs
+// there with a barrier between passes:
 //   1. relaxation passes, alternately in raster and anti-raster order, update
 //      R in place until a pass changes nothing (monotone updates from below,
 //      so the fixed point reached is the reconstruction);
-//   2. plateaus by union-find over the work words (roots are the smallest
-//      index, i.e. the first pixel), a flag on the root of every plateau with
-//      a higher neighbour;
+//   2. markers: what a few passes cannot rule out is joined by union-find over
+//      the work words (roots are the smallest index, i.e. the first pixel);
 //   3. flooding: the work word holds (wave stamp, name); a pass names the
 //      pixels of F at level L with stamp = wave, and only neighbours with an
-//      older stamp count, so a pass is exactly one synchronous wave; a pass
-//      that names nothing yields the next L from the same reads.  F itself
+//      older stamp count, so a pass is exactly one synchronous wave.  F itself
 //      is kept as a list (double-buffered, pixels entered once through an
 //      atomic flag), so a wave costs the frontier, not the box;
 //   4. each basin's first pixel by atomicMin on its root's word, a ballot
 //      prefix over the box in raster order for the ranks.
-// Boxes up to WS_STAGE pixels (with margin) go to four-warp CTAs; larger
-// ones to one-warp CTAs with a large dynamic stage, launched on a side
-// stream so that the few large objects overlap the many small ones; boxes
-// beyond that stage run the same steps (with a full-box scan per wave) on
-// image-sized scratch planes in global memory.  A scan of the per-object
-// basin counts and a pass adding each object's offset finish the numbering.
+// Boxes up to WS_STAGE pixels (with margin) are split by one warp; larger ones
+// by the four warps of a CTA, with a stage of WS_MIDDLE pixels or a larger one,
+// launched on a side stream so that the few large objects overlap the many
+// small ones; boxes beyond that stage run the same steps (with a full-box scan
+// per wave) on image-sized scratch planes in global memory.  A scan of the
+// per-object basin counts and a pass adding each object's offset finish the
+// numbering.
+// Bound: the latency of an object's chain of passes over shared memory; the
+// zeros of the split plane, the boxes and the offsets (about 250 us of the 596
+// for 8 tiles of 4096^2) move the labels and the plane once each.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -49,7 +51,12 @@ namespace nucseg {
 
 constexpr int WS_WARPS = 4;      // warps per CTA: one object each (small boxes) or one together
 constexpr int WS_STAGE = 384;    // staged box (with margin) capacity per warp of the small-box kernel, pixels
-constexpr int WS_MIDDLE = 1024;  // staged box capacity of a CTA with the small stage
+// Staged box capacity of a CTA with the small stage.  The large stage leaves room
+// for two CTAs per SM and waits for that room behind the small boxes, so it is
+// kept for the rare boxes beyond this (8 tiles of 4096^2, and 4 with chains of
+// nuclei: 691 and 917 us at 1024, 592 and 943 at 1536, 609 and 946 at 2048, 596
+// and 812 at 3072).
+constexpr int WS_MIDDLE = 3072;
 constexpr int WS_PX_BYTES = 14;  // stage bytes per pixel: e 4, w 4, dr 2, two frontier lists 2 + 2
 constexpr int WS_LARGE_SMEM = 96 * 1024;  // dynamic stage of a CTA with the large stage
 constexpr int WS_OUT_PASSES = 8;  // passes that spread "on no marker" before the union-find
@@ -192,6 +199,18 @@ __device__ __forceinline__ int ws_find(const B& b, int x) {
         const int gp = (int)(b.w[p] & IDX);
         if (gp != p) b.w[x] = (typename B::Wt)gp;
         x = gp;
+    }
+}
+
+// The root of x without shortening links: while other warps replace links by
+// roots, a shortcut written late could put an older ancestor over a root.
+template <class B>
+__device__ __forceinline__ int ws_root(const B& b, int x) {
+    constexpr typename B::Wt IDX = ((typename B::Wt)1 << B::SH) - 1;
+    for (;;) {
+        const int p = (int)(b.w[x] & IDX);
+        if (p == x) return x;
+        x = p;
     }
 }
 
@@ -341,7 +360,7 @@ __device__ int ws_object(const B& b, const Team<NW>& team, int32_t* out, int* st
     team.sync();
     for (Walk it(t, b.ww); it.f < b.n; it.next()) {
         const int s = b.stor(it);
-        if (b.in(s) && b.w[s] != OUT) b.w[s] = (Wt)ws_find(b, s);
+        if (b.in(s) && b.w[s] != OUT) b.w[s] = (Wt)ws_root(b, s);
     }
     team.sync();
     if (!settled) {

@@ -210,3 +210,24 @@ def test_argument_checks(pipe):
         pipe.watershed(L, E, 0, L, n)            # out overlaps labels
     with pytest.raises(P.PipeError):
         pipe.watershed(L, E, -1, out, n)
+
+
+@pytest.mark.parametrize("bw,bh", [(14, 22), (13, 24), (46, 62), (39, 73), (63, 106), (62, 108)])
+@pytest.mark.parametrize("h", [0, 1])
+def test_boxes_at_the_stage_sizes(pipe, bw, bh, h):
+    """Objects whose box with its margin just fits, or just misses, the stages
+    of 384, 3072 and 7021 pixels: combs (plateaus as long as a tooth) with
+    bites, beside small discs."""
+    rng = np.random.default_rng(bw * 1000 + bh)
+    lab = np.zeros((bh + 8, 3 * bw + 40), np.int32)
+    for k in range(2):
+        x0 = 3 + k * (bw + 4)
+        obj = np.zeros((bh, bw), bool)
+        obj[:, :4] = True
+        for y in range(0, bh, 7):
+            obj[y:y + 5, :int(rng.integers(bw // 2, bw + 1))] = True
+        obj[0, :] = obj[bh - 1, :4] = True
+        lab[4:4 + bh, x0:x0 + bw][obj] = k + 1
+    yy, xx = np.mgrid[0:lab.shape[0], 0:lab.shape[1]]
+    lab[(np.hypot(xx - (2 * bw + 25), yy - 12) <= 7)] = 3
+    check(pipe, lab, h=h, K=3)
