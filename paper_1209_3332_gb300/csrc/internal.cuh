@@ -207,9 +207,10 @@ void launch_recon(const Launch& L, int grid_cap, cudaStream_t s, Profiler* pf);
 void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cudaStream_t s, Profiler* pf);
 size_t edt_rows_smem(int RB, int Wmax);
 void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf);
-size_t morph_open_smem(int r);
-// tmp: a W x H scratch plane (the radius-9 form runs two passes through it); may be null
-void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, int H, int r, cudaStream_t s,
+// The opening (1 <= r <= MORPH_RMAX in two passes through tmp, morph_scratch bytes).
+inline int morph_pitch(int W) { return (W + 15) & ~15; }  // rows of its scratch planes
+size_t morph_scratch(const uint8_t* src, int W, int H);
+void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, int H, int r, int sms, cudaStream_t s,
                        Profiler* pf);
 void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, int H, int K, float* feats,
                            int4* bbox, int sms, cudaStream_t s, Profiler* pf);

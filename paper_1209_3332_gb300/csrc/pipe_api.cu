@@ -834,12 +834,13 @@ int morph_open_tile(pipe_t p, const uint8_t* src_dev, int W, int H, int radius, 
     if (src_dev < dst_dev + N && dst_dev < src_dev + N) return PIPE_EINVAL;  // the planes overlap
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(p->device));
-    if (p->morph_tmp.n < N) {  // the scratch plane of the two-pass form grows to the largest plane seen
+    const size_t need = morph_scratch(src_dev, W, H);
+    if (p->morph_tmp.n < need) {  // the scratch planes grow to the largest call seen
         CK(cudaStreamSynchronize(s));
-        const int rc = p->morph_tmp.ensure(N);
+        const int rc = p->morph_tmp.ensure(need);
         if (rc) return rc;
     }
-    launch_morph_open(src_dev, dst_dev, (uint8_t*)p->morph_tmp.p, W, H, radius, s, &p->prof);
+    launch_morph_open(src_dev, dst_dev, (uint8_t*)p->morph_tmp.p, W, H, radius, p->sms, s, &p->prof);
     CK(cudaGetLastError());
     return PIPE_OK;
 }

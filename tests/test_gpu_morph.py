@@ -77,3 +77,21 @@ def test_argument_checks(pipe):
     assert L.morph_open_tile(pipe.h, a.data_ptr(), 48, 32, 9, a.data_ptr() + 100, None) == P.PIPE_EINVAL
     assert L.morph_open_tile(pipe.h, a.data_ptr(), 0, 32, 9, b.data_ptr(), None) == P.PIPE_EINVAL
     assert L.morph_open_tile(pipe.h, a.data_ptr(), 48, 32, 9, b.data_ptr(), None) == P.PIPE_OK
+
+
+@pytest.mark.parametrize("r", range(1, 16))
+@pytest.mark.parametrize("W,H,off", [(256, 129, 0), (133, 70, 0), (130, 33, 1), (127, 64, 3)])
+def test_every_radius(pipe, W, H, off, r):
+    """Every radius has a pass of its own: strips of 128 columns and segments
+    of 32 rows just full, just over and just short; rows and planes that start
+    on no 4-byte boundary."""
+    import torch
+    rng = np.random.default_rng(r * 100 + W)
+    a = rng.integers(0, 256, (H, W), dtype=np.uint8)
+    buf = torch.full((2, off + H * W + 64), 7, dtype=torch.uint8, device="cuda")
+    src, dst = (buf[i, off:off + H * W].view(H, W) for i in range(2))
+    src.copy_(torch.from_numpy(a))
+    pipe.morph_open(src, dst, radius=r)
+    torch.cuda.synchronize()
+    assert np.array_equal(dst.cpu().numpy(), oracle.morph_open(a, r))
+    assert bool((buf[1, :off] == 7).all()) and bool((buf[1, off + H * W:] == 7).all())
