@@ -202,8 +202,10 @@ struct Profiler {
 
 void upload_deconv_tables(const int32_t* lut256, const int32_t* wq3);
 void launch_deconv(const Launch& L, cudaStream_t s, Profiler* pf);
-int recon_grid(int device);
-void launch_recon(const Launch& L, int grid_cap, cudaStream_t s, Profiler* pf);
+void recon_grid(int device, int* warps, int* teams);
+// warps: resident one-warp workers to use, of warps_cap; launches with few work
+// tiles per worker use teams of four warps instead, the same share of teams_cap
+void launch_recon(const Launch& L, int warps, int warps_cap, int teams_cap, cudaStream_t s, Profiler* pf);
 void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cudaStream_t s, Profiler* pf);
 size_t edt_rows_smem(int RB, int Wmax);
 void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf);

@@ -3,9 +3,10 @@
 // queue-based wave propagation, Sec. V-A).  R = lim R_k with
 // R_{k+1} = min(dilate8(R_k), hem8), R_0 = max(hem8 - h, 0) (written by K1).
 //
-// Design (GB300): a persistent kernel whose warps are independent workers.
+// Design (GB300): a persistent kernel of independent workers, each a warp, or
+// in launches of few tiles a team of four (see k_recon).
 // The image is cut into 64x64 work tiles; a device-wide queue holds the
-// tiles that may still change.  A warp pops a tile, stages R and hem8 (M) of
+// tiles that may still change.  A worker pops a tile, stages R and hem8 (M) of
 // the tile and a one-pixel halo in its own shared memory, and runs rounds of
 // four directional sweeps over the whole tile (down, up, right, left), each
 // an exact sequential sweep along one axis:
@@ -20,7 +21,7 @@
 //  * a sweep reads each block once per two lines and never reads what
 //    another lane stored during it.
 // After each round an exact, chain-free test decides whether another is
-// needed.  The warp then writes the tile back and queues each neighbouring
+// needed.  The worker then writes the tile back and queues each neighbouring
 // tile that one of the changed border pixels can still raise.  Values only
 // grow and are bounded by hem8, so any order of tile processings reaches the
 // same unique fixed point; a per-tile state machine (idle / queued / running
@@ -28,6 +29,8 @@
 // once and never misses a raise of its halo.  Every spin wait is bounded by
 // the pipe's cycle budget, after which the worker records ST_TIMEOUT and
 // returns.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace nucseg {
@@ -36,6 +39,12 @@ constexpr int NB = RT / 2;        // blocks per tile side
 constexpr int BS = NB + 1;        // block row stride: 33 8-byte blocks (odd: column sweeps are conflict-free)
 constexpr int HL = RT + 2;        // halo line length: index = coordinate + 1, coordinates -1..RT
 constexpr int MAX_ROUNDS = 256;   // sweep rounds before a tile re-queues itself
+constexpr int TEAM_MIN_BLOCKS = 8;  // resident teams per SM the register budget must allow
+// Work tiles per resident warp below which teams take them: 16 tiles, 67 us by
+// warps and 42 us by teams; 1024, 154 and 130; 3072, 221 and 203; 4096, 282 and
+// 260; 5120, 255 and 272; 8192, 389 and 411; 16384, 507 and 672; 65536, 1822 and
+// 2569 (2432 resident warps)
+constexpr int TEAM_TILES = 2;
 constexpr unsigned FULL = 0xffffffffu;
 
 // A worker's staged tile.  Block (j, i) covers pixels (2j + a, 2i + b),
@@ -54,6 +63,35 @@ struct WarpTile {
     uint8_t HMc[2][HL + 2];  // M of the halo columns
     uint8_t B0[4][RT];
     int flags[9];            // neighbours to queue: up, down, left, right, UL, UR, DL, DR, self
+    int msg[2];              // from a team's first thread to the others
+};
+
+// The worker of a tile: one warp, or the NW warps of a CTA (the arguments are
+// at k_recon).
+template <int NW>
+struct Worker {
+    static constexpr int T = 32 * NW;
+    int t, lane, warp;
+    __device__ __forceinline__ Worker() : t(threadIdx.x), lane(NW == 1 ? t : t & 31), warp(NW == 1 ? 0 : t >> 5) {}
+    __device__ __forceinline__ void sync() const {
+        if constexpr (NW == 1) __syncwarp(); else __syncthreads();
+    }
+    // whether p holds for some thread; with NW > 1 also a barrier
+    __device__ __forceinline__ bool any(bool p) const {
+        if constexpr (NW == 1) return __any_sync(FULL, p); else return __syncthreads_or(p);
+    }
+    // thread 0's value
+    __device__ __forceinline__ int from_first(WarpTile& S, int v) const {
+        if constexpr (NW == 1) {
+            return __shfl_sync(FULL, v, 0);
+        } else {
+            if (t == 0) S.msg[0] = v;
+            __syncthreads();
+            v = *(volatile int*)&S.msg[0];
+            __syncthreads();
+            return v;
+        }
+    }
 };
 
 // R of halo pixel (hy, hx), and setting its R and M
@@ -253,17 +291,30 @@ __global__ void k_wl_init(Launch L) {
 
 
 // ---- staging ----------------------------------------------------------------------
-// Halo pixel q (0..8) of a lane: q 0-1 top row (-1, 2l + q), q 2-3 bottom row
-// (RT, 2l + q - 2), q 4-5 left column (2l + q - 4, -1), q 6-7 right column
-// (2l + q - 6, RT), q 8 the corners, one each on lanes 0-3.
-__device__ __forceinline__ void halo_coord(int q, int lane, int& hy, int& hx) {
-    if (q < 2) { hy = -1; hx = 2 * lane + q; }
-    else if (q < 4) { hy = RT; hx = 2 * lane + q - 2; }
-    else if (q < 6) { hy = 2 * lane + q - 4; hx = -1; }
-    else if (q < 8) { hy = 2 * lane + q - 6; hx = RT; }
-    else { hy = (lane & 2) ? RT : -1; hx = (lane & 1) ? RT : -1; }
+// Halo pixels of a thread.  One warp: q (0..8) 0-1 top row (-1, 2l + q), 2-3
+// bottom row (RT, 2l + q - 2), 4-5 left column (2l + q - 4, -1), 6-7 right column
+// (2l + q - 6, RT), 8 the corners, one each on lanes 0-3.  Four warps: q 0 the
+// rows, 1 the columns, 2 the corners.
+template <int NW>
+__host__ __device__ constexpr int halo_count() { return NW == 1 ? 9 : 3; }
+template <int NW>
+__device__ __forceinline__ void halo_coord(int q, int t, int& hy, int& hx) {
+    if constexpr (NW == 1) {
+        if (q < 2) { hy = -1; hx = 2 * t + q; }
+        else if (q < 4) { hy = RT; hx = 2 * t + q - 2; }
+        else if (q < 6) { hy = 2 * t + q - 4; hx = -1; }
+        else if (q < 8) { hy = 2 * t + q - 6; hx = RT; }
+        else { hy = (t & 2) ? RT : -1; hx = (t & 1) ? RT : -1; }
+    } else {
+        static_assert(NW == 4, "two lines of 64 pixels per turn");
+        const int far = t >> 6, i = t & 63;
+        if (q == 0) { hy = far ? RT : -1; hx = i; }
+        else if (q == 1) { hy = i; hx = far ? RT : -1; }
+        else { hy = (t & 2) ? RT : -1; hx = (t & 1) ? RT : -1; }
+    }
 }
-__device__ __forceinline__ bool halo_lane(int q, int lane) { return q < 8 || lane < 4; }
+template <int NW>
+__device__ __forceinline__ bool halo_lane(int q, int t) { return q < halo_count<NW>() - 1 || t < 4; }
 
 // the image of a visit, in registers (a descriptor in memory would be read
 // again after every fence)
@@ -273,31 +324,33 @@ struct Img {
     int W, H, rp;
 };
 
-// R (and M) of this lane's halo pixels, 0 outside the image
-__device__ __forceinline__ void load_halo(uint8_t hr[9], uint8_t* hm, const Img& T, int x0, int y0, int lane) {
+// R (and M) of this thread's halo pixels, 0 outside the image
+template <int NW>
+__device__ __forceinline__ void load_halo(uint8_t* hr, uint8_t* hm, const Img& T, int x0, int y0, int t) {
 #pragma unroll
-    for (int q = 0; q < 9; q++) {
+    for (int q = 0; q < halo_count<NW>(); q++) {
         int hy, hx;
-        halo_coord(q, lane, hy, hx);
+        halo_coord<NW>(q, t, hy, hx);
         const int gy = y0 + hy, gx = x0 + hx;
-        const bool in = gy >= 0 && gy < T.H && gx >= 0 && gx < T.W && halo_lane(q, lane);
+        const bool in = gy >= 0 && gy < T.H && gx >= 0 && gx < T.W && halo_lane<NW>(q, t);
         hr[q] = in ? __ldcg(T.R + (size_t)gy * T.rp + gx) : (uint8_t)0;
         if (hm) hm[q] = in ? __ldg(T.hem8 + (size_t)gy * T.W + gx) : (uint8_t)0;
     }
 }
 
-// Stages the tile.  Lane: block row jj of a group of 8, 16-pixel segment seg;
+// Stages the tile.  Thread: block row jj of a group of 8 NW, 16-pixel segment seg;
 // rows 2j and 2j + 1 of R and M, eight blocks built from them.  R's rows are
 // 16-byte aligned; hem8's are where W is a multiple of 16 (odd widths read the
 // aligned words around them: with byte loads for both planes a 1025 x 2049
 // image took 381 us).
-__device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int y0, int lane) {
-    uint8_t hr[9], hm[9];
-    load_halo(hr, hm, T, x0, y0, lane);
+template <int NW>
+__device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int y0, int t) {
+    uint8_t hr[halo_count<NW>()], hm[halo_count<NW>()];
+    load_halo<NW>(hr, hm, T, x0, y0, t);
     const uint8_t* const Rg = T.R;
     const uint8_t* const Mg = T.hem8;
     const int W = T.W, H = T.H;
-    const int jj = lane >> 2, seg = lane & 3, x = x0 + seg * 16;
+    const int jj = t >> 2, seg = t & 3, x = x0 + seg * 16;
     const uint4 z = make_uint4(0, 0, 0, 0);
     auto put = [&](int j, uint4 rt, uint4 rb, uint4 mt, uint4 mb) {
         const uint32_t rtw[4] = {rt.x, rt.y, rt.z, rt.w}, rbw[4] = {rb.x, rb.y, rb.z, rb.w};
@@ -311,8 +364,8 @@ __device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int
     };
     if ((W & 15) == 0 && x0 + RT <= W && (reinterpret_cast<uintptr_t>(Mg) & 15) == 0) {
 #pragma unroll 2
-        for (int g = 0; g < NB / 8; g++) {
-            const int j = g * 8 + jj, gy = y0 + 2 * j;
+        for (int g = 0; g < NB / (8 * NW); g++) {
+            const int j = g * 8 * NW + jj, gy = y0 + 2 * j;
             const size_t o = (size_t)gy * W + x;
             const uint4 rt = gy < H ? __ldcg(reinterpret_cast<const uint4*>(Rg + o)) : z;
             const uint4 rb = gy + 1 < H ? __ldcg(reinterpret_cast<const uint4*>(Rg + o + W)) : z;
@@ -322,8 +375,8 @@ __device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int
         }
     } else {
 #pragma unroll 1
-        for (int g = 0; g < NB / 8; g++) {
-            const int j = g * 8 + jj, gy = y0 + 2 * j;
+        for (int g = 0; g < NB / (8 * NW); g++) {
+            const int j = g * 8 * NW + jj, gy = y0 + 2 * j;
             const bool in0 = x < W && gy < H, in1 = x < W && gy + 1 < H;
             const uint8_t* r = Rg + (size_t)gy * T.rp + x;
             uint4 rt = in0 ? __ldcg(reinterpret_cast<const uint4*>(r)) : z;
@@ -337,22 +390,23 @@ __device__ __forceinline__ void load_tile(WarpTile& S, const Img& T, int x0, int
         }
     }
 #pragma unroll
-    for (int q = 0; q < 9; q++) {
-        if (!halo_lane(q, lane)) continue;
+    for (int q = 0; q < halo_count<NW>(); q++) {
+        if (!halo_lane<NW>(q, t)) continue;
         int hy, hx;
-        halo_coord(q, lane, hy, hx);
+        halo_coord<NW>(q, t, hy, hx);
         set_halo_r(S, hy, hx, hr[q]);
         set_halo_m(S, hy, hx, hm[q]);
     }
 }
 
 // Writes the tile's R back (row padding takes zeros).
-__device__ __forceinline__ void store_tile(WarpTile& S, const Img& T, int x0, int y0, int lane) {
-    const int jj = lane >> 2, seg = lane & 3, x = x0 + seg * 16;
+template <int NW>
+__device__ __forceinline__ void store_tile(WarpTile& S, const Img& T, int x0, int y0, int t) {
+    const int jj = t >> 2, seg = t & 3, x = x0 + seg * 16;
     if (x >= T.W) return;
 #pragma unroll 1
-    for (int g = 0; g < NB / 8; g++) {
-        const int j = g * 8 + jj, gy = y0 + 2 * j;
+    for (int g = 0; g < NB / (8 * NW); g++) {
+        const int j = g * 8 * NW + jj, gy = y0 + 2 * j;
         uint32_t top[4], bot[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
@@ -368,13 +422,14 @@ __device__ __forceinline__ void store_tile(WarpTile& S, const Img& T, int x0, in
 }
 
 // Raises the staged halo pixels to the values just read; true if any grew.
-__device__ __forceinline__ bool merge_halo(WarpTile& S, const uint8_t hr[9], int lane) {
+template <int NW>
+__device__ __forceinline__ bool merge_halo(WarpTile& S, const uint8_t* hr, int t) {
     bool grew = false;
 #pragma unroll
-    for (int q = 0; q < 9; q++) {
-        if (!halo_lane(q, lane)) continue;
+    for (int q = 0; q < halo_count<NW>(); q++) {
+        if (!halo_lane<NW>(q, t)) continue;
         int hy, hx;
-        halo_coord(q, lane, hy, hx);
+        halo_coord<NW>(q, t, hy, hx);
         if (hr[q] > halo_r(S, hy, hx)) {
             set_halo_r(S, hy, hx, hr[q]);
             grew = true;
@@ -409,13 +464,21 @@ __device__ __forceinline__ void line_step(uint32_t& A, uint32_t& B, uint32_t RA,
     B = min2(__vimax3_u16x2(__byte_perm(L, P, LEFT_B), __byte_perm(P, Rt, RIGHT_B), max2(B, RB)), MB);
 }
 
-__device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
+// With several warps, each takes a band of block rows, and its chains start from
+// the lines beside the band as they are (whatever the neighbouring warp has made
+// of them meanwhile: any value there is a lower bound).
+template <int NW>
+__device__ __forceinline__ void row_sweeps(WarpTile& S, int lane, int warp) {
+    constexpr int N = NB / NW;
+    const int j0 = warp * N;
     uint32_t Pd = 0u, Pu = 0u;
-    uint2 bd = S.B[lane], bu = S.B[(NB - 1) * BS + lane];
+    if (NW > 1 && warp > 0) Pd = __byte_perm(S.B[(j0 - 1) * BS + lane].x, 0u, ROW1);
+    if (NW > 1 && warp < NW - 1) Pu = __byte_perm(S.B[(j0 + N) * BS + lane].x, 0u, ROW0);
+    uint2 bd = S.B[j0 * BS + lane], bu = S.B[(j0 + N - 1) * BS + lane];
 #pragma unroll 4
-    for (int k = 0; k < NB; k++) {  // down: rows 2jd, 2jd + 1; up: rows 2ju + 1, 2ju
-        const int jd = k, ju = NB - 1 - k;
-        uint2 nd = S.B[min(jd + 1, NB - 1) * BS + lane], nu = S.B[max(ju - 1, 0) * BS + lane];
+    for (int k = 0; k < N; k++) {  // down: rows 2jd, 2jd + 1; up: rows 2ju + 1, 2ju
+        const int jd = j0 + k, ju = j0 + N - 1 - k;
+        uint2 nd = S.B[min(jd + 1, j0 + N - 1) * BS + lane], nu = S.B[max(ju - 1, j0) * BS + lane];
         line_step(Pd, Pu, __byte_perm(bd.x, 0u, ROW0), __byte_perm(bd.y, 0u, ROW0), __byte_perm(bu.x, 0u, ROW1),
                   __byte_perm(bu.y, 0u, ROW1));
         const uint32_t d0 = Pd, u1 = Pu;
@@ -424,7 +487,7 @@ __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
         const uint32_t wd = __byte_perm(d0, Pd, PACK_ROWS), wu = __byte_perm(Pu, u1, PACK_ROWS);
         S.B[jd * BS + lane].x = wd;
         S.B[ju * BS + lane].x = wu;
-        if (k == NB / 2 - 1) { nd.x = wu; nu.x = wd; }
+        if (k == N / 2 - 1) { nd.x = wu; nu.x = wd; }
         bd = nd;
         bu = nu;
     }
@@ -432,21 +495,26 @@ __device__ __forceinline__ void row_sweeps(WarpTile& S, int lane) {
 
 // The column sweep pair: right (columns 0 -> RT-1) and left (RT-1 -> 0) at
 // once, lane l owning block row l (rows 2l, 2l + 1) in both chains.
-__device__ __forceinline__ void col_sweeps(WarpTile& S, int lane) {
+template <int NW>
+__device__ __forceinline__ void col_sweeps(WarpTile& S, int lane, int warp) {
+    constexpr int N = NB / NW;
+    const int i0 = warp * N;
     uint32_t Cr = 0u, Cl = 0u;
     uint2* const B = S.B + lane * BS;
-    uint2 br = B[0], bl = B[NB - 1];
+    if (NW > 1 && warp > 0) Cr = B[i0 - 1].x;
+    if (NW > 1 && warp < NW - 1) Cl = __byte_perm(B[i0 + N].x, 0u, COL0);
+    uint2 br = B[i0], bl = B[i0 + N - 1];
 #pragma unroll 4
-    for (int k = 0; k < NB; k++) {
-        const int ir = k, il = NB - 1 - k;
-        uint2 nr = B[min(ir + 1, NB - 1)], nl = B[max(il - 1, 0)];
+    for (int k = 0; k < N; k++) {
+        const int ir = i0 + k, il = i0 + N - 1 - k;
+        uint2 nr = B[min(ir + 1, i0 + N - 1)], nl = B[max(il - 1, i0)];
         line_step(Cr, Cl, __byte_perm(br.x, 0u, COL0), __byte_perm(br.y, 0u, COL0), bl.x, bl.y);
         const uint32_t r0 = Cr, l1 = Cl;
         line_step(Cr, Cl, br.x, br.y, __byte_perm(bl.x, 0u, COL0), __byte_perm(bl.y, 0u, COL0));
         const uint32_t wr = __byte_perm(r0, Cr, PACK_COLS), wl = __byte_perm(Cl, l1, PACK_COLS);
         B[ir].x = wr;
         B[il].x = wl;
-        if (k == NB / 2 - 1) { nr.x = wl; nl.x = wr; }
+        if (k == N / 2 - 1) { nr.x = wl; nl.x = wr; }
         br = nr;
         bl = nl;
     }
@@ -455,17 +523,23 @@ __device__ __forceinline__ void col_sweeps(WarpTile& S, int lane) {
 // One round: the row sweep pair, then the column sweep pair.  __syncwarp
 // orders each pair's stores before the next pair's loads (the pairs map
 // lanes to blocks differently).
-__device__ __forceinline__ void sweep_round(WarpTile& S, int lane) {
-    row_sweeps(S, lane);
-    __syncwarp();
-    col_sweeps(S, lane);
-    __syncwarp();
+template <int NW>
+__device__ __forceinline__ void sweep_round(WarpTile& S, const Worker<NW>& me) {
+    row_sweeps<NW>(S, me.lane, me.warp);
+    me.sync();
+    col_sweeps<NW>(S, me.lane, me.warp);
+    me.sync();
 }
 
 // Whether some pixel of the tile can still be raised by one of its 8
 // neighbours in the tile: the exact convergence test, two pixels per lane and
 // row, with no dependent chain; it stops at the first 16-row group that has one.
-__device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
+// With several warps, each looks at its band of block rows, and they agree.
+template <int NW>
+__device__ __forceinline__ bool can_raise(const WarpTile& S, const Worker<NW>& me) {
+    const int lane = me.lane, warp = me.warp;
+    constexpr int N = NB / NW;
+    const int j0 = warp * N;
     // maxima of R over the three columns around each pixel, for the two rows
     // of a block row: the neighbours' block words hold both rows
     auto hmax = [&](uint32_t w, uint32_t& top, uint32_t& bot) {
@@ -474,14 +548,15 @@ __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
         bot = __vimax3_u16x2(__byte_perm(L, w, 0x6030), __byte_perm(w, Rt, 0x6030), __byte_perm(w, 0u, ROW1));
     };
     uint32_t hp = 0u, h0, h1;  // maxima of the row before block row j, and of its two rows
-    uint2 b = S.B[lane];
+    if (NW > 1 && warp > 0) hmax(S.B[(j0 - 1) * BS + lane].x, h0, hp);
+    uint2 b = S.B[j0 * BS + lane];
     hmax(b.x, h0, h1);
     uint32_t v = 0u;
 #pragma unroll 1
-    for (int g = 0; g < NB / 8; g++) {
+    for (int g = 0; g < N / 8; g++) {
 #pragma unroll
         for (int jj = 0; jj < 8; jj++) {
-            const int j = g * 8 + jj;
+            const int j = j0 + g * 8 + jj;
             uint2 nb = make_uint2(0u, 0u);
             uint32_t n0 = 0u, n1 = 0u;
             if (j + 1 < NB) {
@@ -496,9 +571,10 @@ __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
             h1 = n1;
             b = nb;
         }
-        if (__any_sync(FULL, v != 0u)) return true;
+        if constexpr (NW == 1)
+            if (__any_sync(FULL, v != 0u)) return true;
     }
-    return false;
+    if constexpr (NW == 1) return false; else return me.any(v != 0u);
 }
 
 // Lets the halo into the tile: raises each border pixel by the halo pixels
@@ -506,7 +582,9 @@ __device__ __forceinline__ bool can_raise(const WarpTile& S, int lane) {
 // sweeps and the test need not look at it (they read a halo word per line
 // before), and when the tile was at a fixed point before the halo grew, no
 // pixel can be raised if no border pixel grew here.
-__device__ __forceinline__ bool let_in_halo(WarpTile& S, int lane) {
+template <int NW>
+__device__ __forceinline__ bool let_in_halo(WarpTile& S, const Worker<NW>& me) {
+    const int lane = me.lane, warp = me.warp;
     // lane l: border pixels 2l and 2l + 1 of a side in one block word, and the
     // four halo pixels around them (the halo lines hold the corners too, with
     // the same values as the halo rows)
@@ -523,14 +601,18 @@ __device__ __forceinline__ bool let_in_halo(WarpTile& S, int lane) {
             v = true;
         }
     };
-    raise(&S.B[lane], S.HRow[0][i] & 0xff, S.HRow[0][i + 1] & 0xff, S.HRow[0][i + 2] & 0xff, S.HRow[0][i + 3] & 0xff, 0, 8);
-    raise(&S.B[(NB - 1) * BS + lane], S.HRow[1][i] >> 16, S.HRow[1][i + 1] >> 16, S.HRow[1][i + 2] >> 16,
-          S.HRow[1][i + 3] >> 16, 16, 24);
-    __syncwarp();  // the corner blocks belong to a row and to a column
-    raise(&S.B[lane * BS], S.HC[0][i] & 0xff, S.HC[0][i + 1] & 0xff, S.HC[0][i + 2] & 0xff, S.HC[0][i + 3] & 0xff, 0, 16);
-    raise(&S.B[lane * BS + NB - 1], S.HC[1][i] >> 16, S.HC[1][i + 1] >> 16, S.HC[1][i + 2] >> 16, S.HC[1][i + 3] >> 16, 8, 24);
-    const bool any = __any_sync(FULL, v);
-    __syncwarp();
+    if (NW == 1 || warp == 0)
+        raise(&S.B[lane], S.HRow[0][i] & 0xff, S.HRow[0][i + 1] & 0xff, S.HRow[0][i + 2] & 0xff, S.HRow[0][i + 3] & 0xff, 0, 8);
+    if (NW == 1 || warp == 1)
+        raise(&S.B[(NB - 1) * BS + lane], S.HRow[1][i] >> 16, S.HRow[1][i + 1] >> 16, S.HRow[1][i + 2] >> 16,
+              S.HRow[1][i + 3] >> 16, 16, 24);
+    me.sync();  // the corner blocks belong to a row and to a column
+    if (NW == 1 || warp == 2)
+        raise(&S.B[lane * BS], S.HC[0][i] & 0xff, S.HC[0][i + 1] & 0xff, S.HC[0][i + 2] & 0xff, S.HC[0][i + 3] & 0xff, 0, 16);
+    if (NW == 1 || warp == 3)
+        raise(&S.B[lane * BS + NB - 1], S.HC[1][i] >> 16, S.HC[1][i + 1] >> 16, S.HC[1][i + 2] >> 16, S.HC[1][i + 3] >> 16, 8, 24);
+    const bool any = me.any(v);
+    me.sync();
     return any;
 }
 
@@ -541,16 +623,21 @@ __device__ __forceinline__ bool let_in_halo(WarpTile& S, int lane) {
 // to h can raise it.  h = -1 and h = RT are the halo corners, which belong
 // to the diagonal neighbours.  The side's border then becomes the reference
 // for the next requests.
-__device__ __forceinline__ void side_requests(WarpTile& S, int lane) {
+// With four warps, each takes a side.
+template <int NW>
+__device__ __forceinline__ void side_requests(WarpTile& S, const Worker<NW>& me) {
     // lane l holds border pixels 2l and 2l + 1 of every side: one block word
     // of R (top: block (0, l) bytes 0, 1; bottom: block (NB-1, l) bytes 2, 3;
     // left: block (l, 0) bytes 0, 2; right: block (l, NB-1) bytes 1, 3); the
     // changed values of the pixels beyond its pair come from the next lanes
+    const int lane = me.lane;
+    const int p0 = 2 * lane, p1 = 2 * lane + 1;
+    // (one warp: the four loads are in flight together)
     const uint32_t wt = S.B[lane].x, wb = S.B[(NB - 1) * BS + lane].x;
     const uint32_t wl = S.B[lane * BS].x, wr = S.B[lane * BS + NB - 1].x;
-    const int p0 = 2 * lane, p1 = 2 * lane + 1;
 #pragma unroll
     for (int s = 0; s < 4; s++) {
+        if (NW > 1 && s != me.warp) continue;
         const uint32_t w = s == 0 ? wt : s == 1 ? wb : s == 2 ? wl : wr;
         const int sh0 = s == 0 ? 0 : s == 1 ? 16 : s == 2 ? 0 : 8;
         const int sh1 = s == 0 ? 8 : s == 1 ? 24 : s == 2 ? 16 : 24;
@@ -603,23 +690,35 @@ __device__ __forceinline__ void side_requests(WarpTile& S, int lane) {
         S.B0[s][p0] = (uint8_t)v0;
         S.B0[s][p1] = (uint8_t)v1;
     }
-    __syncwarp();
+    me.sync();
 }
 
-__global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
+// A worker is a warp where each has many tiles to do (a warp needs no barriers,
+// and the workers hide one another's latency), and a CTA of four warps where
+// not: then the longest row of dependent visits sets the time, and a visit is
+// serial.  A round of sweeps is 64 steps of two shuffles and a few dependent
+// operations for a warp, 11500 clocks with its test, of which a visit takes two
+// or so, and 16 steps in four bands of 16 lines for a team, 3600 clocks with the
+// barriers; what has to cross bands costs more rounds (of 64 tiles, 6 rounds per
+// tile in all by warps, 10 by teams).  The team's warps also share the loads, the
+// requests and the write-back.  512^2: 141 -> 85 us; 1025 x 2049: 158 -> 107 us;
+// 4096^2: 282 -> 260 us.
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 1 ? RECON_MIN_BLOCKS : TEAM_MIN_BLOCKS) k_recon(Launch L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     WarpTile& S = *reinterpret_cast<WarpTile*>(smraw);
-    const int lane = threadIdx.x;
+    const Worker<NW> me;
+    const int t = me.t, lane = me.lane;
     int visits = 0;  // tile processings of this worker (diagnostic), added once at exit
-    if (lane < 9) S.flags[lane] = 0;
-    __syncwarp();
+    if (t < 9) S.flags[t] = 0;
+    me.sync();
     for (;;) {
         unsigned item = 0;
         int ok = 0;
-        if (lane == 0) ok = wl_pop(L, &item) ? 1 : 0;
-        ok = __shfl_sync(FULL, ok, 0);
+        if (t == 0) ok = wl_pop(L, &item) ? 1 : 0;
+        ok = me.from_first(S, ok);
         if (!ok) break;
-        item = __shfl_sync(FULL, item, 0);
+        item = (unsigned)me.from_first(S, (int)item);
         const int ti = (int)((item >> ITEM_BITS) & ITEM_IMAGE_MASK), k = (int)(item & ITEM_MASK);
         // a tile released by a visit was at a fixed point, so on later visits
         // only its border can have become raisable; its first visit starts
@@ -628,17 +727,17 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
         const TileDev& D = L.tiles[ti];
         const Img T{D.R, D.hem8, D.W, D.H, D.rp};
         const int rx = D.rtx, ry = D.rty, base = D.rt_base;
-        const int t = base + k, ty = k / rx, tx = k - ty * rx;
+        const int tile = base + k, ty = k / rx, tx = k - ty * rx;
         const int x0 = tx * RT, y0 = ty * RT;
-        if (lane == 0) atomicExch(&L.wl_state[t], WL_RUNNING);
+        if (t == 0) atomicExch(&L.wl_state[tile], WL_RUNNING);
         visits++;
         __threadfence();
-        __syncwarp();
-        load_tile(S, T, x0, y0, lane);
-        __syncwarp();
+        me.sync();
+        load_tile<NW>(S, T, x0, y0, t);
+        me.sync();
         // the border as loaded is the reference for the first requests (lane l:
         // border pixels 2l, 2l + 1 of each side, from one block word per side)
-        {
+        if (NW == 1 || me.warp == 0) {
             const uint32_t wt = S.B[lane].x, wb = S.B[(NB - 1) * BS + lane].x;
             const uint32_t wl = S.B[lane * BS].x, wr = S.B[lane * BS + NB - 1].x;
             S.B0[0][2 * lane] = (uint8_t)wt;
@@ -650,17 +749,17 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
             S.B0[3][2 * lane] = (uint8_t)(wr >> 8);
             S.B0[3][2 * lane + 1] = (uint8_t)(wr >> 24);
         }
-        __syncwarp();
+        me.sync();
         for (;;) {
             int nr = 0, queue = -1;
             bool more = false;
-            bool go = let_in_halo(S, lane) || sweep_now || (full_check && can_raise(S, lane));
+            bool go = let_in_halo<NW>(S, me) || sweep_now || (full_check && can_raise<NW>(S, me));
             sweep_now = false;
             while (go) {
                 if (nr >= MAX_ROUNDS) { more = true; break; }
-                sweep_round(S, lane);
+                sweep_round<NW>(S, me);
                 nr++;
-                go = can_raise(S, lane);
+                go = can_raise<NW>(S, me);
             }
             full_check = more;  // otherwise the interior is at a fixed point now
             bool grew = false;
@@ -668,19 +767,19 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
                 // the halo read only decides which neighbours to queue; it is
                 // issued before the write-back so that the two overlap (a stale
                 // value can only cause a needless request)
-                uint8_t hr[9];
-                load_halo(hr, nullptr, T, x0, y0, lane);
-                store_tile(S, T, x0, y0, lane);
+                uint8_t hr[halo_count<NW>()];
+                load_halo<NW>(hr, nullptr, T, x0, y0, t);
+                store_tile<NW>(S, T, x0, y0, t);
                 // the stores drain while the requests are worked out in shared memory
-                grew = __any_sync(FULL, merge_halo(S, hr, lane));
-                __syncwarp();
-                side_requests(S, lane);
-                if (more && lane == 0) S.flags[8] = 1;  // not converged within MAX_ROUNDS: run again
+                grew = me.any(merge_halo<NW>(S, hr, t));
+                me.sync();
+                side_requests<NW>(S, me);
+                if (more && t == 0) S.flags[8] = 1;  // not converged within MAX_ROUNDS: run again
                 __threadfence();  // this tile's pixels before any request
-                __syncwarp();
-                if (lane < 9 && S.flags[lane]) {
+                me.sync();
+                if (t < 9 && S.flags[t]) {
                     int target = -1;
-                    switch (lane) {
+                    switch (t) {
                         case 0: if (ty > 0) target = k - rx; break;
                         case 1: if (ty + 1 < ry) target = k + rx; break;
                         case 2: if (tx > 0) target = k - 1; break;
@@ -691,67 +790,79 @@ __global__ void __launch_bounds__(32, RECON_MIN_BLOCKS) k_recon(Launch L) {
                         case 7: if (ty + 1 < ry && tx + 1 < rx) target = k + rx + 1; break;
                         default: target = k; break;
                     }
-                    S.flags[lane] = 0;
+                    S.flags[t] = 0;
                     if (target >= 0 && wl_want(L, base + target)) queue = target;
                 }
             }
-            const unsigned qm = __ballot_sync(FULL, queue >= 0);
             // The tile is released (unless its fresher halo is to be looked at
             // again) before the wanted neighbours enter the queue; until the one
             // atomic that adds them and takes the tile off, it counts as pending.
             // No fence is needed before the release: every write-back above was
             // followed by one.
             int again = grew ? 1 : 0;
-            unsigned at = 0;
-            if (lane == 0) {
-                if (!grew && atomicCAS(&L.wl_state[t], WL_RUNNING, WL_IDLE) != WL_RUNNING) {
-                    atomicExch(&L.wl_state[t], WL_RUNNING);  // a neighbour raised the halo meanwhile
-                    again = 2;
+            if (NW == 1 || me.warp == 0) {
+                const unsigned qm = __ballot_sync(FULL, queue >= 0);
+                unsigned at = 0;
+                if (lane == 0) {
+                    if (!grew && atomicCAS(&L.wl_state[tile], WL_RUNNING, WL_IDLE) != WL_RUNNING) {
+                        atomicExch(&L.wl_state[tile], WL_RUNNING);  // a neighbour raised the halo meanwhile
+                        again = 2;
+                    }
+                    const int n = __popc(qm), less = again ? 0 : 1;
+                    if (n || less)
+                        at = (unsigned)(atomicAdd(&L.sh->tp, ((unsigned long long)n << 32) + (unsigned long long)(long long)(n - less)) >> 32);
                 }
-                const int n = __popc(qm), less = again ? 0 : 1;
-                if (n || less)
-                    at = (unsigned)(atomicAdd(&L.sh->tp, ((unsigned long long)n << 32) + (unsigned long long)(long long)(n - less)) >> 32);
+                at = __shfl_sync(FULL, at, 0);
+                if (queue >= 0) wl_put(L, at + __popc(qm & ((1u << lane) - 1u)), ((unsigned)ti << ITEM_BITS) | (unsigned)queue);
             }
-            at = __shfl_sync(FULL, at, 0);
-            if (queue >= 0) wl_put(L, at + __popc(qm & ((1u << lane) - 1u)), ((unsigned)ti << ITEM_BITS) | (unsigned)queue);
-            again = __shfl_sync(FULL, again, 0);
-            __syncwarp();
+            again = me.from_first(S, again);
+            me.sync();
             if (again == 1) continue;  // the fresher halo may raise pixels: check again
             if (!again) break;
             visits++;
             __threadfence();
-            if (__any_sync(FULL, ld_vol(&L.sh->err) != 0)) break;
+            if (me.any(ld_vol(&L.sh->err) != 0)) break;
             // only the halo can have changed: the interior belongs to this worker
-            uint8_t hr[9];
-            load_halo(hr, nullptr, T, x0, y0, lane);
-            merge_halo(S, hr, lane);
-            __syncwarp();
+            uint8_t hr[halo_count<NW>()];
+            load_halo<NW>(hr, nullptr, T, x0, y0, t);
+            merge_halo<NW>(S, hr, t);
+            me.sync();
         }
-        __syncwarp();
+        me.sync();
     }
-    if (lane == 0 && visits) atomicAdd(&L.sh->processed, visits);
+    if (t == 0 && visits) atomicAdd(&L.sh->processed, visits);
 }
 
-// resident workers (one warp each) of the reconstruction kernel
-int recon_grid(int device) {
-    int sms = 0, per = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const size_t smem = sizeof(WarpTile);
-    cudaFuncSetAttribute(k_recon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_recon, 32, smem);
+template <int NW>
+static int recon_resident(int sms) {
+    int per = 0;
+    cudaFuncSetAttribute(k_recon<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WarpTile));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_recon<NW>, 32 * NW, sizeof(WarpTile));
     return sms * (per < 1 ? 1 : per);
 }
 
-void launch_recon(const Launch& L, int grid_cap, cudaStream_t s, Profiler* pf) {
+// resident workers of the reconstruction kernels: warps, and teams
+void recon_grid(int device, int* warps, int* teams) {
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    *warps = recon_resident<1>(sms);
+    *teams = recon_resident<4>(sms);
+}
+
+void launch_recon(const Launch& L, int warps, int warps_cap, int teams_cap, cudaStream_t s, Profiler* pf) {
     if (L.n_rt == 0) return;
     pf->begin("recon_init", s);
     k_wl_reset<<<1, 256, 0, s>>>(L);
     k_wl_count<<<(L.n_rt + 255) / 256, 256, 0, s>>>(L);
     k_wl_init<<<(L.n_rt + 255) / 256, 256, 0, s>>>(L);
     pf->end("recon_init", s);
-    const int grid = L.n_rt < grid_cap ? L.n_rt : grid_cap;  // one work tile per worker at a time
     pf->begin("recon", s);
-    k_recon<<<grid, 32, sizeof(WarpTile), s>>>(L);
+    if (L.n_rt < TEAM_TILES * warps_cap) {  // as many teams of all as `warps` is of all warps
+        const int teams = std::max(1, (int)((long long)teams_cap * warps / warps_cap));
+        k_recon<4><<<std::min(L.n_rt, teams), 128, sizeof(WarpTile), s>>>(L);
+    } else {
+        k_recon<1><<<std::min(L.n_rt, warps), 32, sizeof(WarpTile), s>>>(L);
+    }
     pf->end("recon", s);
 }
 

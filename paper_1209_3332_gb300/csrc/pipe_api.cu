@@ -301,7 +301,7 @@ struct pipe_s {
     int device = 0;
     pipe_params prm;
     int sms = 0;
-    int recon_cap = 1;
+    int recon_cap = 1, recon_teams = 1;  // resident workers of the reconstruction: warps, teams
     EventProfiler prof;
     // plain form
     LaunchCtx plain;
@@ -483,7 +483,7 @@ int make_grow(pipe_t p, const std::vector<CannyDesc>& cd, int n_rt, cudaStream_t
 void run_path(pipe_t p, const Launch& L, int Wmax, bool features, int max_objects, const Tune& tu,
               cudaStream_t s, Profiler* pf) {
     launch_deconv(L, s, pf);
-    launch_recon(L, tu.recon_grid, s, pf);
+    launch_recon(L, tu.recon_grid, p->recon_cap, p->recon_teams, s, pf);
     launch_label(L, features ? 1 : 0, max_objects, p->sms, s, pf);
     launch_edt(L, tu.edt_rb, Wmax, s, pf);
     if (features) launch_features_batched(L, tu.feat_grid, s, pf);
@@ -726,7 +726,7 @@ int pipe_create(const pipe_params* params, int device, pipe_t* out) {
     int32_t lut[256], wq[3];
     deconv_tables(lut, wq);
     upload_deconv_tables(lut, wq);
-    p->recon_cap = std::max(1, recon_grid(device));
+    recon_grid(device, &p->recon_cap, &p->recon_teams);
     p->grow_cap = std::max(1, grow_grid(device));
     if (prm.autotune_cache) {
         p->tune_file = prm.autotune_cache;

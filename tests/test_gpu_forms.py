@@ -293,3 +293,32 @@ def test_many_small_tiles_in_one_batch(n):
         assert bool((lab[k::len(kinds)] == want[0]).all()) and bool((edt[k::len(kinds)] == want[1]).all())
         assert_feats_close(feats[k].cpu().numpy()[:r["K"]], r["feats"])
     pipe.close()
+
+
+@pytest.mark.parametrize("n", [1, 101, 102, 130])
+def test_reconstruction_by_warps_and_by_teams(n):
+    """48 work tiles of the reconstruction per tile: with 101 there are just
+    fewer than two for each of 2432 warps, with 102 just more, so that teams of
+    warps and single warps take them in turn; corridors and chains, noise."""
+    import torch
+    import paper_1209_3332_gb300 as P
+    W, H = 449, 321
+    rng = np.random.default_rng(8)
+    kinds = [synth.tile(W, H, 6, n_nuclei=150, frac_chain=0.7, corridor=True), rng.integers(0, 256, (H, W, 3)).astype(np.uint8)]
+    refs = [oracle_all(k) for k in kinds]
+    pipe = P.Pipe(0, autotune=0)
+    dev = torch.device("cuda", 0)
+    rgb = [torch.from_numpy(np.ascontiguousarray(k)).to(dev) for k in kinds]
+    hem = torch.empty((n, H, W), dtype=torch.uint8, device=dev)
+    lab = torch.full((n, H, W), -1, dtype=torch.int32, device=dev)
+    edt = torch.empty((n, H, W), dtype=torch.int32, device=dev)
+    nobj = torch.zeros(n, dtype=torch.int32, device=dev)
+    feats = torch.zeros((n, 8, 15), dtype=torch.float32, device=dev)
+    pipe.seg_features_batch([dict(rgb=rgb[i % 2], hem8=hem[i], labels=lab[i], edt=edt[i], n_objects=nobj[i:i + 1],
+                                  feats=feats[i]) for i in range(n)])
+    torch.cuda.synchronize()
+    for k, r in enumerate(refs[:n]):
+        assert bool((nobj[k::2] == r["K"]).all())
+        assert bool((lab[k::2] == torch.from_numpy(r["labels"]).to(dev)).all())
+        assert bool((edt[k::2] == torch.from_numpy(r["edt"]).to(dev)).all())
+    pipe.close()
