@@ -68,6 +68,7 @@ __device__ void meijster_row(const uint16_t* g, int W, int32_t* out) {
 }
 
 __global__ void __launch_bounds__(256) k_edt_rows(Launch L, int RB, int Wmax) {
+    if (L.early) after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
     uint16_t* gs = reinterpret_cast<uint16_t*>(smraw);  // [RB][WMAX + Wmax + WMAX]
     const int Wp = Wmax + 2 * WMAX;
@@ -178,7 +179,7 @@ void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf)
     size_t smem = edt_rows_smem(RB, Wmax);
     cudaFuncSetAttribute(k_edt_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     pf->begin("edt_rows", s);
-    k_edt_rows<<<L.n_rows, 256, smem, s>>>(L, RB, Wmax);
+    launch_behind(L.early && pf->overlap(), k_edt_rows, L.n_rows, 256, smem, s, L, RB, Wmax);
     pf->end("edt_rows", s);
 }
 

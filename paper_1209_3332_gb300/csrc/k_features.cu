@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(FW * 32) k_fobj_plain(ObjJob J, int K) {
 }
 
 __global__ void k_obj_prefix(Launch L) {
+    if (L.early) after_previous();
     if (threadIdx.x != 0) return;
     int run = 0;
     for (int t = 0; t < L.ntiles; t++) {
@@ -316,6 +317,7 @@ __global__ void k_obj_prefix(Launch L) {
 // Batched form: the objects of all tiles, item -> (tile, object) through the
 // obj_base prefixes (the last tile whose base is <= item owns it).
 __global__ void __launch_bounds__(FW * 32) k_fobj_batched(Launch L) {
+    if (L.early) after_previous();
     __shared__ ObjSmem sm[FW];
     const int warp = threadIdx.x >> 5;
     ObjSmem& S = sm[warp];
@@ -358,10 +360,10 @@ void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, in
 
 void launch_features_batched(const Launch& L, int grid, cudaStream_t s, Profiler* pf) {
     pf->begin("feat_prefix", s);
-    k_obj_prefix<<<1, 32, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_obj_prefix, 1, 32, 0, s, L);
     pf->end("feat_prefix", s);
     pf->begin("feat_objects", s);
-    k_fobj_batched<<<grid, FW * 32, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_fobj_batched, grid, FW * 32, 0, s, L);
     pf->end("feat_objects", s);
 }
 

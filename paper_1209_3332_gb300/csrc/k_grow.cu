@@ -192,6 +192,7 @@ __device__ void grow_tile(const GrowLaunch& G, int t, int drop, int lane) {
 constexpr int GROW_WARPS = 4;
 
 __global__ void __launch_bounds__(GROW_WARPS * 32) k_grow(const __grid_constant__ GrowLaunch G) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     int groups = 0;
     for (;; groups++) {  // the tiles of a group that hold a marker pixel
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(GROW_WARPS * 32) k_grow(const __grid_constant_
 __device__ __forceinline__ uint32_t nibble_bytes(unsigned b) { return (b * 0x00204081u) & 0x01010101u; }
 
 __global__ void __launch_bounds__(256) k_grow_out(const __grid_constant__ GrowLaunch G) {
+    after_previous();
     const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (t >= G.n_rt) return;
     const CannyDesc& d = G.tab[G.tab.find(t, &CannyDesc::rt_base)];
@@ -309,10 +311,10 @@ int grow_grid(int device) {
 
 void launch_grow(const GrowLaunch& G, int grid_cap, cudaStream_t s, Profiler* pf) {
     pf->begin("grow", s);
-    k_grow<<<std::min((G.n_rt + GROW_WARPS - 1) / GROW_WARPS, grid_cap), GROW_WARPS * 32, 0, s>>>(G);
+    launch_behind(pf->overlap(), k_grow, std::min((G.n_rt + GROW_WARPS - 1) / GROW_WARPS, grid_cap), GROW_WARPS * 32, 0, s, G);
     pf->end("grow", s);
     pf->begin("grow_out", s);
-    k_grow_out<<<(G.n_rt + 7) / 8, 256, 0, s>>>(G);
+    launch_behind(pf->overlap(), k_grow_out, (G.n_rt + 7) / 8, 256, 0, s, G);
     pf->end("grow_out", s);
 }
 

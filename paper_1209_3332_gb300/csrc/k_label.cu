@@ -285,6 +285,7 @@ __device__ __forceinline__ int register_roots(const TileDev& T, const WarpGeo& g
 
 // ---- K3a: foreground from the h-dome, background local components ---------------
 __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_fill_local(Launch L) {
+    if (L.early) after_previous();
     __shared__ int par_sm[CCL_WARPS][CB * CB];
     __shared__ uint32_t touch_sm[CCL_WARPS][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -418,6 +419,7 @@ __device__ __forceinline__ void merge_edge(const TileDev& T, int bx, int by, int
 // walks all of its edge pixels).  Bound: the latency of the finds.
 template <int CONN>
 __global__ void __launch_bounds__(CCL_WARPS * 32) k_merge(Launch L, int per) {
+    if (L.early) after_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int first = (blockIdx.x * CCL_WARPS + warp) * per, gb = first + lane;
     if (first >= L.n_cb) return;
@@ -534,6 +536,7 @@ __device__ __forceinline__ bool root_pass(const Launch& L, const TileDev& T, int
 
 template <int MODE>
 __global__ void __launch_bounds__(CCL_WARPS * 32) k_roots(Launch L, int per) {
+    if (L.early) after_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int first = (blockIdx.x * CCL_WARPS + warp) * per, gb = first + lane;
     if (first >= L.n_cb) return;
@@ -576,6 +579,7 @@ __global__ void __launch_bounds__(CCL_WARPS * 32) k_roots(Launch L, int per) {
 
 // ---- K4a: holes -> filled; foreground local components ----------------------------
 __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_label_local(Launch L) {
+    if (L.early) after_previous();
     __shared__ int par_sm[CCL_WARPS][CB * CB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gb = blockIdx.x * CCL_WARPS + warp;
@@ -658,6 +662,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* tmp /*[32]*/, in
 // (pass 1); each thread takes four consecutive words (one 16-byte load where
 // the chunk lies inside the bitmap: chunks start at multiples of 16 KB)
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(Launch L, int pass) {
+    if (L.early) after_previous();
     __shared__ int tmp[32];
     int gc = blockIdx.x;
     int ti = find_tile(L.tiles, L.ntiles, gc, &TileDev::chunk_base);
@@ -692,6 +697,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(Launch L, int pass
 
 // one block per tile: exclusive scan of the chunk sums; K = total
 __global__ void __launch_bounds__(1024) k_scan_tiles(Launch L) {
+    if (L.early) after_previous();
     __shared__ int tmp[32];
     const TileDev& T = L.tiles[blockIdx.x];
     int carry = 0;
@@ -713,6 +719,7 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(Launch L) {
 // writes its row of labels from registers, four labels per 16-byte store.
 constexpr int LAB_FLAG = (int)0x80000000u;
 __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int want_bbox) {
+    if (L.early) after_previous();
     __shared__ int par_sm[CCL_WARPS][CB * CB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gb = blockIdx.x * CCL_WARPS + warp;
@@ -855,6 +862,7 @@ __global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int wa
 
 // every box slot a tile can use (feats_cap of them) starts empty
 __global__ void k_bbox_init(Launch L) {
+    if (L.early) after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     for (int ti = 0; ti < L.ntiles; ti++) {
         const TileDev& T = L.tiles[ti];
@@ -865,6 +873,7 @@ __global__ void k_bbox_init(Launch L) {
 }
 
 __global__ void k_counters_reset(Launch L) {
+    if (L.early) after_previous();
     for (int i = threadIdx.x; i < L.ntiles; i += blockDim.x) L.tile_status[i] = 0;
 }
 
@@ -890,15 +899,15 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
     if (L.n_cb == 0) return;
     const int rgrid = sms * 8;
     pf->begin("label_reset", s);
-    k_counters_reset<<<1, 1024, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_counters_reset, 1, 1024, 0, s, L);
     pf->end("label_reset", s);
     if (want_bbox) {
         pf->begin("bbox_init", s);
-        k_bbox_init<<<rgrid, 256, 0, s>>>(L);
+        launch_behind(L.early && pf->overlap(), k_bbox_init, rgrid, 256, 0, s, L);
         pf->end("bbox_init", s);
     }
     pf->begin("fill_local", s);
-    k_fill_local<<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_fill_local, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L);
     pf->end("fill_local", s);
     // Blocks per warp of the merge and root passes: as many as leave one wave of
     // resident warps, up to 8.  On 16 tiles of 4096^2 more blocks per warp mean
@@ -908,39 +917,39 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
     while (per < 8 && L.n_cb > per * sms * 64) per *= 2;
     const int pg = (L.n_cb + CCL_WARPS * per - 1) / (CCL_WARPS * per), pt = CCL_WARPS * 32;
     pf->begin("fill_merge", s);
-    k_merge<4><<<pg, pt, 0, s>>>(L, per);
+    launch_behind(L.early && pf->overlap(), k_merge<4>, pg, pt, 0, s, L, per);
     pf->end("fill_merge", s);
     pf->begin("fill_roots_flag", s);
-    k_roots<0><<<pg, pt, 0, s>>>(L, per);
+    launch_behind(L.early && pf->overlap(), k_roots<0>, pg, pt, 0, s, L, per);
     pf->end("fill_roots_flag", s);
     pf->begin("fill_roots_copy", s);
-    k_roots<1><<<pg, pt, 0, s>>>(L, per);
+    launch_behind(L.early && pf->overlap(), k_roots<1>, pg, pt, 0, s, L, per);
     pf->end("fill_roots_copy", s);
     pf->begin("label_local", s);
-    k_label_local<<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_label_local, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L);
     pf->end("label_local", s);
     pf->begin("label_merge", s);
     // (a warp per block: edges with foreground are all walked, and 8 blocks per
     // warp take 102 us instead of 38 on four tiles dense with nuclei)
-    k_merge<8><<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, pt, 0, s>>>(L, 1);
+    launch_behind(L.early && pf->overlap(), k_merge<8>, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, pt, 0, s, L, 1);
     pf->end("label_merge", s);
     pf->begin("label_roots_area", s);
-    k_roots<2><<<pg, pt, 0, s>>>(L, per);
+    launch_behind(L.early && pf->overlap(), k_roots<2>, pg, pt, 0, s, L, per);
     pf->end("label_roots_area", s);
     pf->begin("label_roots_keep", s);
-    k_roots<3><<<pg, pt, 0, s>>>(L, per);
+    launch_behind(L.early && pf->overlap(), k_roots<3>, pg, pt, 0, s, L, per);
     pf->end("label_roots_keep", s);
     pf->begin("scan_chunks", s);
-    k_scan_chunks<<<L.n_chunks, SCAN_THREADS, 0, s>>>(L, 0);
+    launch_behind(L.early && pf->overlap(), k_scan_chunks, L.n_chunks, SCAN_THREADS, 0, s, L, 0);
     pf->end("scan_chunks", s);
     pf->begin("scan_tiles", s);
-    k_scan_tiles<<<L.ntiles, 1024, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_scan_tiles, L.ntiles, 1024, 0, s, L);
     pf->end("scan_tiles", s);
     pf->begin("scan_words", s);
-    k_scan_chunks<<<L.n_chunks, SCAN_THREADS, 0, s>>>(L, 1);
+    launch_behind(L.early && pf->overlap(), k_scan_chunks, L.n_chunks, SCAN_THREADS, 0, s, L, 1);
     pf->end("scan_words", s);
     pf->begin("relabel", s);
-    k_relabel<<<(L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s>>>(L, want_bbox);
+    launch_behind(L.early && pf->overlap(), k_relabel, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L, want_bbox);
     pf->end("relabel", s);
 }
 

@@ -20,6 +20,7 @@ constexpr int RB_WARPS = 8;  // work tiles per CTA
 __global__ void __launch_bounds__(RB_WARPS * 32) k_rbc_planes(const __grid_constant__ GrowLaunch G,
                                                               const uint8_t* __restrict__ rgb, size_t pitch, int t_lo,
                                                               int t_hi) {
+    cudaTriggerProgrammaticLaunchCompletion();  // the growth may be prepared
     const int t = blockIdx.x * RB_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x == 0) grow_reset(G);
     if (t >= G.n_rt) return;

@@ -244,6 +244,7 @@ __device__ __forceinline__ int order_class(const Launch& L, int i, int* ti_out, 
 }
 
 __global__ void k_wl_reset(Launch L) {
+    if (L.early) after_previous();
     for (int t = threadIdx.x; t < L.ntiles; t += blockDim.x)
 #pragma unroll
         for (int j = 0; j < 8; j++) L.tiles[t].cls[j] = L.tiles[t].cls_pos[j] = 0;
@@ -253,6 +254,7 @@ __global__ void k_wl_reset(Launch L) {
 // and class, so the counters see one atomic per group instead of one per
 // work tile.
 __global__ void k_wl_count(Launch L) {
+    if (L.early) after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     int ti = -1, k = 0, c = 0;
     if (i < L.n_rt) c = order_class(L, i, &ti, &k);
@@ -262,6 +264,7 @@ __global__ void k_wl_count(Launch L) {
 }
 
 __global__ void k_wl_init(Launch L) {
+    if (L.early) after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     if (i == 0) {
         L.sh->head = 0;
@@ -705,6 +708,7 @@ __device__ __forceinline__ void side_requests(WarpTile& S, const Worker<NW>& me)
 // 4096^2: 282 -> 260 us.
 template <int NW>
 __global__ void __launch_bounds__(32 * NW, NW == 1 ? RECON_MIN_BLOCKS : TEAM_MIN_BLOCKS) k_recon(Launch L) {
+    if (L.early) after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
     WarpTile& S = *reinterpret_cast<WarpTile*>(smraw);
     const Worker<NW> me;
@@ -852,16 +856,16 @@ void recon_grid(int device, int* warps, int* teams) {
 void launch_recon(const Launch& L, int warps, int warps_cap, int teams_cap, cudaStream_t s, Profiler* pf) {
     if (L.n_rt == 0) return;
     pf->begin("recon_init", s);
-    k_wl_reset<<<1, 256, 0, s>>>(L);
-    k_wl_count<<<(L.n_rt + 255) / 256, 256, 0, s>>>(L);
-    k_wl_init<<<(L.n_rt + 255) / 256, 256, 0, s>>>(L);
+    launch_behind(L.early && pf->overlap(), k_wl_reset, 1, 256, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_wl_count, (L.n_rt + 255) / 256, 256, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_wl_init, (L.n_rt + 255) / 256, 256, 0, s, L);
     pf->end("recon_init", s);
     pf->begin("recon", s);
     if (L.n_rt < TEAM_TILES * warps_cap) {  // as many teams of all as `warps` is of all warps
         const int teams = std::max(1, (int)((long long)teams_cap * warps / warps_cap));
-        k_recon<4><<<std::min(L.n_rt, teams), 128, sizeof(WarpTile), s>>>(L);
+        launch_behind(L.early && pf->overlap(), k_recon<4>, std::min(L.n_rt, teams), 128, sizeof(WarpTile), s, L);
     } else {
-        k_recon<1><<<std::min(L.n_rt, warps), 32, sizeof(WarpTile), s>>>(L);
+        launch_behind(L.early && pf->overlap(), k_recon<1>, std::min(L.n_rt, warps), 32, sizeof(WarpTile), s, L);
     }
     pf->end("recon", s);
 }

@@ -94,6 +94,7 @@ struct EventProfiler : Profiler {
         pending_name = name;
         cudaEventRecord(pending_begin, s);
     }
+    bool overlap() const override { return !enabled; }  // events between kernels time them one by one
     void end(const char* name, cudaStream_t s) override {
         if (!enabled || !pending_begin) return;
         cudaEvent_t b = get();
@@ -799,6 +800,7 @@ int seg_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
     t.feats = nullptr;
     const Tune tu = default_tune(p, W);
     Launch L = make_launch(p, p->plain, td, n_rt, tu.edt_rb);
+    L.early = 1;
     if ((rc = upload_desc(L, td, s))) return rc;
     run_path(p, L, W, false, 0, tu, s, &p->prof);
     CK(cudaGetLastError());

@@ -322,3 +322,44 @@ def test_reconstruction_by_warps_and_by_teams(n):
         assert bool((lab[k::2] == torch.from_numpy(r["labels"]).to(dev)).all())
         assert bool((edt[k::2] == torch.from_numpy(r["edt"]).to(dev)).all())
     pipe.close()
+
+
+@pytest.mark.parametrize("how", ["direct", "profiled", "captured"])
+def test_passes_back_to_back(pipe, how):
+    """Passes of different sizes on one stream and one workspace, none waited
+    for on the host: a kernel that is launched before the one ahead of it is
+    complete may not read or write anything of that pass too early.  Launched
+    directly, with events between the kernels, and as a captured graph."""
+    import torch
+    dev = torch.device("cuda", 0)
+    kinds = [synth.tile(512, 384, 31, n_nuclei=120, frac_chain=0.4), synth.tile(77, 133, 32, n_nuclei=6),
+             synth.tile(1030, 517, 33, n_nuclei=300, frac_cluster=0.3), synth.tile(64, 64, 34, n_nuclei=0)]
+    refs = [oracle_all(k) for k in kinds]
+    rgb = [torch.from_numpy(np.ascontiguousarray(k)).to(dev) for k in kinds]
+    passes = []
+    for i in range(24):
+        H, W = rgb[i % 4].shape[:2]
+        passes.append((rgb[i % 4], torch.empty((H, W), dtype=torch.uint8, device=dev), torch.full((H, W), -1, dtype=torch.int32, device=dev),
+                       torch.full((H, W), -1, dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)))
+    for p in passes[:4]:  # workspaces grow here
+        pipe.seg_tile(*p)
+    torch.cuda.synchronize()
+    for p in passes[:4]:
+        p[2].fill_(-1)
+    pipe.profile(how == "profiled")
+    if how == "captured":
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for p in passes:
+                pipe.seg_tile(*p, stream=torch.cuda.current_stream())
+        g.replay()
+    else:
+        for p in passes:
+            pipe.seg_tile(*p)
+    torch.cuda.synchronize()
+    pipe.profile(False)
+    for i, p in enumerate(passes):
+        r = refs[i % 4]
+        assert int(p[4].item()) == r["K"]
+        assert np.array_equal(p[1].cpu().numpy(), r["hem8"])
+        assert np.array_equal(p[2].cpu().numpy(), r["labels"]) and np.array_equal(p[3].cpu().numpy(), r["edt"])
