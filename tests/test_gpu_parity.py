@@ -136,3 +136,22 @@ def test_unaligned_buffers(pipe, W, H, off, pad):
     ref = oracle_all(rgb)
     assert_planes_equal(dict(hem8=hem.cpu().numpy(), R=R.cpu().numpy(), labels=lab.cpu().numpy(), edt=edt.cpu().numpy(),
                              K=int(nobj.item())), ref)
+
+
+@pytest.mark.parametrize("W", [720, 721, 722, 8, 4])
+def test_distances_of_large_objects(W):
+    """Objects wider and taller than several 32-row chunks, whose pixels look
+    for background far beyond their own group of four columns, up to and past
+    the widest search (128), at the image's sides too; widths that are and are
+    not a multiple of four."""
+    import paper_1209_3332_gb300 as P
+    rgb = ring_tile(720, 530)
+    yy, xx = np.mgrid[:530, :720]
+    for cx, cy, rad in ((150, 330, 140), (700, 120, 90), (0, 0, 50)):
+        rgb[(xx - cx) ** 2 + (yy - cy) ** 2 <= rad * rad] = 0
+    rgb = np.concatenate([rgb, np.full((530, 2, 3), 255, np.uint8)], 1)[:, :W] if W > 720 else rgb[:, :W]
+    p = P.Pipe(0, area_max=10 ** 6)
+    g, r = check(p, np.ascontiguousarray(rgb), amax=10 ** 6)
+    if W >= 720:
+        assert int(r["edt"].max()) > 128 * 128
+    p.close()
