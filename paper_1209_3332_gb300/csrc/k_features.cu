@@ -19,8 +19,17 @@
 // non-negative terms, and the gradient mean and variance come from one pass
 // of Welford updates per lane, the lanes combined pairwise (a sum of
 // non-negative terms).
+//
+// A warp's pixels are few and its finishing is long: 36 sums over the warp for
+// the co-occurrence statistics and seven FP64 divisions and roots.  In 32 bits,
+// one instruction per sum, and with a feature per lane (an FP64 instruction
+// takes as long for one lane as for 32), they took 331 -> 203 us for the 48000
+// objects of 16 tiles of 4096^2, and with a stage small enough for 32 warps per
+// SM instead of 20, 173 us.  What bounds it now is the pixel walk: a chain of
+// shared-memory reads and a Welford update with a division per pixel.
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -74,13 +83,29 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-constexpr int STAGE_PX = 5120;  // staged region (box + 1-px margin) capacity per warp
+// A warp stages at most STAGE_PX pixels at a time: with the counters 26 KB per
+// CTA, eight of which fit on an SM (all of a region of 5120 pixels at once: five;
+// objects of 16 tiles of 4096^2 203 us, and 171).
+constexpr int STAGE_PX = 2816;
+constexpr int REGION_PX = 5120;  // largest region (box + 1-px margin) that is staged
+constexpr int HOM_LCM = 408850;  // lcm of 1 + d^2 for d = 0..7
+
+// A sum over the warp of non-negative whole numbers.  Those of a staged object
+// (at most REGION_PX pixels) are below 2^32, so that one instruction adds them.
+template <bool STAGED>
+__device__ __forceinline__ long long whole_sum(long long v) {
+    static_assert((long long)HOM_LCM * REGION_PX < (1LL << 32) && 255LL * 255 * REGION_PX < (1LL << 32) &&
+                  (long long)REGION_PX * REGION_PX < (1LL << 32), "the largest sums");
+    if constexpr (STAGED) return (long long)__reduce_add_sync(FULLF, (unsigned)v);
+    else return warp_sum<long long>(v);
+}
 
 // Features of object `obj` by one warp; glcm: this warp's 4x64 counters;
 // spx: this warp's staging buffer.  When the object's box plus a
-// 1-pixel margin (clipped to the image) fits, it is staged once with
-// coalesced row loads as one 16-bit word per pixel (hem8 and an in-object
-// bit), and every neighbourhood read comes from shared memory; larger boxes read global
+// 1-pixel margin (clipped to the image) has at most REGION_PX pixels, it is
+// staged with coalesced row loads as one 16-bit word per pixel (hem8 and an
+// in-object bit), in bands of rows if it is larger than the buffer, and every
+// neighbourhood read comes from shared memory; larger boxes read global
 // memory directly.  Sobel neighbours (clamped to the image), 4-neighbours and
 // co-occurrence partners of box pixels all lie inside that region.
 template <bool STAGED>
@@ -101,17 +126,20 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     const int rw = min(box.z + 1, W - 1) - rx0 + 1, rh = min(box.w + 1, H - 1) - ry0 + 1;
     constexpr bool staged = STAGED;
     for (int i = lane; i < 4 * 64; i += 32) glcm[i] = 0;
-    if (staged) {
-        // the region as one index space, four pixels per lane per step with
-        // all their loads issued before the stores, so their latencies overlap
-        const int nreg = rh * rw;
+    int sy0 = 0;  // first staged row
+    // stages rows [from, to] of the region's columns
+    auto stage = [&](int from, int to) {
+        sy0 = from;
+        // one index space, four pixels per lane per step with all their loads
+        // issued before the stores, so their latencies overlap
+        const int nreg = (to - from + 1) * rw;
         int sy = lane / rw, sx = lane - sy * rw;
         for (int base = lane; base < nreg; base += 4 * 32) {
             int lab[4], hv[4], at[4];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 at[u] = base + 32 * u < nreg ? sy * rw + sx : -1;
-                const size_t g = (size_t)(ry0 + sy) * W + rx0 + sx;
+                const size_t g = (size_t)(from + sy) * W + rx0 + sx;
                 lab[u] = at[u] >= 0 ? J.labels[g] : 0;
                 hv[u] = at[u] >= 0 ? J.hem8[g] : 0;
                 sx += 32;
@@ -121,22 +149,30 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
             for (int u = 0; u < 4; u++)
                 if (at[u] >= 0) spx[at[u]] = (uint16_t)(hv[u] | (lab[u] == l ? 0x100 : 0));
         }
-    }
-    __syncwarp();
+    };
     // pixel (y, x) of the region as hem8 | (in object) << 8: the 3x3
     // neighbourhood of a pixel serves its Sobel sums, its perimeter test and
     // its co-occurrence partners
     auto PX = [&](int y, int x) -> uint32_t {
-        if (staged) return spx[(y - ry0) * rw + (x - rx0)];
+        if (staged) return spx[(y - sy0) * rw + (x - rx0)];
         const size_t o = (size_t)y * W + x;
         return (uint32_t)J.hem8[o] | (J.labels[o] == l ? 0x100u : 0u);
     };
     int cnt = 0, per = 0, mn = 255, mx = 0, gmn = 0x7fffffff, gmx = 0;
-    long long S = 0, Q = 0;
+    using Whole = typename std::conditional<STAGED, unsigned, long long>::type;
+    Whole S = 0, Q = 0;
     float wm = 0.f, wq = 0.f;  // this lane's running mean and sum of squared deviations of |Sobel|
     // lane walks the box row-major with stride 32, advancing (y, x) without divisions
     int y = box.y + lane / bw, x = box.x + lane % bw;
-    for (long long idx = lane; idx < npx; idx += 32) {
+    // a band: box rows [yb, ye], staged with the rows beside them
+    const int band = staged ? (rw * rh <= STAGE_PX ? bh : STAGE_PX / rw - 2) : bh;
+    long long idx = lane;
+    for (int yb = box.y; yb <= box.w; yb += band) {
+    const int ye = min(yb + band - 1, box.w);
+    __syncwarp();
+    if (staged) stage(max(yb - 1, 0), min(ye + 1, H - 1));
+    __syncwarp();
+    for (; idx < npx && y <= ye; idx += 32) {
         const int cy = y, cx = x;
         x += 32;
         while (x > box.z) { x -= bw; y++; }
@@ -173,9 +209,10 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
         if (cy + 1 < H && cx + 1 < W && (i >> 8)) atomicAdd(&glcm[2 * 64 + vb + ((i & 0xffu) >> 5)], 1);
         if (cy > 0 && cx + 1 < W && (c >> 8)) atomicAdd(&glcm[3 * 64 + vb + ((c & 0xffu) >> 5)], 1);
     }
-    const long long N = warp_sum<long long>(cnt);
-    const long long Ssum = warp_sum<long long>(S), Qsum = warp_sum<long long>(Q);
-    const long long Per = warp_sum<long long>(per);
+    }
+    const long long N = whole_sum<STAGED>(cnt);
+    const long long Ssum = whole_sum<STAGED>(S), Qsum = whole_sum<STAGED>(Q);
+    const long long Per = whole_sum<STAGED>(per);
     const int Mn = __reduce_min_sync(FULLF, mn), Mx = __reduce_max_sync(FULLF, mx);
     const int Gmn = __reduce_min_sync(FULLF, gmn), Gmx = __reduce_max_sync(FULLF, gmx);
     // the lanes' (count, mean, squared deviations) combined pairwise (Chan,
@@ -217,25 +254,25 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     int used = 0;
     const int i0 = lane >> 3, j0 = lane & 7, i1 = i0 + 4, j1 = j0;
     const int d0 = (i0 - j0) * (i0 - j0), d1 = (i1 - j1) * (i1 - j1);
-    const long long HL = 408850;  // lcm of 1+d^2 for d = 0..7
+    const Whole HL = HOM_LCM;
     auto ent = [](long long C, long long T) -> float {
         return C > 0 ? __fmul_rn(__fdiv_rn((float)C, (float)T), log1pf(__fdiv_rn((float)(T - C), (float)C))) : 0.f;
     };
 #pragma unroll
     for (int o = 0; o < 4; o++) {
         const int* cc = glcm + o * 64;
-        const long long v0 = cc[lane], v1 = cc[lane + 32];
-        const long long T = warp_sum<long long>(v0 + v1);
+        const Whole v0 = cc[lane], v1 = cc[lane + 32];
+        const long long T = whole_sum<STAGED>(v0 + v1);
         if (T == 0) continue;
         used++;
-        const long long si = warp_sum<long long>(i0 * v0 + i1 * v1);
-        const long long sj = warp_sum<long long>(j0 * v0 + j1 * v1);
-        const long long sii = warp_sum<long long>(i0 * i0 * v0 + i1 * i1 * v1);
-        const long long sjj = warp_sum<long long>(j0 * j0 * v0 + j1 * j1 * v1);
-        const long long sij = warp_sum<long long>(i0 * j0 * v0 + i1 * j1 * v1);
-        const long long scon = warp_sum<long long>(d0 * v0 + d1 * v1);
-        const long long sene = warp_sum<long long>(v0 * v0 + v1 * v1);
-        const long long shom = warp_sum<long long>((HL / (1 + d0)) * v0 + (HL / (1 + d1)) * v1);
+        const long long si = whole_sum<STAGED>(i0 * v0 + i1 * v1);
+        const long long sj = whole_sum<STAGED>(j0 * v0 + j1 * v1);
+        const long long sii = whole_sum<STAGED>(i0 * i0 * v0 + i1 * i1 * v1);
+        const long long sjj = whole_sum<STAGED>(j0 * j0 * v0 + j1 * j1 * v1);
+        const long long sij = whole_sum<STAGED>(i0 * j0 * v0 + i1 * j1 * v1);
+        const long long scon = whole_sum<STAGED>(d0 * v0 + d1 * v1);
+        const long long sene = whole_sum<STAGED>(v0 * v0 + v1 * v1);
+        const long long shom = whole_sum<STAGED>((HL / (1 + d0)) * v0 + (HL / (1 + d1)) * v1);
         const float sent = warp_sum<float>(__fadd_rn(ent(v0, T), ent(v1, T)));
         const float Tf = (float)T;
         const long long vi = T * sii - si * si, vj = T * sjj - sj * sj, cv = T * sij - si * sj;
@@ -246,23 +283,21 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
         acc[4] = __fadd_rn(acc[4], (vi == 0 || vj == 0) ? 0.f
                                    : __fdiv_rn((float)cv, sqrtf(__fmul_rn((float)vi, (float)vj))));
     }
-    if (lane == 0) {
-        const double n = (double)N;
-        __int128 var_num = (__int128)N * Qsum - (__int128)Ssum * Ssum;
-        double f[NFEAT];
-        f[0] = n;
-        f[1] = (double)Per;
-        f[2] = (double)Ssum / n;
-        f[3] = sqrt((double)var_num) / n;
-        f[4] = Mn;
-        f[5] = Mx;
-        f[6] = (double)gm;
-        f[7] = sqrt(__ddiv_rn((double)gq, n));
-        f[8] = sqrt((double)Gmn);
-        f[9] = sqrt((double)Gmx);
-        for (int k = 0; k < 5; k++) f[10 + k] = used ? __fdiv_rn(acc[k], (float)used) : 0.f;
-        for (int k = 0; k < NFEAT; k++) out[k] = (float)f[k];
-    }
+    // one feature per lane: FP64 instructions cost the same for one lane as for
+    // all, so the divisions and roots of all features are taken together
+    const double n = (double)N;
+    const __int128 var_num = (__int128)N * Qsum - (__int128)Ssum * Ssum;
+    // sqrt(var) / n, sqrt(gq / n), sqrt(Gmn), sqrt(Gmx) on lanes 3, 7, 8, 9
+    const double num = lane == 2 ? (double)Ssum : lane == 3 ? (double)var_num : lane == 7 ? (double)gq : lane == 8 ? (double)Gmn : (double)Gmx;
+    const double quo = __ddiv_rn(num, n);  // lanes 2, 7
+    const double root = sqrt(lane == 7 ? quo : num);
+    const double rn = __ddiv_rn(root, n);
+    const int k = lane - 10;
+    const float a = k == 0 ? acc[0] : k == 1 ? acc[1] : k == 2 ? acc[2] : k == 3 ? acc[3] : acc[4];
+    const float tex = used ? __fdiv_rn(a, (float)used) : 0.f;
+    const float f = lane == 0 ? (float)n : lane == 1 ? (float)Per : lane == 2 ? (float)quo : lane == 3 ? (float)rn : lane == 4 ? (float)Mn
+                  : lane == 5 ? (float)Mx : lane == 6 ? gm : lane < 10 ? (float)root : tex;
+    if (lane < NFEAT) out[lane] = f;
     __syncwarp();
 }
 
@@ -276,7 +311,7 @@ __device__ __forceinline__ void object_features(const ObjJob& J, int obj, int* g
     const int4 box = J.bbox[obj];
     const int rx0 = max(box.x - 1, 0), ry0 = max(box.y - 1, 0);
     const long long rw = (long long)min(box.z + 1, J.W - 1) - rx0 + 1, rh = (long long)min(box.w + 1, J.H - 1) - ry0 + 1;
-    if (rw > 0 && rh > 0 && rw * rh <= STAGE_PX)
+    if (rw > 0 && rh > 0 && rw * rh <= REGION_PX && (rw * rh <= STAGE_PX || 3 * rw <= STAGE_PX))
         object_features_impl<true>(J, obj, glcm, spx);
     else
         object_features_global(J, obj, glcm);
@@ -290,7 +325,7 @@ struct ObjSmem {
     uint16_t px[STAGE_PX];  // hem8 | (in object) << 8
 };
 
-__global__ void __launch_bounds__(FW * 32) k_fobj_plain(ObjJob J, int K) {
+__global__ void __launch_bounds__(FW * 32, 8) k_fobj_plain(ObjJob J, int K) {
     __shared__ ObjSmem sm[FW];
     const int warp = threadIdx.x >> 5;
     ObjSmem& S = sm[warp];
@@ -316,7 +351,7 @@ __global__ void k_obj_prefix(Launch L) {
 
 // Batched form: the objects of all tiles, item -> (tile, object) through the
 // obj_base prefixes (the last tile whose base is <= item owns it).
-__global__ void __launch_bounds__(FW * 32) k_fobj_batched(Launch L) {
+__global__ void __launch_bounds__(FW * 32, 8) k_fobj_batched(Launch L) {
     if (L.early) after_previous();
     __shared__ ObjSmem sm[FW];
     const int warp = threadIdx.x >> 5;

@@ -4,6 +4,7 @@ relative or 1e-6 absolute of the FP64 oracle."""
 import numpy as np
 import pytest
 
+import oracle
 import synth
 from tests.gpu_util import assert_feats_close, assert_planes_equal, oracle_all, run_gpu
 
@@ -155,3 +156,25 @@ def test_distances_of_large_objects(W):
     if W >= 720:
         assert int(r["edt"].max()) > 128 * 128
     p.close()
+
+
+@pytest.mark.parametrize("bw,bh", [(62, 42), (63, 42), (54, 51), (78, 62), (79, 62), (936, 1), (937, 2), (1, 1200), (1, 1), (300, 15)])
+def test_features_at_the_stage_sizes(pipe, bw, bh):
+    """Objects whose box plus margin just fits the features' stage (2816
+    pixels), is staged in bands of rows (up to 5120), or is not staged: full
+    and ragged ones, inside the image and in its corners, under noise."""
+    import torch
+    rng = np.random.default_rng(bw * 1000 + bh)
+    W, H = 2 * bw + 12, 2 * bh + 12
+    hem8 = rng.integers(0, 256, (H, W)).astype(np.uint8)
+    labels = np.zeros((H, W), np.int32)
+    for k, (x, y) in enumerate(((0, 0), (W - bw, 0), (3, H - bh - 3), (W - bw, H - bh))):
+        m = rng.random((bh, bw)) < (1.0 if k % 2 else 0.6)
+        m[0, 0] = m[-1, -1] = True
+        labels[y:y + bh, x:x + bw][m] = k + 1
+    ref = oracle.features(hem8, labels, 4)
+    dev = torch.device("cuda", 0)
+    out = torch.zeros((4, 15), dtype=torch.float32, device=dev)
+    pipe.features_tile(torch.from_numpy(hem8).to(dev), torch.from_numpy(labels).to(dev), 4, out)
+    torch.cuda.synchronize()
+    assert_feats_close(out.cpu().numpy(), ref)
