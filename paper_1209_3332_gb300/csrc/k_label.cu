@@ -18,7 +18,7 @@
 //    instead of storing a full plane of provisional labels;
 //  * a warp's only large shared array is its 1024-entry union-find table
 //    (4 KB), whose root entries also carry a component's payload in bits
-//    16 and up, so that 14 CTAs of 4 warps fit on an SM.
+//    16 and up, so that 48 such warps fit on an SM.
 // Fill holes labels the background with 4-connectivity (dual of the 8-conn
 // foreground) and marks components that touch the image border; every
 // background pixel of an unmarked component is a hole.  Labelling then
@@ -29,6 +29,14 @@
 
 namespace nucseg {
 
+// Labelling blocks (one per warp) per CTA of the local passes.  A block without
+// foreground takes a fraction of the time of one with many runs, and a CTA keeps
+// its warps' places until its slowest is done, so that few warps per CTA keep
+// more places busy: with 4, 2 and 1 on 16 tiles of 4096^2, the fill takes 383, 327
+// and 287 us (32 CTAs per SM allow 64 registers then), the labelling 195, 168 and
+// 172, the relabelling 242, 208 and 211.  The merge and root passes, whose warps
+// are short, keep CCL_WARPS = 4 (label merge 67 us, with 2 82).
+constexpr int FILL_WARPS = 1, LOCAL_WARPS = 2;
 constexpr unsigned FULLM = 0xffffffffu;
 
 // ---- shared-memory union-find ---------------------------------------------------
@@ -284,12 +292,12 @@ __device__ __forceinline__ int register_roots(const TileDev& T, const WarpGeo& g
 
 
 // ---- K3a: foreground from the h-dome, background local components ---------------
-__global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_fill_local(Launch L) {
+__global__ void __launch_bounds__(FILL_WARPS * 32, 32 / FILL_WARPS) k_fill_local(Launch L) {
     if (L.early) after_previous();
-    __shared__ int par_sm[CCL_WARPS][CB * CB];
-    __shared__ uint32_t touch_sm[CCL_WARPS][32];
+    __shared__ int par_sm[FILL_WARPS][CB * CB];
+    __shared__ uint32_t touch_sm[FILL_WARPS][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gb = blockIdx.x * CCL_WARPS + warp;
+    const int gb = blockIdx.x * FILL_WARPS + warp;
     if (gb >= L.n_cb) return;
     const UF par{par_sm[warp]};
     uint32_t* touch = touch_sm[warp];
@@ -578,11 +586,11 @@ __global__ void __launch_bounds__(CCL_WARPS * 32) k_roots(Launch L, int per) {
 }
 
 // ---- K4a: holes -> filled; foreground local components ----------------------------
-__global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_label_local(Launch L) {
+__global__ void __launch_bounds__(LOCAL_WARPS * 32, 48 / LOCAL_WARPS) k_label_local(Launch L) {
     if (L.early) after_previous();
-    __shared__ int par_sm[CCL_WARPS][CB * CB];
+    __shared__ int par_sm[LOCAL_WARPS][CB * CB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gb = blockIdx.x * CCL_WARPS + warp;
+    const int gb = blockIdx.x * LOCAL_WARPS + warp;
     if (gb >= L.n_cb) return;
     const UF par{par_sm[warp]};
     const WarpGeo g = warp_geo(L, gb);
@@ -718,11 +726,11 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(Launch L) {
 // set; every run then takes its root's label from shared memory.  Each lane
 // writes its row of labels from registers, four labels per 16-byte store.
 constexpr int LAB_FLAG = (int)0x80000000u;
-__global__ void __launch_bounds__(CCL_WARPS * 32, 12) k_relabel(Launch L, int want_bbox) {
+__global__ void __launch_bounds__(LOCAL_WARPS * 32, 48 / LOCAL_WARPS) k_relabel(Launch L, int want_bbox) {
     if (L.early) after_previous();
-    __shared__ int par_sm[CCL_WARPS][CB * CB];
+    __shared__ int par_sm[LOCAL_WARPS][CB * CB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gb = blockIdx.x * CCL_WARPS + warp;
+    const int gb = blockIdx.x * LOCAL_WARPS + warp;
     if (gb >= L.n_cb) return;
     const UF par{par_sm[warp]};
     const WarpGeo g = warp_geo(L, gb);
@@ -907,7 +915,7 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
         pf->end("bbox_init", s);
     }
     pf->begin("fill_local", s);
-    launch_behind(L.early && pf->overlap(), k_fill_local, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_fill_local, (L.n_cb + FILL_WARPS - 1) / FILL_WARPS, FILL_WARPS * 32, 0, s, L);
     pf->end("fill_local", s);
     // Blocks per warp of the merge and root passes: as many as leave one wave of
     // resident warps, up to 8.  On 16 tiles of 4096^2 more blocks per warp mean
@@ -926,7 +934,7 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
     launch_behind(L.early && pf->overlap(), k_roots<1>, pg, pt, 0, s, L, per);
     pf->end("fill_roots_copy", s);
     pf->begin("label_local", s);
-    launch_behind(L.early && pf->overlap(), k_label_local, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_label_local, (L.n_cb + LOCAL_WARPS - 1) / LOCAL_WARPS, LOCAL_WARPS * 32, 0, s, L);
     pf->end("label_local", s);
     pf->begin("label_merge", s);
     // (a warp per block: edges with foreground are all walked, and 8 blocks per
@@ -949,7 +957,7 @@ void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cuda
     launch_behind(L.early && pf->overlap(), k_scan_chunks, L.n_chunks, SCAN_THREADS, 0, s, L, 1);
     pf->end("scan_words", s);
     pf->begin("relabel", s);
-    launch_behind(L.early && pf->overlap(), k_relabel, (L.n_cb + CCL_WARPS - 1) / CCL_WARPS, CCL_WARPS * 32, 0, s, L, want_bbox);
+    launch_behind(L.early && pf->overlap(), k_relabel, (L.n_cb + LOCAL_WARPS - 1) / LOCAL_WARPS, LOCAL_WARPS * 32, 0, s, L, want_bbox);
     pf->end("relabel", s);
 }
 
