@@ -241,14 +241,16 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_canny_nms(const __grid_con
 // bits under the disk's chord of each row pick the labels to look at.  Each
 // edge pixel adds one to every distinct object in its disk (the first four
 // remembered in registers, beyond that an object is new iff no earlier disk
-// offset holds it).  8 tiles of 4096^2: 223 us (465 with a CTA per block, a
-// thread per pixel and a label read for every disk offset; 246 with four label
-// loads of a lane in flight instead of seven).  Bound: the latency of the label
-// loads of the blocks that hold edges (about half), 24 warps per SM by shared
-// memory.
+// offset holds it).  8 tiles of 4096^2: 146 us (465 with a CTA per block, a
+// thread per pixel and a label read for every disk offset).  Bound: the latency
+// of the label loads of the blocks that hold edges (about half; seven of a lane
+// in flight), 24 warps per SM by shared memory.
 constexpr int CR_MAX = 4;                 // largest disk radius of the counts
 constexpr int CC_S = CT + 2 * CR_MAX;     // staged labels: the block and a CR_MAX-pixel margin (40 x 40)
-constexpr int CC_WARPS = 4;
+// Blocks (one per warp) per CTA: most blocks hold no edge pixel and end at once, and
+// a CTA keeps its warps' places until its slowest is done (8 tiles of 4096^2: 224
+// us with four, 170 with two, 146 with one).
+constexpr int CC_WARPS = 1;
 
 struct CountStage {
     int32_t lab[CC_S][CC_S];
