@@ -323,8 +323,7 @@ def morph_open_run(torch, pipe, stream, planes, steps, hbm_peak, want_cpu):
     """The opening by the 19x19 disk (Table I "Morph. Open") of every hem8
     plane of the batch through morph_open_tile, timed with CUDA events on the
     launching stream (planes larger than L2 in all).  The passes are bound by
-    instruction issue (ncu: issue active 66%, ALU and load/store pipes near
-    55%, DRAM 4%), so the roofline is the SMs' issue rate, against the warp
+    instruction issue (ncu: issue active 58%, ALU pipe 71%, DRAM 8%), so the roofline is the SMs' issue rate, against the warp
     instructions the committed ncu capture counted per plane."""
     outs = [torch.empty_like(p) for p in planes]
 
