@@ -148,7 +148,9 @@ typedef struct {
     float* feats; int feats_cap;
 } tile_dev;
 /* Launch shapes (the number of persistent reconstruction workers, the rows
- * one distance-transform block solves, the blocks of the feature pass)
+ * one distance-transform block solves, the blocks of the feature pass; where a
+ * batch has few work tiles for each worker and teams of warps take them, as
+ * large a share of all teams as the workers are of all workers)
  * never change a result.  With params.autotune set, the first call with a
  * new list of tile sizes synchronises `stream` and picks them by timing the
  * whole path on this batch (about 30 extra passes; the outputs are
