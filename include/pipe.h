@@ -345,7 +345,9 @@ int batch_release(pipe_t p, uint64_t ticket);
 /* ---- introspection used by tests and the benchmark ---------------------- */
 
 /* Synchronises the pipe's streams and returns (then clears) the device
- * status word: PIPE_OK or the first device-side error since the last read. */
+ * status word: PIPE_OK or the first device-side error since the last read,
+ * whatever calls have followed it.  Errors of the served form are in the
+ * tiles' results instead. */
 int pipe_status_read(pipe_t p);
 
 /* Copies an internal plane of the most recent seg_tile call into dst_dev

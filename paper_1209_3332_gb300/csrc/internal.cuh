@@ -71,7 +71,7 @@ struct Shared {
     alignas(256) int head;              // worklist head
     alignas(256) int next_obj;          // the batched feature pass draws its objects from this counter
     alignas(256) int nobj;              // object items of a batched feature pass
-    int err;                            // first device-side error
+    int err;                            // first error of this launch: ends its waits
     int processed;                      // tile processings (diagnostic)
 };
 
@@ -83,7 +83,7 @@ struct Launch {
     int* rt_src;           // [n_rt] work tiles holding a strong marker (queued first)
     Shared* sh;
     int* tile_status;      // [ntiles]
-    int* status;           // global status word
+    int* status;           // the pipe's status word (set_status); null for served groups, whose results carry theirs
     // totals (host-computed) for grid sizing
     int n_rt, n_cb, n_chunks, n_cols, n_rows, n_px;
     int early;             // each kernel is launched before the one ahead of it is complete (launch_behind)
@@ -104,8 +104,15 @@ __device__ __forceinline__ int find_tile(const TileDev* t, int n, int gid, int T
     return lo;
 }
 
+// The pipe's status word keeps the first error of any call until the host reads
+// it: no launch clears it.
 __device__ __forceinline__ void set_status(int* status, int code) {
-    atomicCAS(status, 0, code);
+    if (status) atomicCAS(status, 0, code);
+}
+// A wait of a launch whose error word is err ran out.
+__device__ __forceinline__ void wait_over(int* err, int* status) {
+    atomicCAS(err, 0, ST_TIMEOUT);
+    set_status(status, ST_TIMEOUT);
 }
 
 // 4 N consecutive bytes from p on, any alignment, from N + 1 aligned words; all
@@ -292,7 +299,7 @@ CannyTab make_canny_tab(const std::vector<CannyDesc>& v, CannyDesc* far, cudaStr
 // per work tile, and the state of its queue.
 struct GrowShared {  // the words that every worker's atomics meet at, in lines of their own
     unsigned long long tp;          // tail << 32 | groups not finished and tiles queued or running
-    int err;                        // first device-side error
+    int err;                        // first error of this launch: ends its waits
     alignas(256) int head;          // queue head
     alignas(256) int next;          // next group of tiles
 };
@@ -303,6 +310,7 @@ struct GrowLaunch {
     int* state;                         // [n_rt], zeroed
     uint8_t* any;                       // [n_rt] the work tile holds a marker pixel
     GrowShared* sh;
+    int* status;                        // the pipe's status word
     int n_rt;
     int group;                          // work tiles drawn at a time at the start, 1 to 32
     long long wait_budget;

@@ -341,7 +341,10 @@ __global__ void k_obj_prefix(Launch L) {
         TileDev& T = L.tiles[t];
         int K = *T.n_objects;
         int m = min(K, T.feats_cap);
-        if (K > T.feats_cap) L.tile_status[t] = ST_OVERFLOW;
+        if (K > T.feats_cap) {
+            L.tile_status[t] = ST_OVERFLOW;
+            set_status(L.status, ST_OVERFLOW);
+        }
         T.obj_base = run;
         run += m;
     }

@@ -43,7 +43,7 @@ __device__ void grow_put(const GrowLaunch& G, unsigned i, unsigned item) {
     u64* slot = G.slots + (i - lap * cap);
     const long long t0 = clock64();
     while ((unsigned)(vol64(slot) >> 32) != 2u * lap) {
-        if (clock64() - t0 > G.wait_budget) { atomicCAS(&G.sh->err, 0, ST_TIMEOUT); return; }
+        if (clock64() - t0 > G.wait_budget) { wait_over(&G.sh->err, G.status); return; }
         __nanosleep(32);
     }
     *(volatile u64*)slot = ((u64)(2u * lap + 1u) << 32) | item;
@@ -57,7 +57,7 @@ __device__ bool grow_want(const GrowLaunch& G, int t) {
         if (s == WL_QUEUED || s == WL_DIRTY) return false;
         if (atomicCAS(&G.state[t], WL_RUNNING, WL_DIRTY) == WL_RUNNING) return false;
     }
-    atomicCAS(&G.sh->err, 0, ST_TIMEOUT);
+    wait_over(&G.sh->err, G.status);
     return false;
 }
 
@@ -73,7 +73,7 @@ __device__ int grow_pop(const GrowLaunch& G) {
             return (int)(unsigned)v;
         }
         if ((unsigned)vol64(&G.sh->tp) == 0u || *(const volatile int*)&G.sh->err) return -1;
-        if (clock64() - t0 > G.wait_budget) { atomicCAS(&G.sh->err, 0, ST_TIMEOUT); return -1; }
+        if (clock64() - t0 > G.wait_budget) { wait_over(&G.sh->err, G.status); return -1; }
         __nanosleep(64);
     }
 }

@@ -178,7 +178,7 @@ __device__ void wl_put(const Launch& L, unsigned i, unsigned item) {
     unsigned long long* slot = L.wl_slots + i % cap;
     long long t0 = clock64();
     while ((unsigned)(ld_vol64(slot) >> 32) != i) {
-        if (budget_over(t0, L.wait_budget)) { atomicCAS(&L.sh->err, 0, ST_TIMEOUT); return; }
+        if (budget_over(t0, L.wait_budget)) { wait_over(&L.sh->err, L.status); return; }
         __nanosleep(32);
     }
     st_vol64(slot, ((unsigned long long)(i + 1) << 32) | item);
@@ -192,7 +192,7 @@ __device__ bool wl_want(const Launch& L, int t) {
         if (s == WL_QUEUED || s == WL_DIRTY) return false;
         if (atomicCAS(&L.wl_state[t], WL_RUNNING, WL_DIRTY) == WL_RUNNING) return false;
     }
-    atomicCAS(&L.sh->err, 0, ST_TIMEOUT);
+    wait_over(&L.sh->err, L.status);
     return false;
 }
 
@@ -210,7 +210,7 @@ __device__ bool wl_pop(const Launch& L, unsigned* item) {
             return true;
         }
         if ((unsigned)ld_vol64(&L.sh->tp) == 0u || ld_vol(&L.sh->err)) return false;
-        if (budget_over(t0, L.wait_budget)) { atomicCAS(&L.sh->err, 0, ST_TIMEOUT); return false; }
+        if (budget_over(t0, L.wait_budget)) { wait_over(&L.sh->err, L.status); return false; }
         __nanosleep(64);
     }
 }

@@ -255,7 +255,7 @@ __global__ void k_set_desc(TileDev* dst, DescPack p) {
 
 // Everything one launch sequence needs besides the descriptors.
 struct LaunchCtx {
-    DevBuf tiles, wl, shared;  // TileDev[], slots+state, Shared + statuses
+    DevBuf tiles, wl, shared;  // TileDev[], slots+state, Shared + tile statuses
     DevBuf arena;
     int ntiles_cap = 0;
 };
@@ -304,6 +304,7 @@ struct pipe_s {
     int sms = 0;
     int recon_cap = 1, recon_teams = 1;  // resident workers of the reconstruction: warps, teams
     EventProfiler prof;
+    DevBuf status;      // the first device-side error since pipe_status_read
     // plain form
     LaunchCtx plain;
     TileDev last_plain{};
@@ -312,7 +313,6 @@ struct pipe_s {
     DevBuf morph_tmp;  // scratch plane of morph_open_tile
     DevBuf ws_obj;      // watershed_tile: per-object boxes and basin counts
     DevBuf ws_scratch;  // watershed_tile: planes for boxes larger than the shared-memory stage
-    DevBuf ws_status;   // watershed_tile: device status word
     DevBuf ws_desc;     // watershed_batch: tile descriptors
     cudaStream_t ws_side = nullptr;        // watershed_tile: large boxes overlap the small ones here
     DevBuf grow;        // rbc_tile, canny_tile, canny_batch: bit planes and queue of the growth
@@ -322,7 +322,6 @@ struct pipe_s {
     // batched form
     LaunchCtx batch;
     GraphCache graphs;
-    int batch_ntiles = 0;
     // served form
     std::mutex mu;
     std::vector<std::unique_ptr<Ctx>> ctxs;
@@ -347,12 +346,14 @@ namespace {
 // Reconstruction queue per launch: a 64-bit slot, a state word and a source
 // flag per work tile.
 size_t wl_bytes(int n_rt) { return sizeof(int) * 4 * (size_t)std::max(n_rt, 1); }
+size_t tiles_bytes(int n) { return sizeof(TileDev) * (size_t)std::max(n, 1); }
+size_t shared_bytes(int n) { return sizeof(Shared) + sizeof(int) * (size_t)std::max(n, 1); }
 
 int ensure_ctx(LaunchCtx& c, int ntiles, int n_rt, size_t arena_bytes) {
     int rc;
-    if ((rc = c.tiles.ensure(sizeof(TileDev) * std::max(ntiles, 1)))) return rc;
+    if ((rc = c.tiles.ensure(tiles_bytes(ntiles)))) return rc;
     if ((rc = c.wl.ensure(wl_bytes(n_rt)))) return rc;
-    if ((rc = c.shared.ensure(sizeof(Shared) + sizeof(int) * (2 + std::max(ntiles, 1))))) return rc;
+    if ((rc = c.shared.ensure(shared_bytes(ntiles)))) return rc;
     if ((rc = c.arena.ensure(std::max(arena_bytes, (size_t)256)))) return rc;
     return PIPE_OK;
 }
@@ -362,8 +363,6 @@ int ensure_ctx(LaunchCtx& c, int ntiles, int n_rt, size_t arena_bytes) {
 // ws: workspace arena, n_rt: reconstruction work tiles).  ensure() only
 // grows a buffer, so each part becomes the larger of the two.
 
-size_t tiles_bytes(int n) { return sizeof(TileDev) * (size_t)std::max(n, 1); }
-size_t shared_bytes(int n) { return sizeof(Shared) + sizeof(int) * (2 + (size_t)std::max(n, 1)); }
 size_t ctx_need(size_t io, size_t ws, int n, int n_rt) {
     return io + std::max(ws, (size_t)256) + tiles_bytes(n) + wl_bytes(n_rt) + shared_bytes(n);
 }
@@ -396,8 +395,15 @@ size_t serve_allocated(pipe_t p) {
     return s;
 }
 
-// Fill launch-wide bases of the descriptors and the Launch totals.
-Launch make_launch(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt_total, int RB) {
+// done when it returns: a stream that does not wait for the default one may be next
+cudaError_t zero_status(pipe_t p) {
+    const cudaError_t e = cudaMemset(p->status.p, 0, sizeof(int));
+    return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
+}
+
+// Fill launch-wide bases of the descriptors and the Launch totals.  status:
+// where errors are kept beyond the launch, or null.
+Launch make_launch(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt_total, int RB, int* status) {
     Launch L{};
     L.tiles = (TileDev*)c.tiles.p;
     L.ntiles = (int)td.size();
@@ -405,8 +411,8 @@ Launch make_launch(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt_to
     L.wl_state = (int*)c.wl.p + 2 * std::max(n_rt_total, 1);
     L.rt_src = L.wl_state + std::max(n_rt_total, 1);
     L.sh = (Shared*)c.shared.p;
-    L.status = (int*)((char*)c.shared.p + sizeof(Shared));
-    L.tile_status = L.status + 2;
+    L.tile_status = (int*)((char*)c.shared.p + sizeof(Shared));
+    L.status = status;
     int rt = 0, cb = 0, ch = 0, col = 0, row = 0, px = 0;
     for (auto& t : td) {
         t.rt_base = rt;
@@ -471,6 +477,7 @@ int make_grow(pipe_t p, const std::vector<CannyDesc>& cd, int n_rt, cudaStream_t
     out->slots = (unsigned long long*)b;
     out->state = (int*)(b + (size_t)n_rt * 8);
     out->any = (uint8_t*)(b + al256(queue));
+    out->status = (int*)p->status.p;
     out->n_rt = n_rt;
     out->group = grow_group(n_rt);
     out->wait_budget = p->prm.wait_budget_cycles;
@@ -580,7 +587,7 @@ int autotune(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt, int Wma
     cp.counter = &p->prof.launches;
     int rc = PIPE_OK;
     auto timeit = [&](const Tune& tu, float* ms) -> int {
-        Launch L = make_launch(p, c, td, n_rt, tu.edt_rb);
+        Launch L = make_launch(p, c, td, n_rt, tu.edt_rb, (int*)p->status.p);
         int r = upload_desc(L, td, s);
         if (r) return r;
         float b = 1e30f;
@@ -724,6 +731,11 @@ int pipe_create(const pipe_params* params, int device, pipe_t* out) {
     p->device = device;
     p->prm = prm;
     cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, device);
+    if (p->status.ensure(sizeof(int)) != PIPE_OK) {
+        delete p;
+        return PIPE_ENOMEM;
+    }
+    zero_status(p);
     int32_t lut[256], wq[3];
     deconv_tables(lut, wq);
     upload_deconv_tables(lut, wq);
@@ -734,6 +746,7 @@ int pipe_create(const pipe_params* params, int device, pipe_t* out) {
         load_tune_file(p);
     }
     if (cudaGetLastError() != cudaSuccess) {
+        p->status.release();
         delete p;
         return PIPE_ECUDA;
     }
@@ -755,7 +768,7 @@ void pipe_destroy(pipe_t p) {
     p->grow.release();
     p->canny_desc.release();
     p->ws_scratch.release();
-    p->ws_status.release();
+    p->status.release();
     p->ws_desc.release();
     if (p->ws_side) cudaStreamDestroy(p->ws_side);
     if (p->ws_fork) cudaEventDestroy(p->ws_fork);
@@ -799,7 +812,7 @@ int seg_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
     t.n_objects = n_objects_dev;
     t.feats = nullptr;
     const Tune tu = default_tune(p, W);
-    Launch L = make_launch(p, p->plain, td, n_rt, tu.edt_rb);
+    Launch L = make_launch(p, p->plain, td, n_rt, tu.edt_rb, (int*)p->status.p);
     L.early = 1;
     if ((rc = upload_desc(L, td, s))) return rc;
     run_path(p, L, W, false, 0, tu, s, &p->prof);
@@ -889,16 +902,12 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
     const size_t need_obj = std::max(objs, (size_t)1) * (sizeof(int4) + 2 * sizeof(int)) + WS_COUNTERS * sizeof(int);
     const size_t need_scr = px * (sizeof(unsigned long long) + sizeof(uint16_t));
     const size_t need_desc = sizeof(WsDesc) * (size_t)n;
-    if (p->ws_obj.n < need_obj || p->ws_scratch.n < need_scr || p->ws_desc.n < need_desc || !p->ws_status.p) {
+    if (p->ws_obj.n < need_obj || p->ws_scratch.n < need_scr || p->ws_desc.n < need_desc) {
         CK(cudaStreamSynchronize(s));
         int rc;
         if ((rc = p->ws_obj.ensure(need_obj)) || (rc = p->ws_scratch.ensure(need_scr)) ||
             (rc = p->ws_desc.ensure(need_desc)))
             return rc;
-        if (!p->ws_status.p) {
-            if ((rc = p->ws_status.ensure(sizeof(int)))) return rc;
-            CK(cudaMemset(p->ws_status.p, 0, sizeof(int)));
-        }
     }
     if (!p->ws_side) {
         int lo_pri = 0, hi_pri = 0;  // the large boxes go first when SM room frees up
@@ -910,7 +919,7 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
     int4* bbox = (int4*)p->ws_obj.p;
     int* cnt = (int*)(bbox + std::max(objs, (size_t)1));
     int* next = cnt + std::max(objs, (size_t)1);
-    launch_watershed_batch(d, (WsDesc*)p->ws_desc.p, h, bbox, cnt, next, p->ws_scratch.p, px, (int*)p->ws_status.p, p->sms,
+    launch_watershed_batch(d, (WsDesc*)p->ws_desc.p, h, bbox, cnt, next, p->ws_scratch.p, px, (int*)p->status.p, p->sms,
                            s, p->ws_side, p->ws_fork, p->ws_join, &p->prof);
     CK(cudaGetLastError());
     return PIPE_OK;
@@ -1032,7 +1041,7 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
                std::to_string(tiles[i].feats_cap) + (tiles[i].edt ? "e" : "n") + ";";
     }
     bool grow = p->batch.arena.n < total || p->batch.wl.n < wl_bytes(n_rt) ||
-                p->batch.tiles.n < sizeof(TileDev) * n || p->batch.shared.n < sizeof(Shared) + sizeof(int) * (2 + n);
+                p->batch.tiles.n < tiles_bytes(n) || p->batch.shared.n < shared_bytes(n);
     if (grow) {
         CK(cudaStreamSynchronize(s));
         clear_graphs(p->graphs);
@@ -1055,7 +1064,6 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
         t.feats = tiles[i].feats;
         max_obj = std::max(max_obj, t.feats_cap);
     }
-    p->batch_ntiles = n;
     int rc;
     Tune tu = default_tune(p, Wmax);
     {
@@ -1070,7 +1078,7 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
         }
     }
     p->last_tune = tu;
-    Launch L = make_launch(p, p->batch, td, n_rt, tu.edt_rb);
+    Launch L = make_launch(p, p->batch, td, n_rt, tu.edt_rb, (int*)p->status.p);
     if ((rc = upload_desc(L, td, s))) return rc;
     if (p->prof.enabled) {
         // profiled runs launch eagerly so that each kernel is bracketed by events
@@ -1087,36 +1095,8 @@ int pipe_status_read(pipe_t p) {
     CK(cudaSetDevice(p->device));
     CK(cudaDeviceSynchronize());
     int result = PIPE_OK;
-    auto check = [&](LaunchCtx& c, int ntiles) {
-        if (!c.shared.p) return;
-        Shared sh;
-        if (cudaMemcpy(&sh, c.shared.p, sizeof(sh), cudaMemcpyDeviceToHost) != cudaSuccess) {
-            result = PIPE_ECUDA;
-            return;
-        }
-        if (sh.err && result == PIPE_OK) result = sh.err;
-        std::vector<int> st(2 + ntiles);
-        cudaMemcpy(st.data(), (char*)c.shared.p + sizeof(Shared), sizeof(int) * st.size(), cudaMemcpyDeviceToHost);
-        for (int i = 2; i < (int)st.size(); i++)
-            if (st[i] && result == PIPE_OK) result = st[i];
-        int zero = 0;
-        cudaMemcpy((char*)c.shared.p + offsetof(Shared, err), &zero, sizeof(int), cudaMemcpyHostToDevice);
-        cudaMemset((char*)c.shared.p + sizeof(Shared), 0, sizeof(int) * st.size());
-    };
-    check(p->plain, 1);
-    check(p->batch, p->batch_ntiles);
-    if (p->grow.p) {
-        GrowShared sh;
-        if (cudaMemcpy(&sh, p->grow.p, sizeof(sh), cudaMemcpyDeviceToHost) != cudaSuccess) return PIPE_ECUDA;
-        if (sh.err && result == PIPE_OK) result = sh.err;
-        cudaMemset((char*)p->grow.p + offsetof(GrowShared, err), 0, sizeof(int));
-    }
-    if (p->ws_status.p) {
-        int st = 0;
-        if (cudaMemcpy(&st, p->ws_status.p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return PIPE_ECUDA;
-        if (st && result == PIPE_OK) result = st;
-        cudaMemset(p->ws_status.p, 0, sizeof(int));
-    }
+    CK(cudaMemcpy(&result, p->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(zero_status(p));
     return result;
 }
 
@@ -1371,7 +1351,7 @@ int batch_submit(pipe_t p, const tile_desc* tiles, int n, uint64_t* ticket) {
         auto it = p->tuned.find(tune_key(p, geos));
         if (it != p->tuned.end() && tune_ok(p, it->second, Wmax)) tu = it->second;
     }
-    Launch L = make_launch(p, c.lc, td, n_rt, tu.edt_rb);
+    Launch L = make_launch(p, c.lc, td, n_rt, tu.edt_rb, nullptr);
     if ((rc = upload_desc(L, td, cs))) return rc;
     {
         std::string key;
