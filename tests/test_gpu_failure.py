@@ -135,3 +135,36 @@ def test_status_outlives_the_calls_behind(late, then):
     small()
     assert pipe.status() == P.PIPE_OK
     pipe.close()
+
+
+@pytest.mark.parametrize("form", ["teams", "warps", "canny", "rbc"])
+def test_wait_budget_exhaustion_of_every_queue(form):
+    """Both kernels of the reconstruction -- teams of warps take a launch of
+    less than two work tiles per resident warp, single warps the larger ones --
+    and the growth under Canny and red blood cells."""
+    import oracle
+    import paper_1209_3332_gb300 as P
+    tight, normal = P.Pipe(0, autotune=0, wait_budget_cycles=300), P.Pipe(0, autotune=0)
+    tile = synth.tile(512, 512, 62, n_nuclei=60, frac_cluster=0.2)  # 64 work tiles
+    if form in ("teams", "warps"):
+        Calls(normal).batch([tile], 200)
+        warps = normal.autotune_info()["recon_workers"]
+        n = -(-2 * warps // 64) - (form == "teams")  # 2 * warps work tiles, or just fewer
+        Calls(tight).batch([tile] * n, 200)
+    elif form == "canny":
+        Calls(tight).canny(spiral(768))
+    else:
+        Calls(tight).rbc(snake_rgb(768))
+    assert tight.status() == P.PIPE_ETIMEOUT
+    assert tight.status() == P.PIPE_OK
+    tight.close()
+    if form == "canny":
+        assert np.array_equal(Calls(normal).canny(spiral(768)).cpu().numpy(), oracle.canny(spiral(768)))
+    elif form == "rbc":
+        assert np.array_equal(Calls(normal).rbc(snake_rgb(768)).cpu().numpy(), oracle.rbc(snake_rgb(768)))
+    else:
+        want = oracle_all(tile)
+        for t in Calls(normal).batch([tile] * n, 200):
+            assert np.array_equal(t["labels"].cpu().numpy(), want["labels"])
+    assert normal.status() == P.PIPE_OK
+    normal.close()
