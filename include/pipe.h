@@ -169,7 +169,9 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
  * in-image pixels only.
  *  src_dev, dst_dev: W x H uint8 planes, row pitch W, caller-owned device
  *    memory; they must not overlap.
- *  0 <= radius <= 15; W, H as for seg_tile.
+ *  0 <= radius <= 15; W, H as for seg_tile.  The pipe owns the scratch (two
+ *  planes with padded rows), allocated on the first call of more pixels,
+ *  which synchronises `stream`.
  * Returns PIPE_EINVAL on a bad argument (nothing is launched); otherwise
  * the work is asynchronous on `stream`. */
 int morph_open_tile(pipe_t p, const uint8_t* src_dev, int W, int H, int radius, uint8_t* dst_dev,

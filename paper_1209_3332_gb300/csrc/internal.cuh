@@ -17,6 +17,7 @@ constexpr int CB_THREADS = 256;
 constexpr int CCL_WARPS = 4;      // labelling blocks (one per warp) per CTA
 constexpr int RL_CAP = 512;       // root-list slots per labelling block
 constexpr int NFEAT = 15;
+constexpr int MAX_SIDE = 16384;   // largest width and height of an image
 constexpr int MORPH_RMAX = 15;   // largest disk radius of the opening (chords of up to 31 pixels)
 
 // worklist tile states
@@ -255,7 +256,14 @@ size_t edt_rows_smem(int RB, int Wmax);
 void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf);
 // The opening (1 <= r <= MORPH_RMAX in two passes through tmp, morph_scratch bytes).
 inline int morph_pitch(int W) { return (W + 15) & ~15; }  // rows of its scratch planes
-size_t morph_scratch(const uint8_t* src, int W, int H);
+// The scratch of any plane of up to `px` pixels, whatever its shape and alignment, so
+// that a call allocates only where it has more pixels than every one before: two
+// planes of padded rows, which are at most W + W / 16 bytes from W = 240 on, and 240
+// bytes below.
+inline size_t morph_scratch(size_t px) {
+    const size_t narrow = (size_t)240 * MAX_SIDE, plane = px + px / 16 > narrow ? px + px / 16 : narrow;
+    return 2 * ((plane + 255) & ~(size_t)255);
+}
 void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, int H, int r, int sms, cudaStream_t s,
                        Profiler* pf);
 void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, int H, int K, float* feats,

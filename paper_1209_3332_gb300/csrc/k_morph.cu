@@ -62,11 +62,6 @@ static MorphPass pass_of(int r) {
 
 static bool morph_direct(const uint8_t* src, int W) { return ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)W) & 3) == 0; }
 
-size_t morph_scratch(const uint8_t* src, int W, int H) {
-    const size_t plane = ((size_t)morph_pitch(W) * H + 255) & ~(size_t)255;
-    return morph_direct(src, W) ? plane : 2 * plane;
-}
-
 void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, int H, int r, int sms, cudaStream_t s,
                        Profiler* pf) {
     if (r == 0) {  // the disk is one pixel

@@ -310,7 +310,7 @@ struct pipe_s {
     TileDev last_plain{};
     bool have_last = false;
     DevBuf fbbox;
-    DevBuf morph_tmp;  // scratch plane of morph_open_tile
+    DevBuf morph_tmp;  // scratch planes of morph_open_tile
     DevBuf ws_obj;      // watershed_tile: per-object boxes and basin counts
     DevBuf ws_scratch;  // watershed_tile: planes for boxes larger than the shared-memory stage
     DevBuf ws_desc;     // watershed_batch: tile descriptors
@@ -648,7 +648,7 @@ done:
     return rc;
 }
 
-bool valid_size(int W, int H) { return W >= 1 && H >= 1 && W <= 16384 && H <= 16384; }
+bool valid_size(int W, int H) { return W >= 1 && H >= 1 && W <= MAX_SIDE && H <= MAX_SIDE; }
 
 // where one tile's results go in mapped host memory
 struct ResultSlot {
@@ -849,7 +849,7 @@ int morph_open_tile(pipe_t p, const uint8_t* src_dev, int W, int H, int radius, 
     if (src_dev < dst_dev + N && dst_dev < src_dev + N) return PIPE_EINVAL;  // the planes overlap
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(p->device));
-    const size_t need = morph_scratch(src_dev, W, H);
+    const size_t need = morph_scratch(N);
     if (p->morph_tmp.n < need) {  // the scratch planes grow to the largest call seen
         CK(cudaStreamSynchronize(s));
         const int rc = p->morph_tmp.ensure(need);

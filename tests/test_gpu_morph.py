@@ -95,3 +95,27 @@ def test_every_radius(pipe, W, H, off, r):
     torch.cuda.synchronize()
     assert np.array_equal(dst.cpu().numpy(), oracle.morph_open(a, r))
     assert bool((buf[1, :off] == 7).all()) and bool((buf[1, off + H * W:] == 7).all())
+
+
+@pytest.mark.parametrize("W,H,off", [(256, 256, 1), (255, 256, 0), (253, 251, 3), (300, 218, 0), (3, 16384, 1)])
+def test_captured_after_a_larger_plane(pipe, W, H, off):
+    """The scratch that a plane leaves serves any other of no more pixels, whatever
+    its shape and where its rows start: such a call does not allocate, so that it
+    can be captured."""
+    import torch
+    import paper_1209_3332_gb300 as P
+    p = P.Pipe(0)
+    big = torch.zeros((256, 256), dtype=torch.uint8, device="cuda")
+    p.morph_open(big, torch.empty_like(big), radius=4)
+    a = np.random.default_rng(W + H).integers(0, 256, (H, W), dtype=np.uint8)
+    buf = torch.zeros((2, 256 * 256 + 8), dtype=torch.uint8, device="cuda")
+    src, dst = (buf[i, off:off + H * W].view(H, W) for i in range(2))
+    src.copy_(torch.from_numpy(a))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.morph_open(src, dst, radius=4, stream=torch.cuda.current_stream())
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(dst.cpu().numpy(), oracle.morph_open(a, 4))
+    p.close()
