@@ -245,8 +245,8 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
  *  W x H uint8 plane, caller-owned, not overlapping the input;
  *  0 <= t_lo <= t_hi <= 255 (the workload uses 40 and 100).  The pipe owns
  *  the scratch (marker and mask as bit planes and a queue of 64x64 work
- *  tiles, shared with the Canny calls), allocated on the first call of a
- *  larger size, which synchronises `stream`.
+ *  tiles), allocated on the first call of a larger size, which synchronises
+ *  `stream`.
  * Returns PIPE_EINVAL on a bad argument (nothing is launched); otherwise
  * the work is asynchronous on `stream`. */
 int rbc_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes, int t_lo, int t_hi,

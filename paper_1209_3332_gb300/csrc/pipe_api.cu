@@ -315,7 +315,9 @@ struct pipe_s {
     DevBuf ws_scratch;  // watershed_tile: planes for boxes larger than the shared-memory stage
     DevBuf ws_desc;     // watershed_batch: tile descriptors
     cudaStream_t ws_side = nullptr;        // watershed_tile: large boxes overlap the small ones here
-    DevBuf grow;        // rbc_tile, canny_tile, canny_batch: bit planes and queue of the growth
+    // bit planes and queue of the growth: one for each of the two, so that a larger
+    // call of the one leaves what a captured call of the other uses
+    DevBuf rbc_grow, canny_grow;
     DevBuf canny_desc;  // canny_batch: tile descriptors
     int grow_cap = 1;   // resident CTAs of the growth
     cudaEvent_t ws_fork = nullptr, ws_join = nullptr;
@@ -457,18 +459,18 @@ int upload_desc(const Launch& L, const std::vector<TileDev>& td, cudaStream_t s)
 }
 
 // The growth of binary markers over the tiles of cd, n_rt work tiles in all:
-// bit planes, queue and descriptors (a larger call than any before grows them,
-// which synchronises s).
-int make_grow(pipe_t p, const std::vector<CannyDesc>& cd, int n_rt, cudaStream_t s, GrowLaunch* out) {
+// bit planes and queue in `scratch`, and descriptors (a larger call than any
+// before grows them, which synchronises s).
+int make_grow(pipe_t p, DevBuf& scratch, const std::vector<CannyDesc>& cd, int n_rt, cudaStream_t s, GrowLaunch* out) {
     const size_t plane = al256((size_t)n_rt * RT * 8), queue = (size_t)n_rt * 12;
     const size_t need = al256(sizeof(GrowShared)) + 2 * plane + al256(queue) + al256((size_t)n_rt);
     const size_t desc = cd.size() > CannyTab::NEAR ? sizeof(CannyDesc) * cd.size() : 0;
-    if (p->grow.n < need || p->canny_desc.n < desc) {
+    if (scratch.n < need || p->canny_desc.n < desc) {
         CK(cudaStreamSynchronize(s));
         int rc;
-        if ((rc = p->grow.ensure(need)) || (rc = p->canny_desc.ensure(desc))) return rc;
+        if ((rc = scratch.ensure(need)) || (rc = p->canny_desc.ensure(desc))) return rc;
     }
-    char* b = (char*)p->grow.p;
+    char* b = (char*)scratch.p;
     out->sh = (GrowShared*)b;
     b += al256(sizeof(GrowShared));
     out->mask = (unsigned long long*)b;
@@ -765,7 +767,8 @@ void pipe_destroy(pipe_t p) {
     p->fbbox.release();
     p->morph_tmp.release();
     p->ws_obj.release();
-    p->grow.release();
+    p->rbc_grow.release();
+    p->canny_grow.release();
     p->canny_desc.release();
     p->ws_scratch.release();
     p->status.release();
@@ -940,7 +943,7 @@ int rbc_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
     cd[0].H = H;
     cd[0].edges = out_dev;
     GrowLaunch G;
-    const int rc = make_grow(p, cd, ((W + RT - 1) / RT) * ((H + RT - 1) / RT), s, &G);
+    const int rc = make_grow(p, p->rbc_grow, cd, ((W + RT - 1) / RT) * ((H + RT - 1) / RT), s, &G);
     if (rc) return rc;
     // red dominance into the marker and the mask, then the growth of the marker
     launch_rbc_planes(G, rgb_dev, pitch_bytes, t_lo, t_hi, s, &p->prof);
@@ -977,7 +980,7 @@ int canny_run(pipe_t p, const edge_tile* tiles, int n, int low, int high, int ra
         counts |= t.n_objects > 0;
     }
     GrowLaunch G;
-    const int rc = make_grow(p, cd, rt, s, &G);
+    const int rc = make_grow(p, p->canny_grow, cd, rt, s, &G);
     if (rc) return rc;
     // 1. gradient and non-maximum suppression: strong pixels and candidates; counts zeroed
     launch_canny_nms(G, nw, low, high, s, &p->prof);

@@ -211,3 +211,44 @@ def test_growth_draws_of_several_tiles(pipe, W, H):
     rng = np.random.default_rng(W)
     img = np.kron(rng.integers(0, 256, ((H + 15) // 16, (W + 15) // 16), dtype=np.uint8), np.ones((16, 16), np.uint8))[:H, :W]
     check(pipe, img)
+
+
+@pytest.mark.parametrize("first", ["canny", "rbc"])
+def test_captured_call_outlives_the_other_kind(first):
+    """A captured Canny call replays after a red blood cell call on a larger
+    plane has allocated its scratch, and the other way round."""
+    import torch
+    import paper_1209_3332_gb300 as P
+    p = P.Pipe(0)
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(17)
+
+    def kron(n, c):
+        return np.kron(rng.integers(0, 256, (n, n, c), dtype=np.uint8), np.ones((9, 9, 1), np.uint8))
+
+    def call(kind, a, capture=False):
+        src = torch.from_numpy(np.ascontiguousarray(a)).to(dev)
+        out = torch.full(a.shape[:2], 7, dtype=torch.uint8, device=dev)
+        run = p.canny if kind == "canny" else p.rbc
+        run(src, out)  # the scratch grows here
+        torch.cuda.synchronize()
+        if not capture:
+            return src, out, None
+        out.fill_(7)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            run(src, out, stream=torch.cuda.current_stream())
+        return src, out, g
+
+    ref = dict(canny=lambda a: oracle.canny(a), rbc=lambda a: oracle.rbc(a))
+    other = "rbc" if first == "canny" else "canny"
+    small, large = (kron(n, 3) for n in (30, 120))
+    small, large = (small[..., 0], large) if first == "canny" else (small, large[..., 0])
+    _, out, g = call(first, small, capture=True)
+    _, out2, _ = call(other, large)
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy(), ref[first](small))
+    assert np.array_equal(out2.cpu().numpy(), ref[other](large))
+    p.close()
