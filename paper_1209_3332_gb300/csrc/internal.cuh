@@ -18,6 +18,7 @@ constexpr int CCL_WARPS = 4;      // labelling blocks (one per warp) per CTA
 constexpr int RL_CAP = 512;       // root-list slots per labelling block
 constexpr int NFEAT = 15;
 constexpr int MAX_SIDE = 16384;   // largest width and height of an image
+constexpr int MAX_TILES = 4096;   // tiles of a batched call
 constexpr int MORPH_RMAX = 15;   // largest disk radius of the opening (chords of up to 31 pixels)
 
 // worklist tile states

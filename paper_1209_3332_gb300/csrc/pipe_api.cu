@@ -870,7 +870,7 @@ int watershed_tile(pipe_t p, const int32_t* labels_dev, const int32_t* edt_dev, 
 }
 
 int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t stream) {
-    if (!p || !tiles || n < 1 || n > 4096 || h < 0 || h > 255) return PIPE_EINVAL;
+    if (!p || !tiles || n < 1 || n > MAX_TILES || h < 0 || h > 255) return PIPE_EINVAL;
     std::vector<WsDesc> d(n);
     size_t objs = 0, px = 0;
     for (int i = 0; i < n; i++) {
@@ -904,7 +904,8 @@ int watershed_batch(pipe_t p, const ws_tile* tiles, int n, int h, pipe_stream_t 
     CK(cudaSetDevice(p->device));
     const size_t need_obj = std::max(objs, (size_t)1) * (sizeof(int4) + 2 * sizeof(int)) + WS_COUNTERS * sizeof(int);
     const size_t need_scr = px * (sizeof(unsigned long long) + sizeof(uint16_t));
-    const size_t need_desc = sizeof(WsDesc) * (size_t)n;
+    // for any number of tiles: a captured call of few tiles outlives one of many
+    const size_t need_desc = sizeof(WsDesc) * MAX_TILES;
     if (p->ws_obj.n < need_obj || p->ws_scratch.n < need_scr || p->ws_desc.n < need_desc) {
         CK(cudaStreamSynchronize(s));
         int rc;
@@ -1011,7 +1012,7 @@ int canny_tile(pipe_t p, const uint8_t* img_dev, const int32_t* labels_dev, int 
 }
 
 int canny_batch(pipe_t p, const edge_tile* tiles, int n, int low, int high, int radius, pipe_stream_t stream) {
-    if (!p || !tiles || n < 1 || n > 4096 || low < 0 || high < low || radius < 0 || radius > 4) return PIPE_EINVAL;
+    if (!p || !tiles || n < 1 || n > MAX_TILES || low < 0 || high < low || radius < 0 || radius > 4) return PIPE_EINVAL;
     for (int i = 0; i < n; i++)
         if (!canny_args_ok(tiles[i])) return PIPE_EINVAL;
     CK(cudaSetDevice(p->device));
@@ -1019,7 +1020,7 @@ int canny_batch(pipe_t p, const edge_tile* tiles, int n, int low, int high, int 
 }
 
 int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t stream) {
-    if (!p || !tiles || n < 1 || n > 4096) return PIPE_EINVAL;
+    if (!p || !tiles || n < 1 || n > MAX_TILES) return PIPE_EINVAL;
     for (int i = 0; i < n; i++) {
         const tile_dev& d = tiles[i];
         if (!d.rgb || !d.hem8 || !d.labels || !d.n_objects || !valid_size(d.W, d.H) || d.pitch < (size_t)d.W * 3 ||

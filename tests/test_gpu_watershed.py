@@ -231,3 +231,34 @@ def test_boxes_at_the_stage_sizes(pipe, bw, bh, h):
     yy, xx = np.mgrid[0:lab.shape[0], 0:lab.shape[1]]
     lab[(np.hypot(xx - (2 * bw + 25), yy - 12) <= 7)] = 3
     check(pipe, lab, h=h, K=3)
+
+
+def test_captured_tile_outlives_a_batch():
+    """A captured call of one tile replays after a batch of more, smaller
+    tiles on the same pipe."""
+    import torch
+    import paper_1209_3332_gb300 as P
+    p = P.Pipe(0)
+    dev = torch.device("cuda", 0)
+    lab = lab_of(discs(200, 300, [(30 + 45 * j, 30 + 34 * i) for i in range(8) for j in range(4)], 11))
+    K = int(lab.max())
+    L = torch.from_numpy(np.ascontiguousarray(lab, np.int32)).to(dev)
+    E = torch.from_numpy(oracle.edt(lab)).to(dev)
+    out, n = torch.full_like(L, -7), torch.full((1,), -7, dtype=torch.int32, device=dev)
+    p.watershed(L, E, K, out, n)  # the scratch grows here
+    torch.cuda.synchronize()
+    out.fill_(-7)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.watershed(L, E, K, out, n, stream=torch.cuda.current_stream())
+    small = lab_of(discs(20, 20, [(9, 9)], 6))
+    want, wn = oracle.watershed(small, oracle.edt(small), 1)
+    for got, gn in _ws_batch(p, [small] * 20, [1] * 20, 1):
+        assert gn == wn and np.array_equal(got, want)
+    g.replay()
+    torch.cuda.synchronize()
+    want, wn = oracle.watershed(lab, oracle.edt(lab), 1)
+    assert int(n.item()) == wn and np.array_equal(out.cpu().numpy(), want)
+    assert p.status() == P.PIPE_OK
+    p.close()
