@@ -252,3 +252,14 @@ def test_captured_call_outlives_the_other_kind(first):
     assert np.array_equal(out.cpu().numpy(), ref[first](small))
     assert np.array_equal(out2.cpu().numpy(), ref[other](large))
     p.close()
+
+
+@pytest.mark.parametrize("K", [3, 9, 70, 4999])
+def test_counts_of_label_noise(pipe, K):
+    """A label on every other pixel: disks of 25 objects and more, with few
+    labels that return at many offsets and with many that share hash bits."""
+    rng = np.random.default_rng(K)
+    img = rng.integers(0, 256, (150, 170), dtype=np.uint8)
+    lab = (rng.integers(0, 2, img.shape) * rng.integers(1, K + 3, img.shape)).astype(np.int32)  # some above K
+    for r in (0, 2, 4):
+        check(pipe, img, lab, K, r=r)
