@@ -262,3 +262,17 @@ def test_captured_tile_outlives_a_batch():
     assert int(n.item()) == wn and np.array_equal(out.cpu().numpy(), want)
     assert p.status() == P.PIPE_OK
     p.close()
+
+
+@pytest.mark.parametrize("n,K", [(1, 0), (1, 300), (16, 0), (17, 0), (16, 20), (17, 20)])
+def test_start_of_a_call(pipe, n, K):
+    """No object at all, more objects than the first block of the starting
+    launch, as many tiles as one launch takes and one more."""
+    lab = np.zeros((60, 90), np.int32)
+    lab[2:4, 3:6] = 1
+    lab[30:40, 20:33] = min(K, 20)
+    lab = np.where(lab <= K, lab, 0).astype(np.int32)
+    want, wn = oracle.watershed(lab, oracle.edt(lab), 1)
+    for _ in range(2):  # the second call on what the first one left
+        for got, gn in _ws_batch(pipe, [lab] * n, [K] * n, 1):
+            assert gn == wn and np.array_equal(got, want)
