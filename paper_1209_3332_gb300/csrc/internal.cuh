@@ -269,7 +269,7 @@ void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, in
                        Profiler* pf);
 void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, int H, int K, float* feats,
                            int4* bbox, int sms, cudaStream_t s, Profiler* pf);
-void launch_features_batched(const Launch& L, int grid, cudaStream_t s, Profiler* pf);
+void launch_features_batched(const Launch& L, int grid, int sms, cudaStream_t s, Profiler* pf);
 // per object 1..K of a label plane: its box (xmin, ymin, xmax, ymax); empty (xmax < xmin) if absent
 void launch_object_boxes(const int32_t* labels, int W, int H, int K, int4* bbox, cudaStream_t s, Profiler* pf);
 // One tile of a Canny launch (plain: one tile; batched: many), or of another

@@ -26,7 +26,10 @@
 // takes as long for one lane as for 32), they took 331 -> 203 us for the 48000
 // objects of 16 tiles of 4096^2, and with a stage small enough for 32 warps per
 // SM instead of 20, 173 us.  What bounds it now is the pixel walk: a chain of
-// shared-memory reads and a Welford update with a division per pixel.
+// shared-memory reads and a Welford update with a division per pixel, 0.6 us per
+// step of 32 pixels.  Regions beyond the stage are walked in bands of rows
+// (objects of 80 x 80 pixels: one 109 us, 64 of them 120; 134 and 143 when they were
+// read from global memory).
 #include <cmath>
 #include <mutex>
 #include <type_traits>
@@ -83,32 +86,41 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-// A warp stages at most STAGE_PX pixels at a time: with the counters 26 KB per
-// CTA, eight of which fit on an SM (all of a region of 5120 pixels at once: five;
-// objects of 16 tiles of 4096^2 203 us, and 171).
-constexpr int STAGE_PX = 2816;
-constexpr int REGION_PX = 5120;  // largest region (box + 1-px margin) that is staged
+constexpr int FW = 4;  // object warps per CTA
+// A warp stages at most MANY_PX pixels at a time where there are many objects: with
+// the counters 26 KB per CTA, eight of which fit on an SM.  FEW_PX at a time: five
+// (objects of 16 tiles of 4096^2 203 us, and 171); for few objects, where a warp's
+// own time is what counts, and more registers shorten it.
+constexpr int MANY_PX = 2816, MANY_CTAS = 8;
+constexpr int FEW_PX = 5120, FEW_CTAS = 5;
+constexpr int BANDS_PX = 1 << 20;  // a lane's share of 255^2 each is below 2^32
+// How an object's pixels are read and its whole numbers added: staged at once, or in
+// bands of rows (up to FEW_PX pixels), in 32 bits; staged in bands, in 64 bits; from
+// global memory, in 64 bits.  The paths are apart so that the common one has the
+// registers to itself: with bands in it, 167 us instead of 157 for the objects of 16
+// tiles of 4096^2.
+enum class Px { STAGED, BANDS, WIDE_BANDS, GLOBAL };
 constexpr int HOM_LCM = 408850;  // lcm of 1 + d^2 for d = 0..7
 
-// A sum over the warp of non-negative whole numbers.  Those of a staged object
-// (at most REGION_PX pixels) are below 2^32, so that one instruction adds them.
-template <bool STAGED>
+// A sum over the warp of non-negative whole numbers.  Those of an object of a
+// region of up to FEW_PX pixels are below 2^32, so that one instruction adds them.
+template <Px HOW>
 __device__ __forceinline__ long long whole_sum(long long v) {
-    static_assert((long long)HOM_LCM * REGION_PX < (1LL << 32) && 255LL * 255 * REGION_PX < (1LL << 32) &&
-                  (long long)REGION_PX * REGION_PX < (1LL << 32), "the largest sums");
-    if constexpr (STAGED) return (long long)__reduce_add_sync(FULLF, (unsigned)v);
+    static_assert((long long)HOM_LCM * FEW_PX < (1LL << 32) && 255LL * 255 * FEW_PX < (1LL << 32) &&
+                  (long long)FEW_PX * FEW_PX < (1LL << 32) && 255LL * 255 * (BANDS_PX / 32 + 1) < (1LL << 32), "the largest sums");
+    if constexpr (HOW <= Px::BANDS) return (long long)__reduce_add_sync(FULLF, (unsigned)v);
     else return warp_sum<long long>(v);
 }
 
 // Features of object `obj` by one warp; glcm: this warp's 4x64 counters;
-// spx: this warp's staging buffer.  When the object's box plus a
-// 1-pixel margin (clipped to the image) has at most REGION_PX pixels, it is
-// staged with coalesced row loads as one 16-bit word per pixel (hem8 and an
-// in-object bit), in bands of rows if it is larger than the buffer, and every
-// neighbourhood read comes from shared memory; larger boxes read global
-// memory directly.  Sobel neighbours (clamped to the image), 4-neighbours and
-// co-occurrence partners of box pixels all lie inside that region.
-template <bool STAGED>
+// spx: this warp's staging buffer.  The object's box plus a 1-pixel margin
+// (clipped to the image) is staged with coalesced row loads as one 16-bit word
+// per pixel (hem8 and an in-object bit), in bands of rows if it is larger than
+// the buffer, and every neighbourhood read comes from shared memory; boxes so
+// wide that the buffer does not hold three rows read global memory directly.
+// Sobel neighbours (clamped to the image), 4-neighbours and co-occurrence
+// partners of box pixels all lie inside that region.
+template <Px HOW, int STAGE_PX>
 __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, int* glcm, uint16_t* spx) {
     const int lane = threadIdx.x & 31;
     const int l = obj + 1;
@@ -124,12 +136,11 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     const long long npx = (long long)bw * bh;
     const int rx0 = max(box.x - 1, 0), ry0 = max(box.y - 1, 0);
     const int rw = min(box.z + 1, W - 1) - rx0 + 1, rh = min(box.w + 1, H - 1) - ry0 + 1;
-    constexpr bool staged = STAGED;
+    constexpr bool staged = HOW != Px::GLOBAL, bands = HOW == Px::BANDS || HOW == Px::WIDE_BANDS;
     for (int i = lane; i < 4 * 64; i += 32) glcm[i] = 0;
     int sy0 = 0;  // first staged row
-    // stages rows [from, to] of the region's columns
-    auto stage = [&](int from, int to) {
-        sy0 = from;
+    // stages rows [from, to] of the region's columns from the buffer's pixel p0 on
+    auto stage = [&](int from, int to, int p0) {
         // one index space, four pixels per lane per step with all their loads
         // issued before the stores, so their latencies overlap
         const int nreg = (to - from + 1) * rw;
@@ -138,7 +149,7 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
             int lab[4], hv[4], at[4];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
-                at[u] = base + 32 * u < nreg ? sy * rw + sx : -1;
+                at[u] = base + 32 * u < nreg ? p0 + sy * rw + sx : -1;
                 const size_t g = (size_t)(from + sy) * W + rx0 + sx;
                 lab[u] = at[u] >= 0 ? J.labels[g] : 0;
                 hv[u] = at[u] >= 0 ? J.hem8[g] : 0;
@@ -159,20 +170,36 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
         return (uint32_t)J.hem8[o] | (J.labels[o] == l ? 0x100u : 0u);
     };
     int cnt = 0, per = 0, mn = 255, mx = 0, gmn = 0x7fffffff, gmx = 0;
-    using Whole = typename std::conditional<STAGED, unsigned, long long>::type;
-    Whole S = 0, Q = 0;
+    using Whole = typename std::conditional<HOW <= Px::BANDS, unsigned, long long>::type;
+    using Acc = typename std::conditional<staged, unsigned, long long>::type;  // a lane's sums of pixels and squares
+    Acc S = 0, Q = 0;
     float wm = 0.f, wq = 0.f;  // this lane's running mean and sum of squared deviations of |Sobel|
     // lane walks the box row-major with stride 32, advancing (y, x) without divisions
     int y = box.y + lane / bw, x = box.x + lane % bw;
     // a band: box rows [yb, ye], staged with the rows beside them
-    const int band = staged ? (rw * rh <= STAGE_PX ? bh : STAGE_PX / rw - 2) : bh;
+    const int band = bands ? STAGE_PX / rw - 2 : bh;
     long long idx = lane;
     for (int yb = box.y; yb <= box.w; yb += band) {
-    const int ye = min(yb + band - 1, box.w);
+    const int ye = bands ? min(yb + band - 1, box.w) : box.w;
     __syncwarp();
-    if (staged) stage(max(yb - 1, 0), min(ye + 1, H - 1));
-    __syncwarp();
-    for (; idx < npx && y <= ye; idx += 32) {
+    if (staged) {
+        const int from = max(yb - 1, 0);
+        int p0 = 0;
+        if (bands && yb > box.y) {  // rows yb - 1 and yb are the last two staged for the band before
+            const int off = (from - sy0) * rw;
+            for (int i = lane; i < ((2 * rw + 31) & ~31); i += 32) {
+                const uint16_t v = spx[off + min(i, 2 * rw - 1)];
+                __syncwarp();  // (a chunk may overlap the place it moves to)
+                if (i < 2 * rw) spx[i] = v;
+                __syncwarp();
+            }
+            p0 = 2 * rw;
+        }
+        sy0 = from;
+        stage(from + (p0 ? 2 : 0), min(ye + 1, H - 1), p0);
+        __syncwarp();
+    }
+    for (; idx < npx && (!bands || y <= ye); idx += 32) {
         const int cy = y, cx = x;
         x += 32;
         while (x > box.z) { x -= bw; y++; }
@@ -210,9 +237,9 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
         if (cy > 0 && cx + 1 < W && (c >> 8)) atomicAdd(&glcm[3 * 64 + vb + ((c & 0xffu) >> 5)], 1);
     }
     }
-    const long long N = whole_sum<STAGED>(cnt);
-    const long long Ssum = whole_sum<STAGED>(S), Qsum = whole_sum<STAGED>(Q);
-    const long long Per = whole_sum<STAGED>(per);
+    const long long N = whole_sum<HOW>(cnt);
+    const long long Ssum = whole_sum<HOW>(S), Qsum = whole_sum<HOW>(Q);
+    const long long Per = whole_sum<HOW>(per);
     const int Mn = __reduce_min_sync(FULLF, mn), Mx = __reduce_max_sync(FULLF, mx);
     const int Gmn = __reduce_min_sync(FULLF, gmn), Gmx = __reduce_max_sync(FULLF, gmx);
     // the lanes' (count, mean, squared deviations) combined pairwise (Chan,
@@ -262,17 +289,17 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     for (int o = 0; o < 4; o++) {
         const int* cc = glcm + o * 64;
         const Whole v0 = cc[lane], v1 = cc[lane + 32];
-        const long long T = whole_sum<STAGED>(v0 + v1);
+        const long long T = whole_sum<HOW>(v0 + v1);
         if (T == 0) continue;
         used++;
-        const long long si = whole_sum<STAGED>(i0 * v0 + i1 * v1);
-        const long long sj = whole_sum<STAGED>(j0 * v0 + j1 * v1);
-        const long long sii = whole_sum<STAGED>(i0 * i0 * v0 + i1 * i1 * v1);
-        const long long sjj = whole_sum<STAGED>(j0 * j0 * v0 + j1 * j1 * v1);
-        const long long sij = whole_sum<STAGED>(i0 * j0 * v0 + i1 * j1 * v1);
-        const long long scon = whole_sum<STAGED>(d0 * v0 + d1 * v1);
-        const long long sene = whole_sum<STAGED>(v0 * v0 + v1 * v1);
-        const long long shom = whole_sum<STAGED>((HL / (1 + d0)) * v0 + (HL / (1 + d1)) * v1);
+        const long long si = whole_sum<HOW>(i0 * v0 + i1 * v1);
+        const long long sj = whole_sum<HOW>(j0 * v0 + j1 * v1);
+        const long long sii = whole_sum<HOW>(i0 * i0 * v0 + i1 * i1 * v1);
+        const long long sjj = whole_sum<HOW>(j0 * j0 * v0 + j1 * j1 * v1);
+        const long long sij = whole_sum<HOW>(i0 * j0 * v0 + i1 * j1 * v1);
+        const long long scon = whole_sum<HOW>(d0 * v0 + d1 * v1);
+        const long long sene = whole_sum<HOW>(v0 * v0 + v1 * v1);
+        const long long shom = whole_sum<HOW>((HL / (1 + d0)) * v0 + (HL / (1 + d1)) * v1);
         const float sent = warp_sum<float>(__fadd_rn(ent(v0, T), ent(v1, T)));
         const float Tf = (float)T;
         const long long vi = T * sii - si * si, vj = T * sjj - sj * sj, cv = T * sij - si * sj;
@@ -301,39 +328,47 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     __syncwarp();
 }
 
-// boxes larger than the stage read global memory; that rare path is kept out
-// of line so the common one stays small in the instruction cache
-__device__ __noinline__ void object_features_global(const ObjJob& J, int obj, int* glcm) {
-    object_features_impl<false>(J, obj, glcm, nullptr);
+// larger regions: rare, and kept out of line so that the common path stays small
+// in the instruction cache
+template <Px HOW, int STAGE_PX>
+__device__ __noinline__ void object_features_large(const ObjJob& J, int obj, int* glcm, uint16_t* spx) {
+    __builtin_assume(__isShared(glcm));  // which the call hides
+    __builtin_assume(__isShared(spx));
+    object_features_impl<HOW, STAGE_PX>(J, obj, glcm, spx);
 }
 
+template <int STAGE_PX>
 __device__ __forceinline__ void object_features(const ObjJob& J, int obj, int* glcm, uint16_t* spx) {
     const int4 box = J.bbox[obj];
     const int rx0 = max(box.x - 1, 0), ry0 = max(box.y - 1, 0);
     const long long rw = (long long)min(box.z + 1, J.W - 1) - rx0 + 1, rh = (long long)min(box.w + 1, J.H - 1) - ry0 + 1;
-    if (rw > 0 && rh > 0 && rw * rh <= REGION_PX && (rw * rh <= STAGE_PX || 3 * rw <= STAGE_PX))
-        object_features_impl<true>(J, obj, glcm, spx);
+    if (rw > 0 && rh > 0 && rw * rh <= STAGE_PX)
+        object_features_impl<Px::STAGED, STAGE_PX>(J, obj, glcm, spx);
+    else if (3 * rw <= STAGE_PX && rw * rh <= FEW_PX)
+        object_features_impl<Px::BANDS, STAGE_PX>(J, obj, glcm, spx);
+    else if (3 * rw <= STAGE_PX && rw * rh <= BANDS_PX)
+        object_features_large<Px::WIDE_BANDS, STAGE_PX>(J, obj, glcm, spx);
     else
-        object_features_global(J, obj, glcm);
+        object_features_large<Px::GLOBAL, STAGE_PX>(J, obj, glcm, spx);
 }
 
-constexpr int FW = 4;  // object warps per CTA
-
-// Plain form: objects [0, K) of one tile, one warp each.
+template <int STAGE_PX>
 struct ObjSmem {
     int glcm[4 * 64];
     uint16_t px[STAGE_PX];  // hem8 | (in object) << 8
 };
 
-__global__ void __launch_bounds__(FW * 32, 8) k_fobj_plain(ObjJob J, int K) {
-    __shared__ ObjSmem sm[FW];
+// Plain form: objects [0, K) of one tile, one warp each.
+template <int STAGE_PX, int CTAS>
+__global__ void __launch_bounds__(FW * 32, CTAS) k_fobj_plain(ObjJob J, int K) {
+    __shared__ ObjSmem<STAGE_PX> sm[FW];
     const int warp = threadIdx.x >> 5;
-    ObjSmem& S = sm[warp];
+    ObjSmem<STAGE_PX>& S = sm[warp];
     for (int obj = blockIdx.x * FW + warp; obj < K; obj += gridDim.x * FW)
-        object_features(J, obj, S.glcm, S.px);
+        object_features<STAGE_PX>(J, obj, S.glcm, S.px);
 }
 
-__global__ void k_obj_prefix(Launch L) {
+__global__ void k_obj_prefix(Launch L, int first) {
     if (L.early) after_previous();
     if (threadIdx.x != 0) return;
     int run = 0;
@@ -349,29 +384,33 @@ __global__ void k_obj_prefix(Launch L) {
         run += m;
     }
     L.sh->nobj = run;
-    L.sh->next_obj = 0;
+    L.sh->next_obj = first;
 }
 
 // Batched form: the objects of all tiles, item -> (tile, object) through the
 // obj_base prefixes (the last tile whose base is <= item owns it).
-__global__ void __launch_bounds__(FW * 32, 8) k_fobj_batched(Launch L) {
+__global__ void __launch_bounds__(FW * 32, MANY_CTAS) k_fobj_batched(Launch L, int first) {
     if (L.early) after_previous();
-    __shared__ ObjSmem sm[FW];
+    __shared__ ObjSmem<MANY_PX> sm[FW];
     const int warp = threadIdx.x >> 5;
-    ObjSmem& S = sm[warp];
+    ObjSmem<MANY_PX>& S = sm[warp];
     const int total = L.sh->nobj;
     const int lane = threadIdx.x & 31;
     // objects are drawn one at a time from a counter, so a warp that drew
-    // large boxes does not hold back the end of the pass
-    for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&L.sh->next_obj, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+    // large boxes does not hold back the end of the pass; the first `first` go
+    // to the first warps of the grid, which spreads few objects evenly over the SMs
+    // (a 2048^2 tile with 900 of 60 x 60 pixels: 300 -> 244 us)
+    for (int item = blockIdx.x * FW + warp;;) {
+        if (item >= first) {
+            if (lane == 0) item = atomicAdd(&L.sh->next_obj, 1);
+            item = __shfl_sync(0xffffffffu, item, 0);
+        }
         if (item >= total) break;
         const int t = find_tile(L.tiles, L.ntiles, item, &TileDev::obj_base);
         const TileDev& T = L.tiles[t];
         ObjJob J{T.hem8, T.labels, T.W, T.H, T.bbox, T.feats};
-        object_features(J, item - T.obj_base, S.glcm, S.px);
+        object_features<MANY_PX>(J, item - T.obj_base, S.glcm, S.px);
+        item = first;
     }
 }
 
@@ -392,16 +431,22 @@ void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, in
     ObjJob J{hem8, labels, W, H, bbox, feats};
     int grid = (K + FW - 1) / FW < sms * 16 ? (K + FW - 1) / FW : sms * 16;
     pf->begin("feat_objects", s);
-    k_fobj_plain<<<grid, FW * 32, 0, s>>>(J, K);
+    // No more objects than warps of the large-stage form fit on the GPU: each is
+    // done soonest there.  More: the form of more warps.  3000 objects of 24 x 24
+    // and 60 x 60 pixels, 52 and 131 us by the first and 57 and 137 by the
+    // second; 3500, 68 and 183, and 58 and 152.
+    if (K <= sms * FEW_CTAS * FW) k_fobj_plain<FEW_PX, FEW_CTAS><<<grid, FW * 32, 0, s>>>(J, K);
+    else k_fobj_plain<MANY_PX, MANY_CTAS><<<grid, FW * 32, 0, s>>>(J, K);
     pf->end("feat_objects", s);
 }
 
-void launch_features_batched(const Launch& L, int grid, cudaStream_t s, Profiler* pf) {
+void launch_features_batched(const Launch& L, int grid, int sms, cudaStream_t s, Profiler* pf) {
+    const int first = FW * (grid < sms * MANY_CTAS ? grid : sms * MANY_CTAS);  // warps resident at once
     pf->begin("feat_prefix", s);
-    launch_behind(L.early && pf->overlap(), k_obj_prefix, 1, 32, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_obj_prefix, 1, 32, 0, s, L, first);
     pf->end("feat_prefix", s);
     pf->begin("feat_objects", s);
-    launch_behind(L.early && pf->overlap(), k_fobj_batched, grid, FW * 32, 0, s, L);
+    launch_behind(L.early && pf->overlap(), k_fobj_batched, grid, FW * 32, 0, s, L, first);
     pf->end("feat_objects", s);
 }
 

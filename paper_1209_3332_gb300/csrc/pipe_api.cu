@@ -496,7 +496,7 @@ void run_path(pipe_t p, const Launch& L, int Wmax, bool features, int max_object
     launch_recon(L, tu.recon_grid, p->recon_cap, p->recon_teams, s, pf);
     launch_label(L, features ? 1 : 0, max_objects, p->sms, s, pf);
     launch_edt(L, tu.edt_rb, Wmax, s, pf);
-    if (features) launch_features_batched(L, tu.feat_grid, s, pf);
+    if (features) launch_features_batched(L, tu.feat_grid, p->sms, s, pf);
 }
 
 int run_path_graph(pipe_t p, GraphCache& cache, const std::string& shape_key, const Launch& L, int Wmax,

@@ -178,3 +178,26 @@ def test_features_at_the_stage_sizes(pipe, bw, bh):
     pipe.features_tile(torch.from_numpy(hem8).to(dev), torch.from_numpy(labels).to(dev), 4, out)
     torch.cuda.synchronize()
     assert_feats_close(out.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("bw,bh", [(79, 64), (80, 64), (100, 100), (300, 200), (936, 6), (937, 6), (1200, 5), (4, 1500), (1, 4000)])
+def test_features_of_objects_beyond_the_stage(pipe, bw, bh):
+    """Regions of more than 5120 pixels, whose sums are taken in 64 bits: staged
+    in bands of many rows down to one, whose first two rows are the last two of
+    the band before, and read from global memory where not even three rows fit;
+    at the image's sides, and touching other objects."""
+    import torch
+    rng = np.random.default_rng(bw * 1000 + bh)
+    W, H = 2 * bw + 5, 2 * bh + 1
+    hem8 = rng.integers(0, 256, (H, W)).astype(np.uint8)
+    labels = np.zeros((H, W), np.int32)
+    for k, (x, y) in enumerate(((0, 0), (W - bw, 0), (2, H - bh), (W - bw, H - bh))):
+        m = rng.random((bh, bw)) < (1.0 if k % 2 else 0.6)
+        m[0, 0] = m[-1, -1] = True
+        labels[y:y + bh, x:x + bw][m] = k + 1
+    ref = oracle.features(hem8, labels, 4)
+    dev = torch.device("cuda", 0)
+    out = torch.zeros((4, 15), dtype=torch.float32, device=dev)
+    pipe.features_tile(torch.from_numpy(hem8).to(dev), torch.from_numpy(labels).to(dev), 4, out)
+    torch.cuda.synchronize()
+    assert_feats_close(out.cpu().numpy(), ref)
