@@ -240,13 +240,14 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_canny_nms(const __grid_con
 // an object, and takes the listed pixels 32 at a time, one per lane: the
 // bits under the disk's chord of each row pick the labels to look at.  Each
 // edge pixel adds one to every distinct object in its disk: the first four are
-// remembered in registers, all of them as a hash in 64 bits, and only an object
-// whose bit is taken is looked for at the earlier disk offsets (1024^2 of noise
-// with a label on every other pixel, disks of radius 4 with 25 objects: 1047 us;
-// 2350 with every object looked for).  8 tiles of 4096^2: 146 us (465 with a CTA per block, a
-// thread per pixel and a label read for every disk offset).  Bound: the latency
-// of the label loads of the blocks that hold edges (about half; seven of a lane
-// in flight), 24 warps per SM by shared memory.
+// remembered in registers, the others as a bit of 64 (a hash where there are more
+// objects than bits), and only an object whose bit is taken is looked for at the
+// earlier disk offsets (1024^2 of noise with a label on every other pixel, disks
+// of radius 4 with 25 objects: 1047 us; 2350 with every object looked for).
+// 8 tiles of 4096^2: 146 us (465 with a CTA per block, a thread per pixel and a
+// label read for every disk offset).  Bound: the latency of the label loads of
+// the blocks that hold edges (about half; seven of a lane in flight), 24 warps
+// per SM by shared memory.
 constexpr int CR_MAX = 4;                 // largest disk radius of the counts
 constexpr int CC_S = CT + 2 * CR_MAX;     // staged labels: the block and a CR_MAX-pixel margin (40 x 40)
 // Blocks (one per warp) per CTA: most blocks hold no edge pixel and end at once, and
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(CC_WARPS * 32) k_canny_counts(const __grid_con
     }
     __syncwarp();
     const int r2 = r * r;
+    const bool exact = K <= 64;  // a bit for every object
     for (int i0 = 0; i0 < n; i0 += 32) {
         if (i0 + lane >= n) break;
         const int p = S.list[i0 + lane], ly = p >> 5, lx = p & 31;
@@ -345,19 +347,22 @@ __global__ void __launch_bounds__(CC_WARPS * 32) k_canny_counts(const __grid_con
                 const int dx = __ffsll((long long)m) - 1 - w;
                 const int v = S.lab[ly + CR_MAX + dy][lx + CR_MAX + dx];
                 if (v == seen0 || v == seen1 || v == seen2 || v == seen3) continue;
-                const u64 bit = 1ull << (((unsigned)v * 0x9e3779b1u) >> 26);
-                bool fresh = true;
-                if (nseen >= 4 && (seen & bit)) {  // look for v at an earlier disk offset
-                    for (int ey = -r; ey <= dy && fresh; ey++) {
-                        int we;
-                        u64 e = chord(ey, we);
-                        if (ey == dy) e &= (1ull << (dx + w)) - 1ull;
-                        for (; e && fresh; e &= e - 1)
-                            fresh = S.lab[ly + CR_MAX + ey][lx + CR_MAX + __ffsll((long long)e) - 1 - we] != v;
+                if (nseen >= 4) {
+                    const u64 bit = 1ull << (exact ? v - 1 : (int)(((unsigned)v * 0x9e3779b1u) >> 26));
+                    bool fresh = !(seen & bit);
+                    if (!fresh && !exact) {  // look for v at an earlier disk offset
+                        fresh = true;
+                        for (int ey = -r; ey <= dy && fresh; ey++) {
+                            int we;
+                            u64 e = chord(ey, we);
+                            if (ey == dy) e &= (1ull << (dx + w)) - 1ull;
+                            for (; e && fresh; e &= e - 1)
+                                fresh = S.lab[ly + CR_MAX + ey][lx + CR_MAX + __ffsll((long long)e) - 1 - we] != v;
+                        }
                     }
+                    if (!fresh) continue;
+                    seen |= bit;
                 }
-                if (!fresh) continue;
-                seen |= bit;
                 atomicAdd(&d.counts[v - 1], 1);
                 if (nseen == 0) seen0 = v; else if (nseen == 1) seen1 = v; else if (nseen == 2) seen2 = v;
                 else if (nseen == 3) seen3 = v;
