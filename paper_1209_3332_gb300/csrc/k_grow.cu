@@ -8,7 +8,12 @@
 // rows above and below (shuffles) and along whole runs of the mask inside a
 // row: adding the marker to the mask carries through each run from its first
 // marker bit upwards, and the same on bit-reversed words fills downwards.
-// Steps repeat until none changes a bit.
+// Steps repeat until none changes a bit; where 16 were not enough in a mask of a
+// quarter of the tile and more, whole runs of the columns are filled between
+// further steps, by doubling over the lanes: one marker pixel in a mask of 2048^2,
+// 279 us by steps alone and 173 so (152 from the eighth step on, but then eight
+// edge planes of 4096^2, whose tiles need few, take 1 % longer; thin masks that
+// wind through a tile gain nothing from it).
 //
 // The tiles are driven by a ticket queue as in the reconstruction (k_recon.cu):
 // workers first draw groups of tiles from a counter and process those whose
@@ -18,7 +23,7 @@
 // it reaches zero, so the work never depends on which workers are resident.
 // Every spin wait is bounded by the pipe's cycle budget (ST_TIMEOUT).
 //
-// Bound: the latency of a visit (loads, about twenty steps, fence and state
+// Bound: the latency of a visit (loads, up to about twenty steps, fence and state
 // atomics) and of a few dependent visits; the planes are 2/8 B per pixel in,
 // 1 B out by k_grow_out.  Eight 4096^2 edge planes: 177 us and 31 for the bytes,
 // one red blood cell plane 28 and 9 (414 and 54 us on bytes with the grayscale
@@ -87,6 +92,33 @@ __device__ __forceinline__ u64 fill_runs(u64 s, u64 c, u64 rc) {
     return __brevll(fill_up(__brevll(s), rc));
 }
 __device__ __forceinline__ u64 spread(u64 v) { return v | (v << 1) | (v >> 1); }
+// The same along the columns: rows 2 l and 2 l + 1 in lane l, runs joined over
+// 1, 2, 4, 8 and 16 lanes in either direction.
+__device__ __forceinline__ void fill_columns(u64& s0, u64& s1, const ulonglong2 c, int lane) {
+#pragma unroll
+    for (int up = 0; up < 2; up++) {
+        // the row of the lane that the next lane looks at: its marker, and whether it lets through
+        u64 g = up ? s0 | (c.x & s1) : s1 | (c.y & s0), p = c.x & c.y;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const u64 gn = up ? __shfl_down_sync(FULLG, g, d) : __shfl_up_sync(FULLG, g, d);
+            const u64 pn = up ? __shfl_down_sync(FULLG, p, d) : __shfl_up_sync(FULLG, p, d);
+            if (up ? lane + d < 32 : lane >= d) {
+                g |= p & gn;
+                p &= pn;
+            }
+        }
+        u64 in = up ? __shfl_down_sync(FULLG, g, 1) : __shfl_up_sync(FULLG, g, 1);
+        if (lane == (up ? 31 : 0)) in = 0ull;
+        if (up) {
+            s1 |= c.y & in;
+            s0 |= c.x & s1;
+        } else {
+            s0 |= c.x & in;
+            s1 |= c.y & s0;
+        }
+    }
+}
 __device__ __forceinline__ ulonglong2 rows2(const u64* plane, int t, int lane) {
     return __ldcg(reinterpret_cast<const ulonglong2*>(plane + (size_t)t * RT) + lane);
 }
@@ -125,7 +157,7 @@ __device__ void grow_tile(const GrowLaunch& G, int t, int drop, int lane) {
         const u64 in0 = (u64)(la | l0 | l1) | ((u64)(ra | r0 | r1) << 63);
         const u64 in1 = (u64)(l0 | l1 | lb) | ((u64)(r0 | r1 | rb) << 63);
         u64 s0 = s.x, s1 = s.y;
-        for (;;) {
+        auto step = [&]() -> bool {
             u64 a = __shfl_up_sync(FULLG, s1, 1), b = __shfl_down_sync(FULLG, s0, 1);
             if (lane == 0) a = sv;
             if (lane == 31) b = sv;
@@ -134,7 +166,19 @@ __device__ void grow_tile(const GrowLaunch& G, int t, int drop, int lane) {
             const bool ch = ((n0 ^ s0) | (n1 ^ s1)) != 0ull;
             s0 = n0;
             s1 = n1;
-            if (!__any_sync(FULLG, ch)) break;
+            return __any_sync(FULLG, ch);
+        };
+        bool go = true;
+#pragma unroll 1
+        for (int i = 0; go && i < 16; i++) go = step();
+        if (go) {
+            const bool wide = __reduce_add_sync(FULLG, (unsigned)(__popcll(c.x) + __popcll(c.y))) >= RT * RT / 4;
+#pragma unroll 1
+            do {
+                if (wide) fill_columns(s0, s1, c, lane);
+#pragma unroll 1
+                for (int i = 0; go && i < 8; i++) go = step();
+            } while (go);
         }
         if (__any_sync(FULLG, ((s0 ^ s.x) | (s1 ^ s.y)) != 0ull))
             __stcg(reinterpret_cast<ulonglong2*>(G.marker + (size_t)t * RT) + lane, make_ulonglong2(s0, s1));
@@ -189,9 +233,9 @@ __device__ void grow_tile(const GrowLaunch& G, int t, int drop, int lane) {
     }
 }
 
-constexpr int GROW_WARPS = 4;
+constexpr int GROW_WARPS = 4, GROW_CTAS = 2;  // per CTA, per SM (grow_grid)
 
-__global__ void __launch_bounds__(GROW_WARPS * 32) k_grow(const __grid_constant__ GrowLaunch G) {
+__global__ void __launch_bounds__(GROW_WARPS * 32, GROW_CTAS) k_grow(const __grid_constant__ GrowLaunch G) {
     after_previous();
     const int lane = threadIdx.x & 31;
     int groups = 0;
@@ -306,7 +350,7 @@ int grow_grid(int device) {
     int sms = 0, per = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_grow, GROW_WARPS * 32, 0);
-    return sms * std::min(std::max(per, 1), 2);
+    return sms * std::min(std::max(per, 1), GROW_CTAS);
 }
 
 void launch_grow(const GrowLaunch& G, int grid_cap, cudaStream_t s, Profiler* pf) {

@@ -159,3 +159,24 @@ def test_argument_checks(pipe):
     assert L.rbc_tile(pipe.h, rgb.data_ptr(), 0, 8, 24, 40, 100, out.data_ptr(), s) == P.PIPE_EINVAL
     assert L.rbc_tile(pipe.h, rgb.data_ptr(), 8, 8, 24, 40, 100, rgb.data_ptr() + 8, s) == P.PIPE_EINVAL  # overlap
     assert L.rbc_tile(pipe.h, None, 8, 8, 24, 40, 100, out.data_ptr(), s) == P.PIPE_EINVAL
+
+
+@pytest.mark.parametrize("W,H", [(64, 64), (64, 65), (200, 333), (517, 130)])
+def test_masks_wide_and_tall(pipe, W, H):
+    """Masks that need more steps in a tile than a few: everything, columns
+    and combs of columns joined at either end, columns with gaps at the rows
+    that neighbouring lanes share, mazes; one marker pixel anywhere."""
+    rng = np.random.default_rng(W + H)
+    yy, xx = np.mgrid[0:H, 0:W]
+    masks = [np.ones((H, W), bool), xx % 2 == 0, (xx % 3 == 0) | (yy == 0), (xx % 2 == 1) | (yy == H - 1),
+             (xx % 2 == 0) & (yy % 17 != 5), (xx % 2 == 0) & (yy % 16 != 2) | (yy % 32 == 2),
+             np.where((xx // 2) % 2 == 0, yy > 0, yy < H - 1) & (xx % 2 == 0) | ((yy == 0) | (yy == H - 1)),
+             rng.random((H, W)) < 0.9, rng.random((H, W)) < 0.62]
+    for m in masks:
+        for _ in range(3):
+            rgb = np.full((H, W, 3), 200, np.uint8)
+            rgb[m] = (200, 140, 140)
+            y, x = int(rng.integers(H)), int(rng.integers(W))
+            rgb[y, x] = (250, 100, 100)
+            want = oracle.rbc(rgb)
+            assert_same(gpu_rbc(pipe, rgb), want, "mask")
