@@ -13,7 +13,6 @@ namespace nucseg {
 constexpr int RT = 64;            // reconstruction work tile: RT x RT pixels, one warp
 constexpr int RECON_MIN_BLOCKS = 16;  // resident reconstruction workers (one-warp CTAs) per SM the register budget must allow
 constexpr int CB = 32;            // labelling block: CB x CB pixels (one bitmap word per row)
-constexpr int CB_THREADS = 256;
 constexpr int CCL_WARPS = 4;      // labelling blocks (one per warp) per CTA
 constexpr int RL_CAP = 512;       // root-list slots per labelling block
 constexpr int NFEAT = 15;
@@ -25,7 +24,7 @@ constexpr int MORPH_RMAX = 15;   // largest disk radius of the opening (chords o
 constexpr int WL_IDLE = 0, WL_QUEUED = 1, WL_RUNNING = 2, WL_DIRTY = 3;
 
 // device status codes (same values as pipe_status)
-constexpr int ST_OK = 0, ST_TIMEOUT = 5, ST_OVERFLOW = 6;
+constexpr int ST_TIMEOUT = 5, ST_OVERFLOW = 6;
 
 // One image of a launch: pointers into caller buffers and the pipe's arena.
 struct TileDev {
@@ -56,7 +55,6 @@ struct TileDev {
     int rtx, rty, rt_base;        // reconstruction tiles and global base id
     int cbx, cby, cb_base;        // labelling blocks and global base id
     int nchunks, chunk_base;      // scan chunks (of SCAN_CHUNK words)
-    int col_base;                 // EDT column strips base
     int row_base;                 // EDT rows base
     int px_base;                  // deconvolution work items base
     int obj_base;                 // first object item of this tile (batched features)
@@ -87,7 +85,7 @@ struct Launch {
     int* tile_status;      // [ntiles]
     int* status;           // the pipe's status word (set_status); null for served groups, whose results carry theirs
     // totals (host-computed) for grid sizing
-    int n_rt, n_cb, n_chunks, n_cols, n_rows, n_px;
+    int n_rt, n_cb, n_chunks, n_rows, n_px;
     int early;             // each kernel is launched before the one ahead of it is complete (launch_behind)
     long long wait_budget;
     int h, thr, amin, amax;
@@ -252,7 +250,7 @@ void recon_grid(int device, int* warps, int* teams);
 // warps: resident one-warp workers to use, of warps_cap; launches with few work
 // tiles per worker use teams of four warps instead, the same share of teams_cap
 void launch_recon(const Launch& L, int warps, int warps_cap, int teams_cap, cudaStream_t s, Profiler* pf);
-void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cudaStream_t s, Profiler* pf);
+void launch_label(const Launch& L, int want_bbox, int sms, cudaStream_t s, Profiler* pf);
 size_t edt_rows_smem(int RB, int Wmax);
 void launch_edt(const Launch& L, int RB, int Wmax, cudaStream_t s, Profiler* pf);
 // The opening (1 <= r <= MORPH_RMAX in two passes through tmp, morph_scratch bytes).
@@ -270,8 +268,6 @@ void launch_morph_open(const uint8_t* src, uint8_t* dst, uint8_t* tmp, int W, in
 void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, int H, int K, float* feats,
                            int4* bbox, int sms, cudaStream_t s, Profiler* pf);
 void launch_features_batched(const Launch& L, int grid, int sms, cudaStream_t s, Profiler* pf);
-// per object 1..K of a label plane: its box (xmin, ymin, xmax, ymax); empty (xmax < xmin) if absent
-void launch_object_boxes(const int32_t* labels, int W, int H, int K, int4* bbox, cudaStream_t s, Profiler* pf);
 // One tile of a Canny launch (plain: one tile; batched: many), or of another
 // growth of a binary marker through a binary mask.
 struct CannyDesc {

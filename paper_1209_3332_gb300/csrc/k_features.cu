@@ -66,19 +66,6 @@ struct ObjJob {
     float* feats;
 };
 
-__device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
-__device__ __forceinline__ int sobel_m2(const uint8_t* I, int W, int H, int y, int x) {
-    int ym = max(y - 1, 0), yp = min(y + 1, H - 1), xm = max(x - 1, 0), xp = min(x + 1, W - 1);
-    const uint8_t* rm = I + (size_t)ym * W;
-    const uint8_t* r0 = I + (size_t)y * W;
-    const uint8_t* rp = I + (size_t)yp * W;
-    int a = rm[xm], b = rm[x], c = rm[xp], d = r0[xm], f = r0[xp], g = rp[xm], h = rp[x], i = rp[xp];
-    int gx = (c + 2 * f + i) - (a + 2 * d + g);
-    int gy = (g + 2 * h + i) - (a + 2 * b + c);
-    return gx * gx + gy * gy;
-}
-
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -369,7 +356,6 @@ __global__ void __launch_bounds__(FW * 32, CTAS) k_fobj_plain(ObjJob J, int K) {
 }
 
 __global__ void k_obj_prefix(Launch L, int first) {
-    if (L.early) after_previous();
     if (threadIdx.x != 0) return;
     int run = 0;
     for (int t = 0; t < L.ntiles; t++) {
@@ -390,7 +376,6 @@ __global__ void k_obj_prefix(Launch L, int first) {
 // Batched form: the objects of all tiles, item -> (tile, object) through the
 // obj_base prefixes (the last tile whose base is <= item owns it).
 __global__ void __launch_bounds__(FW * 32, MANY_CTAS) k_fobj_batched(Launch L, int first) {
-    if (L.early) after_previous();
     __shared__ ObjSmem<MANY_PX> sm[FW];
     const int warp = threadIdx.x >> 5;
     ObjSmem<MANY_PX>& S = sm[warp];
@@ -414,7 +399,7 @@ __global__ void __launch_bounds__(FW * 32, MANY_CTAS) k_fobj_batched(Launch L, i
     }
 }
 
-void launch_object_boxes(const int32_t* labels, int W, int H, int K, int4* bbox, cudaStream_t s, Profiler* pf) {
+static void launch_object_boxes(const int32_t* labels, int W, int H, int K, int4* bbox, cudaStream_t s, Profiler* pf) {
     pf->begin("feat_bbox_init", s);
     k_fbbox_init<<<(K + 255) / 256, 256, 0, s>>>(bbox, K);
     pf->end("feat_bbox_init", s);
@@ -443,10 +428,10 @@ void launch_features_plain(const uint8_t* hem8, const int32_t* labels, int W, in
 void launch_features_batched(const Launch& L, int grid, int sms, cudaStream_t s, Profiler* pf) {
     const int first = FW * (grid < sms * MANY_CTAS ? grid : sms * MANY_CTAS);  // warps resident at once
     pf->begin("feat_prefix", s);
-    launch_behind(L.early && pf->overlap(), k_obj_prefix, 1, 32, 0, s, L, first);
+    k_obj_prefix<<<1, 32, 0, s>>>(L, first);
     pf->end("feat_prefix", s);
     pf->begin("feat_objects", s);
-    launch_behind(L.early && pf->overlap(), k_fobj_batched, grid, FW * 32, 0, s, L, first);
+    k_fobj_batched<<<grid, FW * 32, 0, s>>>(L, first);
     pf->end("feat_objects", s);
 }
 

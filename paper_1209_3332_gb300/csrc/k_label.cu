@@ -870,7 +870,6 @@ __global__ void __launch_bounds__(LOCAL_WARPS * 32, 48 / LOCAL_WARPS) k_relabel(
 
 // every box slot a tile can use (feats_cap of them) starts empty
 __global__ void k_bbox_init(Launch L) {
-    if (L.early) after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     for (int ti = 0; ti < L.ntiles; ti++) {
         const TileDev& T = L.tiles[ti];
@@ -903,15 +902,14 @@ void launch_unpack_bits(const uint32_t* bits, int W, int H, int cbx, uint8_t* ou
     pf->end("unpack_bits", s);
 }
 
-void launch_label(const Launch& L, int want_bbox, int max_objects, int sms, cudaStream_t s, Profiler* pf) {
+void launch_label(const Launch& L, int want_bbox, int sms, cudaStream_t s, Profiler* pf) {
     if (L.n_cb == 0) return;
-    const int rgrid = sms * 8;
     pf->begin("label_reset", s);
     launch_behind(L.early && pf->overlap(), k_counters_reset, 1, 1024, 0, s, L);
     pf->end("label_reset", s);
     if (want_bbox) {
         pf->begin("bbox_init", s);
-        launch_behind(L.early && pf->overlap(), k_bbox_init, rgrid, 256, 0, s, L);
+        k_bbox_init<<<sms * 8, 256, 0, s>>>(L);
         pf->end("bbox_init", s);
     }
     pf->begin("fill_local", s);

@@ -63,7 +63,7 @@ struct WarpTile {
     uint8_t HMc[2][HL + 2];  // M of the halo columns
     uint8_t B0[4][RT];
     int flags[9];            // neighbours to queue: up, down, left, right, UL, UR, DL, DR, self
-    int msg[2];              // from a team's first thread to the others
+    int msg;                 // from a team's first thread to the others
 };
 
 // The worker of a tile: one warp, or the NW warps of a CTA (the arguments are
@@ -85,9 +85,9 @@ struct Worker {
         if constexpr (NW == 1) {
             return __shfl_sync(FULL, v, 0);
         } else {
-            if (t == 0) S.msg[0] = v;
+            if (t == 0) S.msg = v;
             __syncthreads();
-            v = *(volatile int*)&S.msg[0];
+            v = *(volatile int*)&S.msg;
             __syncthreads();
             return v;
         }

@@ -415,19 +415,17 @@ Launch make_launch(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt_to
     L.sh = (Shared*)c.shared.p;
     L.tile_status = (int*)((char*)c.shared.p + sizeof(Shared));
     L.status = status;
-    int rt = 0, cb = 0, ch = 0, col = 0, row = 0, px = 0;
+    int rt = 0, cb = 0, ch = 0, row = 0, px = 0;
     for (auto& t : td) {
         t.rt_base = rt;
         t.cb_base = cb;
         t.chunk_base = ch;
-        t.col_base = col;
         t.row_base = row;
         t.px_base = px;
         t.obj_base = 0;
         rt += t.rtx * t.rty;
         cb += t.cbx * t.cby;
         ch += t.nchunks;
-        col += t.W;
         row += (t.H + RB - 1) / RB;
         px += t.H * ((t.W + 15) / 16);
     }
@@ -435,7 +433,6 @@ Launch make_launch(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt_to
     L.n_rt = rt;
     L.n_cb = cb;
     L.n_chunks = ch;
-    L.n_cols = col;
     L.n_rows = row;
     L.n_px = px;
     L.wait_budget = p->prm.wait_budget_cycles;
@@ -490,17 +487,16 @@ int make_grow(pipe_t p, DevBuf& scratch, const std::vector<CannyDesc>& cd, int n
 
 // The whole path over the descriptors of L (segmentation, and features when
 // `features` is set: boxes come from the relabel pass).
-void run_path(pipe_t p, const Launch& L, int Wmax, bool features, int max_objects, const Tune& tu,
-              cudaStream_t s, Profiler* pf) {
+void run_path(pipe_t p, const Launch& L, int Wmax, bool features, const Tune& tu, cudaStream_t s, Profiler* pf) {
     launch_deconv(L, s, pf);
     launch_recon(L, tu.recon_grid, p->recon_cap, p->recon_teams, s, pf);
-    launch_label(L, features ? 1 : 0, max_objects, p->sms, s, pf);
+    launch_label(L, features ? 1 : 0, p->sms, s, pf);
     launch_edt(L, tu.edt_rb, Wmax, s, pf);
     if (features) launch_features_batched(L, tu.feat_grid, p->sms, s, pf);
 }
 
 int run_path_graph(pipe_t p, GraphCache& cache, const std::string& shape_key, const Launch& L, int Wmax,
-                   int max_obj, const Tune& tu, cudaStream_t s, long long* launches) {
+                   const Tune& tu, cudaStream_t s, long long* launches) {
     const std::string key = shape_key + "|" + tune_str(tu);
     auto it = cache.find(key);
     if (it == cache.end()) {
@@ -514,7 +510,7 @@ int run_path_graph(pipe_t p, GraphCache& cache, const std::string& shape_key, co
             cudaStreamDestroy(cs);
             return PIPE_ECUDA;
         }
-        run_path(p, L, Wmax, true, max_obj, tu, cs, &cp);
+        run_path(p, L, Wmax, true, tu, cs, &cp);
         cudaError_t e = cudaStreamEndCapture(cs, &graph);
         cudaStreamDestroy(cs);
         if (e != cudaSuccess) return PIPE_ECUDA;
@@ -576,8 +572,7 @@ void save_tune(pipe_t p, const std::string& key, const Tune& t) {
 // two runs with CUDA events.  Every candidate computes the same results, so
 // the runs only rewrite the caller's outputs with identical values.  A
 // candidate replaces the current choice only if it is 2% faster.
-int autotune(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt, int Wmax, int max_obj, cudaStream_t s,
-             Tune* out) {
+int autotune(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt, int Wmax, cudaStream_t s, Tune* out) {
     Tune best = default_tune(p, Wmax);
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
@@ -595,7 +590,7 @@ int autotune(pipe_t p, LaunchCtx& c, std::vector<TileDev>& td, int n_rt, int Wma
         float b = 1e30f;
         for (int k = 0; k < 3; k++) {
             if (cudaEventRecord(e0, s) != cudaSuccess) return PIPE_ECUDA;
-            run_path(p, L, Wmax, true, max_obj, tu, s, &cp);
+            run_path(p, L, Wmax, true, tu, s, &cp);
             if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return PIPE_ECUDA;
             float t = 0;
             if (cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) return PIPE_ECUDA;
@@ -818,7 +813,7 @@ int seg_tile(pipe_t p, const uint8_t* rgb_dev, int W, int H, size_t pitch_bytes,
     Launch L = make_launch(p, p->plain, td, n_rt, tu.edt_rb, (int*)p->status.p);
     L.early = 1;
     if ((rc = upload_desc(L, td, s))) return rc;
-    run_path(p, L, W, false, 0, tu, s, &p->prof);
+    run_path(p, L, W, false, tu, s, &p->prof);
     CK(cudaGetLastError());
     p->last_plain = td[0];
     p->have_last = true;
@@ -1053,7 +1048,6 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
         if (rc) return rc;
     }
     std::vector<TileDev> td(n);
-    int max_obj = 1;
     for (int i = 0; i < n; i++) {
         TileDev& t = td[i];
         std::memset(&t, 0, sizeof(t));
@@ -1066,7 +1060,6 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
         t.edt = tiles[i].edt;
         t.n_objects = tiles[i].n_objects;
         t.feats = tiles[i].feats;
-        max_obj = std::max(max_obj, t.feats_cap);
     }
     int rc;
     Tune tu = default_tune(p, Wmax);
@@ -1076,7 +1069,7 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
         if (it != p->tuned.end() && tune_ok(p, it->second, Wmax)) {
             tu = it->second;
         } else if (p->prm.autotune) {
-            if ((rc = autotune(p, p->batch, td, n_rt, Wmax, max_obj, s, &tu))) return rc;
+            if ((rc = autotune(p, p->batch, td, n_rt, Wmax, s, &tu))) return rc;
             p->tuned[tk] = tu;
             save_tune(p, tk, tu);
         }
@@ -1086,8 +1079,8 @@ int seg_features_batch(pipe_t p, const tile_dev* tiles, int n, pipe_stream_t str
     if ((rc = upload_desc(L, td, s))) return rc;
     if (p->prof.enabled) {
         // profiled runs launch eagerly so that each kernel is bracketed by events
-        run_path(p, L, Wmax, true, max_obj, tu, s, &p->prof);
-    } else if ((rc = run_path_graph(p, p->graphs, key, L, Wmax, max_obj, tu, s, &p->prof.launches))) {
+        run_path(p, L, Wmax, true, tu, s, &p->prof);
+    } else if ((rc = run_path_graph(p, p->graphs, key, L, Wmax, tu, s, &p->prof.launches))) {
         return rc;
     }
     CK(cudaGetLastError());
@@ -1361,7 +1354,7 @@ int batch_submit(pipe_t p, const tile_desc* tiles, int n, uint64_t* ticket) {
         std::string key;
         for (int i = 0; i < n; i++)
             key += std::to_string(tiles[i].W) + "x" + std::to_string(tiles[i].H) + (tiles[i].want_planes ? "p;" : ";");
-        rc = run_path_graph(p, c.graphs, key, L, Wmax, *std::max_element(caps.begin(), caps.end()), tu, cs,
+        rc = run_path_graph(p, c.graphs, key, L, Wmax, tu, cs,
                             &p->serve_prof.launches);
         if (rc) return rc;
     }
