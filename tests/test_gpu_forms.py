@@ -295,11 +295,11 @@ def test_many_small_tiles_in_one_batch(n):
     pipe.close()
 
 
-@pytest.mark.parametrize("n", [1, 101, 102, 130])
+@pytest.mark.parametrize("n", ["one", "just fewer", "just enough", "more"])
 def test_reconstruction_by_warps_and_by_teams(n):
-    """48 work tiles of the reconstruction per tile: with 101 there are just
-    fewer than two for each of 2432 warps, with 102 just more, so that teams of
-    warps and single warps take them in turn; corridors and chains, noise."""
+    """48 work tiles of the reconstruction per tile, in batches of just fewer
+    than two work tiles for each resident warp, which teams of warps take, and
+    of just enough for single warps; corridors and chains, noise."""
     import torch
     import paper_1209_3332_gb300 as P
     W, H = 449, 321
@@ -309,6 +309,11 @@ def test_reconstruction_by_warps_and_by_teams(n):
     pipe = P.Pipe(0, autotune=0)
     dev = torch.device("cuda", 0)
     rgb = [torch.from_numpy(np.ascontiguousarray(k)).to(dev) for k in kinds]
+    one = torch.empty((9, H, W), dtype=torch.int32, device=dev)
+    pipe.seg_features_batch([dict(rgb=rgb[0], hem8=one[0].view(torch.uint8), labels=one[4], edt=one[5], n_objects=one[6, 0, :1],
+                                  feats=torch.zeros((8, 15), dtype=torch.float32, device=dev))])
+    enough = -(-2 * pipe.autotune_info()["recon_workers"] // 48)
+    n = {"one": 1, "just fewer": enough - 1, "just enough": enough, "more": enough + 28}[n]
     hem = torch.empty((n, H, W), dtype=torch.uint8, device=dev)
     lab = torch.full((n, H, W), -1, dtype=torch.int32, device=dev)
     edt = torch.empty((n, H, W), dtype=torch.int32, device=dev)

@@ -83,7 +83,7 @@ def test_argument_checks(pipe):
 @pytest.mark.parametrize("W,H,off", [(256, 129, 0), (133, 70, 0), (130, 33, 1), (127, 64, 3)])
 def test_every_radius(pipe, W, H, off, r):
     """Every radius has a pass of its own: strips of 128 columns and segments
-    of 32 rows just full, just over and just short; rows and planes that start
+    of 16 rows just full, just over and just short; rows and planes that start
     on no 4-byte boundary."""
     import torch
     rng = np.random.default_rng(r * 100 + W)
@@ -95,6 +95,19 @@ def test_every_radius(pipe, W, H, off, r):
     torch.cuda.synchronize()
     assert np.array_equal(dst.cpu().numpy(), oracle.morph_open(a, r))
     assert bool((buf[1, :off] == 7).all()) and bool((buf[1, off + H * W:] == 7).all())
+
+
+@pytest.mark.parametrize("r", [4, 9, 12, 15])
+def test_longer_segments(pipe, r):
+    """A plane so tall and wide that its segments have more than the least 16
+    rows (22 to 36 here), on bands of rows at its ends and between."""
+    rng = np.random.default_rng(r)
+    W, H = 385, 16384
+    a = rng.integers(0, 256, (H, W), dtype=np.uint8)
+    got = gpu_open(pipe, a, r)
+    for y0, y1 in ((0, 150), (H // 2, H // 2 + 150), (H - 150, H)):
+        a0, a1 = max(0, y0 - 2 * r), min(H, y1 + 2 * r)
+        assert np.array_equal(got[y0:y1], oracle.morph_open(a[a0:a1], r)[y0 - a0:y1 - a0]), (y0, y1)
 
 
 @pytest.mark.parametrize("W,H,off", [(256, 256, 1), (255, 256, 0), (253, 251, 3), (300, 218, 0), (3, 16384, 1)])
