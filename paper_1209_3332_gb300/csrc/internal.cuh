@@ -217,11 +217,10 @@ struct Profiler {
 // be seen, so that no access comes before it (what such a kernel reads through
 // __ldg lies behind a pointer that it loads from a descriptor first).  As every
 // kernel waits so before the next one may be prepared, completion is transitive.
-// The plain form launches its kernels so: 512^2, 270 -> 232 us; 4096^2, 610 -> 573;
-// 8192^2, 1272 -> 1236 us.  In a graph it changes nothing (1, 4 and 16 tiles of
-// 4096^2 per batch: 518, 1174 and 3856 us either way), and the two statements cost
-// kernels of many short blocks up to a fifth of their time, so that the batched
-// and the served forms do without (Launch::early).
+// The plain form launches its kernels so: 512^2, 233 -> 195 us; 1024^2, 250 -> 212;
+// 4096^2, 490 -> 458; 8192^2, 1054 -> 1029 us.  In a graph it gains nothing (1, 4 and
+// 16 tiles of 4096^2 per batch: 486, 1072 and 3515 us without, 486, 1087 and 3550
+// with), so that the batched and the served forms do without (Launch::early).
 template <typename... P>
 inline void launch_behind(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                           typename std::common_type<P>::type... args) {

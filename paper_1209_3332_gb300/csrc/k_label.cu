@@ -18,7 +18,7 @@
 //    instead of storing a full plane of provisional labels;
 //  * a warp's only large shared array is its 1024-entry union-find table
 //    (4 KB), whose root entries also carry a component's payload in bits
-//    16 and up, so that 48 such warps fit on an SM.
+//    16 and up, so that 32 (the fill) to 48 such warps fit on an SM.
 // Fill holes labels the background with 4-connectivity (dual of the 8-conn
 // foreground) and marks components that touch the image border; every
 // background pixel of an unmarked component is a hole.  Labelling then
