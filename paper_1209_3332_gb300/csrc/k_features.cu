@@ -81,11 +81,13 @@ constexpr int FW = 4;  // object warps per CTA
 constexpr int MANY_PX = 2816, MANY_CTAS = 8;
 constexpr int FEW_PX = 5120, FEW_CTAS = 5;
 constexpr int BANDS_PX = 1 << 20;  // a lane's share of 255^2 each is below 2^32
-// How an object's pixels are read and its whole numbers added: staged at once, or in
-// bands of rows (up to FEW_PX pixels), in 32 bits; staged in bands, in 64 bits; from
-// global memory, in 64 bits.  The paths are apart so that the common one has the
-// registers to itself: with bands in it, 167 us instead of 157 for the objects of 16
-// tiles of 4096^2.
+// How an object's pixels are read and its whole numbers added: up to FEW_PX pixels
+// staged, in 32 bits, in one piece or in bands of eight rows and more that are read
+// in full; in narrower bands that keep the two rows they share with the band
+// before, in 32 bits; in such bands, in 64 bits; from global memory, in 64 bits.
+// The last three are out of line: which code the common path shares its registers
+// with decides 5 to 10 % of it (objects of two sets of 16 tiles of 4096^2: 167 and
+// 160 us; 183 and 157 with no bands in the common path and the second kind inline).
 enum class Px { STAGED, BANDS, WIDE_BANDS, GLOBAL };
 constexpr int HOM_LCM = 408850;  // lcm of 1 + d^2 for d = 0..7
 
@@ -120,10 +122,12 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
         return;
     }
     const int bw = box.z - box.x + 1, bh = box.w - box.y + 1;
-    const long long npx = (long long)bw * bh;
+    using Idx = typename std::conditional<HOW != Px::GLOBAL, int, long long>::type;
+    const Idx npx = (Idx)bw * bh;
     const int rx0 = max(box.x - 1, 0), ry0 = max(box.y - 1, 0);
     const int rw = min(box.z + 1, W - 1) - rx0 + 1, rh = min(box.w + 1, H - 1) - ry0 + 1;
-    constexpr bool staged = HOW != Px::GLOBAL, bands = HOW == Px::BANDS || HOW == Px::WIDE_BANDS;
+    constexpr bool staged = HOW != Px::GLOBAL, keep = HOW == Px::BANDS || HOW == Px::WIDE_BANDS;
+    constexpr bool bands = keep || (HOW == Px::STAGED && STAGE_PX < FEW_PX);  // the region may not fit in one piece
     for (int i = lane; i < 4 * 64; i += 32) glcm[i] = 0;
     int sy0 = 0;  // first staged row
     // stages rows [from, to] of the region's columns from the buffer's pixel p0 on
@@ -164,15 +168,15 @@ __device__ __forceinline__ void object_features_impl(const ObjJob& J, int obj, i
     // lane walks the box row-major with stride 32, advancing (y, x) without divisions
     int y = box.y + lane / bw, x = box.x + lane % bw;
     // a band: box rows [yb, ye], staged with the rows beside them
-    const int band = bands ? STAGE_PX / rw - 2 : bh;
-    long long idx = lane;
+    const int band = !bands || rw * rh <= STAGE_PX ? bh : STAGE_PX / rw - 2;
+    Idx idx = lane;
     for (int yb = box.y; yb <= box.w; yb += band) {
     const int ye = bands ? min(yb + band - 1, box.w) : box.w;
     __syncwarp();
     if (staged) {
         const int from = max(yb - 1, 0);
         int p0 = 0;
-        if (bands && yb > box.y) {  // rows yb - 1 and yb are the last two staged for the band before
+        if (keep && yb > box.y) {  // rows yb - 1 and yb are the last two staged for the band before
             const int off = (from - sy0) * rw;
             for (int i = lane; i < ((2 * rw + 31) & ~31); i += 32) {
                 const uint16_t v = spx[off + min(i, 2 * rw - 1)];
@@ -329,10 +333,10 @@ __device__ __forceinline__ void object_features(const ObjJob& J, int obj, int* g
     const int4 box = J.bbox[obj];
     const int rx0 = max(box.x - 1, 0), ry0 = max(box.y - 1, 0);
     const long long rw = (long long)min(box.z + 1, J.W - 1) - rx0 + 1, rh = (long long)min(box.w + 1, J.H - 1) - ry0 + 1;
-    if (rw > 0 && rh > 0 && rw * rh <= STAGE_PX)
+    if (rw > 0 && rh > 0 && rw * rh <= FEW_PX && (rw * rh <= STAGE_PX || rw <= STAGE_PX / 10))
         object_features_impl<Px::STAGED, STAGE_PX>(J, obj, glcm, spx);
     else if (3 * rw <= STAGE_PX && rw * rh <= FEW_PX)
-        object_features_impl<Px::BANDS, STAGE_PX>(J, obj, glcm, spx);
+        object_features_large<Px::BANDS, STAGE_PX>(J, obj, glcm, spx);
     else if (3 * rw <= STAGE_PX && rw * rh <= BANDS_PX)
         object_features_large<Px::WIDE_BANDS, STAGE_PX>(J, obj, glcm, spx);
     else
