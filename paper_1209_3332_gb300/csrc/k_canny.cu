@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_canny_nms(const __grid_con
 // remembered in registers, the others as a bit of 64 (a hash where there are more
 // objects than bits), and only an object whose bit is taken is looked for at the
 // earlier disk offsets (1024^2 of noise with a label on every other pixel, disks
-// of radius 4 with 25 objects: 1047 us; 2350 with every object looked for).
+// of radius 4 with 25 objects: 1004 us; 2350 with every object looked for).
 // 8 tiles of 4096^2: 146 us (465 with a CTA per block, a thread per pixel and a
 // label read for every disk offset).  Bound: the latency of the label loads of
 // the blocks that hold edges (about half; seven of a lane in flight), 24 warps
