@@ -53,9 +53,11 @@ def snake_rgb(n):
     return rgb
 
 
-# Every call is one whose idle workers wait far longer than WAIT cycles for
-# work, or, of one work tile, one that is done long before.
-WAIT = 40000
+# Wait budgets in cycles that the idle workers of a large call exceed many times
+# and a call of one work tile does not: the growth of a long path takes milliseconds,
+# and its idle warps wait for one tile in the small call; the reconstruction of
+# one tile has one worker, which waits for nobody.
+WAIT = dict(canny=400000, rbc=400000, plain=300, batch=300, overflow=1 << 32)
 
 
 class Calls:
@@ -120,7 +122,7 @@ def test_status_outlives_the_calls_behind(late, then):
     """The status word holds the first error since it was last read, whatever
     runs between the call that failed and the read."""
     import paper_1209_3332_gb300 as P
-    pipe = P.Pipe(0, autotune=0, wait_budget_cycles=WAIT if late != "overflow" else 1 << 32)
+    pipe = P.Pipe(0, autotune=0, wait_budget_cycles=WAIT[late])
     c = Calls(pipe)
     tile = synth.tile(1024, 1024, 61, **NUCLEI)
     small = dict(canny=lambda: c.canny(BLANK[..., 0]), rbc=lambda: c.rbc(BLANK), plain=lambda: c.plain(BLANK),
